@@ -282,6 +282,13 @@ typedef struct gbt_sum_args {
 
 gbt_status gbt_sum(const gbt_trace_t *trace, const gbt_sum_args *args, void *stream);
 
+/* gbt_sum in F32 with the very beams, to their rounding, that gbt_sum_backward
+ * recomputes: the forward pass to take a loss of when its gradient follows (a
+ * gradient depends on the field's rounding through the loss).  Slower than
+ * gbt_sum, whose evaluation differs by rounding only.  GBT_ERR_INVALID_ARG for
+ * GBT_PRECISION_F64. */
+gbt_status gbt_sum_differentiable(const gbt_trace_t *trace, const gbt_sum_args *args, void *stream);
+
 /* Spatially coherent processing order of receivers (Morton order of their
  * positions quantised to their bounding box), written to order_out (device,
  * n_recv int32).  The order changes results only by rounding: each warp of 64

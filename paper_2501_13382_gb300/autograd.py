@@ -1,4 +1,4 @@
-"""torch.autograd.Function over gbt_sum / gbt_sum_backward.
+"""torch.autograd.Function over gbt_sum_differentiable / gbt_sum_backward.
 
     p = gbs_field(trace, recv, freqs, beam_b, gamma, ray_weight, ...)   # complex64 [F, Nr]
     loss = (p - target).abs().pow(2).sum(); loss.backward()
@@ -29,10 +29,11 @@ class GBTSum(torch.autograd.Function):
     def forward(ctx, gamma, ray_weight, beam_b, trace, recv, freqs, order, window, cutoff,
                 tile_cull=False, absorption=None, flow_resistivity=None):
         b = [float(v) for v in beam_b.detach().cpu().tolist()]
-        p = G.gbs_sum(trace, recv, list(freqs), b, gamma.detach().contiguous(),
-                      ray_weight=None if ray_weight is None else ray_weight.detach().contiguous(),
-                      order=order, window=window, cutoff=cutoff, tile_cull=tile_cull,
-                      absorption=absorption, flow_resistivity=flow_resistivity)
+        p = G.gbs_sum_differentiable(
+            trace, recv, list(freqs), b, gamma.detach().contiguous(),
+            ray_weight=None if ray_weight is None else ray_weight.detach().contiguous(),
+            order=order, window=window, cutoff=cutoff, tile_cull=tile_cull,
+            absorption=absorption, flow_resistivity=flow_resistivity)
         ctx.absorption, ctx.flow_resistivity = absorption, flow_resistivity
         ctx.save_for_backward(gamma, ray_weight if ray_weight is not None else torch.empty(0))
         ctx.has_w = ray_weight is not None

@@ -26,8 +26,13 @@ SOURCES = {
     "api.cu": [],
     "trace.cu": ["--fmad=false"],
     "gbs.cu": [],
+    "pair_fwd.cu": [],
+    "pair_field.cu": [],
+    "pair_bwd.cu": [],
+    "pair_batched.cu": [],
 }
-HEADERS = ["gbt_internal.h", "bvh_build.h"]
+HEADERS = ["gbt_internal.h", "bvh_build.h", "pair_common.cuh", "pair_stream.cuh",
+           "pair_exact.cuh", "pair.cuh"]
 
 
 def _nvcc():

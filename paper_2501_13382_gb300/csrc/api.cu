@@ -642,19 +642,32 @@ gbt_status gbt_trace_destroy(gbt_trace_t *trace)
     });
 }
 
-gbt_status gbt_sum(const gbt_trace_t *trace, const gbt_sum_args *args, void *stream)
+static gbt_status sum_call(const char *name, const gbt_trace_t *trace, const gbt_sum_args *args,
+                           void *stream, bool differentiable)
 {
-    NvtxRange nvtx_range("gbt_sum");
+    NvtxRange nvtx_range(name);
     return guarded([&] {
         validate_sum(trace, args);
+        if (differentiable)
+            GBT_REQUIRE(args->precision == GBT_PRECISION_F32, "differentiable sums are F32 only");
         cudaStream_t s = static_cast<cudaStream_t>(stream);
         gbt_trace_t *tr = const_cast<gbt_trace_t *>(trace);
         const SceneDev &sd = tr->d.scene->d;
         const int splits = choose_splits(tr->d, *args);
         void *w = tr->d.work.ensure(sum_workspace_bytes(tr->d, *args, splits), s);
-        sum_launch(tr->d, sd, *args, splits, w, s);
+        sum_launch(tr->d, sd, *args, splits, w, s, nullptr, differentiable);
         mark_trace_used(tr, s);
     });
+}
+
+gbt_status gbt_sum(const gbt_trace_t *trace, const gbt_sum_args *args, void *stream)
+{
+    return sum_call("gbt_sum", trace, args, stream, false);
+}
+
+gbt_status gbt_sum_differentiable(const gbt_trace_t *trace, const gbt_sum_args *args, void *stream)
+{
+    return sum_call("gbt_sum_differentiable", trace, args, stream, true);
 }
 
 gbt_status gbt_synthesize(const float *p, int32_t n_freq, int64_t n_recv, const double *freq_hz,

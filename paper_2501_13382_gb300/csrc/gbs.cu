@@ -1,38 +1,16 @@
-// gbs.cu -- Gaussian beam summation (Eq. 3 with the beam of Eq. 1 / Eq. 2)
-// for every (receiver, segment, frequency) triple, its adjoint, and the
-// receiver order they use.
+// gbs.cu -- everything around the pair kernel (pair.cuh): the prepass of traced segments
+// into kernel records, the tile order and the pre-cull's segment lists, the counting pass,
+// the all-FP64 path, the merge of partial sums, the adjoint's per-ray map, batches, time
+// synthesis and the receiver order.
 //
-// GB300 design of the FP32 pair kernel:
-//  * A prepass turns every traced segment into an 80-byte record (origin and
-//    start distance as float-float, direction, length, amplitude).
-//  * Receivers are visited in Morton order, in warp tiles of 64 (two per lane:
-//    receivers lane and lane + 32) held in registers, absolute (exact path) and
-//    relative to the warp tile's first receiver (prefilter).
-//  * Persistent CTAs of 16 warps, and every warp works on its own: it takes
-//    (warp tile, segment split) items from a global queue, split s owning record
-//    batches s, s + splits, ...  CTA tiles of 15 warp tiles are dispatched
-//    heaviest first and splits are sized for about 16 items per warp, so no warp
-//    waits for another and the queue drains on short items.
-//  * A warp double-buffers its own 32-record batches (a bulk asynchronous copy
-//    completed on a per-warp mbarrier, or per-lane cp.async gathers from the
-//    tile's segment list with the pre-cull) and stages each batch itself.  Every
-//    wait is bounded and raises a status flag instead of hanging.
-//  * Prefilter (every pair, frequency independent): a paired FP32 (f32x2)
-//    evaluation of the union of the per-frequency Gaussian cutoffs and the
-//    window, conservative by a margin, gives one keep bit per pair.  With the
-//    pre-cull, per-tile segment lists with per-entry warp-tile masks and a
-//    per-warp ball test skip segments that can reach none of its receivers.
-//  * Survivors (typically a few percent of pairs) are evaluated exactly, the two
-//    receivers of a lane side by side in paired FP32, in the warp's frame: the
-//    staging forms per segment, relative to the warp tile's first receiver c,
-//    A = (c - o).t and S = s0 + A in float-float and the compensated
-//    N = (c - o) x t, so a receiver at c + x' needs only x'.t (float-float) and
-//    N + x' x t; then float-float s and phase (reduced in turns before the MUFU
-//    sin/cos).  FP32 sums per lane fold into the item's float-float partials every 16
-//    batches, and the per-split partials are merged in float-float (error-free
-//    FP32 sums) in a fixed order by a second kernel, so results do not depend on
-//    scheduling.
-//  * The kernel holds the sums of up to 8 frequencies in registers; more (up to 16)
+//  * A prepass turns every traced segment into an 80-byte record (origin, start distance,
+//    direction and length as float-float, amplitude) and a 32-byte cull record.
+//  * Receivers are visited in Morton order, in warp tiles of 64; CTA tiles of 15 warp tiles
+//    are dispatched heaviest first, with segment splits sized so that the queue drains on
+//    short items.
+//  * The per-split partials are merged in float-float (error-free FP32 sums) in a fixed
+//    order, so results do not depend on scheduling.
+//  * The pair kernel holds the sums of up to 8 frequencies in registers; more (up to 16)
 //    run as one launch per group of 8, each with its own partials and output rows.
 
 #include <math.h>
@@ -44,387 +22,25 @@
 #include <cmath>
 #include <string>
 
-#include "gbt_internal.h"
+#include "pair_exact.cuh"
 
 namespace gbt {
 namespace {
 
-constexpr int kWarpsFwd = 16;               // warps per CTA of the pair kernel (one CTA per SM)
-constexpr size_t kSmemBudget = 227 * 1024;  // dynamic shared memory of one pair-kernel CTA (the maximum)
-constexpr int kWRaw = 2;                    // raw record buffers per warp (double buffering)
-constexpr int kR = 2;                       // receivers per lane
-constexpr int kWarpRecv = 32 * kR;          // receivers per warp tile
-constexpr int kTileWarps = 15;              // warp tiles per CTA tile (dispatch order, lists)
-constexpr int kChunkWords = 16;             // warp-tile words per 32-entry chunk of a tile list
-constexpr int kCtaRecv = kTileWarps * kWarpRecv;
-constexpr int kBatch = 32;                  // segments per staged batch
-constexpr long long kSpinLimit = 1LL << 22; // bounded mbarrier waits
-enum { kFwd = 0, kStats = 1, kBwd = 2 };    // what the pair kernel does with survivors
-constexpr int kFoldEvery = 16;              // batches between float-float folds
-constexpr float kWinMargin = 0.01f;         // prefilter window slack (m)
-// A warp item takes the FP32 local projection x'.t (instead of float-float) when
-// K_max max|x'| <= kFastTurns.  Its rounding, at most about 3 ulp of |x'|, moves a term's
-// phase by at most 3 x 2^-24 x 90 turns = 1.0e-4 rad; the roundings of different terms are
-// independent, so the field moves far less (2e-7 relative on the city, 3.5e-5 with the
-// projection in FP32 everywhere at 4 kHz).  The window test is a hard cutoff, so a pair
-// within the FP32 projection's error bound of an end of its window is decided and
-// evaluated with the float-float projection.  On that path n = N + x' x t also leaves out
-// the products of the lo parts (about 1.3 ulp of |x'|; with |n| <= s the phase moves by
-// at most K x 1.3 ulp(|x'|) <= 9e-5 rad).  Past the limit the float-float products stay.
-constexpr float kFastTurns = 90.0f;
+// ------------------------------------------------------ counting pass --
+// Every pair (or, with the pre-cull, every pair of the segments that reach a warp tile)
+// goes through a paired FP32 prefilter, the union of the bands' cutoffs and the window with
+// a margin, and the survivors through the exact test in float-float (pair_exact.cuh); only
+// counts come out (gbt_sum_stats_get).
 
-// Per-frequency constants, grouped in 16-byte words in the order the survivor
-// path needs them (cutoff test, then the beam), so a kernel that reads them from
-// shared memory (the batched launch) needs two vector loads per kept frequency.
-struct alignas(16) FreqConst {
-    float kb2;            // k b / 2  (Gaussian exponent factor)
-    float b2;             // b^2
-    float K_hi, K_lo;     // f / c in turns per metre, float-float
-    float halfK;          // K / 2: second phase term K n^2 s / (2 D) in turns
-    float kb2l2e;         // k b / 2 * log2(e)
-    float scale;          // k b / (8 pi^2)
-    float b;              // b
-    float kh, invb;       // k / 2, 1 / b  (adjoint)
-    float al2e;           // amplitude decay rate of air a (Np/m) * log2(e), 0 when lossless
-    float pad1;
-};
-static_assert(sizeof(FreqConst) == 48, "three 16-byte words");
-
-struct alignas(16) FwdParams {
-    const float *recv;
-    const int32_t *order;
-    int64_t n_recv;
-    const int32_t *n_seg_ptr;
-    const float *rec;          // AoS records, kRecFloats per segment
-    const float4 *crec;        // cull records: (o_hi, s0_hi), (t_hi, L_hi) per segment
-    int nf;
-    int uniform_b;             // all b equal: frequencies sorted by k, loop stops at first cull
-    int tile_cull;             // skip segments that reach none of a warp's receivers
-    float cutoff;
-    float pre_alpha, pre_beta; // prefilter: keep iff alpha n^2 <= s^2 + beta
-    float kmax_turns;          // largest f / c of the launch's frequencies, turns per metre
-    int splits;
-    int64_t n_items;           // CTA tiles x splits
-    int *work_counter;         // zeroed before launch; CTAs take items from it
-    const int32_t *tile_perm;  // dispatch rank -> CTA tile (heaviest first), or null
-    // tile pre-cull: per CTA tile, the segments whose beams can reach its receivers
-    const int32_t *list;       // segment indices, each tile's in segment order, or null
-    const int64_t *list_off;   // per tile: first entry in list
-    const int32_t *list_n;     // per tile: entries, or -1 (no list: stream every segment)
-    // per 32-entry chunk of a tile's list (every list starts on a chunk boundary), one
-    // word per warp tile w: bit b set if entry b of the chunk can reach warp tile w
-    const uint32_t *list_words;
-    float4 *partial;           // [splits][nf][n_recv]: re_hi, im_hi, re_lo, im_lo
-    unsigned long long *stats; // counting mode when non-null: [1] prefiltered, [2] kept
-    unsigned int *status;      // device status word (timeouts)
-    // adjoint mode
-    const float2 *grad_out;    // g = dL/dRe p + i dL/dIm p, [user frequency][n_recv]
-    float *seg_G;              // per segment: sum over (r, f) of Re(conj(g) c~)
-    float *seg_H;              // per (sorted frequency, segment): sum over r of Re(conj(g) dc~/db)
-    int64_t seg_stride;        // stride of seg_H rows
-    int fperm[GBT_MAX_FREQ];   // sorted frequency slot -> user frequency index
-    // losses of porous surfaces (lossy instantiation): per user frequency f and segment j,
-    // seg_rf[f * rf_stride + j] = (log2 |R|, arg R / 2 pi) of the path's reflection factor
-    const float2 *seg_rf;
-    int64_t rf_stride;
-    // batched launch: per-instance parameters and the first global item of each
-    const struct FwdParams *inst;
-    const int64_t *inst_off;   // n_inst + 1 entries
-    int n_inst;
-    FreqConst fc[GBT_MAX_FREQ];
-};
-
-static_assert(sizeof(FwdParams) % 16 == 0, "instance parameters are copied as 16-byte words");
-
-// Error-free transformations depend on every operation being rounded as written:
-// nvcc contracts a product feeding an add into one FMA by default, which would
-// round differently in each inlined copy.  The __f*_rn intrinsics are never
-// contracted, so these sites use them wherever a rounding is relied upon.
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
-{
-    s = __fadd_rn(a, b);
-    const float bv = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bv)), __fsub_rn(b, bv));
-}
-
-__device__ __forceinline__ float rcp_approx(float x)
-{
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
-__device__ __forceinline__ float ex2_approx(float x)
-{
-    float r;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
-// Kahan's difference of products a*b - c*d, accurate to about one ulp.
-__device__ __forceinline__ float dop(float a, float b, float c, float d)
-{
-    const float w = __fmul_rn(c, d);
-    const float e = fmaf(-c, d, w);
-    const float f = fmaf(a, b, -w);
-    return f + e;
-}
-
-typedef unsigned long long f2x;   // two packed floats (lo = receiver 0, hi = receiver 1)
-__device__ __forceinline__ f2x pk(float a, float b)
-{
-    f2x r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void upk(f2x v, float &a, float &b)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ f2x fma2(f2x a, f2x b, f2x c)
-{
-    f2x r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ f2x add2(f2x a, f2x b)
-{
-    f2x r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f2x sub2(f2x a, f2x b)
-{
-    f2x r;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f2x mul2(f2x a, f2x b)
-{
-    f2x r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f2x neg2(f2x a) { return mul2(a, 0xbf800000bf800000ull); }
-__device__ __forceinline__ f2x splat(float a) { return pk(a, a); }
-// two_sum on both halves; the paired operations round each half exactly like the
-// scalar ones, so both paths give identical results
-__device__ __forceinline__ void two_sum2(f2x a, f2x b, f2x &s, f2x &e)
-{
-    s = add2(a, b);
-    const f2x bv = sub2(s, a);
-    e = add2(sub2(a, sub2(s, bv)), sub2(b, bv));
-}
-__device__ __forceinline__ f2x rint2(f2x a)
-{
-    float x, y;
-    upk(a, x, y);
-    return pk(rintf(x), rintf(y));
-}
-
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem, int src_bytes)
-{
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa), "l"(gmem),
-                 "r"(src_bytes));
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n"); }
-__device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;\n"); }
-__device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;\n"); }
-
-
-__device__ __forceinline__ uint32_t smem_addr(const void *p)
-{
-    return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes)
-{
-    asm volatile("{\n .reg .b64 st;\n mbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n}\n"
-                 ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-                 " selp.u32 %0, 1, 0, p;\n}\n"
-                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    return ok != 0;
-}
-// Bulk copy (TMA) of `bytes` contiguous bytes into shared memory, completing on `bar`.
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
-                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
-}
-
-// Bounded wait: true when the phase of `parity` completed; false on abort or
-// when the iteration limit ran out (then the device status word is flagged).
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag,
-                                          unsigned int *status)
-{
-    for (long long it = 0; it < kSpinLimit; ++it) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if (*abort_flag) return false;
-    }
-    atomicOr(status, STATUS_TIMEOUT);
-    *abort_flag = 1;
-    return false;
-}
-
-// One staged batch of a warp: the prefilter (hot) view relative to the warp
-// tile's first receiver c and the exact-path view in the same frame.  With
-// d = c - o (float-float) the exact view holds, per segment, A = d.t and
-// S = s0 + A as float-float pairs, AL = A - L (the segment window), the
-// compensated N = d x t and the direction as (hi, lo), so that for a receiver
-// at x = c + x' the pair needs only x'.t and x' x t:
-//   s_loc = A + x'.t,  s = S + x'.t,  n = N + x' x t.
-struct StageSmem {
-    float4 O[kBatch];               // o' = o - c, s0_hi (per-warp ball test)
-    // prefilter constants, each duplicated into both halves of a float pair:
-    // P[0] = t_z, -o'.t;  P[1..2] = 2a o'_x, 2a o'_y, 2a o'_z, beta - a |o'|^2;
-    // P[3] = s0 + margin, L + margin;  P[4] = t_x, t_y (as D[0]: the prefilter reads its
-    // own copy, which measured 6 % faster testing every pair than sharing D[0])
-    float4 P[kBatch][5];
-    // exact-path view, two values per word, each duplicated into both halves of a float
-    // pair (a lane evaluating one segment for its two receivers loads its operands as
-    // pairs); component-major, so lanes loading different segments hit different banks:
-    // D[0] t_hi.x, t_hi.y | D[1] t_hi.z, S_hi | D[2] t_lo.x, t_lo.y | D[3] t_lo.z, S_lo
-    // D[4] N.x, N.y | D[5] N.z, W Gamma_path | D[6] A_hi, A_lo | D[7] AL_hi, AL_lo
-    float4 D[8][kBatch];
-    int32_t seg[kBatch];            // global segment index of each staged record
-};
-
-// Losses of the staged batch (lossy instantiation): per frequency slot and staged
-// segment, log2 |R| and arg R / 2 pi of its porous reflections' factor.
-template <int NF>
-struct LossSmem {
-    float2 rf[NF][kBatch];
-};
-
-// Exact geometry of one (receiver, segment) pair in the warp tile's frame, in
-// float-float: x' = (xh + xl) exactly; returns false when the pair falls outside
-// the window.  `fast`: the warp item's choice of the FP32 local projection, within eps
-// of x'.t; a pair within eps of an end of its window is decided and evaluated with the
-// float-float projection instead, so the window test is as exact as on that path.  The
-// paired twin in survivor_pair rounds each half identically, except that it switches a
-// whole pair to the float-float projection when either half is near a window end (the
-// other half's value then differs by at most the FP32 projection's error, and its window
-// decision is the same).
-template <int WINDOW>
-__device__ __forceinline__ bool frame_geometry(float xh, float yh, float zh, float xl, float yl,
-                                               float zl, const StageSmem &w, int j, bool fast,
-                                               float eps, float &sh, float &sl, float &n2)
-{
-    const float4 d0 = w.D[0][j], d1 = w.D[1][j], d2 = w.D[2][j], d3 = w.D[3][j];
-    const float4 d4 = w.D[4][j], d5 = w.D[5][j];
-    const float4 T = make_float4(d0.x, d0.z, d1.x, d1.z), TL = make_float4(d2.x, d2.z, d3.x, d3.z);
-    const float4 NN = make_float4(d4.x, d4.z, d5.x, d5.z);
-    // u = x'.t as (U + ul)
-    float U, ul;
-    auto exact_u = [&]() {
-        const float p0 = __fmul_rn(xh, T.x), p1 = __fmul_rn(yh, T.y), p2 = __fmul_rn(zh, T.z);
-        const float r0 = fmaf(xh, TL.x, fmaf(xl, T.x, fmaf(xh, T.x, -p0)));
-        const float r1 = fmaf(yh, TL.y, fmaf(yl, T.y, fmaf(yh, T.y, -p1)));
-        const float r2 = fmaf(zh, TL.z, fmaf(zl, T.z, fmaf(zh, T.z, -p2)));
-        float S1, E1, E2;
-        two_sum(p0, p1, S1, E1);
-        two_sum(S1, p2, U, E2);
-        ul = __fadd_rn(__fadd_rn(E1, E2), __fadd_rn(__fadd_rn(r0, r1), r2));
-    };
-    if (fast) {
-        U = fmaf(xh, T.x, fmaf(yh, T.y, __fmul_rn(zh, T.z)));
-        ul = fmaf(xl, T.x, fmaf(yl, T.y, fmaf(zl, T.z, fmaf(xh, TL.x, fmaf(yh, TL.y, __fmul_rn(zh, TL.z))))));
-    } else {
-        exact_u();
-    }
-    if (WINDOW == GBT_WINDOW_SEGMENT) {
-        const float4 d6 = w.D[6][j], d7 = w.D[7][j];
-        float wa = __fadd_rn(__fadd_rn(d6.x, U), __fadd_rn(d6.z, ul));
-        float wb = __fadd_rn(__fadd_rn(d7.x, U), __fadd_rn(d7.z, ul));
-        if (fast && fminf(fabsf(wa), fabsf(wb)) <= eps) {
-            fast = false;
-            exact_u();
-            wa = __fadd_rn(__fadd_rn(d6.x, U), __fadd_rn(d6.z, ul));
-            wb = __fadd_rn(__fadd_rn(d7.x, U), __fadd_rn(d7.z, ul));
-        }
-        if (!(wa >= 0.0f)) return false;
-        if (!(wb < 0.0f)) return false;
-    }
-    float e3;
-    two_sum(T.w, U, sh, e3);
-    sl = __fadd_rn(e3, __fadd_rn(ul, TL.w));
-    if (WINDOW == GBT_WINDOW_LINE) {
-        float ss = __fadd_rn(sh, sl);
-        if (fast && fabsf(ss) <= eps) {
-            fast = false;
-            exact_u();
-            two_sum(T.w, U, sh, e3);
-            sl = __fadd_rn(e3, __fadd_rn(ul, TL.w));
-            ss = __fadd_rn(sh, sl);
-        }
-        if (!(ss >= 0.0f)) return false;
-    }
-    // n = N + x' x t: the small terms first (float-float projection only), then the
-    // main products
-    float n0x = NN.x, n0y = NN.y, n0z = NN.z;
-    if (!fast) {
-        n0x = __fadd_rn(n0x, fmaf(yl, T.z, fmaf(-zl, T.y, fmaf(yh, TL.z, __fmul_rn(-zh, TL.y)))));
-        n0y = __fadd_rn(n0y, fmaf(zl, T.x, fmaf(-xl, T.z, fmaf(zh, TL.x, __fmul_rn(-xh, TL.z)))));
-        n0z = __fadd_rn(n0z, fmaf(xl, T.y, fmaf(-yl, T.x, fmaf(xh, TL.y, __fmul_rn(-yh, TL.x)))));
-    }
-    const float nx = fmaf(yh, T.z, fmaf(-zh, T.y, n0x));
-    const float ny = fmaf(zh, T.x, fmaf(-xh, T.z, n0y));
-    const float nz = fmaf(xh, T.y, fmaf(-yh, T.x, n0z));
-    n2 = fmaf(nx, nx, fmaf(ny, ny, __fmul_rn(nz, nz)));
-    return true;
-}
-
-// Adjoint terms of one beam: with c~ the contribution without W Gamma_path,
-// G += Re(conj(g) c~) and H += Re(conj(g) dc~/db), where
-// d log c / db = 1/b + i/E - k n^2 / (2 E^2), E = s - i b.  With losses c~ carries
-// the porous reflections' factor (rf: log2 |R|, arg R in turns) and exp(-a s); neither
-// depends on b, so the logarithmic derivative is the same.
-template <bool LOSSY>
-__device__ __forceinline__ void beam_adjoint(const FreqConst &q, float sh, float sl, float n2,
-                                             float invD, float2 g, float &G, float &H,
-                                             float2 rf = make_float2(0.f, 0.f))
-{
-    const float n2invD = n2 * invD;
-    float ex = -q.kb2l2e * n2invD;
-    if (LOSSY) ex = fmaf(-q.al2e, sh, ex + rf.x);
-    const float ga = ex2_approx(ex);
-    const float ph = __fmul_rn(q.K_hi, sh);       // rounded: pe below is its exact error
-    const float pe = fmaf(q.K_hi, sh, -ph);
-    const float corr = fmaf(q.K_hi, sl, fmaf(q.K_lo, sh, pe));
-    float tau = __fsub_rn(ph, rintf(ph)) + corr;
-    tau = fmaf(q.halfK * n2invD, sh, tau);
-    if (LOSSY) tau += rf.y;
-    tau = tau - rintf(tau);
-    float sn, cs;
-    __sincosf(6.283185307179586f * tau, &sn, &cs);
-    const float gs = q.scale * ga * invD;
-    const float cr = gs * fmaf(sh, cs, -q.b * sn);
-    const float ci = gs * fmaf(sh, sn, q.b * cs);
-    G = fmaf(g.x, cr, fmaf(g.y, ci, G));
-    const float t = q.kh * n2 * invD * invD;                         // k n^2 / (2 D^2)
-    const float dr = q.invb - q.b * invD - t * (sh * sh - q.b2);      // Re d log c / db
-    const float di = sh * invD - t * (2.0f * sh * q.b);               // Im d log c / db
-    H = fmaf(g.x, cr * dr - ci * di, fmaf(g.y, cr * di + ci * dr, H));
-}
-
-// Counting pass: the kept (pair, frequency) triples of one surviving pair, with
-// the same geometry and cutoff arithmetic as the forward path.
+// The kept (pair, frequency) triples of one surviving pair.
 template <int NF, int WINDOW>
 __device__ __forceinline__ void survivor_count(const FwdParams &p, float xh, float yh, float zh,
                                                float xl, float yl, float zl, const StageSmem &w,
-                                               int j, bool fast, float eps, uint32_t &kept)
+                                               int j, uint32_t &kept)
 {
     float sh, sl, n2;
-    if (!frame_geometry<WINDOW>(xh, yh, zh, xl, yl, zl, w, j, fast, eps, sh, sl, n2)) return;
+    if (!frame_geometry<WINDOW>(xh, yh, zh, xl, yl, zl, w, j, false, 0.f, sh, sl, n2)) return;
     if (p.uniform_b) {
         const float D = fmaf(sh, sh, p.fc[0].b2);
         const float r = n2 * rcp_approx(D);
@@ -445,400 +61,29 @@ __device__ __forceinline__ void survivor_count(const FwdParams &p, float xh, flo
     }
 }
 
-// Two surviving pairs at once in paired FP32: receiver 0 of the lane with
-// segment j0 and receiver 1 with segment j1 (a side without a survivor repeats
-// the other side's segment and is masked out).  Every operation is the paired
-// twin of one pair's evaluation (frame_geometry, then per frequency the Gaussian,
-// the phase reduced in turns and the 1/E factor), so each half rounds as that
-// evaluation would; only the MUFU operations run per half.  accx / accy
-// hold the two receivers' real / imaginary sums per sorted frequency.
-// Two staged words of segments j0 (lo half) and j1 (hi half) as float pairs; with one
-// segment for both halves (SAME) the duplicated word is the pair itself.
-template <bool SAME>
-__device__ __forceinline__ void ld_pairs(const float4 &a, const float4 &b, f2x &u, f2x &v)
-{
-    if (SAME) {
-        const ulonglong2 q = *reinterpret_cast<const ulonglong2 *>(&a);
-        u = q.x;
-        v = q.y;
-    } else {
-        const float4 qa = a, qb = b;
-        u = pk(qa.x, qb.x);
-        v = pk(qa.z, qb.z);
-    }
-}
-
-template <int NF, int WINDOW, bool LOSSY, bool SAME = false>
-__device__ __forceinline__ void survivor_pair(const FwdParams &p, f2x XH, f2x YH, f2x ZH,
-                                              f2x XL, f2x YL, f2x ZL, f2x NXH, f2x NYH, f2x NZH,
-                                              const StageSmem &w,
-                                              const LossSmem<NF> *loss, int j0, int j1, bool h0,
-                                              bool h1, bool fast, float eps, f2x (&accx)[NF],
-                                              f2x (&accy)[NF])
-{
-    f2x THX, THY, THZ, SH, TLX, TLY, TLZ, SL, NX0, NY0, NZ0, AMP;
-    ld_pairs<SAME>(w.D[0][j0], w.D[0][j1], THX, THY);
-    ld_pairs<SAME>(w.D[1][j0], w.D[1][j1], THZ, SH);
-    ld_pairs<SAME>(w.D[2][j0], w.D[2][j1], TLX, TLY);
-    ld_pairs<SAME>(w.D[3][j0], w.D[3][j1], TLZ, SL);
-    // u = x'.t as (U + ul): float-float, or (warp-uniform `fast`, compact warps at low
-    // enough frequencies) the FP32 products with the lo parts' first-order terms, within
-    // eps of x'.t.  A pair with a live half within eps of an end of its window takes the
-    // float-float projection instead (`exact`), so every window decision is as exact as
-    // on that path (frame_geometry does the same for one pair).
-    f2x U, ul;
-    f2x AH, AL, BH, BL;
-    if (WINDOW == GBT_WINDOW_SEGMENT) {
-        ld_pairs<SAME>(w.D[6][j0], w.D[6][j1], AH, AL);
-        ld_pairs<SAME>(w.D[7][j0], w.D[7][j1], BH, BL);
-    }
-    bool exact = !fast;
-    if (fast) {
-        U = fma2(XH, THX, fma2(YH, THY, mul2(ZH, THZ)));
-        ul = fma2(XL, THX, fma2(YL, THY, fma2(ZL, THZ, fma2(XH, TLX, fma2(YH, TLY, mul2(ZH, TLZ))))));
-        float a0, a1, b0, b1;
-        if (WINDOW == GBT_WINDOW_SEGMENT) {
-            upk(add2(add2(AH, U), add2(AL, ul)), a0, a1);
-            upk(add2(add2(BH, U), add2(BL, ul)), b0, b1);
-        } else {
-            upk(add2(add2(SH, U), add2(SL, ul)), a0, a1);   // s, near 0 exact as the sum
-            b0 = a0;
-            b1 = a1;
-        }
-        exact = (h0 && fminf(fabsf(a0), fabsf(b0)) <= eps) || (h1 && fminf(fabsf(a1), fabsf(b1)) <= eps);
-    }
-    if (exact) {
-        const f2x p0 = mul2(XH, THX), p1 = mul2(YH, THY), p2 = mul2(ZH, THZ);
-        const f2x r0 = fma2(XH, TLX, fma2(XL, THX, fma2(XH, THX, neg2(p0))));
-        const f2x r1 = fma2(YH, TLY, fma2(YL, THY, fma2(YH, THY, neg2(p1))));
-        const f2x r2 = fma2(ZH, TLZ, fma2(ZL, THZ, fma2(ZH, THZ, neg2(p2))));
-        f2x S1, E1, E2;
-        two_sum2(p0, p1, S1, E1);
-        two_sum2(S1, p2, U, E2);
-        ul = add2(add2(E1, E2), add2(add2(r0, r1), r2));
-    }
-    bool k0 = h0, k1 = h1;
-    float u0, u1;
-    if (WINDOW == GBT_WINDOW_SEGMENT) {
-        upk(add2(add2(AH, U), add2(AL, ul)), u0, u1);
-        k0 = k0 && u0 >= 0.0f;
-        k1 = k1 && u1 >= 0.0f;
-        upk(add2(add2(BH, U), add2(BL, ul)), u0, u1);
-        k0 = k0 && u0 < 0.0f;
-        k1 = k1 && u1 < 0.0f;
-    }
-    f2x sh, e3;
-    two_sum2(SH, U, sh, e3);
-    const f2x sl = add2(e3, add2(ul, SL));
-    if (WINDOW == GBT_WINDOW_LINE) {
-        upk(add2(sh, sl), u0, u1);
-        k0 = k0 && u0 >= 0.0f;
-        k1 = k1 && u1 >= 0.0f;
-    }
-    if (!(k0 || k1)) return;
-    ld_pairs<SAME>(w.D[4][j0], w.D[4][j1], NX0, NY0);
-    ld_pairs<SAME>(w.D[5][j0], w.D[5][j1], NZ0, AMP);
-    // n = N + x' x t; the lo parts' products (about 1.3 ulp of |x'|) only where the
-    // projection is float-float: on the FP32 path they are below its own rounding
-    f2x n0x = NX0, n0y = NY0, n0z = NZ0;
-    if (exact) {
-        n0x = add2(n0x, fma2(YL, THZ, fma2(neg2(ZL), THY, fma2(YH, TLZ, mul2(neg2(ZH), TLY)))));
-        n0y = add2(n0y, fma2(ZL, THX, fma2(neg2(XL), THZ, fma2(ZH, TLX, mul2(neg2(XH), TLZ)))));
-        n0z = add2(n0z, fma2(XL, THY, fma2(neg2(YL), THX, fma2(XH, TLY, mul2(neg2(YH), TLX)))));
-    }
-    const f2x nx = fma2(YH, THZ, fma2(NZH, THY, n0x));
-    const f2x ny = fma2(ZH, THX, fma2(NXH, THZ, n0y));
-    const f2x nz = fma2(XH, THY, fma2(NYH, THX, n0z));
-    const f2x n2 = fma2(nx, nx, fma2(ny, ny, mul2(nz, nz)));
-    const f2x amp = AMP;
-    float n20, n21;
-    upk(n2, n20, n21);
-
-    // one beam term on both halves, each half kept where its flag is set; with losses
-    // the Gaussian exponent takes log2 |R| - a s log2(e) and the phase arg R / 2 pi
-    auto beam = [&](const FreqConst &q, int f, f2x invD, bool kf0, bool kf1, f2x &bx, f2x &by) {
-        const f2x n2invD = mul2(n2, invD);
-        float e0, e1;
-        f2x ex = mul2(splat(-q.kb2l2e), n2invD);
-        f2x RPH = 0ull;
-        if (LOSSY) {
-            const float2 r0 = loss->rf[f][j0], r1 = loss->rf[f][j1];
-            ex = fma2(splat(-q.al2e), sh, add2(ex, pk(r0.x, r1.x)));
-            RPH = pk(r0.y, r1.y);
-        }
-        upk(ex, e0, e1);
-        const f2x ga = pk(ex2_approx(e0), ex2_approx(e1));
-        const f2x KH = splat(q.K_hi);
-        const f2x nph = mul2(splat(-q.K_hi), sh);    // -K_hi sh, exactly
-        const f2x pe = fma2(KH, sh, nph);
-        const f2x corr = fma2(KH, sl, fma2(splat(q.K_lo), sh, pe));
-        f2x tau = add2(sub2(rint2(nph), nph), corr);   // = ph - rint(ph)
-        tau = fma2(mul2(splat(q.halfK), n2invD), sh, tau);
-        if (LOSSY) tau = add2(tau, RPH);
-        // |tau| < 2^22 turns (beyond it FP32 holds no phase): round by 1.5 x 2^23
-        tau = sub2(tau, sub2(add2(tau, splat(12582912.0f)), splat(12582912.0f)));
-        float t0, t1, s0, c0, s1, c1;
-        upk(mul2(splat(6.283185307179586f), tau), t0, t1);
-        __sincosf(t0, &s0, &c0);
-        __sincosf(t1, &s1, &c1);
-        const f2x SN = pk(s0, s1), CS = pk(c0, c1);
-        const f2x gg = mul2(mul2(mul2(mul2(splat(q.scale), amp), ga), invD),
-                            pk(kf0 ? 1.0f : 0.0f, kf1 ? 1.0f : 0.0f));
-        const f2x B = splat(q.b);
-        bx = fma2(gg, fma2(sh, CS, mul2(splat(-q.b), SN)), bx);
-        by = fma2(gg, fma2(sh, SN, mul2(B, CS)), by);
-    };
-    if (p.uniform_b) {
-        // one b for all frequencies, sorted by k: each half keeps a prefix
-        float d0, d1;
-        upk(fma2(sh, sh, splat(p.fc[0].b2)), d0, d1);
-        const f2x invD = pk(rcp_approx(d0), rcp_approx(d1));
-        float r0_, r1_;
-        upk(mul2(n2, invD), r0_, r1_);
-#pragma unroll
-        for (int f = 0; f < NF; ++f) {
-            if (f >= p.nf) break;
-            const FreqConst &q = p.fc[f];
-            k0 = k0 && !(q.kb2 * r0_ > p.cutoff);
-            k1 = k1 && !(q.kb2 * r1_ > p.cutoff);
-            if (!(k0 || k1)) break;
-            beam(q, f, invD, k0, k1, accx[f], accy[f]);
-        }
-    } else {
-#pragma unroll
-        for (int f = 0; f < NF; ++f) {
-            if (f >= p.nf) break;
-            const FreqConst &q = p.fc[f];
-            float d0, d1;
-            upk(fma2(sh, sh, splat(q.b2)), d0, d1);
-            const bool kf0 = k0 && !(q.kb2 * n20 > p.cutoff * d0);
-            const bool kf1 = k1 && !(q.kb2 * n21 > p.cutoff * d1);
-            if (!(kf0 || kf1)) continue;
-            beam(q, f, pk(rcp_approx(d0), rcp_approx(d1)), kf0, kf1, accx[f], accy[f]);
-        }
-    }
-}
-
-// Adjoint terms of one surviving pair added into G and H[f] (gk: this receiver's
-// g per sorted frequency, stride kR * 32 float2).
-template <int NF, int WINDOW, bool LOSSY>
-__device__ __forceinline__ void survivor_adjoint(const FwdParams &p, float xh, float yh, float zh,
-                                                 float xl, float yl, float zl, const StageSmem &w,
-                                                 const LossSmem<NF> *loss, int j, bool fast,
-                                                 float eps, const float2 *gk, float &G,
-                                                 float (&H)[NF])
-{
-    float sh, sl, n2;
-    if (!frame_geometry<WINDOW>(xh, yh, zh, xl, yl, zl, w, j, fast, eps, sh, sl, n2)) return;
-#pragma unroll
-    for (int f = 0; f < NF; ++f) {
-        if (f >= p.nf) break;
-        const FreqConst &q = p.fc[f];
-        const float D = fmaf(sh, sh, q.b2);
-        if (q.kb2 * n2 > p.cutoff * D) {
-            if (p.uniform_b) break;
-            continue;
-        }
-        beam_adjoint<LOSSY>(q, sh, sl, n2, rcp_approx(D), gk[f * (kR * 32)], G, H[f],
-                            LOSSY ? loss->rf[f][j] : make_float2(0.f, 0.f));
-    }
-}
-
-__device__ __forceinline__ float warp_sum(float v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// Adds an FP32 partial sum into a float-float accumulator (hi, hi, lo, lo).
-__device__ __forceinline__ void fold(float4 *acc, float2 &t)
-{
-    if (t.x != 0.0f || t.y != 0.0f) {
-        float4 a = *acc;
-        float s, e;
-        two_sum(a.x, t.x, s, e);
-        a.x = s;
-        a.z += e;
-        two_sum(a.y, t.y, s, e);
-        a.y = s;
-        a.w += e;
-        *acc = a;
-        t = make_float2(0.0f, 0.0f);
-    }
-}
-
-
-// Conservative test: can the segment (origin (ox, oy, oz) relative to the frame
-// of `sphere`, record words r0 / r1) keep any receiver inside the ball `sphere`
-// (centre xyz, radius w)?  The distance from the segment line to a point is
-// 1-Lipschitz, so shrinking the ball's centre distance by the radius bounds n
-// from below and |s| from above over the whole ball; the radius carries slack
-// for FP32 rounding at these magnitudes.
-template <int WINDOW>
-__device__ __forceinline__ bool ball_may_keep(const float4 &r0, const float4 &r1, float ox, float oy,
-                                              float oz, const float4 &sphere, float alpha, float beta)
-{
-    const float dx = sphere.x - ox, dy = sphere.y - oy, dz = sphere.z - oz;
-    const float sc = fmaf(dx, r1.x, fmaf(dy, r1.y, dz * r1.z));
-    const float cxr = dy * r1.z - dz * r1.y, cyr = dz * r1.x - dx * r1.z, czr = dx * r1.y - dy * r1.x;
-    // |d x t| from below: the approximate square root is within a few ulp, and the
-    // factor takes it under the exact root
-    float nc;
-    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(nc) : "f"(fmaf(cxr, cxr, fmaf(cyr, cyr, czr * czr))));
-    nc *= 0.999999f;
-    const float R = sphere.w * 1.0001f + 0.05f + 1e-5f * (fabsf(ox) + fabsf(oy) + fabsf(oz));
-    bool win;
-    if (WINDOW == GBT_WINDOW_LINE) win = r0.w + sc + R >= -kWinMargin;
-    else win = (sc + R >= -kWinMargin) && (sc - R <= r1.w + kWinMargin);
-    const float sabs = fabsf(r0.w + sc) + R;
-    const float nn = nc - R;
-    return win && (nn <= 0.f || alpha * nn * nn <= fmaf(sabs, sabs, beta));
-}
-
-// Two values, each duplicated into both halves of a float pair.
-__device__ __forceinline__ float4 dup2(float a, float b) { return make_float4(a, a, b, b); }
-
-// Stage lane's raw record for the warp: the prefilter view relative to the frame
-// c = (cx, cy, cz) (the warp tile's first receiver), the origin in that frame for the
-// per-warp ball test and the direction.  A record past the segment count becomes one no
-// receiver can keep.  Returns L_hi.
-__device__ __forceinline__ float stage_batch(StageSmem &w, const float4 (&raw)[kRecFloats / 4],
-                                             int lane, bool valid, int32_t seg, float cx,
-                                             float cy, float cz, float alpha, float beta)
-{
-    const float4 r0 = raw[0], r1 = raw[1], r2 = raw[2];
-    float4 *P = w.P[lane];
-    w.seg[lane] = valid ? seg : -1;
-    if (valid) {
-        const float ox = (r0.x - cx) + r2.x, oy = (r0.y - cy) + r2.y, oz = (r0.z - cz) + r2.z;
-        w.O[lane] = make_float4(ox, oy, oz, r0.w);
-        const float ot = fmaf(ox, r1.x, fmaf(oy, r1.y, oz * r1.z));
-        const float oo = fmaf(ox, ox, fmaf(oy, oy, oz * oz));
-        const float a2 = 2.f * alpha;
-        w.D[0][lane] = dup2(r1.x, r1.y);
-        P[4] = dup2(r1.x, r1.y);
-        P[0] = dup2(r1.z, -ot);
-        P[1] = dup2(a2 * ox, a2 * oy);
-        P[2] = dup2(a2 * oz, fmaf(-alpha, oo, beta));
-        P[3] = dup2(r0.w + kWinMargin, r1.w + kWinMargin);
-    } else {
-        // far behind its own start
-        w.O[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
-        w.D[0][lane] = dup2(0.f, 0.f);
-        P[4] = dup2(0.f, 0.f);
-        P[0] = dup2(0.f, -1e15f);
-        P[1] = dup2(0.f, 0.f);
-        P[2] = dup2(0.f, 0.f);
-        P[3] = dup2(0.f, 0.f);
-    }
-    return valid ? r1.w : 0.f;
-}
-
-// Stage lane's raw record's exact-path view in the warp's frame: float-float
-// d = c - o, A = d.t, S = s0 + A, AL = A - L and the compensated N = d x t, with the
-// direction as (hi, lo) and the amplitude; finite values past the segment count.
-__device__ __forceinline__ void stage_exact(StageSmem &w, const float4 (&raw)[kRecFloats / 4],
-                                            int lane, bool valid, float cx, float cy, float cz)
-{
-    const float4 r0 = raw[0], r1 = raw[1], r2 = raw[2], r3 = raw[3], r4 = raw[4];
-    if (valid) {
-        // d = c - o as (dh + dl)
-        float dxh, dxe, dyh, dye, dzh, dze;
-        two_sum(cx, -r0.x, dxh, dxe);
-        two_sum(cy, -r0.y, dyh, dye);
-        two_sum(cz, -r0.z, dzh, dze);
-        const float dxl = __fsub_rn(dxe, r2.x), dyl = __fsub_rn(dye, r2.y), dzl = __fsub_rn(dze, r2.z);
-        // A = d.t, float-float
-        const float q0 = __fmul_rn(dxh, r1.x), q1 = __fmul_rn(dyh, r1.y), q2 = __fmul_rn(dzh, r1.z);
-        const float e0 = fmaf(dxh, r3.x, fmaf(dxl, r1.x, fmaf(dxh, r1.x, -q0)));
-        const float e1 = fmaf(dyh, r3.y, fmaf(dyl, r1.y, fmaf(dyh, r1.y, -q1)));
-        const float e2 = fmaf(dzh, r3.z, fmaf(dzl, r1.z, fmaf(dzh, r1.z, -q2)));
-        float S1, E1, Ah, E2;
-        two_sum(q0, q1, S1, E1);
-        two_sum(S1, q2, Ah, E2);
-        const float Al = __fadd_rn(__fadd_rn(E1, E2), __fadd_rn(__fadd_rn(e0, e1), e2));
-        // S = s0 + A, AL = A - L
-        float Sh, es, ALh, ea;
-        two_sum(r0.w, Ah, Sh, es);
-        const float Sl = __fadd_rn(es, __fadd_rn(Al, r2.w));
-        two_sum(Ah, -r1.w, ALh, ea);
-        const float ALl = __fadd_rn(ea, __fsub_rn(Al, r3.w));
-        // N = d x t, compensated
-        const float nx = dop(dyh, r1.z, dzh, r1.y) +
-                         fmaf(dyh, r3.z, fmaf(-dzh, r3.y, fmaf(dyl, r1.z, -dzl * r1.y)));
-        const float ny = dop(dzh, r1.x, dxh, r1.z) +
-                         fmaf(dzh, r3.x, fmaf(-dxh, r3.z, fmaf(dzl, r1.x, -dxl * r1.z)));
-        const float nz = dop(dxh, r1.y, dyh, r1.x) +
-                         fmaf(dxh, r3.y, fmaf(-dyh, r3.x, fmaf(dxl, r1.y, -dyl * r1.x)));
-        w.D[1][lane] = dup2(r1.z, Sh);
-        w.D[2][lane] = dup2(r3.x, r3.y);
-        w.D[3][lane] = dup2(r3.z, Sl);
-        w.D[4][lane] = dup2(nx, ny);
-        w.D[5][lane] = dup2(nz, r4.x);
-        w.D[6][lane] = dup2(Ah, Al);
-        w.D[7][lane] = dup2(ALh, ALl);
-    } else {
-        w.D[1][lane] = dup2(0.f, -1e15f);
-        w.D[2][lane] = dup2(0.f, 0.f);
-        w.D[3][lane] = dup2(0.f, 0.f);
-        w.D[4][lane] = dup2(0.f, 0.f);
-        w.D[5][lane] = dup2(0.f, 0.f);
-        w.D[6][lane] = dup2(-1e15f, 0.f);
-        w.D[7][lane] = dup2(-1e15f, 0.f);
-    }
-}
-
-template <int NF>
-struct AdjSmem {
-    float2 g[NF][kR][32];      // the warp's receivers' g, per sorted frequency
-};
-// Per-warp shared memory of the pair kernel: two raw record buffers (bulk-copy
-// or cp.async targets), the staged batch, and the completion barriers of the
-// bulk copies.
-struct WarpBuf {
+// Per-warp shared memory of the counting pass: two raw record buffers (bulk-copy or
+// cp.async targets), the staged batch, and the completion barriers of the bulk copies.
+struct CountBuf {
     float4 raw[kWRaw][kBatch][kRecFloats / 4];
     StageSmem stg;
     unsigned long long bar[kWRaw];
     int32_t queue[kBatch];           // list positions of the next batch for this warp tile
     int abort_flag, pad[3];
 };
+constexpr size_t kCountPerWarp = (sizeof(CountBuf) + 127) / 128 * 128;
+constexpr int kCountWarps = (int)(kSmemBudget / kCountPerWarp) < kWarpsFwd
+                                ? (int)(kSmemBudget / kCountPerWarp) : kWarpsFwd;
+constexpr size_t kCountSmem = kCountWarps * kCountPerWarp;
 
-template <int NF, int MODE, bool BATCHED, bool LOSSY = false>
-struct PairCfg {
-    static constexpr size_t kAdj = MODE == kBwd ? sizeof(AdjSmem<NF>) : 0;
-    static constexpr size_t kInst = BATCHED ? sizeof(FwdParams) : 0;
-    static constexpr size_t kLoss = LOSSY ? sizeof(LossSmem<NF>) : 0;
-    static constexpr size_t kPerWarp = (sizeof(WarpBuf) + kAdj + kInst + kLoss + 127) / 128 * 128;
-    // as many warps as fit in the shared memory budget, at most kWarpsFwd
-    static constexpr int kFit = (int)(kSmemBudget / kPerWarp);
-    static constexpr int kWarps = kFit < kWarpsFwd ? kFit : kWarpsFwd;
-    static constexpr size_t kSmem = kWarps * kPerWarp;
-};
-
-// Persistent pair kernel.  Every warp works on its own: it takes (warp tile of
-// 64 receivers, segment split) items from a global queue (CTA tiles of 960
-// heaviest first), streams the item's record batches into its own double buffer
-// (one bulk copy per batch for consecutive segments, one 16-byte cp.async per
-// lane and word for a tile's list), stages each batch relative to its first
-// receiver, and runs the prefilter and the exact path for its receivers.  No
-// warp ever waits for another, so warps whose receivers meet more surviving
-// pairs cost only themselves.  The FP32 sums fold into the item's float-float
-// partials (global, resident in L2) every kFoldEvery batches.
-template <int NF, int WINDOW, int MODE, bool BATCHED, bool LOSSY = false>
-__global__ void __maxnreg__(128) gbs_fwd_kernel(const __grid_constant__ FwdParams prm)
+// Persistent and warp-autonomous like the pair kernel: consecutive segments arrive by one
+// bulk copy per batch, a tile list's by one 16-byte cp.async per lane and word.
+template <int NF, int WINDOW>
+__global__ void __maxnreg__(128) gbs_count_kernel(const __grid_constant__ FwdParams prm)
 {
-    using Cfg = PairCfg<NF, MODE, BATCHED, LOSSY>;
-    static_assert(!(LOSSY && BATCHED), "batches with losses run the single-sum kernel");
-    constexpr bool STATS = MODE == kStats;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned char *const mine = smem_raw + (size_t)warp * Cfg::kPerWarp;
-    WarpBuf &B = *reinterpret_cast<WarpBuf *>(mine);
-    AdjSmem<NF> &adj = *reinterpret_cast<AdjSmem<NF> *>(mine + sizeof(WarpBuf));
-    FwdParams &inst = *reinterpret_cast<FwdParams *>(mine + sizeof(WarpBuf) + Cfg::kAdj);
-    LossSmem<NF> *const loss =
-        reinterpret_cast<LossSmem<NF> *>(mine + sizeof(WarpBuf) + Cfg::kAdj + Cfg::kInst);
+    unsigned char *const mine = smem_raw + (size_t)warp * kCountPerWarp;
+    CountBuf &B = *reinterpret_cast<CountBuf *>(mine);
 
     if (lane == 0) {
         for (int i = 0; i < kWRaw; ++i) mbar_init(smem_addr(&B.bar[i]), 1);
@@ -855,25 +100,8 @@ __global__ void __maxnreg__(128) gbs_fwd_kernel(const __grid_constant__ FwdParam
         int64_t it = 0;
         if (lane == 0) it = atomicAdd(prm.work_counter, 1);
         it = __shfl_sync(0xffffffffu, it, 0);
-        if (BATCHED) {
-            if (it < prm.n_items) {
-                int lo = 0, hi = prm.n_inst - 1;      // last instance with inst_off <= it
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (prm.inst_off[mid] <= it) lo = mid;
-                    else hi = mid - 1;
-                }
-                it -= prm.inst_off[lo];
-                const int4 *src = reinterpret_cast<const int4 *>(prm.inst + lo);
-                int4 *dst = reinterpret_cast<int4 *>(&inst);
-                for (int q = lane; q < (int)(sizeof(FwdParams) / 16); q += 32) dst[q] = src[q];
-                __syncwarp();
-            } else {
-                break;
-            }
-        }
-        const FwdParams &p = BATCHED ? inst : prm;
-        if ((!BATCHED && it >= p.n_items) || *abort_flag) break;
+        const FwdParams &p = prm;
+        if (it >= p.n_items || *abort_flag) break;
 
         // item -> (CTA tile by dispatch rank, split, warp tile within the CTA tile)
         const int64_t per_tile = (int64_t)kTileWarps * p.splits;
@@ -903,16 +131,13 @@ __global__ void __maxnreg__(128) gbs_fwd_kernel(const __grid_constant__ FwdParam
 
         // receiver k of the lane at x = c + x', x' = (xp + xl) exactly
         float xa[kR], ya[kR], za[kR], xp[kR], yp[kR], zp[kR], xl[kR], yl[kR], zl[kR], xx[kR];
-        int32_t ridx[kR];
         uint32_t valid = 0;
-        float4 *const part_base = p.partial + (int64_t)split * p.nf * p.n_recv;
 #pragma unroll
         for (int k = 0; k < kR; ++k) {
             // lane holds receivers lane and lane + 32 of the warp tile: the two halves
             // of its Morton patch, so a beam edge splits work evenly over lanes
             const int64_t r = wbase + (int64_t)k * 32 + lane;
             xa[k] = ya[k] = za[k] = xp[k] = yp[k] = zp[k] = xl[k] = yl[k] = zl[k] = xx[k] = 0.0f;
-            ridx[k] = -1;
             if (r < p.n_recv) {
                 const int64_t o = p.order ? p.order[r] : r;
                 xa[k] = p.recv[3 * o]; ya[k] = p.recv[3 * o + 1]; za[k] = p.recv[3 * o + 2];
@@ -921,19 +146,6 @@ __global__ void __maxnreg__(128) gbs_fwd_kernel(const __grid_constant__ FwdParam
                 two_sum(za[k], -cz, zp[k], zl[k]);
                 xx[k] = fmaf(xp[k], xp[k], fmaf(yp[k], yp[k], zp[k] * zp[k]));
                 valid |= 1u << k;
-                ridx[k] = (int32_t)o;
-            }
-            if (MODE == kBwd) {
-#pragma unroll
-                for (int f = 0; f < NF; ++f)
-                    adj.g[f][k][lane] = (f < p.nf && ridx[k] >= 0)
-                                            ? p.grad_out[(int64_t)p.fperm[f] * p.n_recv + ridx[k]]
-                                            : make_float2(0.f, 0.f);
-            } else if (MODE == kFwd) {
-#pragma unroll
-                for (int f = 0; f < NF; ++f)
-                    if (f < p.nf && ridx[k] >= 0)
-                        part_base[(int64_t)f * p.n_recv + ridx[k]] = make_float4(0.f, 0.f, 0.f, 0.f);
             }
         }
         // bounding ball of the warp tile's receivers (relative to its first receiver)
@@ -962,40 +174,11 @@ __global__ void __maxnreg__(128) gbs_fwd_kernel(const __grid_constant__ FwdParam
             for (int o = 16; o > 0; o >>= 1) r2 = fmaxf(r2, __shfl_xor_sync(0xffffffffu, r2, o));
             sphere = make_float4(sx, sy, sz, sqrtf(r2));
         }
-        // the FP32 local projection when the warp is compact enough for its frequencies
-        float xmax2 = fmaxf((valid & 1u) ? xx[0] : 0.f, (valid & 2u) ? xx[1] : 0.f);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) xmax2 = fmaxf(xmax2, __shfl_xor_sync(0xffffffffu, xmax2, o));
-        const bool fast_u = sqrtf(xmax2) * p.kmax_turns <= kFastTurns;
-        // its error bound: the three-term FP32 dot product with |t| = 1 is within about
-        // 3 x 2^-24 max|x'| of x'.t; eps is over five times that
-        const float eps_u = 1e-6f * sqrtf(xmax2);
         static_assert(kR == 2, "the paired prefilter handles two receivers per lane");
         const f2x X2 = pk(xp[0], xp[1]), Y2 = pk(yp[0], yp[1]), Z2 = pk(zp[0], zp[1]);
         const f2x NAXX = pk(-alpha * xx[0], -alpha * xx[1]);
         const f2x AL2 = pk(alpha, alpha);
         const f2x MG2 = pk(kWinMargin, kWinMargin);
-        // per-batch FP32 sums of the lane's two receivers, paired (re, im)
-        f2x accx[NF], accy[NF];
-#pragma unroll
-        for (int f = 0; f < NF; ++f) accx[f] = accy[f] = 0ull;
-        const f2x XL2 = pk(xl[0], xl[1]), YL2 = pk(yl[0], yl[1]), ZL2 = pk(zl[0], zl[1]);
-        const f2x NX2 = neg2(X2), NY2 = neg2(Y2), NZ2 = neg2(Z2);
-        auto fold_all = [&]() {
-#pragma unroll
-            for (int f = 0; f < NF; ++f) {
-                if (f < p.nf) {
-                    float x0, x1, y0, y1;
-                    upk(accx[f], x0, x1);
-                    upk(accy[f], y0, y1);
-                    float2 t0 = make_float2(x0, y0), t1 = make_float2(x1, y1);
-                    if (ridx[0] >= 0) fold(part_base + (int64_t)f * p.n_recv + ridx[0], t0);
-                    if (ridx[1] >= 0) fold(part_base + (int64_t)f * p.n_recv + ridx[1], t1);
-                }
-                accx[f] = accy[f] = 0ull;
-            }
-        };
-
         // Batches of the item, double-buffered: raw buffer k % 2 receives batch k.  Consecutive
         // segments: batch k is split + k * splits, one bulk copy (lane 0) on the buffer's
         // mbarrier.  A tile list: the item takes the list's 32-entry chunks split, split +
@@ -1003,9 +186,7 @@ __global__ void __maxnreg__(128) gbs_fwd_kernel(const __grid_constant__ FwdParam
         // queues the set bits' list positions in order, gathers the entries of each full
         // batch, and every lane copies its own record with 16-byte async copies (one commit
         // group per batch, empty past the end).
-        // Per buffer: records in the batch, and this lane's segment index (or -1).
-        int nrec0 = 0, nrec1 = 0;
-        int32_t seg0 = -1, seg1 = -1;
+        int nrec0 = 0, nrec1 = 0;   // per buffer: records in the batch
         const int64_t n_chunks = (n_seg + kBatch - 1) / kBatch;
         const uint32_t *lw =
             lst ? p.list_words + (p.list_off[tile] / kBatch) * kChunkWords + wl : nullptr;
@@ -1047,11 +228,10 @@ __global__ void __maxnreg__(128) gbs_fwd_kernel(const __grid_constant__ FwdParam
         auto issue = [&](uint32_t k) {   // all lanes, k in increasing order
             const int buf = (int)(k & 1u);
             int n = 0;
-            int32_t idx = -1;
             if (lst) {
                 int32_t pos;
                 n = next_list_batch(pos);
-                idx = pos >= 0 ? lst[pos] : -1;
+                const int32_t idx = pos >= 0 ? lst[pos] : -1;
                 if (idx >= 0) {
                     const float4 *src =
                         reinterpret_cast<const float4 *>(p.rec + (int64_t)idx * kRecFloats);
@@ -1062,7 +242,6 @@ __global__ void __maxnreg__(128) gbs_fwd_kernel(const __grid_constant__ FwdParam
             } else if (k < nb) {
                 const int64_t b = split + (int64_t)k * p.splits;
                 n = (int)min((int64_t)kBatch, n_seg - b * kBatch);
-                idx = lane < n ? (int32_t)(b * kBatch + lane) : -1;
                 if (lane == 0) {
                     const uint32_t bytes = (uint32_t)n * kRecFloats * 4;
                     mbar_arrive_expect_tx(smem_addr(&B.bar[buf]), bytes);
@@ -1070,17 +249,15 @@ __global__ void __maxnreg__(128) gbs_fwd_kernel(const __grid_constant__ FwdParam
                              smem_addr(&B.bar[buf]));
                 }
             }
-            if (buf) { nrec1 = n; seg1 = idx; } else { nrec0 = n; seg0 = idx; }
+            if (buf) nrec1 = n; else nrec0 = n;
         };
         issue(0);
         issue(1);
         uint32_t waited = 0;   // bulk batches whose copy has landed
-        bool dirty = false;    // survivors since the last fold
         for (uint32_t kb_ = 0;; ++kb_) {
             const int buf = (int)(kb_ & 1u);
             const int nrec = buf ? nrec1 : nrec0;
             if (nrec <= 0) break;
-            const int32_t my_seg = buf ? seg1 : seg0;
             if (lst) {
                 cp_async_wait1();   // this lane's copies of batch kb_
             } else {
@@ -1091,19 +268,11 @@ __global__ void __maxnreg__(128) gbs_fwd_kernel(const __grid_constant__ FwdParam
             }
             const bool seg_ok = lane < nrec;
             StageSmem &w = B.stg;
-            const float my_len = stage_batch(w, B.raw[buf][lane], lane, seg_ok, my_seg, cx, cy, cz,
-                                             alpha, beta);
-            // The exact view: with the pre-cull at once (nearly every batch has survivors);
-            // testing every pair only after the prefilter, and only for a batch in which the
-            // warp has a survivor (most such batches have none), before raw[buf] is reused.
+            const float my_len = stage_batch(w, B.raw[buf][lane], lane, seg_ok, -1, cx, cy, cz, alpha,
+                                             beta);
+            // the exact view: with the pre-cull at once, testing every pair only for a batch in
+            // which the warp has a survivor, before raw[buf] is reused
             if (lst) stage_exact(w, B.raw[buf][lane], lane, seg_ok, cx, cy, cz);
-            if (LOSSY && MODE != kStats) {
-#pragma unroll
-                for (int f = 0; f < NF; ++f)
-                    loss->rf[f][lane] = (seg_ok && f < p.nf)
-                                            ? p.seg_rf[(int64_t)p.fperm[f] * p.rf_stride + my_seg]
-                                            : make_float2(0.f, 0.f);
-            }
             uint32_t tmask = 0u;
             if (p.tile_cull) {
                 // this lane's segment against the warp tile's ball (own lane's staging only)
@@ -1156,25 +325,10 @@ __global__ void __maxnreg__(128) gbs_fwd_kernel(const __grid_constant__ FwdParam
                     kb1 = ~(__float_as_uint(g1) | __float_as_uint(a1)) & __float_as_uint(b1_);
                 }
             };
-            if (MODE == kFwd && lst) {
-                // With the pre-cull most tested pairs survive the exact test, so the
-                // prefilter is skipped: every lane takes each segment that reaches the
-                // warp tile's ball, in segment order, for both of its receivers.  The
-                // exact path rejects whatever the prefilter would have, so the kept terms,
-                // their arithmetic and their order per receiver are unchanged.
-                uint32_t T = tmask;
-                dirty |= T != 0u;
-                while (T) {
-                    const int jj = __ffs(T) - 1;
-                    T &= T - 1;
-                    survivor_pair<NF, WINDOW, LOSSY, true>(p, X2, Y2, Z2, XL2, YL2, ZL2, NX2, NY2, NZ2, w, loss, jj,
-                                                           jj, (valid & 1u) != 0u, (valid & 2u) != 0u,
-                                                           fast_u, eps_u, accx, accy);
-                }
-            } else if (p.tile_cull) {
+if (p.tile_cull) {
                 // only the segments that can reach this warp tile's receivers
                 uint32_t T = tmask;
-                if (STATS) n_test += __popc(T) * __popc(valid);
+                n_test += __popc(T) * __popc(valid);
                 while (T) {
                     const int jj = __ffs(T) - 1;
                     T &= T - 1;
@@ -1184,7 +338,7 @@ __global__ void __maxnreg__(128) gbs_fwd_kernel(const __grid_constant__ FwdParam
                     m[1] |= (kb1 >> 31) << (31 - jj);
                 }
             } else {
-                if (STATS) n_test += (uint32_t)nrec * __popc(valid);
+                n_test += (uint32_t)nrec * __popc(valid);
 #pragma unroll 4
                 for (int jj = 0; jj < kBatch; ++jj) {
                     uint32_t kb0, kb1;
@@ -1199,74 +353,15 @@ __global__ void __maxnreg__(128) gbs_fwd_kernel(const __grid_constant__ FwdParam
                 __syncwarp();    // the batch is staged and raw[buf] is free again
                 issue(kb_ + 2);
             }
-            // ---- survivors, in segment order per receiver
-            if (MODE == kFwd && lst) {
-                // evaluated above
-            } else if (MODE == kFwd) {
-                // the two receivers' survivors side by side, each in segment order
-                uint32_t mm0 = (valid & 1u) ? m[0] : 0u, mm1 = (valid & 2u) ? m[1] : 0u;
-                while (mm0 | mm1) {
-                    const bool h0 = mm0 != 0u, h1 = mm1 != 0u;
-                    int j0 = __clz(mm0), j1 = __clz(mm1);
-                    if (h0) mm0 ^= 0x80000000u >> j0;
-                    if (h1) mm1 ^= 0x80000000u >> j1;
-                    if (!h0) j0 = j1;
-                    if (!h1) j1 = j0;
-                    survivor_pair<NF, WINDOW, LOSSY>(p, X2, Y2, Z2, XL2, YL2, ZL2, NX2, NY2, NZ2, w, loss, j0, j1, h0,
-                                                     h1, fast_u, eps_u, accx, accy);
-                }
-            } else if (MODE == kBwd) {
-                // segment by segment: the lanes holding a survivor of segment jj add their
-                // receivers' terms, the warp sums them, and one lane adds the sums to the
-                // segment's global G and H (no shared-memory atomics between lanes)
-                const uint32_t mm0 = (valid & 1u) ? m[0] : 0u, mm1 = (valid & 2u) ? m[1] : 0u;
-                uint32_t any = __reduce_or_sync(0xffffffffu, mm0 | mm1);
-                while (any) {
-                    const int jj = __clz(any);
-                    any ^= 0x80000000u >> jj;
-                    float G = 0.f, H[NF];
+            // ---- survivors
 #pragma unroll
-                    for (int f = 0; f < NF; ++f) H[f] = 0.f;
-                    if ((mm0 << jj) >> 31)
-                        survivor_adjoint<NF, WINDOW, LOSSY>(p, xp[0], yp[0], zp[0], xl[0], yl[0],
-                                                            zl[0], w, loss, jj, fast_u, eps_u,
-                                                            &adj.g[0][0][lane],
-                                                            G, H);
-                    if ((mm1 << jj) >> 31)
-                        survivor_adjoint<NF, WINDOW, LOSSY>(p, xp[1], yp[1], zp[1], xl[1], yl[1],
-                                                            zl[1], w, loss, jj, fast_u, eps_u,
-                                                            &adj.g[0][1][lane],
-                                                            G, H);
-                    G = warp_sum(G);
-#pragma unroll
-                    for (int f = 0; f < NF; ++f)
-                        if (f < p.nf) H[f] = warp_sum(H[f]);
-                    const int32_t jg = w.seg[jj];
-                    if (lane == 0 && jg >= 0) {
-                        if (G != 0.f) atomicAdd(&p.seg_G[jg], G);
-#pragma unroll
-                        for (int f = 0; f < NF; ++f)
-                            if (f < p.nf && H[f] != 0.f) atomicAdd(&p.seg_H[(int64_t)f * p.seg_stride + jg], H[f]);
-                    }
-                }
-            } else {
-#pragma unroll
-                for (int k = 0; k < kR; ++k) {
-                    uint32_t mm = ((valid >> k) & 1u) ? m[k] : 0u;
-                    if (STATS) n_pre += __popc(mm);
-                    while (mm) {
-                        const int jj = __clz(mm);
-                        mm ^= 0x80000000u >> jj;
-                        survivor_count<NF, WINDOW>(p, xp[k], yp[k], zp[k], xl[k], yl[k], zl[k], w, jj,
-                                                   fast_u, eps_u, n_kept);
-                    }
-                }
-            }
-            if (MODE == kFwd) {
-                dirty |= (m[0] | m[1]) != 0u;
-                if ((kb_ % kFoldEvery) == kFoldEvery - 1 && dirty) {
-                    dirty = false;
-                    fold_all();
+            for (int k = 0; k < kR; ++k) {
+                uint32_t mm = ((valid >> k) & 1u) ? m[k] : 0u;
+                n_pre += __popc(mm);
+                while (mm) {
+                    const int jj = __clz(mm);
+                    mm ^= 0x80000000u >> jj;
+                    survivor_count<NF, WINDOW>(p, xp[k], yp[k], zp[k], xl[k], yl[k], zl[k], w, jj, n_kept);
                 }
             }
             __syncwarp();        // before the next batch is staged over this one
@@ -1283,13 +378,10 @@ __global__ void __maxnreg__(128) gbs_fwd_kernel(const __grid_constant__ FwdParam
                 ph ^= 1u << bf;
             }
         }
-        if (MODE == kFwd) fold_all();
     }
-    if (STATS) {
-        atomicAdd(&prm.stats[1], (unsigned long long)n_pre);
-        atomicAdd(&prm.stats[2], (unsigned long long)n_kept);
-        atomicAdd(&prm.stats[3], n_test);
-    }
+    atomicAdd(&prm.stats[1], (unsigned long long)n_pre);
+    atomicAdd(&prm.stats[2], (unsigned long long)n_kept);
+    atomicAdd(&prm.stats[3], n_test);
 }
 
 // ------------------------------------------------------------- prepass --
@@ -1644,16 +736,6 @@ __global__ void grad_out_kernel(GradOutParams p)
 constexpr int kWeightSamples = 1 << 15;        // sampled segments per estimate
 constexpr int64_t kMaxOrderedTiles = 1 << 14;  // beyond this the rank pass is skipped
 
-// A ball with its share of the list test's slack, and a segment's share (seg_reaches_ball).
-__device__ __forceinline__ float4 reach_ball(const float4 &b)
-{
-    return make_float4(b.x, b.y, b.z,
-                       fmaf(b.w, 1.0001f, 0.05f) + 1e-5f * (fabsf(b.x) + fabsf(b.y) + fabsf(b.z)));
-}
-__device__ __forceinline__ float segment_slack(const float4 &r0)
-{
-    return 1e-5f * (fabsf(r0.x) + fabsf(r0.y) + fabsf(r0.z));
-}
 
 // Also each tile's reach ball (the list passes' form, with the ball's share of the slack).
 __global__ void tile_ball_kernel(const float *recv, const int32_t *order, int64_t n_recv,
@@ -1777,51 +859,6 @@ __global__ void tile_rank_kernel(const unsigned int *weight, int64_t n_tiles, in
 // of the list buffer lightest first; a tile that does not fit streams every
 // segment, which gives the same field.
 constexpr int kListChunk = 1024;
-
-// The list passes' form of ball_may_keep, with its slack split between the ball and the
-// segment: a reach ball (centre, W) with W = r 1.0001 + 0.05 + 1e-5 (|cx| + |cy| + |cz|),
-// and the segment's 1e-5 (|ox| + |oy| + |oz|).  Their sum bounds the slack of
-// ball_may_keep (|o - c| <= |o| + |c|), so the test is at least as conservative and
-// costs each (segment, ball) pair a single add for it.  From a segment's cull record
-// (its origin rounded to FP32, which the slack of 5 cm far exceeds).
-// A segment's terms of the test, formed once for all the balls it meets: with d = c - o,
-// d.t = c.t - o.t and d x t = c x t - o x t, whose extra rounding (a few ulp of |c| and
-// |o|) the slack's 1e-5 (|o| + |c|) far exceeds.
-struct SegCull {
-    float tx, ty, tz, len, s0;   // direction, length, start
-    float ot, ox, oy, oz;        // o.t and o x t
-    float slack;                 // the segment's share of the slack
-};
-__device__ __forceinline__ SegCull seg_cull(const float4 &r0, const float4 &r1)
-{
-    SegCull g;
-    g.tx = r1.x; g.ty = r1.y; g.tz = r1.z; g.len = r1.w; g.s0 = r0.w;
-    g.ot = fmaf(r0.x, r1.x, fmaf(r0.y, r1.y, r0.z * r1.z));
-    g.ox = fmaf(r0.y, r1.z, -r0.z * r1.y);
-    g.oy = fmaf(r0.z, r1.x, -r0.x * r1.z);
-    g.oz = fmaf(r0.x, r1.y, -r0.y * r1.x);
-    g.slack = segment_slack(r0);
-    return g;
-}
-template <int WINDOW>
-__device__ __forceinline__ bool seg_reaches_ball(const SegCull &g, const float4 &rb, float alpha,
-                                                 float beta)
-{
-    const float sc = fmaf(rb.x, g.tx, fmaf(rb.y, g.ty, fmaf(rb.z, g.tz, -g.ot)));
-    const float cxr = fmaf(rb.y, g.tz, fmaf(-rb.z, g.ty, -g.ox));
-    const float cyr = fmaf(rb.z, g.tx, fmaf(-rb.x, g.tz, -g.oy));
-    const float czr = fmaf(rb.x, g.ty, fmaf(-rb.y, g.tx, -g.oz));
-    float nc;   // |d x t| from below (see ball_may_keep)
-    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(nc) : "f"(fmaf(cxr, cxr, fmaf(cyr, cyr, czr * czr))));
-    nc *= 0.999999f;
-    const float R = rb.w + g.slack;
-    bool win;
-    if (WINDOW == GBT_WINDOW_LINE) win = g.s0 + sc + R >= -kWinMargin;
-    else win = (sc + R >= -kWinMargin) && (sc - R <= g.len + kWinMargin);
-    const float sabs = fabsf(g.s0 + sc) + R;
-    const float nn = nc - R;
-    return win && (nn <= 0.f || alpha * nn * nn <= fmaf(sabs, sabs, beta));
-}
 
 template <int WINDOW>
 __global__ void __launch_bounds__(kListChunk) list_count_kernel(
@@ -2128,59 +1165,74 @@ struct ReduceParams {
     int64_t n_recv;
     int perm[GBT_MAX_FREQ];    // partial frequency slot -> output frequency
     int splits;
-    const float4 *p32;
-    const double2 *p64;
+    const float4 *p32;         // in processing order of the receivers
+    const int32_t *order;      // processing order -> receiver, or null
+    float scale[GBT_MAX_FREQ]; // per slot: the partials' common factor
+    const double2 *p64;        // F64 path: by receiver
     float2 *out;
     int accumulate;
 };
 
-__global__ void reduce_kernel(ReduceParams p)
+// Float-float partials (hi, running FP32 sum of errors) merged into a float-float total with
+// error-free FP32 sums: about 44 bits, far beyond the complex64 output, and no FP64
+// arithmetic (GB300 issues FP64 at a small fraction of the FP32 rate).  A block takes 32
+// outputs; its kMergeGroups warps each sum a consecutive range of the splits and the first
+// warp adds the groups in order, so a few thousand receivers with hundreds of splits still
+// fill the chip (9,973 receivers, 3 bands, 471 splits: 160 us with one thread per output).
+constexpr int kMergeGroups = 8;
+__device__ __forceinline__ void merge_ff(float4 &a, const float4 &v)   // (rh, ih, rl, il)
+{
+    float t, e;
+    two_sum(a.x, v.x, t, e);
+    a.x = t;
+    a.z = __fadd_rn(a.z, __fadd_rn(e, v.z));
+    two_sum(a.y, v.y, t, e);
+    a.y = t;
+    a.w = __fadd_rn(a.w, __fadd_rn(e, v.w));
+}
+__global__ void __launch_bounds__(32 * kMergeGroups) reduce_kernel(ReduceParams p)
+{
+    __shared__ float4 part[kMergeGroups][32];
+    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+    const int64_t i = blockIdx.x * (int64_t)32 + lane;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (i < p.n) {
+        const int s0 = (int)((int64_t)p.splits * g / kMergeGroups);
+        const int s1 = (int)((int64_t)p.splits * (g + 1) / kMergeGroups);
+        const float4 *src = p.p32 + i;
+#pragma unroll 8
+        for (int s = s0; s < s1; ++s) merge_ff(a, __ldcs(src + (int64_t)s * p.n));
+    }
+    part[g][lane] = a;
+    __syncthreads();
+    if (g != 0 || i >= p.n) return;
+#pragma unroll
+    for (int q = 1; q < kMergeGroups; ++q) merge_ff(a, part[q][lane]);
+    const int64_t f = i / p.n_recv, r = i - f * p.n_recv;
+    const int64_t oi = (int64_t)p.perm[f] * p.n_recv + (p.order ? p.order[r] : r);
+    // times the slot's amplitude factor, in float-float (1 leaves the total as it is)
+    const float k = p.scale[f], x = __fmul_rn(a.x, k), y = __fmul_rn(a.y, k);
+    a = make_float4(x, y, fmaf(a.z, k, fmaf(a.x, k, -x)), fmaf(a.w, k, fmaf(a.y, k, -y)));
+    if (p.accumulate) {
+        const float2 o = p.out[oi];
+        merge_ff(a, make_float4(o.x, o.y, 0.f, 0.f));
+    }
+    p.out[oi] = make_float2(__fadd_rn(a.x, a.z), __fadd_rn(a.y, a.w));
+}
+
+__global__ void reduce64_kernel(ReduceParams p)
 {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= p.n) return;
-    // splits in order (the sums are the same whatever the unrolling); unrolled so the
-    // independent loads are in flight together
     const int64_t f = i / p.n_recv, r = i - f * p.n_recv;
     const int64_t oi = (int64_t)p.perm[f] * p.n_recv + r;
-    if (p.p32) {
-        // float-float partials (hi, running FP32 sum of errors) merged into a float-float
-        // total with error-free FP32 sums: about 44 bits, far beyond the complex64 output,
-        // and no FP64 arithmetic (GB300 issues FP64 at a small fraction of the FP32 rate)
-        const float4 *src = p.p32 + i;
-        float rh = 0.0f, rl = 0.0f, ih = 0.0f, il = 0.0f;
-#pragma unroll 8
-        for (int s = 0; s < p.splits; ++s) {
-            const float4 v = __ldcs(src + (int64_t)s * p.n);
-            float t, e;
-            two_sum(rh, v.x, t, e);
-            rh = t;
-            rl = __fadd_rn(rl, __fadd_rn(e, v.z));
-            two_sum(ih, v.y, t, e);
-            ih = t;
-            il = __fadd_rn(il, __fadd_rn(e, v.w));
-        }
-        if (p.accumulate) {
-            const float2 o = p.out[oi];
-            float t, e;
-            two_sum(rh, o.x, t, e);
-            rh = t;
-            rl = __fadd_rn(rl, e);
-            two_sum(ih, o.y, t, e);
-            ih = t;
-            il = __fadd_rn(il, e);
-        }
-        p.out[oi] = make_float2(__fadd_rn(rh, rl), __fadd_rn(ih, il));
-        return;
-    }
     double re = 0.0, im = 0.0;
-    {
-        const double2 *src = p.p64 + i;
+    const double2 *src = p.p64 + i;
 #pragma unroll 8
-        for (int s = 0; s < p.splits; ++s) {
-            const double2 v = src[(int64_t)s * p.n];
-            re += v.x;
-            im += v.y;
-        }
+    for (int s = 0; s < p.splits; ++s) {
+        const double2 v = src[(int64_t)s * p.n];
+        re += v.x;
+        im += v.y;
     }
     if (p.accumulate) {
         const float2 o = p.out[oi];
@@ -2190,17 +1242,15 @@ __global__ void reduce_kernel(ReduceParams p)
     p.out[oi] = make_float2((float)re, (float)im);
 }
 
-// ------------------------------------------------------ receiver order --
+static void reduce_launch(const ReduceParams &rp, cudaStream_t s)
+{
+    if (rp.p32) reduce_kernel<<<(unsigned)((rp.n + 31) / 32), 32 * kMergeGroups, 0, s>>>(rp);
+    else reduce64_kernel<<<(unsigned)((rp.n + 255) / 256), 256, 0, s>>>(rp);
+    note_launches(1);
+    GBT_CUDA(cudaGetLastError());
+}
 
-__device__ __forceinline__ unsigned int ordered_bits(float f)
-{
-    unsigned int u = __float_as_uint(f);
-    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-__device__ __forceinline__ float from_ordered(unsigned int u)
-{
-    return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
-}
+// ------------------------------------------------------ receiver order --
 
 __global__ void bbox_kernel(const float *recv, int64_t n, unsigned int *bb)
 {
@@ -2349,65 +1399,25 @@ float4 *cull_records(const float *rec, int64_t capacity)
         align_up((size_t)kRecFloats * (size_t)capacity * sizeof(float), 256));
 }
 
-template <int NF, int WINDOW, int MODE, bool BATCHED = false, bool LOSSY = false>
-void launch_fwd_t(const FwdParams &p, cudaStream_t s, bool timed)
+template <int NF, int WINDOW>
+void launch_count(const FwdParams &p, cudaStream_t s)
 {
-    constexpr bool STATS = MODE != kFwd;
-    using Cfg = PairCfg<NF, MODE, BATCHED, LOSSY>;
-    const size_t smem = Cfg::kSmem;
-    const int threads = 32 * Cfg::kWarps;
-    GBT_CUDA(cudaFuncSetAttribute(gbs_fwd_kernel<NF, WINDOW, MODE, BATCHED, LOSSY>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    int per_sm = 0;
-    GBT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &per_sm, gbs_fwd_kernel<NF, WINDOW, MODE, BATCHED, LOSSY>, threads, smem));
-    if (per_sm < 1) fail(GBT_ERR_UNSUPPORTED, "GBS kernel does not fit on one SM");
+    GBT_CUDA(cudaFuncSetAttribute(gbs_count_kernel<NF, WINDOW>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCountSmem));
     const int grid = (int)std::max<int64_t>(
-        1, std::min<int64_t>((p.n_items + Cfg::kWarps - 1) / Cfg::kWarps,
-                             (int64_t)std::max(per_sm, 1) * num_sms()));
+        1, std::min<int64_t>((p.n_items + kCountWarps - 1) / kCountWarps, (int64_t)num_sms()));
     GBT_CUDA(cudaMemsetAsync(p.work_counter, 0, sizeof(int), s));
-    if (MODE != kStats && timed) timing_begin(s);
-    gbs_fwd_kernel<NF, WINDOW, MODE, BATCHED, LOSSY><<<grid, threads, smem, s>>>(p);
+    gbs_count_kernel<NF, WINDOW><<<grid, 32 * kCountWarps, kCountSmem, s>>>(p);
     note_launches(1);
     GBT_CUDA(cudaGetLastError());
-    if (MODE != kStats && timed) timing_end(s);
-    (void)STATS;
-}
-
-template <int NF, int WINDOW>
-void launch_fwd(const FwdParams &p, cudaStream_t s, bool timed)
-{
-    if (p.grad_out) launch_fwd_t<NF, WINDOW, kBwd>(p, s, timed);
-    else if (p.stats) launch_fwd_t<NF, WINDOW, kStats>(p, s, timed);
-    else launch_fwd_t<NF, WINDOW, kFwd>(p, s, timed);
-}
-
-// With losses (seg_rf set) the forward and adjoint launches take the lossy kernel,
-// instantiated for 1, 2, 4 and 8 frequency slots; counting needs no losses.
-template <int NF, int WINDOW>
-void launch_fwd_lossy(const FwdParams &p, cudaStream_t s, bool timed)
-{
-    if (p.grad_out) launch_fwd_t<NF, WINDOW, kBwd, false, true>(p, s, timed);
-    else launch_fwd_t<NF, WINDOW, kFwd, false, true>(p, s, timed);
 }
 
 template <int WINDOW>
-void launch_fwd_nf(const FwdParams &p, cudaStream_t s, bool timed = true)
+void launch_count_nf(const FwdParams &p, cudaStream_t s)
 {
-    if (p.seg_rf && !p.stats) {
-        if (p.nf <= 1) launch_fwd_lossy<1, WINDOW>(p, s, timed);
-        else if (p.nf <= 2) launch_fwd_lossy<2, WINDOW>(p, s, timed);
-        else if (p.nf <= 4) launch_fwd_lossy<4, WINDOW>(p, s, timed);
-        else if (p.nf <= 8) launch_fwd_lossy<8, WINDOW>(p, s, timed);
-        else fail(GBT_ERR_UNSUPPORTED, "pair kernel launched with more than 8 frequencies");
-        return;
-    }
-    if (p.nf <= 1) launch_fwd<1, WINDOW>(p, s, timed);
-    else if (p.nf <= 2) launch_fwd<2, WINDOW>(p, s, timed);
-    else if (p.nf <= 4) launch_fwd<4, WINDOW>(p, s, timed);
-    else if (p.nf <= 6) launch_fwd<6, WINDOW>(p, s, timed);
-    else if (p.nf <= 8) launch_fwd<8, WINDOW>(p, s, timed);
-    else fail(GBT_ERR_UNSUPPORTED, "pair kernel launched with more than 8 frequencies");
+    if (p.nf <= 1) launch_count<1, WINDOW>(p, s);
+    else if (p.nf <= 4) launch_count<4, WINDOW>(p, s);
+    else launch_count<8, WINDOW>(p, s);
 }
 
 // Frequency processing order: when every b is equal, sorted by k so that the kept
@@ -2424,15 +1434,12 @@ bool freq_order(const gbt_sum_args &a, int (&perm)[GBT_MAX_FREQ])
     return uniform;
 }
 
-// Frequencies go through the pair kernel in groups of at most kGroupFreq slots of
-// the processing order; the kernel is instantiated for up to that many.
-constexpr int kGroupFreq = 8;
 
 // Kernel parameters shared by the forward, counting and adjoint launches, for the
 // frequency group that starts at processing slot g0 (fperm maps the group's slots to
 // user frequency indices).
 FwdParams make_pair_params(const TraceDev &td, const SceneDev &sd, const gbt_sum_args &a,
-                           const float *rec, int g0 = 0)
+                           const float *rec, int g0 = 0, bool adjoint = false)
 {
     FwdParams q{};
     q.recv = a.recv; q.order = a.recv_order; q.n_recv = a.n_recv;
@@ -2455,20 +1462,23 @@ FwdParams make_pair_params(const TraceDev &td, const SceneDev &sd, const gbt_sum
         FreqConst &c = q.fc[f];
         c.K_hi = (float)K;
         c.K_lo = (float)(K - (double)c.K_hi);
-        c.halfK = (float)(0.5 * K);
         c.kb2 = (float)(0.5 * k * b);
-        c.kb2l2e = (float)(0.5 * k * b * 1.4426950408889634);
-        c.b = (float)b;
         c.b2 = (float)(b * b);
-        c.scale = (float)(k * b / (8.0 * kPi * kPi));
-        c.kh = (float)(0.5 * k);
         c.invb = (float)(1.0 / b);
-        c.al2e = (float)(a.absorption[g] * 1.4426950408889634);
+        c.b = (float)b;
+        c.nkh = (float)(-0.5 * k);
+        const double unit = adjoint ? 1.0 : b;      // the pass's unit of length for s
+        c.hK = (float)(0.5 * K / unit);
+        c.ne = (float)(-0.5 * k * b * 1.4426950408889634 / (unit * unit));
+        c.rc = (float)(a.cutoff * unit * unit / (0.5 * k * b));
+        c.sA = (float)(k * b / (8.0 * kPi * kPi) / unit);
+        c.nal = (float)(-a.absorption[g] * 1.4426950408889634 * unit);
         amin = std::min(amin, 0.5 * k * b);
         bmax = std::max(bmax, b * b);
         kmax = std::max(kmax, K);
     }
     q.kmax_turns = (float)kmax;
+    q.s_scale = (q.uniform_b && !adjoint) ? (float)(1.0 / a.beam_b[0]) : 1.0f;
     q.pre_alpha = (float)(amin / (a.cutoff + 1.0));
     q.pre_beta = (float)bmax;
     q.status = status_word();
@@ -2727,7 +1737,7 @@ size_t sum_workspace_bytes(const TraceDev &td, const gbt_sum_args &a, int splits
 }
 
 void sum_launch(const TraceDev &td, const SceneDev &sd, const gbt_sum_args &a, int splits,
-                void *work, cudaStream_t s, unsigned long long *stats)
+                void *work, cudaStream_t s, unsigned long long *stats, bool differentiable)
 {
     char *w = static_cast<char *>(work);
     float *rec = reinterpret_cast<float *>(w);
@@ -2753,11 +1763,7 @@ void sum_launch(const TraceDev &td, const SceneDev &sd, const gbt_sum_args &a, i
     rp.out = reinterpret_cast<float2 *>(a.out);
     rp.accumulate = a.accumulate;
     rp.splits = splits;
-    auto reduce = [&]() {
-        reduce_kernel<<<(unsigned)((rp.n + 255) / 256), 256, 0, s>>>(rp);
-        note_launches(1);
-        GBT_CUDA(cudaGetLastError());
-    };
+    rp.order = a.recv_order;
     if (a.precision == GBT_PRECISION_F64) {
         F64Params q{};
         q.recv = a.recv; q.order = a.recv_order; q.n_recv = a.n_recv;
@@ -2782,13 +1788,13 @@ void sum_launch(const TraceDev &td, const SceneDev &sd, const gbt_sum_args &a, i
         rp.n = (int64_t)a.n_freq * a.n_recv;
         for (int f = 0; f < GBT_MAX_FREQ; ++f) rp.perm[f] = f;
         rp.p64 = reinterpret_cast<double2 *>(partial);
-        reduce();
+        reduce_launch(rp, s);
         return;
     }
     // F32: one pair launch and one merge per group of at most 8 frequencies, each
     // group with its own partials (split-major within the group) and output rows
     for (int g0 = 0; g0 < a.n_freq; g0 += kGroupFreq) {
-        FwdParams q = make_pair_params(td, sd, a, rec, g0);
+        FwdParams q = make_pair_params(td, sd, a, rec, g0, differentiable);
         q.splits = splits;
         q.partial = reinterpret_cast<float4 *>(partial) + (int64_t)splits * g0 * a.n_recv;
         q.stats = stats;
@@ -2797,13 +1803,18 @@ void sum_launch(const TraceDev &td, const SceneDev &sd, const gbt_sum_args &a, i
         q.n_items = cta_tiles(a.n_recv) * kTileWarps * splits;
         q.work_counter = counter;
         tile_prep_launch(q, a.window, tile_ws_layout(order_ws, a.n_recv, td.capacity, a.tile_cull != 0), s);
-        if (a.window == GBT_WINDOW_LINE) launch_fwd_nf<GBT_WINDOW_LINE>(q, s);
-        else launch_fwd_nf<GBT_WINDOW_SEGMENT>(q, s);
-        if (stats) continue;
+        if (stats) {
+            if (a.window == GBT_WINDOW_LINE) launch_count_nf<GBT_WINDOW_LINE>(q, s);
+            else launch_count_nf<GBT_WINDOW_SEGMENT>(q, s);
+            continue;
+        }
+        if (differentiable) pair_field_launch(q, a.window, s, true);
+        else pair_fwd_launch(q, a.window, s, true);
         rp.n = (int64_t)q.nf * a.n_recv;
         for (int f = 0; f < GBT_MAX_FREQ; ++f) rp.perm[f] = q.fperm[f];
+        for (int f = 0; f < q.nf; ++f) rp.scale[f] = differentiable ? 1.0f : q.fc[f].sA;
         rp.p32 = q.partial;
-        reduce();
+        reduce_launch(rp, s);
     }
 }
 
@@ -2930,7 +1941,7 @@ void bwd_launch(const TraceDev &td, const SceneDev &sd, const gbt_sum_args &a,
     if (a.n_recv > 0) {
         const int splits = choose_splits(td, a);
         for (int g0 = 0; g0 < a.n_freq; g0 += kGroupFreq) {
-            FwdParams q = make_pair_params(td, sd, a, rec, g0);
+            FwdParams q = make_pair_params(td, sd, a, rec, g0, true);
             q.splits = splits;
             q.n_items = cta_tiles(a.n_recv) * kTileWarps * splits;
             q.work_counter = counter;
@@ -2941,8 +1952,7 @@ void bwd_launch(const TraceDev &td, const SceneDev &sd, const gbt_sum_args &a,
             q.seg_rf = static_cast<const float2 *>(loss);
             q.rf_stride = td.capacity;
             tile_prep_launch(q, a.window, tile_ws_layout(w + off[6], a.n_recv, td.capacity, a.tile_cull != 0), s);
-            if (a.window == GBT_WINDOW_LINE) launch_fwd_nf<GBT_WINDOW_LINE>(q, s);
-            else launch_fwd_nf<GBT_WINDOW_SEGMENT>(q, s);
+            pair_bwd_launch(q, a.window, s, true);
         }
     }
     int fperm[GBT_MAX_FREQ];
@@ -2983,37 +1993,10 @@ void bwd_launch(const TraceDev &td, const SceneDev &sd, const gbt_sum_args &a,
 
 // ------------------------------------------------------------ batched --
 
-// Many (trace, sum arguments) instances in one persistent launch: one global
-// work counter over the items of all instances (instances ordered by cost,
-// longest first), each CTA loading the item's instance parameters.
-template <int NF, int WINDOW>
-int batched_prepare()
-{
-    using Cfg = PairCfg<NF, kFwd, true>;
-    const size_t smem = Cfg::kSmem;
-    GBT_CUDA(cudaFuncSetAttribute(gbs_fwd_kernel<NF, WINDOW, kFwd, true>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    int per_sm = 0;
-    GBT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &per_sm, gbs_fwd_kernel<NF, WINDOW, kFwd, true>, 32 * Cfg::kWarps, smem));
-    if (per_sm < 1) fail(GBT_ERR_UNSUPPORTED, "GBS kernel does not fit on one SM");
-    return per_sm;
-}
-
-template <int NF, int WINDOW>
-void batched_launch(const FwdParams &prm, int grid, cudaStream_t s)
-{
-    GBT_CUDA(cudaMemsetAsync(prm.work_counter, 0, sizeof(int), s));
-    using Cfg = PairCfg<NF, kFwd, true>;
-    gbs_fwd_kernel<NF, WINDOW, kFwd, true><<<grid, 32 * Cfg::kWarps, Cfg::kSmem, s>>>(prm);
-    note_launches(1);
-    GBT_CUDA(cudaGetLastError());
-}
-
-typedef int (*BatchedPrepFn)();
+// Many (trace, sum arguments) instances in one persistent launch (pair_batched.cu), or each
+// on its own kernels over a few branch streams.
 enum { kFused = 0, kConcurrent = 1 };      // how a batch executes
 constexpr int kBranches = 4;               // branch streams of a concurrent batch
-typedef void (*BatchedLaunchFn)(const FwdParams &, int, cudaStream_t);
 
 struct BatchImpl {
     std::vector<const gbt_trace_t *> traces;
@@ -3031,7 +2014,6 @@ struct BatchImpl {
     int64_t *d_off = nullptr;
     int grid = 1;
     int nf_max = 1, window = 0;
-    BatchedLaunchFn launch = nullptr;
     bool use_graph = false;
     cudaStream_t capture_stream = nullptr;   // private stream the graph is recorded on
     cudaGraph_t graph = nullptr;
@@ -3161,14 +2143,14 @@ static void batch_reduce(BatchImpl &B, int k, cudaStream_t s)
     rp.n = (int64_t)a.n_freq * a.n_recv;
     rp.n_recv = a.n_recv;
     for (int f = 0; f < GBT_MAX_FREQ; ++f) rp.perm[f] = B.table[k].fperm[f];
+    for (int f = 0; f < a.n_freq; ++f) rp.scale[f] = B.table[k].fc[f].sA;
     rp.splits = B.splits[i];
     rp.p32 = reinterpret_cast<float4 *>(static_cast<char *>(B.work) + B.part_off[i]);
     rp.p64 = nullptr;
+    rp.order = a.recv_order;
     rp.out = reinterpret_cast<float2 *>(a.out);
     rp.accumulate = a.accumulate;
-    reduce_kernel<<<(unsigned)((rp.n + 255) / 256), 256, 0, s>>>(rp);
-    note_launches(1);
-    GBT_CUDA(cudaGetLastError());
+    reduce_launch(rp, s);
 }
 
 // Concurrent form: instances (longest first) dealt round-robin to branch streams
@@ -3202,8 +2184,7 @@ static void batch_record_concurrent(BatchImpl &B, cudaStream_t s)
                              tile_ws_layout(w + B.ord_off[i], B.args[i].n_recv,
                                             B.traces[i]->d.capacity, B.args[i].tile_cull != 0), bs);
         }
-        if (B.window == GBT_WINDOW_LINE) launch_fwd_nf<GBT_WINDOW_LINE>(q, bs, false);
-        else launch_fwd_nf<GBT_WINDOW_SEGMENT>(q, bs, false);
+        pair_fwd_launch(q, B.window, bs, false);
         batch_reduce(B, k, bs);
     }
     for (int j = 0; j < nb; ++j) {
@@ -3234,7 +2215,7 @@ static void batch_record(BatchImpl &B, cudaStream_t s)
     prm.n_inst = n;
     prm.n_items = B.inst_off.back();
     prm.work_counter = B.counter;
-    B.launch(prm, B.grid, s);
+    pair_batched_launch(prm, B.nf_max, B.window, B.grid, s);
     for (int k = 0; k < n; ++k) batch_reduce(B, k, s);
 }
 
@@ -3284,20 +2265,7 @@ BatchImpl *batch_create(const gbt_batch_desc &d, cudaStream_t s)
         for (int i = 0; i < n; ++i) B->order[i] = i;
         std::stable_sort(B->order.begin(), B->order.end(),
                          [&](int x, int y) { return B->cost[x] > B->cost[y]; });
-        int per_sm = 1;
-        BatchedPrepFn prep = nullptr;
-        const int nf = B->nf_max <= 1 ? 1 : B->nf_max <= 2 ? 2 : B->nf_max <= 4 ? 4 : 8;
-#define GBT_PICK(NFV)                                                                     \
-    if (nf == NFV) {                                                                      \
-        prep = B->window == GBT_WINDOW_LINE ? batched_prepare<NFV, GBT_WINDOW_LINE>       \
-                                            : batched_prepare<NFV, GBT_WINDOW_SEGMENT>;   \
-        B->launch = B->window == GBT_WINDOW_LINE ? batched_launch<NFV, GBT_WINDOW_LINE>   \
-                                                 : batched_launch<NFV, GBT_WINDOW_SEGMENT>; \
-    }
-        GBT_PICK(1) GBT_PICK(2) GBT_PICK(4) GBT_PICK(8)
-#undef GBT_PICK
-        per_sm = prep();
-        B->grid = per_sm * num_sms();
+        B->grid = pair_batched_prepare(B->nf_max, B->window) * num_sms();
         // candidates: the concurrent form, then the fused launch at a few work
         // granularities (items per resident CTA); 0 items marks the concurrent form
         auto plan = [&](double ips) {

@@ -168,7 +168,8 @@ bool has_losses(const gbt_sum_args &a);
 size_t sum_workspace_bytes(const TraceDev &td, const gbt_sum_args &a, int splits);
 int choose_splits(const TraceDev &td, const gbt_sum_args &a);
 void sum_launch(const TraceDev &td, const SceneDev &sd, const gbt_sum_args &a, int splits,
-                void *work, cudaStream_t s, unsigned long long *stats = nullptr);
+                void *work, cudaStream_t s, unsigned long long *stats = nullptr,
+                bool differentiable = false);   // with the adjoint's own evaluation (F32)
 void recv_order_launch(const float *recv, int64_t n, int32_t *order, void *scratch,
                        cudaStream_t s);
 size_t recv_order_scratch_bytes(int64_t n);

@@ -1,0 +1,496 @@
+// pair.cuh -- the FP32 pair kernel: beams of Eq. 1 / Eq. 2 summed over (receiver, segment,
+// frequency), forward and adjoint.
+//
+// Every warp works on its own.  It takes (warp tile of 64 receivers, segment split) items
+// from a global queue (CTA tiles of 960 receivers heaviest first), collects the segments
+// whose beams can reach the warp tile's ball, and evaluates each of them for its 64
+// receivers, two per lane in paired FP32 (f32x2).  Where the segments come from:
+//  * a tile list (the pre-cull): the warp reads its own 32-bit word of 32 list chunks at
+//    once and gathers the entries whose bit is set;
+//  * no list: the warp tests the 32-byte cull records of four chunks of 32 segments at a
+//    time against its ball.  About 35 instructions per 32 segments, where a test of every
+//    (receiver, segment) pair took 15 per segment.
+// Gathered records arrive by per-lane cp.async, double buffered, and each lane stages one.
+//
+// What bounds it: operand reads.  On this chip an FFMA2 with three operand pairs of its own
+// issues every 3.1 cycles (2.1 when it shares one with its neighbour, as in a mul2 or add2),
+// and ALU, MUFU and shared loads add to that instead of hiding behind it (an FFMA2 and a
+// LOP3: 4.9 cycles); more warps or longer chains change little.  So the number of operands
+// per pair is what counts.
+//  * The frame is the centre of the warp tile's bounding box, x = c + x'.  The staging forms
+//    per segment A = (c - o).t and S = s0 + A in float-float, the compensated
+//    N = (c - o) x t, and per band the phase of S reduced to one turn, so a pair needs
+//      u = x'.t,  s = S + u,  n = N + x' x t
+//    and the phase K u + phi_f, reduced by adding and subtracting 1.5 x 2^23: no
+//    float-float arithmetic per pair (32 paired operations with one band, where float-float
+//    geometry and phase took 63).
+//  * u in FP32 is within about 3 x 2^-24 |x'| of x'.t, which moves the phase by at most
+//    3 x 2^-24 x 16 turns = 1.8e-5 rad where K max|x'| <= kFastTurns.  Beyond that, and for
+//    the segments that have an end of their window inside the warp tile's ball (about one
+//    in five on the city), u = Um + Uc: x' and t are split on grids of 11 and 12 bits of
+//    their largest magnitude, so the three products of Um and their sum are exact in FP32,
+//    and Uc holds the rest to about 2^-36 |x'|.  Nine products, where float-float sums took
+//    31 operations; window decisions are then those of the exact arithmetic to 1e-10 m.
+//    Which of the two a segment takes is uniform over the warp.
+//  * Every sum of the phase is rounded near its smallest size (whole turns go before and
+//    after the second term): against 64 bits the relative L2 error of the open plane with 6
+//    bands is 2.5e-7 (float-float phases 2.9e-7), of scattered receivers 3.7e-7 (4.7e-7), of
+//    8 bands on the city 2.5e-7 to 2.8e-7 (2.5e-7 to 2.9e-7).
+//  * The amplitude's common factor k / (8 pi^2) is left to the merge, the pairs' cutoff test
+//    is one comparison (r <= rc), and receivers past the last are computed and not stored.
+// Summation: FP32 per lane and batch group, folded every kFoldEvery batches into the item's
+// float-float partials, merged in split order by reduce_kernel, so results do not depend on
+// scheduling.
+// Measured (kernel alone, before -> after): city, 1,048,576 rays x 512^2 receivers, lists:
+// 31.0 -> 17.4 ms; open plane, 65,536 rays x 256^2 x 6 bands, no lists: 6.04 -> 1.92 ms;
+// city, 65,536 rays x 200^2 x 2 bands, no lists: 6.79 -> 1.6 ms.
+#pragma once
+
+#include "pair_stream.cuh"
+
+namespace gbt {
+namespace {
+
+// K max|x'| up to which u is plain FP32.  The split form everywhere costs the 1M-ray city
+// step 5 % (26.6 against 25.4 ms) and brings the small open plane's error from 4.3e-7 to
+// 1.9e-7; up to this line the plain form's error stays under that of MUFU sine and cosine.
+constexpr float kFastTurns = 16.0f;
+
+// Shape by the number of band slots: segments evaluated together (plain, and of the second
+// class), bands per vote, and warps.  One band needs several segments for independent
+// chains and shared operands (1M-ray city step: one segment, 16 warps 27.4 ms; two 26.0;
+// four, 12 warps 25.1); two or more bands have the chains themselves.  Bands in pairs spare
+// votes where most bands are kept (open plane, 6 bands: 2.06 -> 1.94 ms), and cost where
+// few are or the losses take the registers (9,973 scattered receivers, 3 bands: 0.72 ->
+// 0.76 ms; 8 bands with losses: 10.25 -> 10.43 ms).
+template <int NF, bool LOSSY>
+struct PairShape {
+    static constexpr int NS = NF == 1 ? 4 : 1, NP = NF == 1 ? 2 : 1;
+    static constexpr int FG = NF >= 6 && !LOSSY ? 2 : 1;
+    static constexpr int kWarps = NF == 1 ? 12 : 16;
+};
+
+// Per-warp shared memory: the raw records and the staged batch, every value in both halves of
+// a float pair (a segment is shared by the warp, so the operands of the paired arithmetic are
+// broadcast loads).  Segments sit in slots: those whose u is plain FP32 first, then the
+// others, padded to whole groups with a slot of zero amplitude.
+template <int NF, bool LOSSY>
+struct WarpBuf {
+    static constexpr int kSlots = kBatch + 1;   // padding
+    RawBuf in;
+    // D[0] t.x, t.y | D[1] t.z, S (times s_scale) | D[2] N.x, N.y | D[3] N.z, amplitude |
+    // D[4..6] t on its grid (3) and the rest (3)
+    float4 D[7][kSlots];
+    float4 W[kSlots];               // SEGMENT: A, A - L as (hi, lo); LINE: S as (hi, lo)
+    float4 F[(NF + 1) / 2][kSlots]; // bands 2 i, 2 i + 1: phase of S in turns
+    float4 R[LOSSY ? (NF + 1) / 2 : 1][LOSSY ? kSlots : 1];   // and amplitude with the losses
+};
+
+// A lane's two receivers relative to the frame, as float pairs: x', -x', x' on its grid, the
+// rest.
+struct LaneRecv {
+    f2x X, Y, Z, NX, NY, NZ, XH, YH, ZH, XL, YL, ZL;
+};
+
+// Adds the beams of the staged slots j .. j + NS - 1 to the lane's two receivers' sums per
+// band.  `cross`: slots with an end of their window inside the warp tile's ball.
+template <int NF, int WINDOW, bool LOSSY, bool PREC, int NS, int FG>
+__device__ __forceinline__ void eval_segments(const FwdParams &p, const WarpBuf<NF, LOSSY> &w,
+                                              int j, uint64_t cross, const LaneRecv &x,
+                                              f2x (&ax)[NF], f2x (&ay)[NF])
+{
+    const f2x MAGIC = splat(12582912.0f), ONE = splat(1.0f);
+    f2x U[NS], UC[NS], s[NS], nn[NS], amp[NS];
+    bool k0[NS], k1[NS];
+    auto word = [&](int d, int q, f2x &a, f2x &b) {
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(&w.D[d][j + q]);
+        a = v.x;
+        b = v.y;
+    };
+#pragma unroll
+    for (int q = 0; q < NS; ++q) {
+        k0[q] = k1[q] = true;
+        f2x TX, TY, TZ, S, NX, NY, NZ;
+        word(0, q, TX, TY);
+        word(1, q, TZ, S);
+        word(2, q, NX, NY);
+        word(3, q, NZ, amp[q]);
+        f2x u;
+        if (PREC) {
+            f2x HX, HY, HZ, LX, LY, LZ;
+            word(4, q, HX, HY);
+            word(5, q, HZ, LX);
+            word(6, q, LY, LZ);
+            U[q] = fma2(x.XH, HX, fma2(x.YH, HY, mul2(x.ZH, HZ)));            // exact
+            UC[q] = fma2(x.XL, TX, fma2(x.YL, TY, fma2(x.ZL, TZ,
+                    fma2(x.XH, LX, fma2(x.YH, LY, mul2(x.ZH, LZ))))));
+            u = add2(U[q], UC[q]);
+            if ((cross >> (j + q)) & 1u) {
+                const float4 e = w.W[j + q];
+                float a0, a1;
+                upk(add2(add2(splat(e.x), U[q]), add2(splat(e.y), UC[q])), a0, a1);
+                k0[q] = a0 >= 0.0f;
+                k1[q] = a1 >= 0.0f;
+                if (WINDOW == GBT_WINDOW_SEGMENT) {
+                    upk(add2(add2(splat(e.z), U[q]), add2(splat(e.w), UC[q])), a0, a1);
+                    k0[q] = k0[q] && a0 < 0.0f;
+                    k1[q] = k1[q] && a1 < 0.0f;
+                }
+            }
+        } else {
+            U[q] = u = fma2(x.X, TX, fma2(x.Y, TY, mul2(x.Z, TZ)));
+        }
+        s[q] = fma2(u, splat(p.s_scale), S);
+        // n = N + x' x t
+        const f2x nx = fma2(x.Y, TZ, fma2(x.NZ, TY, NX));
+        const f2x ny = fma2(x.Z, TX, fma2(x.NX, TZ, NY));
+        const f2x nz = fma2(x.X, TY, fma2(x.NY, TX, NZ));
+        nn[q] = fma2(nx, nx, fma2(ny, ny, mul2(nz, nz)));
+    }
+    // FG bands at a time, one vote for each group: their chains interleave
+    f2x sc[NS][FG], nsc[NS][FG], AD[NS][FG], r[NS][FG], rs[NS][FG];
+#pragma unroll
+    for (int f0 = 0; f0 < NF; f0 += FG) {
+        if (NF > 1 && f0 >= p.nf) break;
+        bool m0[NS][FG], m1[NS][FG], any = false;
+#pragma unroll
+        for (int i = 0; i < FG; ++i) {
+            const int f = f0 + i;
+            const FreqConst &c = p.fc[f];
+            const bool live = NF == 1 || FG == 1 || f < p.nf;
+#pragma unroll
+            for (int q = 0; q < NS; ++q) {
+                if (f == 0 || !p.uniform_b) {
+                    sc[q][i] = (NF == 1 || p.uniform_b) ? s[q] : mul2(splat(c.invb), s[q]);
+                    nsc[q][i] = neg2(sc[q][i]);
+                    float d0, d1;
+                    upk(fma2(sc[q][i], sc[q][i], ONE), d0, d1);
+                    const f2x invD = pk(rcp_approx(d0), rcp_approx(d1));
+                    r[q][i] = mul2(nn[q], invD);
+                    rs[q][i] = mul2(r[q][i], sc[q][i]);
+                    AD[q][i] = LOSSY ? invD : mul2(amp[q], invD);
+                } else if (i > 0) {
+                    sc[q][i] = sc[q][0]; nsc[q][i] = nsc[q][0]; AD[q][i] = AD[q][0];
+                    r[q][i] = r[q][0]; rs[q][i] = rs[q][0];
+                }
+                float r0, r1;
+                upk(r[q][i], r0, r1);
+                m0[q][i] = live && (PREC ? k0[q] && r0 <= c.rc : r0 <= c.rc);
+                m1[q][i] = live && (PREC ? k1[q] && r1 <= c.rc : r1 <= c.rc);
+                any = any || m0[q][i] || m1[q][i];
+            }
+        }
+        // narrower bands keep no more (one b: the kept bands are a prefix); a compact warp's
+        // only band seldom misses all its receivers
+        if ((NF > 1 || PREC) && !__any_sync(0xffffffffu, any)) {
+            if (NF == 1 || p.uniform_b) break;
+            continue;
+        }
+#pragma unroll
+        for (int i = 0; i < FG; ++i) {
+            const int f = f0 + i;
+            const FreqConst &c = p.fc[f];
+#pragma unroll
+            for (int q = 0; q < NS; ++q) {
+                const ulonglong2 pp = *reinterpret_cast<const ulonglong2 *>(&w.F[f / 2][j + q]);
+                f2x g = AD[q][i];
+                if (LOSSY) {
+                    const ulonglong2 ra = *reinterpret_cast<const ulonglong2 *>(&w.R[f / 2][j + q]);
+                    g = mul2(f & 1 ? ra.y : ra.x, g);
+                }
+                f2x ex = mul2(splat(c.ne), r[q][i]);
+                if (LOSSY) ex = fma2(splat(c.nal), sc[q][i], ex);
+                float e0, e1;
+                upk(ex, e0, e1);
+                g = mul2(g, pk(m0[q][i] ? ex2_approx(e0) : 0.0f, m1[q][i] ? ex2_approx(e1) : 0.0f));
+                const f2x KH = splat(c.K_hi);
+                f2x ph = f & 1 ? pp.y : pp.x, tau;
+                if (PREC || NF > 1) ph = fma2(splat(c.K_lo), U[q], ph);
+                if (PREC) ph = fma2(KH, UC[q], ph);
+                if (NF == 1) {
+                    // K u + ph less its whole turns, ph with the second term
+                    ph = fma2(splat(c.hK), rs[q][i], ph);
+                    const f2x nr = sub2(MAGIC, add2(fma2(KH, U[q], ph), MAGIC));
+                    tau = add2(fma2(KH, U[q], nr), ph);
+                } else {
+                    // less whole turns before and after the second term: every sum is rounded
+                    // near its smallest size
+                    const f2x nr = sub2(MAGIC, fma2(KH, U[q], MAGIC));
+                    tau = fma2(splat(c.hK), rs[q][i], add2(fma2(KH, U[q], nr), ph));
+                    tau = add2(tau, sub2(MAGIC, add2(tau, MAGIC)));
+                }
+                float t0, t1, sn0, cs0, sn1, cs1;
+                upk(mul2(splat(-6.283185307179586f), tau), t0, t1);
+                __sincosf(t0, &sn0, &cs0);
+                __sincosf(t1, &sn1, &cs1);
+                const f2x NSN = pk(sn0, sn1), CS = pk(cs0, cs1);                // -sin, cos
+                ax[f] = fma2(g, fma2(sc[q][i], CS, NSN), ax[f]);
+                ay[f] = fma2(g, fma2(nsc[q][i], NSN, CS), ay[f]);
+            }
+        }
+    }
+}
+
+// Slots of a staged batch: [0, n_plain) with u in FP32, [n_plain, end) with the split one, and
+// which slots may have an end of their window inside the ball.
+struct StagedBatch {
+    int n_plain, end;
+    uint64_t cross;
+};
+
+// Stages the batch's raw records (a lane each) in the frame c, for the 64 receivers within rad
+// of it: see WarpBuf.  A segment is of the second class where the warp is not compact
+// (`fast`) or an end of its window may lie inside the ball (a margin of 1 mm covers the
+// rounding of the float-float heads).
+template <int NF, int WINDOW, bool LOSSY, int NS, int NP>
+__device__ __forceinline__ StagedBatch stage(const FwdParams &p, WarpBuf<NF, LOSSY> &w, int lane,
+                                             int nrec, int buf, int32_t seg, float cx, float cy,
+                                             float cz, float rad, bool fast)
+{
+    const bool have = lane < nrec;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4 r0 = have ? w.in.raw[buf][0][lane] : zero, r1 = have ? w.in.raw[buf][1][lane] : zero;
+    const float4 r2 = have ? w.in.raw[buf][2][lane] : zero, r3 = have ? w.in.raw[buf][3][lane] : zero;
+    const float amp = have ? w.in.amp[buf][lane] : 0.0f;
+    // d = c - o as (dh + dl)
+    float dxh, dxe, dyh, dye, dzh, dze;
+    two_sum(cx, -r0.x, dxh, dxe);
+    two_sum(cy, -r0.y, dyh, dye);
+    two_sum(cz, -r0.z, dzh, dze);
+    const float dxl = __fsub_rn(dxe, r2.x), dyl = __fsub_rn(dye, r2.y), dzl = __fsub_rn(dze, r2.z);
+    // A = d.t, float-float
+    const float q0 = __fmul_rn(dxh, r1.x), q1 = __fmul_rn(dyh, r1.y), q2 = __fmul_rn(dzh, r1.z);
+    const float e0 = fmaf(dxh, r3.x, fmaf(dxl, r1.x, fmaf(dxh, r1.x, -q0)));
+    const float e1 = fmaf(dyh, r3.y, fmaf(dyl, r1.y, fmaf(dyh, r1.y, -q1)));
+    const float e2 = fmaf(dzh, r3.z, fmaf(dzl, r1.z, fmaf(dzh, r1.z, -q2)));
+    float S1, E1, Ah, E2;
+    two_sum(q0, q1, S1, E1);
+    two_sum(S1, q2, Ah, E2);
+    const float Al = __fadd_rn(__fadd_rn(E1, E2), __fadd_rn(__fadd_rn(e0, e1), e2));
+    // S = s0 + A
+    float Sh, es;
+    two_sum(r0.w, Ah, Sh, es);
+    const float Sl = __fadd_rn(es, __fadd_rn(Al, r2.w));
+    bool cross;
+    float4 W;
+    if (WINDOW == GBT_WINDOW_SEGMENT) {
+        float ALh, ea;
+        two_sum(Ah, -r1.w, ALh, ea);
+        const float ALl = __fadd_rn(ea, __fsub_rn(Al, r3.w));
+        W = make_float4(Ah, Al, ALh, ALl);
+        cross = !(Ah - rad >= 1e-3f && ALh + rad <= -1e-3f);
+    } else {
+        W = make_float4(Sh, Sl, 0.f, 0.f);
+        cross = !(Sh - rad >= 1e-3f);
+    }
+    // slots: whole groups of NS plain segments first, then the others (the last few plain ones
+    // among them), padded to whole groups of NP with slots of zero amplitude
+    const uint32_t xm = __ballot_sync(0xffffffffu, have && cross);
+    const uint32_t all = nrec < 32 ? (1u << nrec) - 1u : 0xffffffffu;
+    const uint32_t below = (1u << lane) - 1u;
+    uint32_t plain = fast ? all & ~xm : 0u;
+    StagedBatch b;
+    b.n_plain = __popc(plain) / NS * NS;
+#pragma unroll
+    for (int q = 1; q < NS; ++q)
+        if (__popc(plain) > b.n_plain) plain &= plain - 1u;
+    b.end = nrec;
+    b.cross = fast ? ~0ull : (uint64_t)xm;     // compact warps: every segment of the second class
+    const bool mine_plain = (plain >> lane) & 1u;
+    const int slot = mine_plain ? __popc(plain & below) : b.n_plain + __popc(all & ~plain & below);
+    // N = d x t, compensated
+    const float nx = dop(dyh, r1.z, dzh, r1.y) +
+                     fmaf(dyh, r3.z, fmaf(-dzh, r3.y, fmaf(dyl, r1.z, -dzl * r1.y)));
+    const float ny = dop(dzh, r1.x, dxh, r1.z) +
+                     fmaf(dzh, r3.x, fmaf(-dxh, r3.z, fmaf(dzl, r1.x, -dxl * r1.z)));
+    const float nz = dop(dxh, r1.y, dyh, r1.x) +
+                     fmaf(dxh, r3.y, fmaf(-dyh, r3.x, fmaf(dxl, r1.y, -dyl * r1.x)));
+    // one band: t times K / K_hi, so that K_hi u is K u (K_lo u would move the phase of every
+    // term alike, by up to 45 x 2^-25 turns); several bands add K_lo u each
+    const float ks = NF == 1 ? p.fc[0].K_lo * rcp_approx(p.fc[0].K_hi) : 0.0f;
+    const float tx = fmaf(r1.x, ks, r3.x) + r1.x, ty = fmaf(r1.y, ks, r3.y) + r1.y,
+                tz = fmaf(r1.z, ks, r3.z) + r1.z;
+    if (have) {
+        w.D[0][slot] = dup2(tx, ty);
+        w.D[1][slot] = dup2(tz, Sh * p.s_scale);
+        w.D[2][slot] = dup2(nx, ny);
+        w.D[3][slot] = dup2(nz, amp);
+        if (!mine_plain) {
+            // t rounded to multiples of 2^-12 (by 1.5 x 2^11, whose ulp that is), and the rest
+            const float hx = __fsub_rn(__fadd_rn(r1.x, 3072.f), 3072.f);
+            const float hy = __fsub_rn(__fadd_rn(r1.y, 3072.f), 3072.f);
+            const float hz = __fsub_rn(__fadd_rn(r1.z, 3072.f), 3072.f);
+            w.D[4][slot] = dup2(hx, hy);
+            w.D[5][slot] = dup2(hz, __fadd_rn(__fsub_rn(r1.x, hx), r3.x));
+            w.D[6][slot] = dup2(__fadd_rn(__fsub_rn(r1.y, hy), r3.y), __fadd_rn(__fsub_rn(r1.z, hz), r3.z));
+            w.W[slot] = W;
+        }
+    }
+#pragma unroll
+    for (int f0 = 0; f0 < NF; f0 += 2) {
+        float phi[2] = {0.f, 0.f}, a[2] = {0.f, 0.f};
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int f = f0 + i;
+            if (f >= NF || (NF > 1 && f >= p.nf)) continue;
+            const FreqConst &c = p.fc[f];
+            const float ph = __fmul_rn(c.K_hi, Sh);
+            const float pe = fmaf(c.K_hi, Sh, -ph);                    // exact
+            phi[i] = __fsub_rn(ph, rintf(ph)) + fmaf(c.K_hi, Sl, fmaf(c.K_lo, Sh, pe));
+            if (LOSSY && have) {
+                const float2 rf = p.seg_rf[(int64_t)p.fperm[f] * p.rf_stride + seg];
+                phi[i] += rf.y;
+                a[i] = amp * exp2f(rf.x);
+            }
+        }
+        if (have) {
+            w.F[f0 / 2][slot] = dup2(phi[0], phi[1]);
+            if (LOSSY) w.R[f0 / 2][slot] = dup2(a[0], a[1]);
+        }
+    }
+    if (NP > 1 && lane < (NP - (b.end - b.n_plain) % NP) % NP) {
+        const int q = b.end + lane;
+#pragma unroll
+        for (int d = 0; d < 7; ++d) w.D[d][q] = zero;
+        w.W[q] = zero;
+#pragma unroll
+        for (int f0 = 0; f0 < NF; f0 += 2) {
+            w.F[f0 / 2][q] = zero;
+            if (LOSSY) w.R[f0 / 2][q] = zero;
+        }
+    }
+    return b;
+}
+
+template <int NF, int WINDOW, bool BATCHED, bool LOSSY>
+__global__ void __launch_bounds__(32 * PairCfg<WarpBuf<NF, LOSSY>, BATCHED, PairShape<NF, LOSSY>::kWarps>::kWarps, 1) gbs_pair_kernel(const __grid_constant__ FwdParams prm)
+{
+    using Cfg = PairCfg<WarpBuf<NF, LOSSY>, BATCHED, PairShape<NF, LOSSY>::kWarps>;
+    static_assert(!(LOSSY && BATCHED), "batches with losses run the single-sum kernel");
+    using Shape = PairShape<NF, LOSSY>;
+    constexpr int NS = Shape::NS, NP = Shape::NP, FG = Shape::FG;
+    static_assert(NF % FG == 0 && NS <= 4, "whole band groups");
+    static_assert(NP <= 2, "one padding slot");
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned char *const mine = smem_raw + (size_t)warp * Cfg::kPerWarp;
+    WarpBuf<NF, LOSSY> &B = *reinterpret_cast<WarpBuf<NF, LOSSY> *>(mine);
+    FwdParams &inst = *reinterpret_cast<FwdParams *>(mine + sizeof(WarpBuf<NF, LOSSY>));
+
+    for (;;) {
+        int64_t it = 0;
+        if (lane == 0) it = atomicAdd(prm.work_counter, 1);
+        it = __shfl_sync(0xffffffffu, it, 0);
+        if (it >= prm.n_items) break;
+        if (BATCHED) {
+            int lo = 0, hi = prm.n_inst - 1;      // last instance with inst_off <= it
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (prm.inst_off[mid] <= it) lo = mid;
+                else hi = mid - 1;
+            }
+            it -= prm.inst_off[lo];
+            __syncwarp();
+            const int4 *src = reinterpret_cast<const int4 *>(prm.inst + lo);
+            int4 *dst = reinterpret_cast<int4 *>(&inst);
+            for (int q = lane; q < (int)(sizeof(FwdParams) / 16); q += 32) dst[q] = src[q];
+            __syncwarp();
+        }
+        const FwdParams &p = BATCHED ? inst : prm;
+        Item item;
+        if (!decode_item(p, it, item)) continue;
+
+        // the lane's receivers: lane and lane + 32 of the warp tile, the two halves of its
+        // Morton patch, so a beam edge splits work evenly over lanes
+        float xr[kR], yr[kR], zr[kR];
+        bool valid[kR];
+        unsigned bb[6] = {~0u, ~0u, ~0u, 0u, 0u, 0u};
+#pragma unroll
+        for (int k = 0; k < kR; ++k) {
+            const int64_t r = item.wbase + (int64_t)k * 32 + lane;
+            valid[k] = r < p.n_recv;
+            xr[k] = yr[k] = zr[k] = 0.0f;
+            if (valid[k]) {
+                const int64_t o = p.order ? p.order[r] : r;
+                xr[k] = p.recv[3 * o]; yr[k] = p.recv[3 * o + 1]; zr[k] = p.recv[3 * o + 2];
+                const unsigned ux = ordered_bits(xr[k]), uy = ordered_bits(yr[k]), uz = ordered_bits(zr[k]);
+                bb[0] = min(bb[0], ux); bb[1] = min(bb[1], uy); bb[2] = min(bb[2], uz);
+                bb[3] = max(bb[3], ux); bb[4] = max(bb[4], uy); bb[5] = max(bb[5], uz);
+            }
+        }
+        f2x ax[NF], ay[NF];     // FP32 sums of the two receivers, per band
+#pragma unroll
+        for (int f = 0; f < NF; ++f) ax[f] = ay[f] = 0ull;
+        // frame: the centre c of the bounding box; rad bounds |x'|
+        float ctr[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const float lo = from_ordered(__reduce_min_sync(0xffffffffu, bb[a]));
+            const float hi = from_ordered(__reduce_max_sync(0xffffffffu, bb[3 + a]));
+            ctr[a] = 0.5f * lo + 0.5f * hi;
+        }
+        const float cx = ctr[0], cy = ctr[1], cz = ctr[2];
+        float xp[kR], yp[kR], zp[kR], xl[kR], yl[kR], zl[kR], xx = 0.0f;
+#pragma unroll
+        for (int k = 0; k < kR; ++k) {
+            xp[k] = yp[k] = zp[k] = xl[k] = yl[k] = zl[k] = 0.0f;
+            if (valid[k]) {
+                two_sum(xr[k], -cx, xp[k], xl[k]);
+                two_sum(yr[k], -cy, yp[k], yl[k]);
+                two_sum(zr[k], -cz, zp[k], zl[k]);
+                xx = fmaxf(xx, fmaf(xp[k], xp[k], fmaf(yp[k], yp[k], zp[k] * zp[k])));
+            }
+        }
+        const float rad = 1.000001f * sqrtf(__uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(xx))));
+        const bool fast = rad * p.kmax_turns <= kFastTurns;
+        // grid of x': a power of two q with |x'| <= 2^11 q, by adding 1.5 x 2^23 q
+        const float grid = rad > 1e-25f ? scalbnf(12582912.0f, (int)ceilf(log2f(rad) + 1e-5f) - 11) : 0.0f;
+        LaneRecv x;
+        {
+            float h[3][kR];
+#pragma unroll
+            for (int k = 0; k < kR; ++k) {
+                h[0][k] = __fsub_rn(__fadd_rn(xp[k], grid), grid);
+                h[1][k] = __fsub_rn(__fadd_rn(yp[k], grid), grid);
+                h[2][k] = __fsub_rn(__fadd_rn(zp[k], grid), grid);
+                xl[k] = __fadd_rn(__fsub_rn(xp[k], h[0][k]), xl[k]);
+                yl[k] = __fadd_rn(__fsub_rn(yp[k], h[1][k]), yl[k]);
+                zl[k] = __fadd_rn(__fsub_rn(zp[k], h[2][k]), zl[k]);
+            }
+            x.X = pk(xp[0], xp[1]); x.Y = pk(yp[0], yp[1]); x.Z = pk(zp[0], zp[1]);
+            x.NX = neg2(x.X); x.NY = neg2(x.Y); x.NZ = neg2(x.Z);
+            x.XH = pk(h[0][0], h[0][1]); x.YH = pk(h[1][0], h[1][1]); x.ZH = pk(h[2][0], h[2][1]);
+            x.XL = pk(xl[0], xl[1]); x.YL = pk(yl[0], yl[1]); x.ZL = pk(zl[0], zl[1]);
+        }
+        const float4 rball = reach_ball(make_float4(cx, cy, cz, rad));
+
+        float4 *const part = p.partial + (int64_t)item.split * p.nf * p.n_recv + item.wbase + lane;
+        bool first = true;
+        auto fold_all = [&]() { fold_bands<NF>(p, part, valid, ax, ay, first); };
+
+        Gather<WINDOW, false> g(item);
+        g.issue(p, item, B.in, lane, rball, 0);
+        g.issue(p, item, B.in, lane, rball, 1);
+        for (uint32_t kb = 0;; ++kb) {
+            const int buf = (int)(kb & 1u);
+            const int nrec = buf ? g.n1 : g.n0;
+            if (nrec <= 0) break;
+            cp_async_wait1();   // this lane's copies of batch kb
+            const StagedBatch b = stage<NF, WINDOW, LOSSY, NS, NP>(p, B, lane, nrec, buf, buf ? g.seg1 : g.seg0,
+                                                                   cx, cy, cz, rad, fast);
+            __syncwarp();       // the batch is staged
+            g.issue(p, item, B.in, lane, rball, buf);   // batch kb + 2 into the buffer just read
+            for (int j = 0; j < b.n_plain; j += NS)
+                eval_segments<NF, WINDOW, LOSSY, false, NS, FG>(p, B, j, 0ull, x, ax, ay);
+            for (int j = b.n_plain; j < b.end; j += NP)
+                eval_segments<NF, WINDOW, LOSSY, true, NP, FG>(p, B, j, b.cross, x, ax, ay);
+            if ((kb % kFoldEvery) == kFoldEvery - 1) fold_all();
+            __syncwarp();        // before the next batch is staged over this one
+        }
+        cp_async_wait0();        // every gather of this item has landed
+        fold_all();
+    }
+}
+
+}  // namespace
+}  // namespace gbt

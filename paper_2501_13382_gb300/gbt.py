@@ -106,6 +106,7 @@ _SIGS = {
                                    C.c_void_p, C.POINTER(C.c_void_p)]),
     "gbt_trace_destroy": (C.c_int, [C.c_void_p]),
     "gbt_sum": (C.c_int, [C.c_void_p, C.POINTER(gbt_sum_args), C.c_void_p]),
+    "gbt_sum_differentiable": (C.c_int, [C.c_void_p, C.POINTER(gbt_sum_args), C.c_void_p]),
     "gbt_synthesize": (C.c_int, [C.c_void_p, C.c_int32, C.c_int64, C.c_void_p, C.c_void_p,
                                  C.c_double, C.c_double, C.c_int64, C.c_void_p, C.c_int32,
                                  C.c_void_p]),
@@ -217,6 +218,11 @@ def gbt_trace_destroy(trace: int):
 
 def gbt_sum(trace: int, args: gbt_sum_args, stream: int = 0):
     _check(load().gbt_sum(C.c_void_p(trace), C.byref(args), C.c_void_p(stream)), "gbt_sum")
+
+
+def gbt_sum_differentiable(trace: int, args: gbt_sum_args, stream: int = 0):
+    _check(load().gbt_sum_differentiable(C.c_void_p(trace), C.byref(args), C.c_void_p(stream)),
+           "gbt_sum_differentiable")
 
 
 def gbt_air_absorption(freqs, temperature_c: float = 20.0, humidity_pct: float = 70.0,
@@ -568,14 +574,8 @@ def _check_out(out, nf: int, nr: int):
     _require(tuple(out.shape) == (nf, nr), f"out must have shape ({nf}, {nr})")
 
 
-def gbs_sum(trace: Trace, recv, freqs, beam_b, gamma, ray_weight=None, order=None,
-            window: int = WINDOW_LINE, cutoff: float = 16.0, precision: int = PRECISION_F32,
-            out=None, accumulate: bool = False, seg_split: int = 0, tile_cull: bool = False,
-            absorption=None, flow_resistivity=None):
-    """Complex pressure p[f, r] (torch complex64 on the device).  absorption: per-frequency
-    amplitude decay rate of air (Np/m, see air_absorption); flow_resistivity: float32 CUDA
-    tensor of per-material flow resistivities (kPa s m^-2, <= 0 hard).  Asynchronous:
-    problems a kernel detects (a bounded wait that ran out) surface at gbt_sync."""
+def _sum(call, trace: Trace, recv, freqs, beam_b, gamma, ray_weight, order, window, cutoff, precision,
+         out, accumulate, seg_split, tile_cull, absorption, flow_resistivity):
     import torch
     _check_tensors(recv, gamma, ray_weight, order, trace.scene.n_materials, trace.n_fan)
     _check_sigma(flow_resistivity, trace.scene.n_materials)
@@ -586,8 +586,29 @@ def gbs_sum(trace: Trace, recv, freqs, beam_b, gamma, ray_weight=None, order=Non
     a = sum_args(recv, freqs, beam_b, gamma, out, ray_weight, order, window, cutoff, precision,
                  accumulate, seg_split, tile_cull=tile_cull, absorption=absorption,
                  flow_resistivity=flow_resistivity)
-    gbt_sum(trace.handle, a, _stream_ptr())
+    call(trace.handle, a, _stream_ptr())
     return out
+
+
+def gbs_sum(trace: Trace, recv, freqs, beam_b, gamma, ray_weight=None, order=None,
+            window: int = WINDOW_LINE, cutoff: float = 16.0, precision: int = PRECISION_F32,
+            out=None, accumulate: bool = False, seg_split: int = 0, tile_cull: bool = False,
+            absorption=None, flow_resistivity=None):
+    """Complex pressure p[f, r] (torch complex64 on the device).  absorption: per-frequency
+    amplitude decay rate of air (Np/m, see air_absorption); flow_resistivity: float32 CUDA
+    tensor of per-material flow resistivities (kPa s m^-2, <= 0 hard).  Asynchronous:
+    problems a kernel detects (a bounded wait that ran out) surface at gbt_sync."""
+    return _sum(gbt_sum, trace, recv, freqs, beam_b, gamma, ray_weight, order, window, cutoff,
+                precision, out, accumulate, seg_split, tile_cull, absorption, flow_resistivity)
+
+
+def gbs_sum_differentiable(trace: Trace, recv, freqs, beam_b, gamma, ray_weight=None, order=None,
+                           window: int = WINDOW_LINE, cutoff: float = 16.0, tile_cull: bool = False,
+                           absorption=None, flow_resistivity=None):
+    """gbs_sum with the very beams that gbs_sum_backward recomputes (gbt_sum_differentiable)."""
+    return _sum(gbt_sum_differentiable, trace, recv, freqs, beam_b, gamma, ray_weight, order,
+                window, cutoff, PRECISION_F32, None, False, 0, tile_cull, absorption,
+                flow_resistivity)
 
 
 def sum_stats(trace: Trace, recv, freqs, beam_b, gamma, ray_weight=None, order=None,

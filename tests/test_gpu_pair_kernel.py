@@ -1,0 +1,63 @@
+"""The forward pair kernel at the sizes where it can go wrong: edges of warp tiles (64
+receivers) and CTA tiles (960), ragged segment batches, every band-slot instantiation, one
+and several beam parameters, compact warps (the FP32 projection) and scattered ones (the
+split projection), with a segment list and without; and the differentiable sum beside it.
+
+Tolerance: a term's phase moves by at most 3 x 2^-24 x 90 turns = 1.0e-4 rad (the FP32
+projection of the differentiable sum at its limit) and its amplitude by a few 2^-22 (MUFU),
+independently from term to term, so 1e-4 bounds the relative L2 error also where terms cancel mildly."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2501_13382_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-4
+
+
+def _receivers(kind, n, seed):
+    rng = np.random.default_rng(seed)
+    if kind == "compact":           # a lattice of 2 m near the source's street
+        k = int(np.ceil(np.sqrt(n)))
+        g = 2.0 * (np.arange(k) - k / 2)
+        xx, yy = np.meshgrid(g, g)
+        return np.stack([xx.ravel(), yy.ravel(), np.full(k * k, 1.5)], 1)[:n].astype(np.float32)
+    return I.random_receivers(rng, n, (-200.0, -200.0, 1.0), (200.0, 200.0, 20.0))
+
+
+@pytest.mark.parametrize("kind,n,rays,nf,uniform,window,cull", [
+    ("compact", 1, 257, 1, True, I.WINDOW_SEGMENT, False),
+    ("compact", 63, 300, 2, True, I.WINDOW_SEGMENT, True),
+    ("compact", 65, 301, 3, False, I.WINDOW_LINE, False),
+    ("compact", 959, 500, 4, True, I.WINDOW_SEGMENT, False),
+    ("compact", 961, 333, 6, False, I.WINDOW_SEGMENT, True),
+    ("scatter", 64, 1023, 1, True, I.WINDOW_SEGMENT, False),
+    ("scatter", 200, 700, 2, False, I.WINDOW_SEGMENT, False),
+    ("scatter", 961, 512, 5, True, I.WINDOW_LINE, True),
+    ("scatter", 1921, 400, 8, True, I.WINDOW_SEGMENT, False),
+    ("scatter", 130, 900, 7, False, I.WINDOW_SEGMENT, True),
+])
+def test_pair_kernel_edges(kind, n, rays, nf, uniform, window, cull):
+    import torch
+    from paper_2501_13382_gb300 import gbt as G
+    sc0, _ = I.city_scene(I.SEED_BASE + 3)
+    src = I.Source(np.array([0.3, -0.2, 3.0]), rays, 4, 600.0)
+    recv = _receivers(kind, n, rays)
+    freqs = list(125.0 * 2.0 ** (np.arange(nf) * (5.0 / max(nf - 1, 1))))[::-1]
+    b = [40.0] * nf if uniform else [20.0 + 9.0 * f for f in range(nf)]
+    ot = O.trace(sc0, src)
+    po = O.gbs_sum(ot, recv, freqs, b, sc0.c, sc0.gamma, window=window)
+    sc = G.Scene(sc0)
+    tr = G.Trace(sc, src)
+    r = torch.as_tensor(recv, device="cuda")
+    gam = torch.as_tensor(sc0.gamma, device="cuda")
+    args = (tr, r, freqs, b, gam)
+    for order in (None, G.recv_order(r)):
+        p = G.gbs_sum(*args, order=order, window=window, tile_cull=cull)
+        q = G.gbs_sum_differentiable(*args, order=order, window=window, tile_cull=cull)
+        torch.cuda.synchronize()
+        G.gbt_sync()
+        for got in (p, q):
+            e = got.cpu().numpy().astype(np.complex128) - po
+            assert np.linalg.norm(e) <= TOL * np.linalg.norm(po)
