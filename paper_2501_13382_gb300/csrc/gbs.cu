@@ -400,52 +400,12 @@ struct PrepParams {
     // F64 path records (nullptr when not needed)
     double *amp64;
     unsigned int *status;
-    // losses: per-material flow resistivity (kPa s m^-2, <= 0 hard) or nullptr, the
-    // primitives that end the segments, the scene's triangles (unit normal at 9..11)
-    const float *sigma;
-    const int32_t *hit;
-    const double *tri;
-    int64_t n_tri;
-    int nf;
-    double freq[GBT_MAX_FREQ];
-    float2 *seg_rf;            // [f][rf_stride] (log2 |R|, arg R / 2 pi), or nullptr
-    double2 *seg_r64;          // [f][rf_stride] R for the F64 path, or nullptr
-    int64_t rf_stride;
 };
 
 __device__ __forceinline__ void split_ff(double v, float &hi, float &lo)
 {
     hi = (float)v;
     lo = (float)(v - (double)hi);
-}
-
-// Cosine of the angle of incidence at the reflection that starts segment j (depth >= 1):
-// |t_j . n| with n the unit normal of the primitive that ended segment j - 1 (ground:
-// +z); a mirror reflection keeps |d . n|.  An unknown primitive is flagged.
-__device__ __forceinline__ double incidence_cos(const PrepParams &p, int64_t j)
-{
-    const int prim = p.hit[j - 1];
-    double nx = 0.0, ny = 0.0, nz = 1.0;
-    if (prim >= 1 && prim <= p.n_tri) {
-        const double *n = p.tri + 12 * (int64_t)(prim - 1) + 9;
-        nx = n[0]; ny = n[1]; nz = n[2];
-    } else if (prim != 0) {
-        atomicOr(p.status, STATUS_BAD_INPUT);
-    }
-    return fabs(p.t[3 * j] * nx + p.t[3 * j + 1] * ny + p.t[3 * j + 2] * nz);
-}
-
-// Plane-wave reflection factor of a porous, locally reacting surface of flow resistivity
-// sigma (kPa s m^-2) at frequency f for incidence cos(theta) = c: the Delany-Bazley
-// normalised impedance Z = 1 + 9.08 (f/sigma)^-0.75 + i 11.9 (f/sigma)^-0.73
-// (exp(-i omega t)) in R = (Z c - 1) / (Z c + 1).
-__device__ __forceinline__ double2 porous_reflection(double f, double sigma, double c)
-{
-    const double x = f / sigma;
-    const double zr = 1.0 + 9.08 * pow(x, -0.75), zi = 11.9 * pow(x, -0.73);
-    const double ar = zr * c - 1.0, ai = zi * c, br = zr * c + 1.0, bi = zi * c;
-    const double inv = 1.0 / (br * br + bi * bi);
-    return make_double2((ar * br + ai * bi) * inv, (ai * br - ar * bi) * inv);
 }
 
 __global__ void prepass_kernel(PrepParams p)
@@ -482,29 +442,88 @@ __global__ void prepass_kernel(PrepParams p)
     p.crec[2 * j] = R[0];
     p.crec[2 * j + 1] = R[1];
     if (p.amp64) p.amp64[j] = amp;
-    if (p.seg_rf || p.seg_r64) {
-        // per frequency: the product of the porous reflections' factors before segment j
-        for (int f = 0; f < p.nf; ++f) {
-            double rr = 1.0, ri = 0.0;
-            if (p.sigma) {
-                for (int q = 1; q <= dep; ++q) {
-                    const int64_t jq = j - dep + q;
-                    const int m = p.bmat[jq];
-                    if (m < 0 || m >= p.n_materials) continue;     // flagged above
-                    const double sg = (double)p.sigma[m];
-                    if (!(sg > 0.0)) continue;                      // hard surface
-                    const double2 r = porous_reflection(p.freq[f], sg, incidence_cos(p, jq));
-                    const double nr = rr * r.x - ri * r.y;
-                    ri = rr * r.y + ri * r.x;
-                    rr = nr;
-                }
+}
+
+// ---- losses of porous surfaces
+struct LossParams {
+    const int32_t *ray_off;
+    int64_t n_rays;
+    const double *t;
+    const int32_t *bmat, *hit;
+    const float *sigma;        // per material, kPa s m^-2 (<= 0 hard), or nullptr: all hard
+    const double *tri;         // the scene's triangles (unit normal at 9..11)
+    int64_t n_tri;
+    int n_materials, nf;
+    double freq[GBT_MAX_FREQ];
+    double2 *z;                // [f][material] impedance
+    float2 *seg_rf;            // [f][rf_stride] (log2 |R|, arg R / 2 pi), or nullptr
+    double2 *seg_r64;          // [f][rf_stride] R for the F64 path, or nullptr
+    int64_t rf_stride;
+    unsigned int *status;
+};
+
+// Normalised impedance of a porous, locally reacting surface of flow resistivity sigma
+// (kPa s m^-2) at frequency f, Delany-Bazley for exp(-i omega t):
+// Z = 1 + 9.08 (f/sigma)^-0.75 + i 11.9 (f/sigma)^-0.73.  Once per (band, material): the two
+// pow() of a bounce were most of the prepass (8 bands, 448,870 segments: 4.45 ms).
+__global__ void porous_impedance_kernel(LossParams p)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= p.nf * p.n_materials) return;
+    const double sg = (double)p.sigma[i % p.n_materials];
+    if (!(sg > 0.0)) return;
+    const double x = p.freq[i / p.n_materials] / sg;
+    p.z[i] = make_double2(1.0 + 9.08 * pow(x, -0.75), 11.9 * pow(x, -0.73));
+}
+
+// Cosine of the angle of incidence at the reflection that starts segment j (depth >= 1):
+// |t_j . n| with n the unit normal of the primitive that ended segment j - 1 (ground:
+// +z); a mirror reflection keeps |d . n|.  An unknown primitive is flagged.
+__device__ __forceinline__ double incidence_cos(const LossParams &p, int64_t j)
+{
+    const int prim = p.hit[j - 1];
+    double nx = 0.0, ny = 0.0, nz = 1.0;
+    if (prim >= 1 && prim <= p.n_tri) {
+        const double *n = p.tri + 12 * (int64_t)(prim - 1) + 9;
+        nx = n[0]; ny = n[1]; nz = n[2];
+    } else if (prim != 0) {
+        atomicOr(p.status, STATUS_BAD_INPUT);
+    }
+    return fabs(p.t[3 * j] * nx + p.t[3 * j + 1] * ny + p.t[3 * j + 2] * nz);
+}
+
+// One thread per (ray, band) walks the ray's segments with the product of the plane-wave
+// reflection factors R = (Z c - 1) / (Z c + 1) of its porous reflections so far; the F32
+// path keeps their logarithms and arguments as running sums, one logarithm and arctangent
+// per porous bounce instead of one per segment.  Bound by FP64 issue.
+__global__ void __launch_bounds__(128) porous_path_kernel(LossParams p)
+{
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= p.n_rays) return;
+    const int f = blockIdx.y;
+    const int32_t a = p.ray_off[i], e = p.ray_off[i + 1];
+    double rr = 1.0, ri = 0.0, lg = 0.0, turns = 0.0;
+    for (int32_t j = a; j < e; ++j) {
+        const int m = j > a ? p.bmat[j] : -1;
+        if (p.sigma && m >= 0 && m < p.n_materials && p.sigma[m] > 0.0f) {
+            const double2 z = p.z[f * p.n_materials + m];
+            const double c = incidence_cos(p, j);
+            const double ar = z.x * c - 1.0, ai = z.y * c, br = z.x * c + 1.0;
+            const double inv = 1.0 / (br * br + ai * ai);
+            const double x = (ar * br + ai * ai) * inv, y = (ai * br - ar * ai) * inv;
+            if (p.seg_rf) {
+                lg += 0.5 * log2(x * x + y * y);
+                turns += atan2(y, x) * (0.5 / kPi);
+                turns -= rint(turns);
+            } else {
+                const double nr = rr * x - ri * y;
+                ri = rr * y + ri * x;
+                rr = nr;
             }
-            const int64_t k = (int64_t)f * p.rf_stride + j;
-            if (p.seg_rf)
-                p.seg_rf[k] = make_float2((float)(0.5 * log2(rr * rr + ri * ri)),
-                                          (float)(atan2(ri, rr) * (0.5 / kPi)));
-            if (p.seg_r64) p.seg_r64[k] = make_double2(rr, ri);
         }
+        const int64_t k = (int64_t)f * p.rf_stride + j;
+        if (p.seg_rf) p.seg_rf[k] = make_float2((float)lg, (float)turns);
+        else p.seg_r64[k] = make_double2(rr, ri);
     }
 }
 
@@ -1496,12 +1515,14 @@ bool has_losses(const gbt_sum_args &a)
 }
 
 // Per (frequency, segment) loss factors of a sum: (log2 |R|, arg R / 2 pi) floats for the
-// F32 path, complex doubles for the F64 path; none without losses.
+// F32 path, complex doubles for the F64 path; then the impedance per (frequency, material);
+// none without losses.
 static size_t loss_bytes(const TraceDev &td, const gbt_sum_args &a)
 {
     if (!has_losses(a)) return 0;
     const size_t per = a.precision == GBT_PRECISION_F64 ? sizeof(double2) : sizeof(float2);
-    return align_up((size_t)a.n_freq * (size_t)td.capacity * per, 256);
+    return align_up((size_t)a.n_freq * (size_t)td.capacity * per, 256) +
+           align_up((size_t)a.n_freq * (size_t)td.scene->d.n_materials * sizeof(double2), 256);
 }
 
 int choose_splits(const TraceDev &td, const gbt_sum_args &a)
@@ -1707,19 +1728,37 @@ static void prepass_launch(const TraceDev &td, const SceneDev &sd, const gbt_sum
     pp.crec = cull_records(rec, td.capacity);
     pp.amp64 = amp64;
     pp.status = status_word();
-    if (loss) {
-        pp.sigma = a.flow_resistivity;
-        pp.hit = td.hit;
-        pp.tri = sd.tri;
-        pp.n_tri = sd.n_tri;
-        pp.nf = a.n_freq;
-        for (int f = 0; f < a.n_freq; ++f) pp.freq[f] = a.freq_hz[f];
-        pp.rf_stride = td.capacity;
-        if (a.precision == GBT_PRECISION_F64) pp.seg_r64 = static_cast<double2 *>(loss);
-        else pp.seg_rf = static_cast<float2 *>(loss);
-    }
     prepass_kernel<<<(unsigned)((td.capacity + 255) / 256), 256, 0, s>>>(pp);
     note_launches(1);
+    if (loss) {
+        LossParams lp{};
+        lp.ray_off = td.ray_off;
+        lp.n_rays = td.n_rays;
+        lp.t = td.t;
+        lp.bmat = td.bmat;
+        lp.hit = td.hit;
+        lp.sigma = a.flow_resistivity;
+        lp.tri = sd.tri;
+        lp.n_tri = sd.n_tri;
+        lp.n_materials = sd.n_materials;
+        lp.nf = a.n_freq;
+        for (int f = 0; f < a.n_freq; ++f) lp.freq[f] = a.freq_hz[f];
+        lp.rf_stride = td.capacity;
+        lp.status = status_word();
+        const bool f64 = a.precision == GBT_PRECISION_F64;
+        if (f64) lp.seg_r64 = static_cast<double2 *>(loss);
+        else lp.seg_rf = static_cast<float2 *>(loss);
+        lp.z = reinterpret_cast<double2 *>(
+            static_cast<char *>(loss) +
+            align_up((size_t)a.n_freq * (size_t)td.capacity * (f64 ? sizeof(double2) : sizeof(float2)), 256));
+        const int nz = a.n_freq * sd.n_materials;
+        if (lp.sigma) {
+            porous_impedance_kernel<<<(unsigned)((nz + 63) / 64), 64, 0, s>>>(lp);
+            note_launches(1);
+        }
+        porous_path_kernel<<<dim3((unsigned)((td.n_rays + 127) / 128), (unsigned)a.n_freq), 128, 0, s>>>(lp);
+        note_launches(1);
+    }
     GBT_CUDA(cudaGetLastError());
 }
 
