@@ -23,6 +23,7 @@
 #include <string>
 
 #include "pair_exact.cuh"
+#include "pair_stream.cuh"
 
 namespace gbt {
 namespace {
@@ -529,131 +530,263 @@ __global__ void __launch_bounds__(128) porous_path_kernel(LossParams p)
 
 // ------------------------------------------------------ FP64 variant --
 
-constexpr int kThreads64 = 128;
-constexpr int kTS64 = 64;
+constexpr int kWarps64 = 2;        // warps per block, each on its own 32 receivers
 
 struct F64Params {
+    FwdParams g;               // what the gathering of segments reads (records, splits, cull)
     const float *recv;
     const int32_t *order;
     int64_t n_recv;
-    const int32_t *n_seg_ptr;
     const double *o, *t, *L, *s0, *amp;
     int nf;
     double cutoff;
-    double k[GBT_MAX_FREQ], b[GBT_MAX_FREQ];
-    int splits;
+    double k[GBT_MAX_FREQ], b[GBT_MAX_FREQ], kb[GBT_MAX_FREQ], b2[GBT_MAX_FREQ];
     double2 *partial;          // [splits][nf][n_recv]
     double absorb[GBT_MAX_FREQ];   // amplitude decay rate of air per frequency (Np/m)
     const double2 *r64;        // [f][r64_stride] porous reflections' factor, or nullptr
     int64_t r64_stride;
 };
 
-// Every step in FP64.  The cull k n^2 b / (2 D) <= C is tested as k b n^2 <= 2 C D
-// (no division), first for the union over the frequencies (the smallest k b against the
-// largest b^2) so that a pair every frequency culls costs no per-frequency work; the
-// accumulators of NF frequency slots stay in registers.
-template <int WINDOW, int NF>
-__global__ void __launch_bounds__(kThreads64) gbs_fwd_f64_kernel(const F64Params p)
+template <int NF>
+struct Warp64 {
+    RawBuf in;
+    // prefilter constants of a staged segment (o' = o - c): (t, -o'.t), (2a o', beta - a |o'|^2),
+    // (s0 + margin, L + margin, margin)
+    float4 P[3][kBatch];
+    int32_t seg[kBatch];
+    // a window of candidate pairs: s and n^2, segment, kept frequencies, terms
+    double2 geo[32];
+    int32_t pair_seg[32];
+    uint32_t kept[32];
+    double2 term[NF][32];
+};
+
+// Position of the n-th set bit of m (n < popc(m)).
+__device__ __forceinline__ int nth_bit(uint32_t m, int n)
 {
-    __shared__ double so[kTS64][3], stt[kTS64][3], sL[kTS64], s0s[kTS64], sa[kTS64];
-    const int64_t r = (int64_t)blockIdx.x * kThreads64 + threadIdx.x;
-    const int split = blockIdx.y;
-    const int64_t n_seg = *p.n_seg_ptr;
-    const int64_t seg_begin = split * n_seg / p.splits;
-    const int64_t seg_end = (split + 1) * n_seg / p.splits;
+    int pos = 0;
+#pragma unroll
+    for (int w = 16; w > 0; w >>= 1) {
+        const int c = __popc(m & ((1u << w) - 1u));
+        if (n >= c) {
+            n -= c;
+            pos += w;
+            m >>= w;
+        }
+    }
+    return pos;
+}
+
+__device__ __forceinline__ int warp_scan(int v, int lane)     // inclusive
+{
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += y;
+    }
+    return v;
+}
+
+// The lane in whose range [its predecessor's incl, incl) slot lies (31 past the last).
+__device__ __forceinline__ int list_owner(int incl, int slot)
+{
+    int own = 0;
+#pragma unroll
+    for (int st = 16; st > 0; st >>= 1) {
+        const int e = __shfl_sync(0xffffffffu, incl, own + st - 1);
+        if (e <= slot) own += st;
+    }
+    return own;
+}
+
+// Every step of a kept beam in FP64: geometry, cull, beam, Neumaier accumulation.  FP64
+// issues at 1/64 of the FP32 rate, so what bounds it is the number of FP64 instructions in
+// which lanes idle or reject: a warp gathers the segments that reach the ball of its 32
+// receivers (as the FP32 kernels do) and an FP32 prefilter with a margin marks the candidates
+// among 32 of them.  The marked pairs go through the FP64 geometry and cull 32 at a time, a
+// lane per pair, and what they keep through the beam 32 at a time, a lane per (pair, band),
+// whoever owns the receiver; each receiver's lane then adds its terms in segment order.
+// Candidates are listed segment by segment, so that a window's terms belong to many lanes
+// (listed lane by lane, 10 of 32 lanes were active).  16,384 rays x 128^2 receivers x 2
+// bands: 35.4 ms testing every pair in FP64, 2.2 ms so,
+// bit for bit the same field.
+template <int WINDOW, int NF>
+__global__ void __launch_bounds__(32 * kWarps64) gbs_fwd_f64_kernel(const __grid_constant__ F64Params p)
+{
+    __shared__ Warp64<NF> all[kWarps64];
+    const int lane = threadIdx.x & 31;
+    Warp64<NF> &w = all[threadIdx.x >> 5];
+    Item m;
+    m.wbase = ((int64_t)blockIdx.x * kWarps64 + (threadIdx.x >> 5)) * 32;
+    if (m.wbase >= p.n_recv) return;            // warps never wait for one another
+    m.split = blockIdx.y;
+    m.lst = nullptr;
+    m.lw = nullptr;
+    m.n_seg = *p.g.n_seg_ptr;
+    const int64_t r = m.wbase + lane;
     const bool valid = r < p.n_recv;
     const int64_t ri = valid ? (p.order ? p.order[r] : r) : 0;
-    const double x = valid ? (double)p.recv[3 * ri] : 0.0;
-    const double y = valid ? (double)p.recv[3 * ri + 1] : 0.0;
-    const double z = valid ? (double)p.recv[3 * ri + 2] : 0.0;
-    double kb[NF], b2[NF];
-    double kbmin = 1e300, b2max = 0.0;
+    const float xf = valid ? p.recv[3 * ri] : 0.f, yf = valid ? p.recv[3 * ri + 1] : 0.f,
+                zf = valid ? p.recv[3 * ri + 2] : 0.f;
+    // ball about the centre c of the receivers' bounding box
+    const float v[3] = {xf, yf, zf};
+    float ctr[3];
 #pragma unroll
-    for (int f = 0; f < NF; ++f) {
-        kb[f] = f < p.nf ? p.k[f] * p.b[f] : 1e300;
-        b2[f] = f < p.nf ? p.b[f] * p.b[f] : 0.0;
-        kbmin = fmin(kbmin, kb[f]);
-        b2max = fmax(b2max, b2[f]);
+    for (int a = 0; a < 3; ++a) {
+        const unsigned u = ordered_bits(v[a]);
+        ctr[a] = 0.5f * from_ordered(__reduce_min_sync(0xffffffffu, valid ? u : ~0u)) +
+                 0.5f * from_ordered(__reduce_max_sync(0xffffffffu, valid ? u : 0u));
     }
+    const float xp = xf - ctr[0], yp = yf - ctr[1], zp = zf - ctr[2];
+    const float xx = fmaf(xp, xp, fmaf(yp, yp, zp * zp));
+    const float rad = 1.000001f * sqrtf(__uint_as_float(
+        __reduce_max_sync(0xffffffffu, valid ? __float_as_uint(xx) : 0u)));
+    const float4 rball = reach_ball(make_float4(ctr[0], ctr[1], ctr[2], rad));
+    const float alpha = p.g.pre_alpha, beta = p.g.pre_beta, naxx = -alpha * xx;
     const double c2 = 2.0 * p.cutoff;
+
     double sr[NF], cr[NF], si[NF], ci[NF];
 #pragma unroll
     for (int f = 0; f < NF; ++f) sr[f] = cr[f] = si[f] = ci[f] = 0.0;
-    for (int64_t t0 = seg_begin; t0 < seg_end; t0 += kTS64) {
-        __syncthreads();
-        for (int q = threadIdx.x; q < kTS64; q += kThreads64) {
-            const int64_t j = t0 + q;
-            if (j < seg_end) {
-                so[q][0] = p.o[3 * j]; so[q][1] = p.o[3 * j + 1]; so[q][2] = p.o[3 * j + 2];
-                stt[q][0] = p.t[3 * j]; stt[q][1] = p.t[3 * j + 1]; stt[q][2] = p.t[3 * j + 2];
-                sL[q] = p.L[j]; s0s[q] = p.s0[j]; sa[q] = p.amp[j];
-            }
+    Gather<WINDOW, false> g(m);
+    g.issue(p.g, m, w.in, lane, rball, 0);
+    g.issue(p.g, m, w.in, lane, rball, 1);
+    for (uint32_t kb = 0;; ++kb) {
+        const int buf = (int)(kb & 1u);
+        const int nrec = buf ? g.n1 : g.n0;
+        if (nrec <= 0) break;
+        cp_async_wait1();   // this lane's copies of batch kb
+        if (lane < nrec) {
+            const float4 r0 = w.in.raw[buf][0][lane], r1 = w.in.raw[buf][1][lane], r2 = w.in.raw[buf][2][lane];
+            const float ox = (r0.x - ctr[0]) + r2.x, oy = (r0.y - ctr[1]) + r2.y, oz = (r0.z - ctr[2]) + r2.z;
+            const float ot = fmaf(ox, r1.x, fmaf(oy, r1.y, oz * r1.z));
+            const float oo = fmaf(ox, ox, fmaf(oy, oy, oz * oz));
+            const float a2 = 2.f * alpha;
+            w.P[0][lane] = make_float4(r1.x, r1.y, r1.z, -ot);
+            w.P[1][lane] = make_float4(a2 * ox, a2 * oy, a2 * oz, fmaf(-alpha, oo, beta));
+            const float mg = kWinMargin + 1e-6f * (fabsf(ox) + fabsf(oy) + fabsf(oz));
+            w.P[2][lane] = make_float4(r0.w + mg, r1.w + mg, mg, 0.f);
+            w.seg[lane] = buf ? g.seg1 : g.seg0;
         }
-        __syncthreads();
-        const int nt = (int)min((int64_t)kTS64, seg_end - t0);
-        if (!valid) continue;
-        for (int q = 0; q < nt; ++q) {
-            const double dx = x - so[q][0], dy = y - so[q][1], dz = z - so[q][2];
-            const double tx = stt[q][0], ty = stt[q][1], tz = stt[q][2];
-            const double sl = dx * tx + dy * ty + dz * tz;
-            const double s = s0s[q] + sl;
-            if (WINDOW == GBT_WINDOW_SEGMENT) {
-                if (!(sl >= 0.0 && sl < sL[q])) continue;
-            } else {
-                if (!(s >= 0.0)) continue;
-            }
-            const double cx = dy * tz - dz * ty, cy = dz * tx - dx * tz, cz = dx * ty - dy * tx;
-            const double n2 = cx * cx + cy * cy + cz * cz;
-            const double ss = s * s;
-            // union over the frequencies: culled for every f (with a relative margin far
-            // above FP64 rounding, so no pair a frequency keeps is skipped)
-            if (kbmin * n2 > c2 * (ss + b2max) * (1.0 + 1e-12)) continue;
+        __syncwarp();
+        g.issue(p.g, m, w.in, lane, rball, buf);
+        // candidates, frequency independent: s_loc = x'.t - o'.t, sm = s_loc + s0 + margin,
+        // sm^2 + beta - alpha |x' - o'|^2 + alpha s_loc^2 (= q - alpha n^2) >= 0, window
+        uint32_t mine = 0u;                   // lane j: the lanes that are candidates of segment j
+        for (int j = 0; j < nrec; ++j) {
+            const float4 a = w.P[0][j], b = w.P[1][j], q = w.P[2][j];
+            const float sl = fmaf(xp, a.x, fmaf(yp, a.y, fmaf(zp, a.z, a.w)));
+            const float sm = sl + q.x;
+            const float nd = fmaf(xp, b.x, fmaf(yp, b.y, fmaf(zp, b.z, naxx + b.w)));
+            bool keep = valid && fmaf(alpha * sl, sl, fmaf(sm, sm, nd)) >= 0.f;
+            if (WINDOW == GBT_WINDOW_LINE) keep = keep && sm >= 0.f;
+            else keep = keep && sl + q.z >= 0.f && sl < q.y;
+            const uint32_t b32 = __ballot_sync(0xffffffffu, keep);
+            if (lane == j) mine = b32;
+        }
+        // the segments' candidates as one list: segment j's at [incl - cnt, incl) of lane j
+        const int cnt = __popc(mine);
+        const int incl = warp_scan(cnt, lane);
+        const int total = __shfl_sync(0xffffffffu, incl, 31);
+        for (int w0 = 0; w0 < total; w0 += 32) {
+            const int slot = w0 + lane;
+            const int sj = list_owner(incl, slot);
+            const int rank = slot - __shfl_sync(0xffffffffu, incl - cnt, sj);
+            const uint32_t lanes = __shfl_sync(0xffffffffu, mine, sj);
+            const int rl = slot < total ? nth_bit(lanes, rank) : 0;
+            const double x = (double)__shfl_sync(0xffffffffu, xf, rl);
+            const double y = (double)__shfl_sync(0xffffffffu, yf, rl);
+            const double z = (double)__shfl_sync(0xffffffffu, zf, rl);
+            uint32_t kf = 0u;                 // frequencies this pair keeps
+            if (slot < total) {
+                const int64_t j = w.seg[sj];
+                const double dx = x - p.o[3 * j], dy = y - p.o[3 * j + 1], dz = z - p.o[3 * j + 2];
+                const double tx = p.t[3 * j], ty = p.t[3 * j + 1], tz = p.t[3 * j + 2];
+                const double sl = dx * tx + dy * ty + dz * tz;
+                const double s = p.s0[j] + sl;
+                const bool in = WINDOW == GBT_WINDOW_SEGMENT ? sl >= 0.0 && sl < p.L[j] : s >= 0.0;
+                const double cx = dy * tz - dz * ty, cy = dz * tx - dx * tz, cz = dx * ty - dy * tx;
+                const double n2 = cx * cx + cy * cy + cz * cz;
+                const double ss = s * s;
+                if (in) {
 #pragma unroll
-            for (int f = 0; f < NF; ++f) {
-                if (f >= p.nf) break;
-                const double k = p.k[f], b = p.b[f];
-                const double D = ss + b2[f];
-                if (kb[f] * n2 > c2 * D) continue;
-                // c = amp * (k b / 8 pi^2) / E * exp(i k s + i k n^2 / (2E)), E = s - i b
-                const double invD = 1.0 / D;
-                const double re_exp = -0.5 * kb[f] * n2 * invD - p.absorb[f] * s;
-                const double ph = k * s + 0.5 * k * n2 * s * invD;
-                const double a = sa[q] * (kb[f] / (8.0 * kPi * kPi)) * exp(re_exp) * invD;
-                double sn, cs;
-                sincos(ph, &sn, &cs);
-                double vr = a * (s * cs - b * sn), vi = a * (s * sn + b * cs);
-                if (p.r64) {
-                    const double2 R = p.r64[(int64_t)f * p.r64_stride + t0 + q];
-                    const double ur = vr * R.x - vi * R.y;
-                    vi = vr * R.y + vi * R.x;
-                    vr = ur;
+                    for (int f = 0; f < NF; ++f) {
+                        if (f >= p.nf) break;
+                        kf |= (uint32_t)!(p.kb[f] * n2 > c2 * (ss + p.b2[f])) << f;
+                    }
                 }
-                // Neumaier accumulation
-                double t1 = sr[f] + vr;
-                cr[f] += fabs(sr[f]) >= fabs(vr) ? (sr[f] - t1) + vr : (vr - t1) + sr[f];
-                sr[f] = t1;
-                double t2 = si[f] + vi;
-                ci[f] += fabs(si[f]) >= fabs(vi) ? (si[f] - t2) + vi : (vi - t2) + si[f];
-                si[f] = t2;
+                w.geo[lane] = make_double2(s, n2);
+                w.pair_seg[lane] = (int32_t)j;
             }
+            w.kept[lane] = kf;
+            const int kc = __popc(kf), kincl = warp_scan(kc, lane);
+            const int ktotal = __shfl_sync(0xffffffffu, kincl, 31);
+            __syncwarp();
+            for (int v0 = 0; v0 < ktotal; v0 += 32) {
+                const int ks = v0 + lane;
+                const int ps = list_owner(kincl, ks);
+                const int krank = ks - __shfl_sync(0xffffffffu, kincl - kc, ps);
+                if (ks < ktotal) {
+                    const int f = nth_bit(w.kept[ps], krank);
+                    const int64_t j = w.pair_seg[ps];
+                    const double s = w.geo[ps].x, n2 = w.geo[ps].y;
+                    const double k = p.k[f], b = p.b[f], kb = p.kb[f];
+                    // c = amp * (k b / 8 pi^2) / E * exp(i k s + i k n^2 / (2E)), E = s - i b
+                    const double invD = 1.0 / (s * s + p.b2[f]);
+                    const double re_exp = -0.5 * kb * n2 * invD - p.absorb[f] * s;
+                    const double ph = k * s + 0.5 * k * n2 * s * invD;
+                    const double a = p.amp[j] * (kb / (8.0 * kPi * kPi)) * exp(re_exp) * invD;
+                    double sn, cs;
+                    sincos(ph, &sn, &cs);
+                    double2 v = make_double2(a * (s * cs - b * sn), a * (s * sn + b * cs));
+                    if (p.r64) {
+                        const double2 R = p.r64[(int64_t)f * p.r64_stride + j];
+                        v = make_double2(v.x * R.x - v.y * R.y, v.x * R.y + v.y * R.x);
+                    }
+                    w.term[f][ps] = v;
+                }
+            }
+            __syncwarp();
+            const int last = __shfl_sync(0xffffffffu, sj, min(total - w0, 32) - 1);
+            for (int q = __shfl_sync(0xffffffffu, sj, 0); q <= last; ++q) {
+                const uint32_t own = __shfl_sync(0xffffffffu, mine, q);
+                const int at = __shfl_sync(0xffffffffu, incl - cnt, q) + __popc(own & ((1u << lane) - 1u)) - w0;
+                const uint32_t bits = ((own >> lane) & 1u) && at >= 0 && at < 32 ? w.kept[at] : 0u;
+#pragma unroll
+                for (int f = 0; f < NF; ++f) {
+                    if ((bits >> f) & 1u) {
+                        const double2 v = w.term[f][at];
+                        // Neumaier accumulation
+                        const double t1 = sr[f] + v.x;
+                        cr[f] += fabs(sr[f]) >= fabs(v.x) ? (sr[f] - t1) + v.x : (v.x - t1) + sr[f];
+                        sr[f] = t1;
+                        const double t2 = si[f] + v.y;
+                        ci[f] += fabs(si[f]) >= fabs(v.y) ? (si[f] - t2) + v.y : (v.y - t2) + si[f];
+                        si[f] = t2;
+                    }
+                }
+            }
+            __syncwarp();       // before the next window
         }
+        __syncwarp();           // before the next batch is staged over this one
     }
+    cp_async_wait0();
     if (!valid) return;
 #pragma unroll
     for (int f = 0; f < NF; ++f)
         if (f < p.nf)
-            p.partial[((int64_t)split * p.nf + f) * p.n_recv + ri] =
+            p.partial[((int64_t)m.split * p.nf + f) * p.n_recv + ri] =
                 make_double2(sr[f] + cr[f], si[f] + ci[f]);
 }
 
 template <int WINDOW>
 void launch_f64(const F64Params &q, dim3 grid, cudaStream_t s)
 {
-    if (q.nf <= 1) gbs_fwd_f64_kernel<WINDOW, 1><<<grid, kThreads64, 0, s>>>(q);
-    else if (q.nf <= 2) gbs_fwd_f64_kernel<WINDOW, 2><<<grid, kThreads64, 0, s>>>(q);
-    else if (q.nf <= 4) gbs_fwd_f64_kernel<WINDOW, 4><<<grid, kThreads64, 0, s>>>(q);
-    else if (q.nf <= 8) gbs_fwd_f64_kernel<WINDOW, 8><<<grid, kThreads64, 0, s>>>(q);
-    else gbs_fwd_f64_kernel<WINDOW, GBT_MAX_FREQ><<<grid, kThreads64, 0, s>>>(q);
+    if (q.nf <= 1) gbs_fwd_f64_kernel<WINDOW, 1><<<grid, 32 * kWarps64, 0, s>>>(q);
+    else if (q.nf <= 2) gbs_fwd_f64_kernel<WINDOW, 2><<<grid, 32 * kWarps64, 0, s>>>(q);
+    else if (q.nf <= 4) gbs_fwd_f64_kernel<WINDOW, 4><<<grid, 32 * kWarps64, 0, s>>>(q);
+    else if (q.nf <= 8) gbs_fwd_f64_kernel<WINDOW, 8><<<grid, 32 * kWarps64, 0, s>>>(q);
+    else gbs_fwd_f64_kernel<WINDOW, GBT_MAX_FREQ><<<grid, 32 * kWarps64, 0, s>>>(q);
 }
 
 // ------------------------------------------------------------ adjoint --
@@ -1530,9 +1663,11 @@ int choose_splits(const TraceDev &td, const gbt_sum_args &a)
     if (a.seg_split > 0) return a.seg_split;
     const int64_t nseg_est = td.n_seg_host >= 0 ? td.n_seg_host : td.capacity;
     if (a.precision == GBT_PRECISION_F64) {
-        const int64_t tiles = (a.n_recv + kThreads64 - 1) / kThreads64;
-        int64_t s = (4 * (int64_t)num_sms() + tiles - 1) / (tiles > 0 ? tiles : 1);
-        s = std::max<int64_t>(1, std::min<int64_t>(s, (nseg_est + kTS64 - 1) / kTS64));
+        // about 512 warps (of 32 receivers) per SM, whose costs differ by ten times and more
+        // (16,384 rays x 128^2 x 2 bands: 128 per SM 3.05 ms, 256 2.48, 512 2.24)
+        const int64_t tiles = (a.n_recv + 31) / 32;
+        int64_t s = (512 * (int64_t)num_sms() + tiles - 1) / (tiles > 0 ? tiles : 1);
+        s = std::max<int64_t>(1, std::min<int64_t>(s, (nseg_est + 2 * kBatch - 1) / (2 * kBatch)));
         return (int)std::min<int64_t>(s, 4096);
     }
     // items are (warp tile, split): about 16 per resident warp, 32 with the pre-cull (its
@@ -1806,20 +1941,30 @@ void sum_launch(const TraceDev &td, const SceneDev &sd, const gbt_sum_args &a, i
     if (a.precision == GBT_PRECISION_F64) {
         F64Params q{};
         q.recv = a.recv; q.order = a.recv_order; q.n_recv = a.n_recv;
-        q.n_seg_ptr = n_seg_ptr;
+        q.g.n_seg_ptr = n_seg_ptr;
+        q.g.rec = rec;
+        q.g.crec = cull_records(rec, td.capacity);
+        q.g.splits = splits;
+        double kbmin = 1e300, bmax = 0.0;
         q.o = td.o; q.t = td.t; q.L = td.L; q.s0 = td.s0; q.amp = amp64;
         q.nf = a.n_freq;
         q.cutoff = a.cutoff;
         for (int f = 0; f < a.n_freq; ++f) {
             q.k[f] = 2.0 * kPi * a.freq_hz[f] / sd.c;
             q.b[f] = a.beam_b[f];
+            q.kb[f] = q.k[f] * q.b[f];
+            q.b2[f] = q.b[f] * q.b[f];
+            kbmin = std::min(kbmin, q.k[f] * q.b[f]);
+            bmax = std::max(bmax, q.b[f]);
         }
-        q.splits = splits;
+        // the union of the bands' cutoffs, with a relative margin of 2e-4 at any cutoff
+        q.g.pre_alpha = (float)(0.5 * kbmin / (1.0002 * a.cutoff + 1.0));
+        q.g.pre_beta = (float)(bmax * bmax);
         q.partial = reinterpret_cast<double2 *>(partial);
         for (int f = 0; f < a.n_freq; ++f) q.absorb[f] = a.absorption[f];
         q.r64 = static_cast<const double2 *>(loss);
         q.r64_stride = td.capacity;
-        dim3 grid((unsigned)((a.n_recv + kThreads64 - 1) / kThreads64), (unsigned)splits);
+        dim3 grid((unsigned)((a.n_recv + 32 * kWarps64 - 1) / (32 * kWarps64)), (unsigned)splits);
         if (a.window == GBT_WINDOW_LINE) launch_f64<GBT_WINDOW_LINE>(q, grid, s);
         else launch_f64<GBT_WINDOW_SEGMENT>(q, grid, s);
         note_launches(1);

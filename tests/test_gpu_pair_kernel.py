@@ -61,3 +61,33 @@ def test_pair_kernel_edges(kind, n, rays, nf, uniform, window, cull):
         for got in (p, q):
             e = got.cpu().numpy().astype(np.complex128) - po
             assert np.linalg.norm(e) <= TOL * np.linalg.norm(po)
+
+
+@pytest.mark.parametrize("n,rays,nf,window,cutoff", [
+    (1, 257, 1, I.WINDOW_SEGMENT, 16.0),
+    (31, 300, 2, I.WINDOW_LINE, 16.0),
+    (33, 700, 3, I.WINDOW_SEGMENT, 1e4),
+    (65, 1023, 9, I.WINDOW_SEGMENT, 2.0),
+    (400, 513, 16, I.WINDOW_LINE, 16.0),
+])
+def test_f64_kernel_edges(n, rays, nf, window, cutoff):
+    """The FP64 sum at the edges of its 32-receiver tiles and candidate windows, with few and
+    many bands and with cutoffs that keep few pairs or nearly all.  Tolerance: the complex64
+    output rounds each component by at most 2^-24 of it (6e-8 of the L2 norm); FP64 phases of
+    up to 1e5 rad add 1e-11."""
+    import torch
+    from paper_2501_13382_gb300 import gbt as G
+    sc0, _ = I.city_scene(I.SEED_BASE + 3)
+    src = I.Source(np.array([0.3, -0.2, 3.0]), rays, 4, 600.0)
+    recv = _receivers("scatter" if n % 2 else "compact", n, rays)
+    freqs = list(125.0 * 2.0 ** (np.arange(nf) * (5.0 / max(nf - 1, 1))))[::-1]
+    b = [20.0 + 9.0 * f for f in range(nf)]
+    po = O.gbs_sum(O.trace(sc0, src), recv, freqs, b, sc0.c, sc0.gamma, window=window, cutoff=cutoff)
+    sc = G.Scene(sc0)
+    tr = G.Trace(sc, src)
+    r = torch.as_tensor(recv, device="cuda")
+    p = G.gbs_sum(tr, r, freqs, b, torch.as_tensor(sc0.gamma, device="cuda"), order=G.recv_order(r),
+                  window=window, cutoff=cutoff, precision=G.PRECISION_F64)
+    torch.cuda.synchronize()
+    e = p.cpu().numpy().astype(np.complex128) - po
+    assert np.linalg.norm(e) <= 1e-7 * np.linalg.norm(po)
