@@ -448,7 +448,6 @@ gbt_status gbt_scene_create(const gbt_scene_desc *desc, void *stream, gbt_scene_
         try {
             const size_t nt = (size_t)std::max<int64_t>(d.n_tri, 1);
             sd.tri = static_cast<double *>(dalloc(nt * 12 * sizeof(double), s));
-            sd.trif = static_cast<float *>(dalloc(nt * 9 * sizeof(float), s));
             sd.face = static_cast<int32_t *>(dalloc(nt * sizeof(int32_t), s));
             sd.mat = static_cast<int32_t *>(dalloc(nt * sizeof(int32_t), s));
             sd.n_clusters = (d.n_tri + kTriCluster - 1) / kTriCluster;
@@ -501,6 +500,7 @@ gbt_status gbt_scene_create(const gbt_scene_desc *desc, void *stream, gbt_scene_
                     GBT_REQUIRE(sd.bvh_depth + 2 <= kBvhStack, "BVH deeper than the traversal stack");
                     sd.bvh = static_cast<BvhNode *>(dalloc(bb.nodes.size() * sizeof(BvhNode), s));
                     sd.bvh_perm = static_cast<int32_t *>(dalloc(bb.perm.size() * sizeof(int32_t), s));
+                    sd.leaf = static_cast<float4 *>(dalloc(3 * bb.perm.size() * sizeof(float4), s));
                     GBT_CUDA(cudaMemcpyAsync(sd.bvh, bb.nodes.data(), bb.nodes.size() * sizeof(BvhNode),
                                              cudaMemcpyHostToDevice, s));
                     GBT_CUDA(cudaMemcpyAsync(sd.bvh_perm, bb.perm.data(), bb.perm.size() * sizeof(int32_t),
@@ -513,10 +513,11 @@ gbt_status gbt_scene_create(const gbt_scene_desc *desc, void *stream, gbt_scene_
             }
         } catch (...) {
             if (raw) dfree(raw, s);
-            dfree(sd.tri, s); dfree(sd.trif, s); dfree(sd.face, s); dfree(sd.mat, s); dfree(sd.cbox, s);
+            dfree(sd.tri, s); dfree(sd.face, s); dfree(sd.mat, s); dfree(sd.cbox, s);
             dfree(sd.tbox, s);
             if (sd.bvh) dfree(sd.bvh, s);
             if (sd.bvh_perm) dfree(sd.bvh_perm, s);
+            if (sd.leaf) dfree(sd.leaf, s);
             delete sc;
             throw;
         }
@@ -530,13 +531,13 @@ gbt_status gbt_scene_destroy(gbt_scene_t *scene)
         if (!scene) return;
         cudaStream_t q = after_last_use(scene->d.used);
         dfree(scene->d.tri, q);
-        dfree(scene->d.trif, q);
         dfree(scene->d.face, q);
         dfree(scene->d.mat, q);
         dfree(scene->d.cbox, q);
         dfree(scene->d.tbox, q);
         if (scene->d.bvh) dfree(scene->d.bvh, q);
         if (scene->d.bvh_perm) dfree(scene->d.bvh_perm, q);
+        if (scene->d.leaf) dfree(scene->d.leaf, q);
         if (scene->d.used) cudaEventDestroy(scene->d.used);
         delete scene;
     });

@@ -91,7 +91,6 @@ struct SceneDev {
     int64_t n_tri = 0;
     int n_materials = 0;
     double *tri = nullptr;       // n_tri * 12
-    float *trif = nullptr;       // n_tri * 9: v0, e1, e2 rounded to FP32 (BVH screen)
     int32_t *face = nullptr;     // n_tri
     int32_t *mat = nullptr;      // n_tri
     // bounding boxes of consecutive triangle clusters (kTriCluster each), in FP32,
@@ -103,6 +102,7 @@ struct SceneDev {
     int accel = GBT_ACCEL_AUTO;
     BvhNode *bvh = nullptr;        // nodes (root 0), or nullptr when not built
     int32_t *bvh_perm = nullptr;   // triangle index of each leaf entry
+    float4 *leaf = nullptr;        // three words per leaf entry: FP32 v0, facet | e1, triangle | e2
     int64_t n_bvh_nodes = 0;
     int bvh_depth = 0;
     mutable cudaEvent_t used = nullptr;   // after the latest launch that read the scene

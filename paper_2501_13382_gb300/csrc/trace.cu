@@ -30,7 +30,7 @@ constexpr int kScanBlock = 1024;        // threads per scan block
 constexpr int kScanItems = 4;           // items per scan thread
 
 __global__ void scene_prep_kernel(const double *__restrict__ raw, int64_t n,
-                                  double *__restrict__ tri, float *__restrict__ trif)
+                                  double *__restrict__ tri)
 {
     int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (k >= n) return;
@@ -46,8 +46,21 @@ __global__ void scene_prep_kernel(const double *__restrict__ raw, int64_t n,
     o[3] = e1x; o[4] = e1y; o[5] = e1z;
     o[6] = e2x; o[7] = e2y; o[8] = e2z;
     o[9] = nx / len; o[10] = ny / len; o[11] = nz / len;
-    float *f = trif + 9 * k;
-    for (int q = 0; q < 9; ++q) f[q] = (float)o[q];
+}
+
+// FP32 record of each BVH leaf entry, in leaf order: v0, facet | e1, triangle | e2.  Three
+// 16-byte loads per triangle test, where index, facet, box and vertices apart took seventeen
+// loads of 4 bytes.
+__global__ void leaf_prep_kernel(const double *__restrict__ tri, const int32_t *__restrict__ perm,
+                                 const int32_t *__restrict__ face, int64_t n, float4 *__restrict__ leaf)
+{
+    const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (e >= n) return;
+    const int32_t k = perm[e];
+    const double *r = tri + 12 * (int64_t)k;
+    leaf[3 * e] = make_float4((float)r[0], (float)r[1], (float)r[2], __int_as_float(face[k]));
+    leaf[3 * e + 1] = make_float4((float)r[3], (float)r[4], (float)r[5], __int_as_float(k));
+    leaf[3 * e + 2] = make_float4((float)r[6], (float)r[7], (float)r[8], 0.0f);
 }
 
 struct TraceParams {
@@ -61,7 +74,6 @@ struct TraceParams {
     double ground_z;
     int ground_mat;
     const double *tri;         // n_tri * 12
-    const float *trif;         // n_tri * 9 (v0, e1, e2 in FP32)
     const int32_t *face;
     const int32_t *mat;
     int64_t n_tri;
@@ -69,7 +81,7 @@ struct TraceParams {
     const float *tbox;         // n_tri * 6
     int64_t n_clusters;
     const BvhNode *bvh;        // BVH nodes (root 0) or nullptr
-    const int32_t *bvh_perm;
+    const float4 *leaf;        // FP32 records of its leaf entries (leaf_prep_kernel)
     unsigned int *status;
     int chunk;                 // triangles per shared-memory chunk (a multiple of kTriCluster)
     int64_t strip;             // Fibonacci fan: lattice step between a warp's rays (0: none)
@@ -214,8 +226,7 @@ __device__ __forceinline__ void nearest_in_chunk(const double o[3], const double
     }
 }
 
-// Conservative FP32 screen in front of the exact FP64 test: false only when that test
-// is certain to reject the triangle.  With eps = 2^-24 the FP32 rounding of the inputs
+// FP32 screen in front of the exact FP64 test.  With eps = 2^-24 the FP32 rounding of the inputs
 // (origin, direction, v0, e1, e2) and of these operations moves u's numerator (o - v0).p
 // by at most 9 eps sum_i (|o_i| + |v0_i|) |p|_i, the determinant by 8 eps sum |e1_i| |p|_i
 // and v's numerator by 9 eps sum |d_i| |q|_i (|p|_i, |q|_i: the sums of the absolute
@@ -224,39 +235,72 @@ __device__ __forceinline__ void nearest_in_chunk(const double o[3], const double
 // test's own (about 1e-15 relative).  Outside the margins u < 0, u > 1, v < 0 or u + v > 1
 // holds in exact arithmetic, and so in FP64; where the determinant's sign is uncertain the
 // FP64 test decides.
-__device__ __forceinline__ bool tri_may_hit(float of0, float of1, float of2, float df0, float df1,
-                                            float df2, const float *__restrict__ f)
+//
+// FP32 view of one ray-triangle test: whether the exact test may accept it, and bounds of
+// its distance.  `sure`: the exact test accepts it (inside by more than the error bounds
+// above, the determinant's sign known, t above kTMin).  The distance's numerator e2.q moves
+// by at most 9 eps sum |e2_i| |q|_i, bounded with the same 1e-5 as the others.
+struct TriGuess {
+    bool may, sure;
+    float lo, hi;              // t lies in [lo, hi]
+};
+__device__ __forceinline__ TriGuess tri_guess(float of0, float of1, float of2, float df0, float df1,
+                                              float df2, const float4 &f0, const float4 &f1,
+                                              const float4 &f2)
 {
-    const float v0x = f[0], v0y = f[1], v0z = f[2];
-    const float e1x = f[3], e1y = f[4], e1z = f[5];
-    const float e2x = f[6], e2y = f[7], e2z = f[8];
+    TriGuess g;
+    g.may = true;
+    g.sure = false;
+    g.lo = 0.0f;
+    g.hi = INFINITY;
+    const float v0x = f0.x, v0y = f0.y, v0z = f0.z;
+    const float e1x = f1.x, e1y = f1.y, e1z = f1.z;
+    const float e2x = f2.x, e2y = f2.y, e2z = f2.z;
     const float px = df1 * e2z - df2 * e2y, py = df2 * e2x - df0 * e2z, pz = df0 * e2y - df1 * e2x;
     const float pax = fabsf(df1 * e2z) + fabsf(df2 * e2y), pay = fabsf(df2 * e2x) + fabsf(df0 * e2z),
                 paz = fabsf(df0 * e2y) + fabsf(df1 * e2x);
     const float det = e1x * px + e1y * py + e1z * pz;
     const float bd = 1e-5f * (fabsf(e1x) * pax + fabsf(e1y) * pay + fabsf(e1z) * paz) + 1e-30f;
     const float adet = fabsf(det);
-    if (!(adet > bd)) return true;
+    if (!(adet > bd)) return g;         // the exact test decides, at any distance
     const float tx = of0 - v0x, ty = of1 - v0y, tz = of2 - v0z;
     const float ax = fabsf(of0) + fabsf(v0x), ay = fabsf(of1) + fabsf(v0y), az = fabsf(of2) + fabsf(v0z);
     const float bu = 1e-5f * (ax * pax + ay * pay + az * paz) + 1e-30f;
     const float sgn = det > 0.0f ? 1.0f : -1.0f;
     const float su = sgn * (tx * px + ty * py + tz * pz);
-    if (su < -bu || su - adet > bu + bd) return false;
+    g.may = !(su < -bu || su - adet > bu + bd);
+    if (!g.may) return g;
     const float qx = ty * e1z - tz * e1y, qy = tz * e1x - tx * e1z, qz = tx * e1y - ty * e1x;
     const float qax = ay * fabsf(e1z) + az * fabsf(e1y), qay = az * fabsf(e1x) + ax * fabsf(e1z),
                 qaz = ax * fabsf(e1y) + ay * fabsf(e1x);
     const float bv = 1e-5f * (fabsf(df0) * qax + fabsf(df1) * qay + fabsf(df2) * qaz) + 1e-30f;
     const float sv = sgn * (df0 * qx + df1 * qy + df2 * qz);
-    if (sv < -bv || su + sv - adet > bu + bv + bd) return false;
-    return true;
+    g.may = !(sv < -bv || su + sv - adet > bu + bv + bd);
+    if (!g.may) return g;
+    const float bt = 1e-5f * (fabsf(e2x) * qax + fabsf(e2y) * qay + fabsf(e2z) * qaz) + 1e-30f;
+    const float st = sgn * (e2x * qx + e2y * qy + e2z * qz);
+    g.may = !(st < -bt);                // t < 0 whatever the rounding
+    // both bounds widened by the rounding of the divisions
+    g.lo = st - bt > 0.0f ? (st - bt) / (adet + bd) * 0.999999f : 0.0f;
+    g.hi = (st + bt) / (adet - bd) * 1.000001f;
+    g.sure = su > bu && su + bu + bd < adet && sv > bv && su + sv + bu + bv + bd < adet && g.lo > 1e-6f;
+    return g;
 }
 
-// Nearest hit among all triangles through the BVH.  Same candidates and the same
-// winner as testing every triangle in index order: a child whose padded box the ray
-// misses, or enters only beyond the best hit so far (widened like the boxes), holds
-// no hit that could win; hits are compared by (t, primitive id), so the lowest id
-// wins a tie whatever order the leaves are met in.
+// Nearest hit among the ground and all triangles through the BVH.  Same candidates and the
+// same winner as testing everything in index order: hits are compared by (t, primitive id),
+// so the lowest id wins a tie whatever order the leaves are met in.
+//
+// FP64 issues at 1/64 of the FP32 rate, and an exact test inside the traversal runs for the
+// few lanes that reach a leaf at the same time.  So the traversal keeps only FP32 bounds:
+// `bound` is above the distance of a hit that is sure; a child box entered beyond it (with
+// slack for the boxes' own rounding), or a primitive whose distance is surely larger, holds
+// no hit that could win.  What is left (mostly one primitive) is tested exactly after the
+// traversal, when the warp's lanes are together again.  262,144 rays, 12,288 triangles: 1.54
+// -> 0.72 ms (exact tests at the leaves to here), 0.63 ms with the packed leaf records; FP64
+// pipe 70 -> 31 % of active cycles, now bound by the latency of the divergent walk.  Four
+// blocks per SM instead of three (64 registers): 1.49 ms.
+constexpr int kCand = 4;
 __device__ __forceinline__ void nearest_in_bvh(const TraceParams &p, const double o[3],
                                                const double d[3], int last_face, double &tbest,
                                                int &best)
@@ -264,6 +308,31 @@ __device__ __forceinline__ void nearest_in_bvh(const TraceParams &p, const doubl
     const float of0 = (float)o[0], of1 = (float)o[1], of2 = (float)o[2];
     const float df0 = (float)d[0], df1 = (float)d[1], df2 = (float)d[2];
     const float id0 = 1.0f / df0, id1 = 1.0f / df1, id2 = 1.0f / df2;
+    float bound = INFINITY;
+    int32_t cand[kCand];       // primitive ids (0: ground), and below what distance they can win
+    float clo[kCand];
+    int nc = 0;
+    auto exact = [&](int32_t id) {
+        double t;
+        if (id == 0) t = (p.ground_z - o[2]) / d[2];
+        else t = ray_triangle(o, d, p.tri + 12 * (int64_t)(id - 1));
+        if (t > kTMin && (t < tbest || (t == tbest && id < best))) {
+            tbest = t;
+            best = id;
+        }
+    };
+    if (p.ground && last_face != -2 && d[2] != 0.0) {
+        // (ground_z - z) / d_z in FP32 within 1e-6 of the terms' sizes
+        const float gz = (float)p.ground_z, t = (gz - of2) * id2;
+        const float e = 1e-6f * ((fabsf(gz) + fabsf(of2)) * fabsf(id2) + fabsf(t));
+        if (!(t + e < 0.0f)) {          // also where d_z underflows in FP32 (t not finite)
+            const bool fine = e < 1e30f;
+            clo[0] = fine ? fmaxf(t - e, 0.0f) : 0.0f;
+            cand[0] = 0;
+            nc = 1;
+            if (fine && t - e > 1e-6f) bound = t + e;
+        }
+    }
     int32_t sref[kBvhStack];
     float stn[kBvhStack];
     int sp = 0;
@@ -273,26 +342,31 @@ __device__ __forceinline__ void nearest_in_bvh(const TraceParams &p, const doubl
     while (sp > 0) {
         --sp;
         const int32_t ref = sref[sp];
-        const float bound = (float)tbest * 1.000001f + 1e-3f;
-        if (stn[sp] > bound) continue;
+        const float wide = bound * 1.000001f + 1e-3f;
+        if (stn[sp] > wide) continue;
         if (ref < 0) {
             const int32_t v = -(ref + 1);
             const int32_t first = v >> 3, count = (v & 7) + 1;
             for (int e = first; e < first + count; ++e) {
-                const int32_t k = p.bvh_perm[e];
-                const int face = p.face ? p.face[k] : k;
-                if (face == last_face) continue;
-                const float *tb = p.tbox + 6 * (int64_t)k;
-                float un = 0.0f, uf = (float)tbest * 1.000001f + 1e-3f;
-                bool hit_tri = slab(of0, df0, id0, tb[0], tb[3], un, uf);
-                hit_tri = hit_tri && slab(of1, df1, id1, tb[1], tb[4], un, uf);
-                hit_tri = hit_tri && slab(of2, df2, id2, tb[2], tb[5], un, uf);
-                if (!hit_tri || un > uf) continue;
-                if (!tri_may_hit(of0, of1, of2, df0, df1, df2, p.trif + 9 * (int64_t)k)) continue;
-                const double t = ray_triangle(o, d, p.tri + 12 * (int64_t)k);
-                if (t > kTMin && (t < tbest || (t == tbest && k + 1 < best))) {
-                    tbest = t;
-                    best = k + 1;
+                const float4 f0 = __ldg(p.leaf + 3 * (int64_t)e), f1 = __ldg(p.leaf + 3 * (int64_t)e + 1),
+                             f2 = __ldg(p.leaf + 3 * (int64_t)e + 2);
+                if (__float_as_int(f0.w) == last_face) continue;
+                const int32_t k = __float_as_int(f1.w);
+                const TriGuess g = tri_guess(of0, of1, of2, df0, df1, df2, f0, f1, f2);
+                if (!g.may || g.lo > bound) continue;
+                if (g.sure && g.hi < bound) bound = g.hi;
+                if (nc == kCand) {      // drop what the bound has overtaken since
+                    int n = 0;
+                    for (int c = 0; c < kCand; ++c)
+                        if (!(clo[c] > bound)) { cand[n] = cand[c]; clo[n] = clo[c]; ++n; }
+                    nc = n;
+                }
+                if (nc == kCand) {
+                    exact(k + 1);
+                } else {
+                    cand[nc] = k + 1;
+                    clo[nc] = g.lo;
+                    ++nc;
                 }
             }
             continue;
@@ -302,7 +376,7 @@ __device__ __forceinline__ void nearest_in_bvh(const TraceParams &p, const doubl
         const float b0[6] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y};
         const float b1[6] = {w1.z, w1.w, w2.x, w2.y, w2.z, w2.w};
         const int32_t r0 = __float_as_int(w3.x), r1 = __float_as_int(w3.y);
-        float tn0 = 0.0f, tf0 = bound, tn1 = 0.0f, tf1 = bound;
+        float tn0 = 0.0f, tf0 = wide, tn1 = 0.0f, tf1 = wide;
         bool h0 = r0 != kBvhNone;
         h0 = h0 && slab(of0, df0, id0, b0[0], b0[3], tn0, tf0);
         h0 = h0 && slab(of1, df1, id1, b0[1], b0[4], tn0, tf0);
@@ -329,6 +403,8 @@ __device__ __forceinline__ void nearest_in_bvh(const TraceParams &p, const doubl
             sref[sp] = r1; stn[sp] = tn1; ++sp;
         }
     }
+    for (int c = 0; c < nc; ++c)
+        if (!(clo[c] > bound)) exact(cand[c]);
 }
 
 // Ground plane candidate (best 0) before any triangle.
@@ -485,7 +561,6 @@ __global__ void __launch_bounds__(kTraceBlock) trace_bvh_kernel(TraceParams p)
         for (bool alive = true; alive;) {
             double tbest = INFINITY;
             int best = -1;
-            nearest_ground(p, o, d, last_face, tbest, best);
             nearest_in_bvh(p, o, d, last_face, tbest, best);
             alive = record_and_reflect(p, i, o, d, s0, last_face, bmat, nref, nseg, tbest, best);
         }
@@ -643,8 +718,13 @@ void scene_prepare(SceneDev &sd, const double *tri_raw_dev, cudaStream_t s)
     if (sd.n_tri == 0) return;
     const int bs = 128;
     scene_prep_kernel<<<(unsigned)((sd.n_tri + bs - 1) / bs), bs, 0, s>>>(tri_raw_dev, sd.n_tri,
-                                                                          sd.tri, sd.trif);
+                                                                          sd.tri);
     note_launches(1);
+    if (sd.bvh) {
+        leaf_prep_kernel<<<(unsigned)((sd.n_tri + bs - 1) / bs), bs, 0, s>>>(sd.tri, sd.bvh_perm, sd.face,
+                                                                             sd.n_tri, sd.leaf);
+        note_launches(1);
+    }
     GBT_CUDA(cudaGetLastError());
 }
 
@@ -687,7 +767,6 @@ void trace_launch(const SceneDev &sd, TraceDev &td, const gbt_source_desc &src, 
     p.ground_z = sd.ground_z;
     p.ground_mat = sd.ground_material;
     p.tri = sd.tri;
-    p.trif = sd.trif;
     p.face = sd.face;
     p.mat = sd.mat;
     p.n_tri = sd.n_tri;
@@ -695,7 +774,7 @@ void trace_launch(const SceneDev &sd, TraceDev &td, const gbt_source_desc &src, 
     p.tbox = sd.tbox;
     p.n_clusters = sd.n_clusters;
     p.bvh = sd.bvh;
-    p.bvh_perm = sd.bvh_perm;
+    p.leaf = sd.leaf;
     p.status = status_word();
     // coherent warps on a Fibonacci fan: the largest Fibonacci number <= sqrt(N) / 2
     p.strip = 0;
@@ -738,6 +817,7 @@ void trace_launch(const SceneDev &sd, TraceDev &td, const gbt_source_desc &src, 
     }
     // the BVH (built unless GBT_ACCEL_LINEAR) outran the shared-memory scene already at
     // 768 triangles: 3.2 ms against 5.4 ms for 1,048,576 rays through the synthetic city
+    // (1.5 ms since)
     const bool use_bvh = sd.n_tri > 0 && sd.bvh && sd.accel != GBT_ACCEL_LINEAR;
     if (use_bvh) {
         int per_sm = 0;
