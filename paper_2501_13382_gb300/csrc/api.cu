@@ -281,9 +281,10 @@ static void validate_source(const gbt_source_desc &src)
 }
 
 // Device buffers of a trace of up to cnt rays (one allocation); td's ray range is set
-// by the caller before each trace_launch into it.
+// by the caller before each trace_launch into it.  Without `list` only the offsets (a solve
+// that packs its records from the padded rows).
 static void alloc_trace_block(TraceDev &td, const gbt_scene_t *scene, const gbt_source_desc &src,
-                              int64_t cnt, cudaStream_t s)
+                              int64_t cnt, cudaStream_t s, bool list = true)
 {
     td.scene = scene;
     td.n_fan = src.n_rays;
@@ -301,12 +302,13 @@ static void alloc_trace_block(TraceDev &td, const gbt_scene_t *scene, const gbt_
     td.max_path = src.max_path;
     td.capacity = cnt * (int64_t)(src.max_reflections + 1);
     const size_t cap = (size_t)td.capacity;
-    size_t bytes = align_up((size_t)(cnt + 1) * 4, 256) + 2 * align_up(cap * 24, 256) +
-                   2 * align_up(cap * 8, 256) + 4 * align_up(cap * 4, 256);
+    size_t bytes = align_up((size_t)(cnt + 1) * 4, 256);
+    if (list) bytes += 2 * align_up(cap * 24, 256) + 2 * align_up(cap * 8, 256) + 4 * align_up(cap * 4, 256);
     td.block = dalloc(bytes, s);
     char *w = static_cast<char *>(td.block);
     auto take = [&](size_t b) { char *p = w; w += align_up(b, 256); return p; };
     td.ray_off = reinterpret_cast<int32_t *>(take((size_t)(cnt + 1) * 4));
+    if (!list) return;
     td.o = reinterpret_cast<double *>(take(cap * 24));
     td.t = reinterpret_cast<double *>(take(cap * 24));
     td.L = reinterpret_cast<double *>(take(cap * 8));
@@ -343,9 +345,8 @@ static gbt_trace_t *make_trace(const gbt_scene_t *scene, const gbt_source_desc &
     return tr;
 }
 
-static void validate_sum(const gbt_trace_t *trace, const gbt_sum_args *a, bool need_out = true)
+static void validate_sum_args(const gbt_sum_args *a, bool need_out = true)
 {
-    GBT_REQUIRE(trace, "trace is NULL");
     GBT_REQUIRE(a, "args is NULL");
     GBT_REQUIRE(a->n_recv >= 0, "n_recv must be >= 0");
     GBT_REQUIRE(a->n_freq >= 1 && a->n_freq <= GBT_MAX_FREQ, "n_freq must be in [1, 16]");
@@ -369,6 +370,12 @@ static void validate_sum(const gbt_trace_t *trace, const gbt_sum_args *a, bool n
         }
         GBT_REQUIRE(a->n_recv < 2147483647LL, "n_recv must be < 2^31");
     }
+}
+
+static void validate_sum(const gbt_trace_t *trace, const gbt_sum_args *a, bool need_out = true)
+{
+    GBT_REQUIRE(trace, "trace is NULL");
+    validate_sum_args(a, need_out);
 }
 
 }  // namespace gbt
@@ -743,7 +750,7 @@ gbt_status gbt_recv_order(const float *recv, int64_t n_recv, int32_t *order_out,
         GBT_REQUIRE(recv && order_out, "recv and order_out must be non-NULL");
         cudaStream_t s = static_cast<cudaStream_t>(stream);
         const size_t b = recv_order_scratch_bytes(n_recv);
-        void *scr = dalloc(b, s);
+        void *scr = b ? dalloc(b, s) : nullptr;
         try {
             recv_order_launch(recv, n_recv, order_out, scr, s);
         } catch (...) {
@@ -795,6 +802,8 @@ gbt_status gbt_solve(const gbt_scene_t *scene, const gbt_source_desc *src, const
         GBT_REQUIRE(src->fan != GBT_FAN_EXPLICIT,
                     "gbt_solve generates its fan: Fibonacci or lat-long, not explicit");
         GBT_REQUIRE(args->max_device_bytes >= 0, "max_device_bytes must be >= 0");
+        validate_source(*src);
+        validate_sum_args(args);
         cudaStream_t s = static_cast<cudaStream_t>(stream);
         const int64_t N = src->n_rays;
         const int64_t loss = has_losses(*args) ? 16 * (int64_t)args->n_freq : 0;
@@ -807,32 +816,45 @@ gbt_status gbt_solve(const gbt_scene_t *scene, const gbt_source_desc *src, const
         }
         chunk = std::min<int64_t>(chunk, (int64_t)(2147483646LL / (src->max_reflections + 1)));
         gbt_sum_args a = *args;
+        // without losses nothing but the records is needed of the trace
+        const bool packed = !has_losses(a) && a.precision == GBT_PRECISION_F32;
         if (chunk >= N) {
             // one pass: trace and sum on the caller's stream
-            gbt_trace_t *tr = make_trace(scene, *src, s);
+            TraceDev td;
+            void *scratch = nullptr;
+            auto release = [&] {
+                td.work.release(s);
+                dfree(td.block, s);
+                dfree(scratch, s);
+            };
             try {
-                validate_sum(tr, &a);
-                const int splits = choose_splits(tr->d, a);
-                void *w = tr->d.work.ensure(sum_workspace_bytes(tr->d, a, splits), s);
-                sum_launch(tr->d, scene->d, a, splits, w, s);
+                alloc_trace_block(td, scene, *src, N, s, !packed);
+                td.ray_begin = 0;
+                td.n_rays = N;
+                const size_t sb = trace_scratch_bytes(N, src->max_reflections);
+                scratch = dalloc(sb, s);
+                PaddedRays rays;
+                if (packed) {
+                    rays = trace_rays_launch(scene->d, td, *src, scratch, sb, s);
+                } else {
+                    trace_launch(scene->d, td, *src, scratch, sb, s);
+                    dfree(scratch, s);
+                    scratch = nullptr;
+                }
+                const int splits = choose_splits(td, a);
+                void *w = td.work.ensure(sum_workspace_bytes(td, a, splits), s);
+                sum_launch(td, scene->d, a, splits, w, s, nullptr, false, packed ? &rays : nullptr);
             } catch (...) {
-                tr->d.work.release(s);
-                dfree(tr->d.block, s);
-                if (tr->d.used) cudaEventDestroy(tr->d.used);
-                delete tr;
+                release();
                 throw;
             }
-            tr->d.work.release(s);
-            dfree(tr->d.block, s);
-            if (tr->d.used) cudaEventDestroy(tr->d.used);
-            delete tr;
+            release();
             mark_used(scene->d.used, s);
             return;
         }
         // Chunks of rays, double-buffered: chunk i is traced on a private stream into slot
         // i % 2 while the caller's stream sums chunk i - 1 from the other slot; every sum
         // accumulates into out in chunk order on the caller's stream.
-        validate_source(*src);
         const int nslot = 2;
         TraceDev slot[nslot];
         void *scratch[nslot] = {nullptr, nullptr};
@@ -858,7 +880,7 @@ gbt_status gbt_solve(const gbt_scene_t *scene, const gbt_source_desc *src, const
             for (int k = 0; k < nslot; ++k) {
                 GBT_CUDA(cudaEventCreateWithFlags(&traced[k], cudaEventDisableTiming));
                 GBT_CUDA(cudaEventCreateWithFlags(&summed[k], cudaEventDisableTiming));
-                alloc_trace_block(slot[k], scene, *src, chunk, s);
+                alloc_trace_block(slot[k], scene, *src, chunk, s, !packed);
                 scratch[k] = dalloc(sb, s);
                 // the sum workspace for a full chunk, sized once
                 slot[k].ray_begin = 0;
@@ -879,12 +901,15 @@ gbt_status gbt_solve(const gbt_scene_t *scene, const gbt_source_desc *src, const
                 td.ray_begin = cs.ray_begin;
                 td.n_rays = cs.ray_count;
                 td.n_seg_host = -1;
-                trace_launch(scene->d, td, cs, scratch[k], sb, ts);
+                PaddedRays rays;
+                if (packed) rays = trace_rays_launch(scene->d, td, cs, scratch[k], sb, ts);
+                else trace_launch(scene->d, td, cs, scratch[k], sb, ts);
                 GBT_CUDA(cudaEventRecord(traced[k], ts));
                 GBT_CUDA(cudaStreamWaitEvent(s, traced[k], 0));
                 a.accumulate = (i == 0) ? args->accumulate : 1;
                 const int splits = choose_splits(td, a);
-                sum_launch(td, scene->d, a, splits, td.work.ensure(sum_workspace_bytes(td, a, splits), s), s);
+                sum_launch(td, scene->d, a, splits, td.work.ensure(sum_workspace_bytes(td, a, splits), s), s,
+                           nullptr, false, packed ? &rays : nullptr);
                 GBT_CUDA(cudaEventRecord(summed[k], s));
             }
             // the caller's stream is last: every trace was waited for by a sum on it

@@ -401,48 +401,145 @@ struct PrepParams {
     // F64 path records (nullptr when not needed)
     double *amp64;
     unsigned int *status;
+    double w0;                 // weight of every ray of a Fibonacci or explicit fan
+    int *counters;             // kCounters work counters to zero, or nullptr
 };
+constexpr int kCounters = GBT_MAX_FREQ / kGroupFreq;   // one per pair launch of a sum
 
+// v = hi + lo, each rounded to nearest: hi = (float)v, lo = (float)(v - hi).  By integer
+// operations on v's bits in the range where neither part can leave FP32 (2^-60 .. 2^120, and
+// zero): the four FP64 and conversion instructions per value issue at a 64th of the integer
+// rate and were most of the prepass (3.06e6 segments: 405 us with them).
 __device__ __forceinline__ void split_ff(double v, float &hi, float &lo)
 {
-    hi = (float)v;
-    lo = (float)(v - (double)hi);
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(v);
+    const uint32_t h = (uint32_t)(bits >> 32), l = (uint32_t)bits;
+    const uint32_t e = (h >> 20) & 0x7ffu;
+    if (e - 963u <= 180u) {
+        const uint32_t m = ((h & 0xfffffu) << 3) | (l >> 29);      // hi's 23 fraction bits
+        int32_t r = (int32_t)(l & 0x1fffffffu);                    // the 29 below, in 2^(e - 1075)
+        const bool up = r > 0x10000000 || (r == 0x10000000 && (m & 1u));
+        hi = __uint_as_float((h & 0x80000000u) | ((((e - 896u) << 23) | m) + (up ? 1u : 0u)));
+        if (up) r -= 0x20000000;
+        if (h & 0x80000000u) r = -r;
+        lo = __int2float_rn(r) * __uint_as_float((e - 948u) << 23);
+    } else if ((bits << 1) == 0ull) {
+        hi = (float)v;
+        lo = 0.0f;
+    } else {
+        hi = (float)v;
+        lo = (float)(v - (double)hi);
+    }
 }
 
-__global__ void prepass_kernel(PrepParams p)
+// Writes segment j's 80-byte record and 32-byte cull record.
+__device__ __forceinline__ void write_record(float *rec, float4 *crec, int64_t j, const double *o,
+                                             const double *t, double s0, double L, double amp)
 {
-    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t n = *p.n_seg_ptr;
-    if (j >= n) return;
-    // Gamma_path: product of gamma over the reflections before this segment
+    float4 *R = reinterpret_cast<float4 *>(rec + j * kRecFloats);
+    float oh[3], ol[3], th[3], tl[3], s0h, s0l, Lh, Ll;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        split_ff(o[a], oh[a], ol[a]);
+        split_ff(t[a], th[a], tl[a]);
+    }
+    split_ff(s0, s0h, s0l);
+    split_ff(L, Lh, Ll);
+    R[0] = make_float4(oh[0], oh[1], oh[2], s0h);     // R_OXH .. R_S0H
+    R[1] = make_float4(th[0], th[1], th[2], Lh);      // R_TXH .. R_LH
+    R[2] = make_float4(ol[0], ol[1], ol[2], s0l);     // R_OXL .. R_S0L
+    R[3] = make_float4(tl[0], tl[1], tl[2], Ll);      // R_TXL .. R_LL
+    R[4] = make_float4((float)amp, 0.f, 0.f, 0.f);    // R_AMP
+    crec[2 * j] = R[0];
+    crec[2 * j + 1] = R[1];
+}
+
+// Product of gamma over the reflections before a segment: materials bmat[1 .. dep].
+__device__ __forceinline__ double path_gamma(const PrepParams &p, const int32_t *bmat, int dep)
+{
     double g = 1.0;
-    const int dep = p.depth[j];
     for (int q = 1; q <= dep; ++q) {
-        const int m = p.bmat[j - dep + q];
+        const int m = bmat[q];
         if (m < 0 || m >= p.n_materials) {
             atomicOr(p.status, STATUS_BOUNDS);
             continue;
         }
         g *= (double)p.gamma[m];
     }
-    const double w = p.weight ? (double)p.weight[p.ray[j]] : fan_weight(p.fan, p.n_fan, p.ray[j]);
-    const double amp = w * g;
-    float4 *R = reinterpret_cast<float4 *>(p.rec + j * kRecFloats);
-    float oh[3], ol[3], th[3], tl[3], s0h, s0l, Lh, Ll;
-    for (int a = 0; a < 3; ++a) {
-        split_ff(p.o[3 * j + a], oh[a], ol[a]);
-        split_ff(p.t[3 * j + a], th[a], tl[a]);
-    }
-    split_ff(p.s0[j], s0h, s0l);
-    split_ff(p.L[j], Lh, Ll);
-    R[0] = make_float4(oh[0], oh[1], oh[2], s0h);     // R_OXH .. R_S0H
-    R[1] = make_float4(th[0], th[1], th[2], Lh);      // R_TXH .. R_LH
-    R[2] = make_float4(ol[0], ol[1], ol[2], s0l);     // R_OXL .. R_S0L
-    R[3] = make_float4(tl[0], tl[1], tl[2], Ll);      // R_TXL .. R_LL
-    R[4] = make_float4((float)amp, 0.f, 0.f, 0.f);    // R_AMP
-    p.crec[2 * j] = R[0];
-    p.crec[2 * j + 1] = R[1];
+    return g;
+}
+__device__ __forceinline__ double ray_amplitude(const PrepParams &p, int64_t ray)
+{
+    if (p.weight) return (double)p.weight[ray];
+    return p.fan.kind == GBT_FAN_LATLONG ? fan_weight(p.fan, p.n_fan, ray) : p.w0;
+}
+
+__global__ void prepass_kernel(PrepParams p)
+{
+    const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (j < kCounters && p.counters) p.counters[j] = 0;
+    if (j >= *p.n_seg_ptr) return;
+    const int dep = p.depth[j];
+    const double amp = ray_amplitude(p, p.ray[j]) * path_gamma(p, p.bmat + j - dep, dep);
+    write_record(p.rec, p.crec, j, p.o + 3 * j, p.t + 3 * j, p.s0[j], p.L[j], amp);
     if (p.amp64) p.amp64[j] = amp;
+}
+
+// Records straight from the tracer's padded rows (gbt_solve: nobody sees the segment list):
+// a block takes kPackRays rays, finds its first segment from the blocks' counts, and its
+// threads run over its segments, not its slots (most rows are short).  Replaces the scan, the
+// compaction and the prepass: 101 bytes less written and read per segment (1M-ray city: 610
+// us for the five kernels, 258 us).
+__global__ void __launch_bounds__(kPackRays) pack_kernel(PrepParams p, PaddedRays r)
+{
+    __shared__ int32_t first[kPackRays + 1];     // segments of the block before each ray
+    __shared__ int32_t ws[kPackRays / 32];
+    __shared__ int32_t before_s;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (blockIdx.x == 0 && threadIdx.x < kCounters) p.counters[threadIdx.x] = 0;
+    auto block_sum = [&](int32_t v) {            // of every thread's v
+        v = __reduce_add_sync(0xffffffffu, v);
+        if (lane == 0) ws[wid] = v;
+        __syncthreads();
+        int32_t s = 0;
+        for (int w = 0; w < kPackRays / 32; ++w) s += ws[w];
+        __syncthreads();
+        return s;
+    };
+    int32_t before = 0;
+    if (r.scanned) {
+        before = r.bsum[blockIdx.x];
+    } else {
+        for (int64_t q = threadIdx.x; q < blockIdx.x; q += kPackRays) before += r.bsum[q];
+        before = block_sum(before);
+    }
+    const int64_t i = (int64_t)blockIdx.x * kPackRays + threadIdx.x;
+    const int32_t cnt = i < r.n_rays ? r.cnt[i] : 0;
+    int32_t x = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) ws[wid] = x;
+    __syncthreads();
+    for (int w = 0; w < wid; ++w) x += ws[w];
+    first[threadIdx.x + 1] = x;
+    if (threadIdx.x == 0) first[0] = 0;
+    __syncthreads();
+    const int32_t total = first[kPackRays];
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *r.n_seg = before + total;
+    for (int32_t k = threadIdx.x; k < total; k += kPackRays) {
+        int lo = 0;                              // last ray with first[lo] <= k
+#pragma unroll
+        for (int st = kPackRays / 2; st > 0; st >>= 1)
+            if (first[lo + st] <= k) lo += st;
+        const int dep = k - first[lo];
+        const int64_t ray = (int64_t)blockIdx.x * kPackRays + lo;
+        const int64_t slot = ray * r.stride + dep;
+        const double amp = ray_amplitude(p, r.ray_begin + ray) * path_gamma(p, r.bmat + slot - dep, dep);
+        write_record(p.rec, p.crec, before + k, r.o + 3 * slot, r.t + 3 * slot, r.s0[slot], r.L[slot], amp);
+    }
 }
 
 // ---- losses of porous surfaces
@@ -887,6 +984,8 @@ __global__ void grad_out_kernel(GradOutParams p)
 // changes which CTA computes an item, never the arithmetic of any sum.
 constexpr int kWeightSamples = 1 << 15;        // sampled segments per estimate
 constexpr int64_t kMaxOrderedTiles = 1 << 14;  // beyond this the rank pass is skipped
+constexpr int64_t kOrderPairs = int64_t(1) << 31;   // (receiver, segment slot) pairs, see tile_ws_layout
+constexpr int64_t kOrderTiles = 24;
 
 
 // Also each tile's reach ball (the list passes' form, with the ball's share of the slack).
@@ -979,14 +1078,15 @@ __global__ void tile_weight_kernel(const float4 *crec, const int32_t *n_seg_ptr,
         r0 = crec[2 * j];
         r1 = crec[2 * j + 1];
     }
-    for (int64_t t = 0; t < n_tiles; ++t) {
+    for (int64_t t = blockIdx.y; t < n_tiles; t += gridDim.y) {
         const float4 b = ball[t];
         bool pass = false;
         if (ok)
             pass = ball_may_keep<WINDOW>(r0, r1, r0.x - b.x, r0.y - b.y, r0.z - b.z,
                                          make_float4(0.f, 0.f, 0.f, b.w), alpha, beta);
-        const unsigned int m = __ballot_sync(0xffffffffu, pass);
-        if ((threadIdx.x & 31) == 0 && m) atomicAdd(&weight[t], (unsigned int)__popc(m));
+        // one atomic per block: a warp each, on a few dozen tiles, took 23 us in contention
+        const int c = __syncthreads_count(pass);
+        if (threadIdx.x == 0 && c) atomicAdd(&weight[t], (unsigned int)c);
     }
 }
 
@@ -1434,21 +1534,27 @@ __device__ __forceinline__ unsigned int spread10(unsigned int v)
     return v;
 }
 
+// 30-bit code of a position quantised to the bounding box bb (ordered bits, see bbox_kernel).
+__device__ __forceinline__ unsigned int morton_code(const float *x, const unsigned int *bb)
+{
+    unsigned int code = 0;
+    for (int a = 0; a < 3; ++a) {
+        const float lo = from_ordered(bb[a]), hi = from_ordered(bb[3 + a]);
+        const float span = hi - lo;
+        float u = span > 0.f ? (x[a] - lo) / span : 0.f;
+        unsigned int q = (unsigned int)fminf(fmaxf(u * 1023.0f, 0.0f), 1023.0f);
+        code |= spread10(q) << a;
+    }
+    return code;
+}
+
 __global__ void morton_kernel(const float *recv, int64_t n, int64_t npad, const unsigned int *bb,
                               unsigned long long *keys)
 {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= npad) return;
     if (i >= n) { keys[i] = ~0ull; return; }
-    unsigned int code = 0;
-    for (int a = 0; a < 3; ++a) {
-        const float lo = from_ordered(bb[a]), hi = from_ordered(bb[3 + a]);
-        const float span = hi - lo;
-        float u = span > 0.f ? (recv[3 * i + a] - lo) / span : 0.f;
-        unsigned int q = (unsigned int)fminf(fmaxf(u * 1023.0f, 0.0f), 1023.0f);
-        code |= spread10(q) << a;
-    }
-    keys[i] = ((unsigned long long)code << 32) | (unsigned long long)i;
+    keys[i] = ((unsigned long long)morton_code(recv + 3 * i, bb) << 32) | (unsigned long long)i;
 }
 
 __global__ void bitonic_step(unsigned long long *keys, int64_t npad, int64_t j, int64_t k)
@@ -1473,6 +1579,20 @@ __device__ __forceinline__ unsigned int radix_digit(unsigned long long key, int 
     return (unsigned int)(key >> (32 + shift)) & (kRadixBuckets - 1);
 }
 
+// The lanes (of those with ok) that hold the same 8-bit digit: a ballot per bit, a third of
+// the time of __match_any_sync.
+__device__ __forceinline__ unsigned int same_digit(unsigned int d, bool ok)
+{
+    unsigned int m = __ballot_sync(0xffffffffu, ok);
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+        const bool set = (d >> b) & 1u;
+        const unsigned int v = __ballot_sync(0xffffffffu, set);
+        m &= set ? v : ~v;
+    }
+    return m;
+}
+
 // counts[d * nblocks + block]: keys of the block with digit d
 __global__ void __launch_bounds__(kRadixBlock) radix_count_kernel(const unsigned long long *keys,
                                                                   int64_t n, int shift,
@@ -1487,19 +1607,35 @@ __global__ void __launch_bounds__(kRadixBlock) radix_count_kernel(const unsigned
     if (threadIdx.x < kRadixBuckets) counts[(int64_t)threadIdx.x * nblocks + blockIdx.x] = c[threadIdx.x];
 }
 
-// One block: exclusive scan of the counts in place (digit-major, then block).
-__global__ void __launch_bounds__(1024) radix_scan_kernel(uint32_t *counts, int64_t total)
+// One block per digit: exclusive scan of its blocks' counts in place, and its total.  (One
+// block for all digits took 47 us a pass at 262,144 keys.)
+__global__ void __launch_bounds__(256) radix_scan_kernel(uint32_t *counts, int64_t nblocks, uint32_t *total)
 {
-    __shared__ int64_t ws[33];
-    int64_t carry = 0;
-    for (int64_t base = 0; base < total; base += 1024) {
+    __shared__ uint32_t ws[8];
+    uint32_t *row = counts + (int64_t)blockIdx.x * nblocks;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint32_t carry = 0;
+    for (int64_t base = 0; base < nblocks; base += 256) {
         const int64_t c = base + threadIdx.x;
-        const int64_t v = c < total ? counts[c] : 0;
-        int64_t excl;
-        const int64_t tot = block_scan_1024(v, excl, ws);
-        if (c < total) counts[c] = (uint32_t)(carry + excl);
-        carry += tot;
+        const uint32_t v = c < nblocks ? row[c] : 0u;
+        uint32_t x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) ws[wid] = x;
+        __syncthreads();
+        uint32_t before = carry, all = 0;
+        for (int w = 0; w < 8; ++w) {
+            if (w < wid) before += ws[w];
+            all += ws[w];
+        }
+        if (c < nblocks) row[c] = before + x - v;
+        carry += all;
+        __syncthreads();
     }
+    if (threadIdx.x == 0) total[blockIdx.x] = carry;
 }
 
 // Stable scatter: rank within the warp from the lanes holding the same digit, then the
@@ -1508,9 +1644,11 @@ __global__ void __launch_bounds__(kRadixBlock) radix_scatter_kernel(const unsign
                                                                     unsigned long long *out,
                                                                     int64_t n, int shift,
                                                                     const uint32_t *offs,
+                                                                    const uint32_t *total,
                                                                     int64_t nblocks)
 {
     __shared__ uint32_t wc[kRadixBlock / 32][kRadixBuckets];
+    __shared__ uint32_t base[kRadixBuckets];     // keys of smaller digits
     for (int q = threadIdx.x; q < (kRadixBlock / 32) * kRadixBuckets; q += kRadixBlock)
         (&wc[0][0])[q] = 0u;
     __syncthreads();
@@ -1518,8 +1656,8 @@ __global__ void __launch_bounds__(kRadixBlock) radix_scatter_kernel(const unsign
     const int64_t i = (int64_t)blockIdx.x * kRadixBlock + threadIdx.x;
     const bool ok = i < n;
     const unsigned long long key = ok ? in[i] : 0ull;
-    const unsigned int d = ok ? radix_digit(key, shift) : (unsigned int)kRadixBuckets;
-    const unsigned int same = __match_any_sync(0xffffffffu, d);
+    const unsigned int d = radix_digit(key, shift);
+    const unsigned int same = same_digit(d, ok);
     const unsigned int rank = __popc(same & ((1u << lane) - 1u));
     if (ok && rank == 0) wc[wid][d] = __popc(same);
     __syncthreads();
@@ -1531,8 +1669,137 @@ __global__ void __launch_bounds__(kRadixBlock) radix_scatter_kernel(const unsign
             run += c;
         }
     }
+    if (wid == 0) {
+        uint32_t carry = 0;
+#pragma unroll
+        for (int q = 0; q < kRadixBuckets / 32; ++q) {
+            const uint32_t v = total[q * 32 + lane];
+            uint32_t x = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
+            }
+            base[q * 32 + lane] = carry + x - v;
+            carry += __shfl_sync(0xffffffffu, x, 31);
+        }
+    }
     __syncthreads();
-    if (ok) out[offs[(int64_t)d * nblocks + blockIdx.x] + wc[wid][d] + rank] = key;
+    if (ok) out[base[d] + offs[(int64_t)d * nblocks + blockIdx.x] + wc[wid][d] + rank] = key;
+}
+
+// The whole order in one block, for up to kOrderSmall receivers: bounding box, codes and the
+// four radix passes in shared memory.  Each warp owns a contiguous share of the keys and its
+// own digit counters; ranks within a warp come from the lanes holding the same digit, so
+// every pass is stable.  A few thousand receivers are bound by launches: 15 kernels and 2
+// memsets took 72 us for 4,096 receivers (with the present kernels 65 us), this one 29; at
+// 10,000 the two are even.
+constexpr int kOrderSmall = 8192;
+constexpr int kOrderThreads = 1024, kOrderWarps = kOrderThreads / 32;
+struct OrderSmem {
+    uint32_t code[2][kOrderSmall];
+    uint16_t idx[2][kOrderSmall];
+};
+struct OrderCounts {
+    uint32_t c[kRadixBuckets][kOrderWarps + 1];   // padded: a digit's counts in different banks
+    uint32_t ws[kOrderWarps];
+    unsigned int bb[6];
+};
+__global__ void __launch_bounds__(kOrderThreads) order_small_kernel(const float *recv, int n, int32_t *order)
+{
+    extern __shared__ __align__(16) unsigned char order_smem[];
+    OrderCounts &K = *reinterpret_cast<OrderCounts *>(order_smem);
+    const int cap = (n + 1) / 2 * 2;
+    uint32_t *code[2];
+    uint16_t *idx[2];
+    code[0] = reinterpret_cast<uint32_t *>(order_smem + sizeof(OrderCounts));
+    code[1] = code[0] + cap;
+    idx[0] = reinterpret_cast<uint16_t *>(code[1] + cap);
+    idx[1] = idx[0] + cap;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (threadIdx.x < 3) { K.bb[threadIdx.x] = 0xffffffffu; K.bb[3 + threadIdx.x] = 0u; }
+    __syncthreads();
+    unsigned lo[3] = {~0u, ~0u, ~0u}, hi[3] = {0u, 0u, 0u};
+    for (int i = threadIdx.x; i < n; i += kOrderThreads)
+        for (int a = 0; a < 3; ++a) {
+            const unsigned u = ordered_bits(recv[3 * i + a]);
+            lo[a] = min(lo[a], u);
+            hi[a] = max(hi[a], u);
+        }
+    for (int a = 0; a < 3; ++a) {
+        lo[a] = __reduce_min_sync(0xffffffffu, lo[a]);
+        hi[a] = __reduce_max_sync(0xffffffffu, hi[a]);
+        if (lane == 0) {
+            atomicMin(&K.bb[a], lo[a]);
+            atomicMax(&K.bb[3 + a], hi[a]);
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += kOrderThreads) {
+        code[0][i] = morton_code(recv + 3 * i, K.bb);
+        idx[0][i] = (uint16_t)i;
+    }
+    // warp w owns keys [w share, (w + 1) share)
+    const int share = (n + kOrderThreads - 1) / kOrderThreads * 32;
+    const int b = min(n, wid * share), e = min(n, b + share);
+    for (int pass = 0; pass < 4; ++pass) {
+        const int shift = 8 * pass;
+        const uint32_t *ci = code[pass & 1];
+        const uint16_t *ii = idx[pass & 1];
+        for (int q = threadIdx.x; q < kRadixBuckets * kOrderWarps; q += kOrderThreads)
+            K.c[q / kOrderWarps][q % kOrderWarps] = 0u;
+        __syncthreads();
+        for (int i0 = b; i0 < e; i0 += 32) {
+            const bool ok = i0 + lane < e;
+            const unsigned d = ok ? (ci[i0 + lane] >> shift) & 255u : 0u;
+            const unsigned same = same_digit(d, ok);
+            if (ok && (same & ((1u << lane) - 1u)) == 0u) K.c[d][wid] += __popc(same);
+            __syncwarp();
+        }
+        __syncthreads();
+        // exclusive scan over (digit, warp): 8 consecutive counts per thread
+        uint32_t v[8], sum = 0;
+        for (int q = 0; q < 8; ++q) {
+            const int at = threadIdx.x * 8 + q;
+            v[q] = K.c[at / kOrderWarps][at % kOrderWarps];
+            sum += v[q];
+        }
+        uint32_t x = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) K.ws[wid] = x;
+        __syncthreads();
+        uint32_t run = x - sum;
+        for (int w = 0; w < wid; ++w) run += K.ws[w];
+        for (int q = 0; q < 8; ++q) {
+            const int at = threadIdx.x * 8 + q;
+            K.c[at / kOrderWarps][at % kOrderWarps] = run;
+            run += v[q];
+        }
+        __syncthreads();
+        for (int i0 = b; i0 < e; i0 += 32) {
+            const bool ok = i0 + lane < e;
+            const uint32_t cd = ok ? ci[i0 + lane] : 0u;
+            const unsigned d = (cd >> shift) & 255u;
+            const unsigned same = same_digit(d, ok), below = same & ((1u << lane) - 1u);
+            const uint32_t at = ok ? K.c[d][wid] + __popc(below) : 0u;
+            __syncwarp();
+            if (ok) {
+                if (below == 0u) K.c[d][wid] += __popc(same);
+                if (pass == 3) {
+                    order[at] = ii[i0 + lane];
+                } else {
+                    code[1 - (pass & 1)][at] = cd;
+                    idx[1 - (pass & 1)][at] = ii[i0 + lane];
+                }
+            }
+            __syncwarp();
+        }
+        __syncthreads();
+    }
 }
 
 __global__ void extract_order(const unsigned long long *keys, int64_t n, int32_t *order)
@@ -1706,11 +1973,17 @@ struct TileWs {
 
 std::atomic<int64_t> g_list_cap_limit{0};   // set_list_capacity (0: the default)
 
-static TileWs tile_ws_layout(void *ws, int64_t n_recv, int64_t seg_capacity, bool tile_cull)
+static TileWs tile_ws_layout(void *ws, int64_t n_recv, int64_t seg_capacity, bool tile_cull,
+                             bool adjoint = false)
 {
     TileWs t;
     t.tiles = cta_tiles(n_recv);
-    t.order = t.tiles >= 2 && t.tiles <= kMaxOrderedTiles;
+    // The order's three launches (10 to 14 us) pay where a tile's items are many and long: with
+    // few tiles every tile is split finely and the queue drains evenly in any order, until the
+    // whole kernel is long.  Measured without / with the order, 5 to 18 tiles: 1.3e7 pairs 36 /
+    // 46 us, 6e7 69 / 83, 2.4e8 110 / 120, 7e8 155 / 164, 2.1e9 268 / 257, 9.7e9 703 / 697.
+    t.order = t.tiles >= 2 && t.tiles <= kMaxOrderedTiles &&
+              (adjoint || tile_cull || t.tiles >= kOrderTiles || n_recv * seg_capacity >= kOrderPairs);
     t.lists = tile_cull && t.tiles >= 1 && t.tiles <= kMaxOrderedTiles && seg_capacity > 0;
     if (!t.order && !t.lists) return t;
     t.chunks = t.lists ? (seg_capacity + kListChunk - 1) / kListChunk : 0;
@@ -1749,9 +2022,9 @@ static TileWs tile_ws_layout(void *ws, int64_t n_recv, int64_t seg_capacity, boo
     return t;
 }
 
-static size_t tile_ws_bytes(int64_t n_recv, int64_t seg_capacity, bool tile_cull)
+static size_t tile_ws_bytes(int64_t n_recv, int64_t seg_capacity, bool tile_cull, bool adjoint = false)
 {
-    return tile_ws_layout(nullptr, n_recv, seg_capacity, tile_cull).bytes;
+    return tile_ws_layout(nullptr, n_recv, seg_capacity, tile_cull, adjoint).bytes;
 }
 
 // Launches the tile preparation for q's receivers and records (the records must
@@ -1786,10 +2059,10 @@ static void tile_prep_launch(FwdParams &q, int window, const TileWs &t, cudaStre
         n += 2;
     } else {
         if (window == GBT_WINDOW_LINE)
-            tile_weight_kernel<GBT_WINDOW_LINE><<<kWeightSamples / 256, 256, 0, s>>>(
+            tile_weight_kernel<GBT_WINDOW_LINE><<<dim3(kWeightSamples / 256, 8), 256, 0, s>>>(
                 q.crec, q.n_seg_ptr, t.ball, T, q.pre_alpha, q.pre_beta, t.weight);
         else
-            tile_weight_kernel<GBT_WINDOW_SEGMENT><<<kWeightSamples / 256, 256, 0, s>>>(
+            tile_weight_kernel<GBT_WINDOW_SEGMENT><<<dim3(kWeightSamples / 256, 8), 256, 0, s>>>(
                 q.crec, q.n_seg_ptr, t.ball, T, q.pre_alpha, q.pre_beta, t.weight);
         ++n;
     }
@@ -1847,10 +2120,13 @@ static size_t records_bytes(const TraceDev &td)
 // Prepass of a trace's segments into kernel records (and FP64 amplitudes when amp64 is
 // set), with the sum's reflection coefficients and ray weights.
 static void prepass_launch(const TraceDev &td, const SceneDev &sd, const gbt_sum_args &a,
-                           float *rec, double *amp64, cudaStream_t s, void *loss = nullptr)
+                           float *rec, double *amp64, int *counters, cudaStream_t s,
+                           void *loss = nullptr, const PaddedRays *rays = nullptr)
 {
     if (td.capacity == 0) return;
     PrepParams pp{};
+    pp.counters = counters;
+    pp.w0 = 4.0 * kPi / (double)td.n_fan;
     pp.n_seg_ptr = td.ray_off + td.n_rays;
     pp.o = td.o; pp.t = td.t; pp.L = td.L; pp.s0 = td.s0;
     pp.ray = td.ray; pp.depth = td.depth; pp.bmat = td.bmat;
@@ -1863,6 +2139,12 @@ static void prepass_launch(const TraceDev &td, const SceneDev &sd, const gbt_sum
     pp.crec = cull_records(rec, td.capacity);
     pp.amp64 = amp64;
     pp.status = status_word();
+    if (rays) {
+        pack_kernel<<<(unsigned)((rays->n_rays + kPackRays - 1) / kPackRays), kPackRays, 0, s>>>(pp, *rays);
+        note_launches(1);
+        GBT_CUDA(cudaGetLastError());
+        return;
+    }
     prepass_kernel<<<(unsigned)((td.capacity + 255) / 256), 256, 0, s>>>(pp);
     note_launches(1);
     if (loss) {
@@ -1911,7 +2193,8 @@ size_t sum_workspace_bytes(const TraceDev &td, const gbt_sum_args &a, int splits
 }
 
 void sum_launch(const TraceDev &td, const SceneDev &sd, const gbt_sum_args &a, int splits,
-                void *work, cudaStream_t s, unsigned long long *stats, bool differentiable)
+                void *work, cudaStream_t s, unsigned long long *stats, bool differentiable,
+                const PaddedRays *rays)
 {
     char *w = static_cast<char *>(work);
     float *rec = reinterpret_cast<float *>(w);
@@ -1929,7 +2212,7 @@ void sum_launch(const TraceDev &td, const SceneDev &sd, const gbt_sum_args &a, i
     void *loss = loss_bytes(td, a) ? static_cast<void *>(w) : nullptr;
     const int32_t *n_seg_ptr = td.ray_off + td.n_rays;
 
-    prepass_launch(td, sd, a, rec, amp64, s, loss);
+    prepass_launch(td, sd, a, rec, amp64, counter, s, loss, rays);
 
     if (a.n_recv <= 0) return;
     ReduceParams rp{};
@@ -1985,7 +2268,7 @@ void sum_launch(const TraceDev &td, const SceneDev &sd, const gbt_sum_args &a, i
         q.seg_rf = static_cast<const float2 *>(loss);
         q.rf_stride = td.capacity;
         q.n_items = cta_tiles(a.n_recv) * kTileWarps * splits;
-        q.work_counter = counter;
+        q.work_counter = counter + g0 / kGroupFreq;
         tile_prep_launch(q, a.window, tile_ws_layout(order_ws, a.n_recv, td.capacity, a.tile_cull != 0), s);
         if (stats) {
             if (a.window == GBT_WINDOW_LINE) launch_count_nf<GBT_WINDOW_LINE>(q, s);
@@ -2039,13 +2322,31 @@ void synth_launch(const float *p, int nf, int64_t n_recv, const double *freq_hz,
 size_t recv_order_scratch_bytes(int64_t n)
 {
     const int64_t nblocks = (n + kRadixBlock - 1) / kRadixBlock;
+    if (n <= kOrderSmall) return 0;
     return 2 * align_up((size_t)n * sizeof(unsigned long long), 256) +
-           align_up((size_t)kRadixBuckets * nblocks * sizeof(uint32_t), 256) + 256;
+           align_up((size_t)kRadixBuckets * nblocks * sizeof(uint32_t), 256) +
+           align_up(kRadixBuckets * sizeof(uint32_t), 256) + 256;
 }
 
 void recv_order_launch(const float *recv, int64_t n, int32_t *order, void *scratch, cudaStream_t s)
 {
     if (n <= 0) return;
+    if (n <= kOrderSmall) {
+        const size_t sm = sizeof(OrderCounts) + 2 * ((size_t)n + 1) * (sizeof(uint32_t) + sizeof(uint16_t));
+        static std::atomic<bool> set[64] = {};
+        int dev = 0;
+        GBT_CUDA(cudaGetDevice(&dev));
+        if (dev < 0 || dev >= 64) fail(GBT_ERR_UNSUPPORTED, "device index >= 64");
+        if (!set[dev].load(std::memory_order_acquire)) {
+            GBT_CUDA(cudaFuncSetAttribute(order_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)(sizeof(OrderCounts) + sizeof(OrderSmem) + 16)));
+            set[dev].store(true, std::memory_order_release);
+        }
+        order_small_kernel<<<1, kOrderThreads, sm, s>>>(recv, (int)n, order);
+        note_launches(1);
+        GBT_CUDA(cudaGetLastError());
+        return;
+    }
     const int64_t nblocks = (n + kRadixBlock - 1) / kRadixBlock;
     char *w = static_cast<char *>(scratch);
     unsigned long long *keys = reinterpret_cast<unsigned long long *>(w);
@@ -2054,6 +2355,8 @@ void recv_order_launch(const float *recv, int64_t n, int32_t *order, void *scrat
     w += align_up((size_t)n * sizeof(unsigned long long), 256);
     uint32_t *counts = reinterpret_cast<uint32_t *>(w);
     w += align_up((size_t)kRadixBuckets * nblocks * sizeof(uint32_t), 256);
+    uint32_t *total = reinterpret_cast<uint32_t *>(w);
+    w += align_up(kRadixBuckets * sizeof(uint32_t), 256);
     unsigned int *bb = reinterpret_cast<unsigned int *>(w);
     GBT_CUDA(cudaMemsetAsync(bb, 0xff, 3 * sizeof(unsigned int), s));
     GBT_CUDA(cudaMemsetAsync(bb + 3, 0x00, 3 * sizeof(unsigned int), s));
@@ -2063,8 +2366,8 @@ void recv_order_launch(const float *recv, int64_t n, int32_t *order, void *scrat
     note_launches(1);
     for (int shift = 0; shift < 30; shift += 8) {   // 30-bit codes: four passes
         radix_count_kernel<<<(unsigned)nblocks, kRadixBlock, 0, s>>>(keys, n, shift, counts, nblocks);
-        radix_scan_kernel<<<1, 1024, 0, s>>>(counts, (int64_t)kRadixBuckets * nblocks);
-        radix_scatter_kernel<<<(unsigned)nblocks, kRadixBlock, 0, s>>>(keys, tmp, n, shift, counts,
+        radix_scan_kernel<<<kRadixBuckets, 256, 0, s>>>(counts, nblocks, total);
+        radix_scatter_kernel<<<(unsigned)nblocks, kRadixBlock, 0, s>>>(keys, tmp, n, shift, counts, total,
                                                                          nblocks);
         note_launches(3);
         std::swap(keys, tmp);
@@ -2088,7 +2391,7 @@ static size_t bwd_layout(const TraceDev &td, const gbt_sum_args &a, const SceneD
     off[3] = b; b += align_up((size_t)td.capacity * sizeof(float), 256);
     off[4] = b; b += align_up((size_t)a.n_freq * td.capacity * sizeof(float), 256);
     off[5] = b; b += align_up((size_t)((sd ? sd->n_materials : 1024) + GBT_MAX_FREQ) * sizeof(double), 256);
-    off[6] = b; b += tile_ws_bytes(a.n_recv, td.capacity, a.tile_cull != 0);
+    off[6] = b; b += tile_ws_bytes(a.n_recv, td.capacity, a.tile_cull != 0, true);
     off[7] = b; b += loss_bytes(td, a);
     return b;
 }
@@ -2119,7 +2422,7 @@ void bwd_launch(const TraceDev &td, const SceneDev &sd, const gbt_sum_args &a,
     if (grad_w) GBT_CUDA(cudaMemsetAsync(grad_w, 0, (size_t)td.n_fan * sizeof(float), s));
 
     void *loss = loss_bytes(td, a) ? static_cast<void *>(w + off[7]) : nullptr;
-    prepass_launch(td, sd, a, rec, amp64, s, loss);
+    prepass_launch(td, sd, a, rec, amp64, counter, s, loss);
     // per frequency group: seg_G gathers every frequency's terms, seg_H the group's rows
     // (processing slots g0 .. g0 + nf - 1)
     if (a.n_recv > 0) {
@@ -2128,14 +2431,14 @@ void bwd_launch(const TraceDev &td, const SceneDev &sd, const gbt_sum_args &a,
             FwdParams q = make_pair_params(td, sd, a, rec, g0, true);
             q.splits = splits;
             q.n_items = cta_tiles(a.n_recv) * kTileWarps * splits;
-            q.work_counter = counter;
+            q.work_counter = counter + g0 / kGroupFreq;
             q.grad_out = reinterpret_cast<const float2 *>(grad_out);
             q.seg_G = seg_G;
             q.seg_H = seg_H + (int64_t)g0 * td.capacity;
             q.seg_stride = td.capacity;
             q.seg_rf = static_cast<const float2 *>(loss);
             q.rf_stride = td.capacity;
-            tile_prep_launch(q, a.window, tile_ws_layout(w + off[6], a.n_recv, td.capacity, a.tile_cull != 0), s);
+            tile_prep_launch(q, a.window, tile_ws_layout(w + off[6], a.n_recv, td.capacity, a.tile_cull != 0, true), s);
             pair_bwd_launch(q, a.window, s, true);
         }
     }
@@ -2261,7 +2564,8 @@ static void batch_layout(BatchImpl &B, cudaStream_t s)
         B.loss_off[i] = b;
         b += loss_bytes(B.traces[i]->d, B.args[i]);
     }
-    const size_t cnt = align_up((size_t)n * sizeof(int), 256);    // one work counter per instance
+    // work counters per instance (kCounters, of which an instance of one group uses the first)
+    const size_t cnt = align_up((size_t)n * kCounters * sizeof(int), 256);
     const size_t tab = align_up((size_t)n * sizeof(FwdParams), 256);
     const size_t off = align_up((size_t)(n + 1) * sizeof(int64_t), 256);
     const size_t need = b + cnt + tab + off;
@@ -2286,7 +2590,7 @@ static void batch_layout(BatchImpl &B, cudaStream_t s)
         q.splits = B.splits[i];
         q.n_items = cta_tiles(a.n_recv) * kTileWarps * q.splits;
         q.partial = reinterpret_cast<float4 *>(w + B.part_off[i]);
-        q.work_counter = B.mode == kConcurrent ? B.counter + k : B.counter;
+        q.work_counter = B.mode == kConcurrent ? B.counter + k * kCounters : B.counter;
         if (has_losses(a)) {
             q.seg_rf = reinterpret_cast<const float2 *>(w + B.loss_off[i]);
             q.rf_stride = td.capacity;
@@ -2309,12 +2613,12 @@ static void batch_layout(BatchImpl &B, cudaStream_t s)
     GBT_CUDA(cudaStreamSynchronize(s));
 }
 
-static void batch_prepass(BatchImpl &B, int i, cudaStream_t s)
+static void batch_prepass(BatchImpl &B, int i, int *counters, cudaStream_t s)
 {
     const TraceDev &td = B.traces[i]->d;
     char *w = static_cast<char *>(B.work);
     prepass_launch(td, td.scene->d, B.args[i], reinterpret_cast<float *>(w + B.rec_off[i]), nullptr,
-                   s, has_losses(B.args[i]) ? static_cast<void *>(w + B.loss_off[i]) : nullptr);
+                   counters, s, has_losses(B.args[i]) ? static_cast<void *>(w + B.loss_off[i]) : nullptr);
 }
 
 // Merge of instance i (processing index k) into its output.
@@ -2359,9 +2663,9 @@ static void batch_record_concurrent(BatchImpl &B, cudaStream_t s)
     for (int k = 0; k < n; ++k) {
         const int i = B.order[k];
         cudaStream_t bs = B.branch[k % nb];
-        batch_prepass(B, i, bs);
-        if (B.args[i].n_recv == 0) continue;
         const FwdParams &q = B.table[k];
+        batch_prepass(B, i, q.work_counter, bs);
+        if (B.args[i].n_recv == 0) continue;
         {
             FwdParams qq = q;
             tile_prep_launch(qq, B.window,
@@ -2385,7 +2689,7 @@ static void batch_record(BatchImpl &B, cudaStream_t s)
     }
     const int n = (int)B.args.size();
     char *w = static_cast<char *>(B.work);
-    for (int i = 0; i < n; ++i) batch_prepass(B, i, s);
+    for (int i = 0; i < n; ++i) batch_prepass(B, i, nullptr, s);
     for (int k = 0; k < n; ++k) {
         const int i = B.order[k];
         FwdParams qq = B.table[k];

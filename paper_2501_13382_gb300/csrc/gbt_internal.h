@@ -159,6 +159,19 @@ void scene_prepare(SceneDev &sd, const double *tri_raw_dev, cudaStream_t s);
 void trace_launch(const SceneDev &sd, TraceDev &td, const gbt_source_desc &src,
                   void *scratch, size_t scratch_bytes, cudaStream_t s);
 size_t trace_scratch_bytes(int64_t n_rays, int max_refl);
+// The tracer's padded rows (ray r's segments at slots r * stride ..), before the scan and
+// compaction: what a solve packs its records from.
+constexpr int kPackRays = 256;         // rays per block of the packing kernel and per entry of bsum
+struct PaddedRays {
+    int64_t n_rays, ray_begin, stride;
+    const int32_t *cnt, *bmat;         // segments per ray; materials per slot
+    const double *o, *t, *L, *s0;
+    const int32_t *bsum;               // segments per kPackRays rays, or (scanned) before them
+    int scanned;
+    int32_t *n_seg;                    // where the segment count goes
+};
+PaddedRays trace_rays_launch(const SceneDev &sd, TraceDev &td, const gbt_source_desc &src,
+                             void *scratch, size_t scratch_bytes, cudaStream_t s);
 // Fills each segment's ray index and depth from the trace's offsets (imported traces).
 void csr_ray_depth_launch(TraceDev &td, cudaStream_t s);
 
@@ -169,7 +182,8 @@ size_t sum_workspace_bytes(const TraceDev &td, const gbt_sum_args &a, int splits
 int choose_splits(const TraceDev &td, const gbt_sum_args &a);
 void sum_launch(const TraceDev &td, const SceneDev &sd, const gbt_sum_args &a, int splits,
                 void *work, cudaStream_t s, unsigned long long *stats = nullptr,
-                bool differentiable = false);   // with the adjoint's own evaluation (F32)
+                bool differentiable = false,    // with the adjoint's own evaluation (F32)
+                const PaddedRays *rays = nullptr);   // records from these instead of td's list
 void recv_order_launch(const float *recv, int64_t n, int32_t *order, void *scratch,
                        cudaStream_t s);
 size_t recv_order_scratch_bytes(int64_t n);

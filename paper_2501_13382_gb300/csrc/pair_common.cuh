@@ -54,7 +54,7 @@ struct alignas(16) FwdParams {
     float s_scale;             // staged s is s times this: 1 / b when uniform and forward, else 1
     int splits;
     int64_t n_items;           // CTA tiles x splits
-    int *work_counter;         // zeroed before launch; warps take items from it
+    int *work_counter;         // zero at launch (prepass); warps take items from it
     const int32_t *tile_perm;  // dispatch rank -> CTA tile (heaviest first), or null
     // tile pre-cull: per CTA tile, the segments whose beams can reach its receivers
     const int32_t *list;       // segment indices, each tile's in segment order, or null

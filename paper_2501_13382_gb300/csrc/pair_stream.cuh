@@ -229,14 +229,13 @@ int resident_ctas(FN fn, std::atomic<int> (&known)[64])
     return per_sm;
 }
 
-// Launches one persistent kernel over p's items.
+// Launches one persistent kernel over p's items (p.work_counter zeroed by the prepass).
 template <class CFG, class FN>
 void launch_items(FN fn, std::atomic<int> (&known)[64], const FwdParams &p, cudaStream_t s, bool timed)
 {
     const int per_sm = resident_ctas<CFG>(fn, known);
     const int grid = (int)std::max<int64_t>(
         1, std::min<int64_t>((p.n_items + CFG::kWarps - 1) / CFG::kWarps, (int64_t)per_sm * num_sms()));
-    GBT_CUDA(cudaMemsetAsync(p.work_counter, 0, sizeof(int), s));
     if (timed) timing_begin(s);
     fn<<<grid, 32 * CFG::kWarps, CFG::kSmem, s>>>(p);
     note_launches(1);

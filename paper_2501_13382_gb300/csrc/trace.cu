@@ -89,6 +89,7 @@ struct TraceParams {
     int64_t stride;            // max_refl + 1
     double *po, *pt, *pL, *ps0;
     int32_t *pbmat, *phit, *cnt;
+    int32_t *bsum;             // segments per kPackRays rays (zeroed), or nullptr
 };
 
 // Moller-Trumbore test against a triangle given as v0, e1, e2 (12-double record);
@@ -465,6 +466,12 @@ __device__ __forceinline__ bool record_and_reflect(const TraceParams &p, int64_t
     return true;
 }
 
+__device__ __forceinline__ void write_count(const TraceParams &p, int64_t i, int nseg)
+{
+    p.cnt[i] = nseg;
+    if (p.bsum) atomicAdd(&p.bsum[i / kPackRays], nseg);
+}
+
 // Scene too large for one shared-memory chunk: the block streams the triangle chunks
 // for every bounce, so its rays advance bounce by bounce together.
 __global__ void __launch_bounds__(kTraceBlock) trace_kernel(TraceParams p)
@@ -500,7 +507,7 @@ __global__ void __launch_bounds__(kTraceBlock) trace_kernel(TraceParams p)
         if (alive) alive = record_and_reflect(p, i, o, d, s0, last_face, bmat, nref, nseg, tbest, best);
         if (!__syncthreads_or(alive)) break;
     }
-    if (active) p.cnt[i] = nseg;
+    if (active) write_count(p, i, nseg);
 }
 
 // Scene resident in shared memory: after the one load, every warp takes strips of 32
@@ -537,7 +544,7 @@ __global__ void __launch_bounds__(kTraceBlock) trace_resident_kernel(TraceParams
                 nearest_in_chunk(o, d, last_face, st, stbox, sbox, sface, 0, (int)p.n_tri, tbest, best);
             alive = record_and_reflect(p, i, o, d, s0, last_face, bmat, nref, nseg, tbest, best);
         }
-        p.cnt[i] = nseg;
+        write_count(p, i, nseg);
     }
 }
 
@@ -564,7 +571,7 @@ __global__ void __launch_bounds__(kTraceBlock) trace_bvh_kernel(TraceParams p)
             nearest_in_bvh(p, o, d, last_face, tbest, best);
             alive = record_and_reflect(p, i, o, d, s0, last_face, bmat, nref, nseg, tbest, best);
         }
-        p.cnt[i] = nseg;
+        write_count(p, i, nseg);
     }
 }
 
@@ -739,11 +746,15 @@ size_t trace_scratch_bytes(int64_t n_rays, int max_refl)
     b += align_up((size_t)n_rays * sizeof(int32_t), 256);   // cnt
     b += align_up((nb + 1) * sizeof(int32_t), 256);     // block sums
     b += 256;                                           // strip counter
+    b += align_up((size_t)((n_rays + kPackRays - 1) / kPackRays) * sizeof(int32_t), 256);   // pack sums
     return b;
 }
 
-void trace_launch(const SceneDev &sd, TraceDev &td, const gbt_source_desc &src, void *scratch,
-                  size_t scratch_bytes, cudaStream_t s)
+// Launches the tracer into the padded rows of scratch; with `sums`, also the segment counts
+// per kPackRays rays.  p and bsum: where things are.
+static void rays_launch(const SceneDev &sd, TraceDev &td, const gbt_source_desc &src, void *scratch,
+                        size_t scratch_bytes, bool sums, TraceParams &p, int32_t *&bsum,
+                        cudaStream_t s)
 {
     const int64_t n = td.n_rays;
     const int64_t stride = td.max_refl + 1;
@@ -754,7 +765,7 @@ void trace_launch(const SceneDev &sd, TraceDev &td, const gbt_source_desc &src, 
         w += align_up(bytes, 256);
         return p;
     };
-    TraceParams p{};
+    p = TraceParams{};
     p.src[0] = src.pos[0]; p.src[1] = src.pos[1]; p.src[2] = src.pos[2];
     p.n_fan = td.n_fan;
     p.ray_begin = td.ray_begin;
@@ -796,8 +807,12 @@ void trace_launch(const SceneDev &sd, TraceDev &td, const gbt_source_desc &src, 
     p.cnt = reinterpret_cast<int32_t *>(take((size_t)n * sizeof(int32_t)));
     const int64_t per = (int64_t)kScanBlock * kScanItems;
     const int64_t nb = (n + per - 1) / per;
-    int32_t *bsum = reinterpret_cast<int32_t *>(take((size_t)(nb + 1) * sizeof(int32_t)));
-    p.counter = reinterpret_cast<unsigned long long *>(take(sizeof(unsigned long long)));
+    bsum = reinterpret_cast<int32_t *>(take((size_t)(nb + 1) * sizeof(int32_t)));
+    // the strip counter and the pack sums, zeroed together
+    p.counter = reinterpret_cast<unsigned long long *>(take(256));
+    const size_t packs = (size_t)((n + kPackRays - 1) / kPackRays);
+    int32_t *pack = reinterpret_cast<int32_t *>(take(packs * sizeof(int32_t)));
+    p.bsum = sums ? pack : nullptr;
     if ((size_t)(w - static_cast<char *>(scratch)) > scratch_bytes)
         fail(GBT_ERR_INVALID_ARG, "trace scratch too small");
 
@@ -819,6 +834,7 @@ void trace_launch(const SceneDev &sd, TraceDev &td, const gbt_source_desc &src, 
     // 768 triangles: 3.2 ms against 5.4 ms for 1,048,576 rays through the synthetic city
     // (1.5 ms since)
     const bool use_bvh = sd.n_tri > 0 && sd.bvh && sd.accel != GBT_ACCEL_LINEAR;
+    GBT_CUDA(cudaMemsetAsync(p.counter, 0, 256 + (sums ? packs * sizeof(int32_t) : 0), s));
     if (use_bvh) {
         int per_sm = 0;
         GBT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, trace_bvh_kernel, kTraceBlock, 0));
@@ -826,7 +842,6 @@ void trace_launch(const SceneDev &sd, TraceDev &td, const gbt_source_desc &src, 
         const int64_t blocks = std::max<int64_t>(
             1, std::min<int64_t>((int64_t)std::max(per_sm, 1) * num_sms(),
                                  (strips + kTraceBlock / 32 - 1) / (kTraceBlock / 32)));
-        GBT_CUDA(cudaMemsetAsync(p.counter, 0, sizeof(unsigned long long), s));
         trace_bvh_kernel<<<(unsigned)blocks, kTraceBlock, 0, s>>>(p);
     } else if (sd.n_tri <= p.chunk) {
         // resident scene: a persistent grid whose warps take strips of rays
@@ -837,14 +852,47 @@ void trace_launch(const SceneDev &sd, TraceDev &td, const gbt_source_desc &src, 
         const int64_t blocks = std::max<int64_t>(
             1, std::min<int64_t>((int64_t)std::max(per_sm, 1) * num_sms(),
                                  (strips + kTraceBlock / 32 - 1) / (kTraceBlock / 32)));
-        GBT_CUDA(cudaMemsetAsync(p.counter, 0, sizeof(unsigned long long), s));
         trace_resident_kernel<<<(unsigned)blocks, kTraceBlock, smem, s>>>(p);
     } else {
         trace_kernel<<<(unsigned)((n + kTraceBlock - 1) / kTraceBlock), kTraceBlock, smem, s>>>(p);
     }
     note_launches(1);
     GBT_CUDA(cudaGetLastError());
+}
 
+PaddedRays trace_rays_launch(const SceneDev &sd, TraceDev &td, const gbt_source_desc &src,
+                             void *scratch, size_t scratch_bytes, cudaStream_t s)
+{
+    TraceParams p;
+    int32_t *bsum;
+    rays_launch(sd, td, src, scratch, scratch_bytes, true, p, bsum, s);
+    PaddedRays r{};
+    r.n_rays = td.n_rays; r.ray_begin = td.ray_begin; r.stride = p.stride;
+    r.cnt = p.cnt; r.bmat = p.pbmat;
+    r.o = p.po; r.t = p.pt; r.L = p.pL; r.s0 = p.ps0;
+    r.bsum = p.bsum;
+    r.n_seg = td.ray_off + td.n_rays;
+    // each packing block adds up the entries before its own; beyond 4,096 of them (1M rays) a
+    // scan of the entries is the smaller part
+    const int64_t packs = (td.n_rays + kPackRays - 1) / kPackRays;
+    if (packs > 4096) {
+        scan_of_block_sums<<<1, kScanBlock, 0, s>>>(p.bsum, packs);
+        note_launches(1);
+        GBT_CUDA(cudaGetLastError());
+        r.scanned = 1;
+    }
+    return r;
+}
+
+void trace_launch(const SceneDev &sd, TraceDev &td, const gbt_source_desc &src, void *scratch,
+                  size_t scratch_bytes, cudaStream_t s)
+{
+    TraceParams p;
+    int32_t *bsum;
+    rays_launch(sd, td, src, scratch, scratch_bytes, false, p, bsum, s);
+    const int64_t n = td.n_rays, stride = p.stride;
+    const int64_t per = (int64_t)kScanBlock * kScanItems;
+    const int64_t nb = (n + per - 1) / per;
     scan_block_sums<<<(unsigned)nb, kScanBlock, 0, s>>>(p.cnt, n, bsum);
     note_launches(1);
     scan_of_block_sums<<<1, kScanBlock, 0, s>>>(bsum, nb);

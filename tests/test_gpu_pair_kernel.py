@@ -91,3 +91,25 @@ def test_f64_kernel_edges(n, rays, nf, window, cutoff):
     torch.cuda.synchronize()
     e = p.cpu().numpy().astype(np.complex128) - po
     assert np.linalg.norm(e) <= 1e-7 * np.linalg.norm(po)
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 1023, 1024, 1025, 5000, 16383, 16384, 16385, 40001])
+def test_receiver_order_is_the_stable_morton_order(n):
+    """One block up to 16,384 receivers, radix passes over the grid beyond; codes and order
+    from numpy in the same FP32 steps, ties by index.  Integers: no tolerance."""
+    import torch
+    from paper_2501_13382_gb300 import gbt as G
+    rng = np.random.default_rng(n)
+    x = rng.uniform(-300, 300, (n, 3)).astype(np.float32)
+    x[:, 2] = rng.choice(np.float32([1.5, 4.0]), n)
+    x[n // 2:] = x[rng.integers(0, max(n // 2, 1), n - n // 2)] if n > 1 else x[n // 2:]   # ties
+    lo, hi = x.min(0), x.max(0)
+    span = (hi - lo).astype(np.float32)
+    u = np.where(span > 0, (x - lo) / np.where(span > 0, span, np.float32(1)), np.float32(0)).astype(np.float32)
+    q = np.clip(u * np.float32(1023), 0, 1023).astype(np.uint32)
+    code = np.zeros(n, np.uint64)
+    for b in range(10):
+        for a in range(3):
+            code |= ((q[:, a] >> b) & 1).astype(np.uint64) << np.uint64(3 * b + a)
+    got = G.recv_order(torch.as_tensor(x, device="cuda")).cpu().numpy()
+    assert np.array_equal(got, np.argsort(code, kind="stable"))
