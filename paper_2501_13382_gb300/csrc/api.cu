@@ -661,8 +661,8 @@ static gbt_status sum_call(const char *name, const gbt_trace_t *trace, const gbt
         cudaStream_t s = static_cast<cudaStream_t>(stream);
         gbt_trace_t *tr = const_cast<gbt_trace_t *>(trace);
         const SceneDev &sd = tr->d.scene->d;
-        const int splits = choose_splits(tr->d, *args);
-        void *w = tr->d.work.ensure(sum_workspace_bytes(tr->d, *args, splits), s);
+        const int splits = choose_splits(tr->d, *args, differentiable);
+        void *w = tr->d.work.ensure(sum_workspace_bytes(tr->d, *args, splits, differentiable), s);
         sum_launch(tr->d, sd, *args, splits, w, s, nullptr, differentiable);
         mark_trace_used(tr, s);
     });

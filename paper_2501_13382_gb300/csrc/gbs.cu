@@ -717,6 +717,7 @@ __global__ void __launch_bounds__(32 * kWarps64) gbs_fwd_f64_kernel(const __grid
     m.wbase = ((int64_t)blockIdx.x * kWarps64 + (threadIdx.x >> 5)) * 32;
     if (m.wbase >= p.n_recv) return;            // warps never wait for one another
     m.split = blockIdx.y;
+    m.splits = p.g.splits;
     m.lst = nullptr;
     m.lw = nullptr;
     m.n_seg = *p.g.n_seg_ptr;
@@ -1266,11 +1267,21 @@ __global__ void list_words_kernel(const float4 *crec, const float4 *wball, int64
 }
 
 // One block: list ranges, tiles lightest first (perm lists them heaviest first), each
-// starting on a 32-entry chunk boundary.
+// starting on a 32-entry chunk boundary; and, with want > 0, each tile's segment splits,
+// want per tile on average (at most (want + 1) x n_tiles in all), numbered heaviest tile
+// first.  A tile's share goes with the root of its list length, its cost: equal shares make
+// the heavy tiles' items ten times the mean, so that the queue drains well only with three
+// times as many of them, whose per-item work and partial sums then cost more than the tail
+// they save; shares with the cost itself make the last items as long as the first.  Equal
+// (32 items per warp) | root (12) | cost (12), in ms: 1 M rays x 1024^2 x 1 band, city,
+// 22.4 | 19.4 | 20.4; 192^2 x 8 bands with losses 6.40 | 6.42 | 6.94; batch of 8 sources x
+// 128^2 x 8 bands 4.63 | 3.62 | 3.67; 4,096 scattered receivers .724 | .701 | .697.
 __global__ void __launch_bounds__(1024) list_layout_kernel(const unsigned int *total,
                                                            const int32_t *perm, int64_t n_tiles,
                                                            int64_t cap, int64_t *list_off,
-                                                           int32_t *list_n)
+                                                           int32_t *list_n, const int32_t *n_seg_ptr,
+                                                           int64_t want, int32_t *item_off,
+                                                           int32_t *tile_first, int32_t *tile_splits)
 {
     __shared__ int64_t ws[33];
     const int64_t per = (n_tiles + 1023) / 1024;
@@ -1291,6 +1302,31 @@ __global__ void __launch_bounds__(1024) list_layout_kernel(const unsigned int *t
         list_n[t] = off + padded(n) <= cap ? (int32_t)n : -1;
         off += padded(n);
     }
+    if (want <= 0) return;
+    __syncthreads();       // every list_n is written
+    const int64_t scan_cost = *n_seg_ptr / 8;      // a tile without a list tests every segment
+    auto rank_tile = [&](int64_t r) { return perm ? (int64_t)perm[r] : r; };
+    auto cost = [&](int64_t t) { return (int64_t)total[t] + (list_n[t] < 0 ? scan_cost : 0); };
+    auto share = [&](int64_t t) { return (int64_t)(64.0f * sqrtf((float)cost(t))) + 1; };
+    sum = 0;
+    for (int64_t r = i0; r < i0 + per && r < n_tiles; ++r) sum += share(rank_tile(r));
+    int64_t at;
+    const int64_t all = block_scan_1024(sum, at, ws);
+    const int64_t each = max((all + want - 1) / want, (int64_t)1);
+    auto splits = [&](int64_t t) {
+        return max(min((share(t) + each - 1) / each, (cost(t) + 63) / 64), (int64_t)1);
+    };
+    sum = 0;
+    for (int64_t r = i0; r < i0 + per && r < n_tiles; ++r) sum += splits(rank_tile(r));
+    const int64_t n_items = block_scan_1024(sum, at, ws);
+    for (int64_t r = i0; r < i0 + per && r < n_tiles; ++r) {
+        const int64_t t = rank_tile(r), s = splits(t);
+        item_off[r] = (int32_t)at;
+        tile_first[t] = (int32_t)at;
+        tile_splits[t] = (int32_t)s;
+        at += s;
+    }
+    if (threadIdx.x == 0) item_off[n_tiles] = (int32_t)n_items;
 }
 
 template <int WINDOW>
@@ -1480,6 +1516,9 @@ struct ReduceParams {
     const double2 *p64;        // F64 path: by receiver
     float2 *out;
     int accumulate;
+    // weighted splits: per tile its first tile-split and their number, or nullptr
+    const int32_t *tile_first, *tile_splits;
+    int nf;
 };
 
 // Float-float partials (hi, running FP32 sum of errors) merged into a float-float total with
@@ -1506,11 +1545,17 @@ __global__ void __launch_bounds__(32 * kMergeGroups) reduce_kernel(ReduceParams 
     const int64_t i = blockIdx.x * (int64_t)32 + lane;
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
     if (i < p.n) {
-        const int s0 = (int)((int64_t)p.splits * g / kMergeGroups);
-        const int s1 = (int)((int64_t)p.splits * (g + 1) / kMergeGroups);
+        int64_t n = p.splits, stride = p.n;
         const float4 *src = p.p32 + i;
+        if (p.tile_first) {
+            const int64_t f = i / p.n_recv, r = i - f * p.n_recv, t = r / kCtaRecv;
+            n = p.tile_splits[t];
+            stride = (int64_t)p.nf * kCtaRecv;
+            src = p.p32 + p.tile_first[t] * stride + f * kCtaRecv + (r - t * kCtaRecv);
+        }
+        const int s0 = (int)(n * g / kMergeGroups), s1 = (int)(n * (g + 1) / kMergeGroups);
 #pragma unroll 8
-        for (int s = s0; s < s1; ++s) merge_ff(a, __ldcs(src + (int64_t)s * p.n));
+        for (int s = s0; s < s1; ++s) merge_ff(a, __ldcs(src + s * stride));
     }
     part[g][lane] = a;
     __syncthreads();
@@ -1982,7 +2027,7 @@ static size_t loss_bytes(const TraceDev &td, const gbt_sum_args &a)
            align_up((size_t)a.n_freq * (size_t)td.scene->d.n_materials * sizeof(double2), 256);
 }
 
-int choose_splits(const TraceDev &td, const gbt_sum_args &a)
+int choose_splits(const TraceDev &td, const gbt_sum_args &a, bool adjoint)
 {
     if (a.seg_split > 0) return a.seg_split;
     const int64_t nseg_est = td.n_seg_host >= 0 ? td.n_seg_host : td.capacity;
@@ -1994,11 +2039,13 @@ int choose_splits(const TraceDev &td, const gbt_sum_args &a)
         s = std::max<int64_t>(1, std::min<int64_t>(s, (nseg_est + 2 * kBatch - 1) / (2 * kBatch)));
         return (int)std::min<int64_t>(s, 4096);
     }
-    // items are (warp tile, split): about 16 per resident warp, 32 with the pre-cull (its
-    // item costs vary more), so that the last items to finish are short ones
+    // items are (warp tile, split): about 16 per resident warp, so that the last items to
+    // finish are short ones; with the pre-cull 12, shared out by list length (see
+    // list_layout_kernel; 16 and 24: 0-5 % slower for a batch, within 1 % elsewhere), and 32
+    // equal ones for the differentiable sum, whose tiles are split alike
     const int64_t wtiles = std::max<int64_t>(1, (a.n_recv + kCtaRecv - 1) / kCtaRecv) * kTileWarps;
     const int64_t warps = (int64_t)num_sms() * kWarpsFwd;
-    const int64_t per_warp = a.tile_cull ? 32 : 16;
+    const int64_t per_warp = !a.tile_cull ? 16 : adjoint ? 32 : 12;
     int64_t s = (per_warp * warps + wtiles - 1) / wtiles;
     s = std::max<int64_t>(1, std::min<int64_t>(s, (nseg_est + kBatch - 1) / kBatch));
     // partial sums stay under ~1 GiB
@@ -2023,6 +2070,8 @@ struct TileWs {
     uint32_t *words = nullptr;     // per 32-entry list chunk: one word per warp tile
     float4 *wball = nullptr;       // per warp tile: bounding ball
     uint32_t *bits = nullptr;      // [tiles][chunks * 32]: the counting pass's ballots, or null
+    int32_t *item_off = nullptr;   // by rank, tiles + 1: first tile-split of each tile (see list_layout_kernel)
+    int32_t *tile_first = nullptr, *tile_splits = nullptr;   // the same by tile
     int64_t tiles = 0, chunks = 0, cap = 0, wtiles = 0;
     bool order = false, lists = false;
     size_t bytes = 0;              // workspace the layout needs
@@ -2067,6 +2116,9 @@ static TileWs tile_ws_layout(void *ws, int64_t n_recv, int64_t seg_capacity, boo
         t.counts = reinterpret_cast<int32_t *>(take((size_t)(t.tiles * t.chunks) * sizeof(int32_t)));
         t.list_off = reinterpret_cast<int64_t *>(take((size_t)t.tiles * sizeof(int64_t)));
         t.list_n = reinterpret_cast<int32_t *>(take((size_t)t.tiles * sizeof(int32_t)));
+        t.item_off = reinterpret_cast<int32_t *>(take((size_t)(t.tiles + 1) * sizeof(int32_t)));
+        t.tile_first = reinterpret_cast<int32_t *>(take((size_t)t.tiles * sizeof(int32_t)));
+        t.tile_splits = reinterpret_cast<int32_t *>(take((size_t)t.tiles * sizeof(int32_t)));
         t.list = reinterpret_cast<int32_t *>(take((size_t)t.cap * sizeof(int32_t)));
         t.words = reinterpret_cast<uint32_t *>(take((size_t)(t.cap / 32) * kChunkWords * sizeof(uint32_t)));
         t.wball = reinterpret_cast<float4 *>(take((size_t)t.wtiles * sizeof(float4)));
@@ -2084,11 +2136,33 @@ static size_t tile_ws_bytes(int64_t n_recv, int64_t seg_capacity, bool tile_cull
     return tile_ws_layout(nullptr, n_recv, seg_capacity, tile_cull, adjoint).bytes;
 }
 
+// Whether a sum's tiles are split in proportion to their lists (else every tile alike): the
+// automatic split of the pre-culled forward sum.
+static bool weighted_splits(const gbt_sum_args &a, const TileWs &t, bool adjoint)
+{
+    return t.lists && a.seg_split == 0 && !adjoint;
+}
+// Points q at a weighted layout: tile-splits instead of splits per tile.
+static void set_weighted(FwdParams &q, const TileWs &t)
+{
+    q.item_off = t.item_off;
+    q.n_tiles = (int32_t)t.tiles;
+    q.n_items = ((int64_t)q.splits + 1) * t.tiles * kTileWarps;     // at most (sizes the grid)
+}
+// Float-float partials of nf bands: [split][band][receiver], or weighted
+// [tile-split][band][receiver of the tile].
+static size_t partial_count(const gbt_sum_args &a, int nf, int splits, bool weighted)
+{
+    return weighted ? ((size_t)splits + 1) * (size_t)cta_tiles(a.n_recv) * kCtaRecv * nf
+                    : (size_t)splits * nf * (size_t)a.n_recv;
+}
+
 // Launches the tile preparation for q's receivers and records (the records must
 // be written earlier on s) and points q at its results: the dispatch order and,
 // with the pre-cull, the segment lists.  Weights are the exact list sizes when
 // the lists are built, else a sampled count.
-static void tile_prep_launch(FwdParams &q, int window, const TileWs &t, cudaStream_t s)
+static void tile_prep_launch(FwdParams &q, int window, const TileWs &t, cudaStream_t s,
+                             bool weighted = false)
 {
     if (!t.order && !t.lists) return;
     const int64_t T = t.tiles;
@@ -2130,7 +2204,9 @@ static void tile_prep_launch(FwdParams &q, int window, const TileWs &t, cudaStre
     }
     if (t.lists) {
         list_layout_kernel<<<1, 1024, 0, s>>>(t.weight, t.order ? t.perm : nullptr, T, t.cap,
-                                              t.list_off, t.list_n);
+                                              t.list_off, t.list_n, q.n_seg_ptr,
+                                              weighted ? (int64_t)q.splits * T : 0, t.item_off,
+                                              t.tile_first, t.tile_splits);
         warp_ball_kernel<<<(unsigned)((t.wtiles + 7) / 8), 256, 0, s>>>(q.recv, q.order, q.n_recv,
                                                                          t.wtiles, t.wball);
         const dim3 mgrid(128, (unsigned)T);     // many blocks per tile: the gathers overlap
@@ -2160,6 +2236,7 @@ static void tile_prep_launch(FwdParams &q, int window, const TileWs &t, cudaStre
         q.list_off = t.list_off;
         q.list_n = t.list_n;
         q.list_words = t.words;
+        if (weighted) set_weighted(q, t);
     }
     GBT_CUDA(cudaGetLastError());
     note_launches(n);
@@ -2236,14 +2313,21 @@ static void prepass_launch(const TraceDev &td, const SceneDev &sd, const gbt_sum
     GBT_CUDA(cudaGetLastError());
 }
 
-size_t sum_workspace_bytes(const TraceDev &td, const gbt_sum_args &a, int splits)
+// Partials of all of a sum's frequency groups.
+static size_t partial_bytes(const TraceDev &td, const gbt_sum_args &a, int splits, bool adjoint)
+{
+    if (a.precision == GBT_PRECISION_F64)
+        return align_up((size_t)splits * a.n_freq * (size_t)a.n_recv * sizeof(double2), 256);
+    const bool w = weighted_splits(a, tile_ws_layout(nullptr, a.n_recv, td.capacity, a.tile_cull != 0), adjoint);
+    return align_up(partial_count(a, a.n_freq, splits, w) * sizeof(float4), 256);
+}
+
+size_t sum_workspace_bytes(const TraceDev &td, const gbt_sum_args &a, int splits, bool adjoint)
 {
     size_t b = records_bytes(td);
     b += align_up((size_t)td.capacity * sizeof(double), 256);               // amp64
     b += 256;                                                               // work counter
-    const size_t part = (size_t)splits * a.n_freq * (size_t)a.n_recv;
-    b += align_up(part * (a.precision == GBT_PRECISION_F64 ? sizeof(double2) : sizeof(float4)),
-                  256);
+    b += partial_bytes(td, a, splits, adjoint);
     if (a.precision != GBT_PRECISION_F64) b += tile_ws_bytes(a.n_recv, td.capacity, a.tile_cull != 0);
     b += loss_bytes(td, a);
     return b;
@@ -2261,9 +2345,7 @@ void sum_launch(const TraceDev &td, const SceneDev &sd, const gbt_sum_args &a, i
     int *counter = reinterpret_cast<int *>(w);
     w += 256;
     void *partial = w;
-    w += align_up((size_t)splits * a.n_freq * (size_t)a.n_recv *
-                      (a.precision == GBT_PRECISION_F64 ? sizeof(double2) : sizeof(float4)),
-                  256);
+    w += partial_bytes(td, a, splits, differentiable);
     void *order_ws = w;
     if (a.precision != GBT_PRECISION_F64) w += tile_ws_bytes(a.n_recv, td.capacity, a.tile_cull != 0);
     void *loss = loss_bytes(td, a) ? static_cast<void *>(w) : nullptr;
@@ -2320,13 +2402,15 @@ void sum_launch(const TraceDev &td, const SceneDev &sd, const gbt_sum_args &a, i
     for (int g0 = 0; g0 < a.n_freq; g0 += kGroupFreq) {
         FwdParams q = make_pair_params(td, sd, a, rec, g0, differentiable);
         q.splits = splits;
-        q.partial = reinterpret_cast<float4 *>(partial) + (int64_t)splits * g0 * a.n_recv;
+        const TileWs tw = tile_ws_layout(order_ws, a.n_recv, td.capacity, a.tile_cull != 0);
+        const bool weighted = weighted_splits(a, tw, differentiable) && !stats;
+        q.partial = reinterpret_cast<float4 *>(partial) + partial_count(a, g0, splits, weighted);
         q.stats = stats;
         q.seg_rf = static_cast<const float2 *>(loss);
         q.rf_stride = td.capacity;
         q.n_items = cta_tiles(a.n_recv) * kTileWarps * splits;
         q.work_counter = counter + g0 / kGroupFreq;
-        tile_prep_launch(q, a.window, tile_ws_layout(order_ws, a.n_recv, td.capacity, a.tile_cull != 0), s);
+        tile_prep_launch(q, a.window, tw, s, weighted);
         if (stats) {
             if (a.window == GBT_WINDOW_LINE) launch_count_nf<GBT_WINDOW_LINE>(q, s);
             else launch_count_nf<GBT_WINDOW_SEGMENT>(q, s);
@@ -2338,6 +2422,9 @@ void sum_launch(const TraceDev &td, const SceneDev &sd, const gbt_sum_args &a, i
         for (int f = 0; f < GBT_MAX_FREQ; ++f) rp.perm[f] = q.fperm[f];
         for (int f = 0; f < q.nf; ++f) rp.scale[f] = differentiable ? 1.0f : q.fc[f].sA;
         rp.p32 = q.partial;
+        rp.tile_first = weighted ? tw.tile_first : nullptr;
+        rp.tile_splits = tw.tile_splits;
+        rp.nf = q.nf;
         reduce_launch(rp, s);
     }
 }
@@ -2485,7 +2572,7 @@ void bwd_launch(const TraceDev &td, const SceneDev &sd, const gbt_sum_args &a,
     // per frequency group: seg_G gathers every frequency's terms, seg_H the group's rows
     // (processing slots g0 .. g0 + nf - 1)
     if (a.n_recv > 0) {
-        const int splits = choose_splits(td, a);
+        const int splits = choose_splits(td, a, true);
         for (int g0 = 0; g0 < a.n_freq; g0 += kGroupFreq) {
             FwdParams q = make_pair_params(td, sd, a, rec, g0, true);
             q.splits = splits;
@@ -2607,6 +2694,14 @@ static void batch_plan_concurrent(BatchImpl &B)
     for (int i = 0; i < n; ++i) B.splits[i] = choose_splits(B.traces[i]->d, B.args[i]);
 }
 
+// The fused form's table holds each instance's items, so its tiles are split alike.
+static bool batch_weighted(const BatchImpl &B, int i)
+{
+    const gbt_sum_args &a = B.args[i];
+    return B.mode == kConcurrent &&
+           weighted_splits(a, tile_ws_layout(nullptr, a.n_recv, B.traces[i]->d.capacity, a.tile_cull != 0), false);
+}
+
 static void batch_layout(BatchImpl &B, cudaStream_t s)
 {
     const int n = (int)B.args.size();
@@ -2619,7 +2714,7 @@ static void batch_layout(BatchImpl &B, cudaStream_t s)
         B.rec_off[i] = b;
         b += records_bytes(B.traces[i]->d);
         B.part_off[i] = b;
-        b += align_up((size_t)B.splits[i] * B.args[i].n_freq * (size_t)B.args[i].n_recv *
+        b += align_up(partial_count(B.args[i], B.args[i].n_freq, B.splits[i], batch_weighted(B, i)) *
                           sizeof(float4), 256);
         B.ord_off[i] = b;
         b += tile_ws_bytes(B.args[i].n_recv, B.traces[i]->d.capacity, B.args[i].tile_cull != 0);
@@ -2664,6 +2759,7 @@ static void batch_layout(BatchImpl &B, cudaStream_t s)
             q.list_off = t.lists ? t.list_off : nullptr;
             q.list_n = t.lists ? t.list_n : nullptr;
             q.list_words = t.lists ? t.words : nullptr;
+            if (batch_weighted(B, i)) set_weighted(q, t);
         }
         B.table.push_back(q);
         B.inst_off.push_back(B.inst_off.back() + q.n_items);
@@ -2700,6 +2796,13 @@ static void batch_reduce(BatchImpl &B, int k, cudaStream_t s)
     rp.order = a.recv_order;
     rp.out = reinterpret_cast<float2 *>(a.out);
     rp.accumulate = a.accumulate;
+    if (batch_weighted(B, i)) {
+        const TileWs t = tile_ws_layout(static_cast<char *>(B.work) + B.ord_off[i], a.n_recv,
+                                        B.traces[i]->d.capacity, a.tile_cull != 0);
+        rp.tile_first = t.tile_first;
+        rp.tile_splits = t.tile_splits;
+        rp.nf = a.n_freq;
+    }
     reduce_launch(rp, s);
 }
 
@@ -2732,7 +2835,8 @@ static void batch_record_concurrent(BatchImpl &B, cudaStream_t s)
             FwdParams qq = q;
             tile_prep_launch(qq, B.window,
                              tile_ws_layout(w + B.ord_off[i], B.args[i].n_recv,
-                                            B.traces[i]->d.capacity, B.args[i].tile_cull != 0), bs);
+                                            B.traces[i]->d.capacity, B.args[i].tile_cull != 0), bs,
+                             batch_weighted(B, i));
         }
         pair_fwd_launch(q, B.window, bs, false);
         batch_reduce(B, k, bs);

@@ -178,8 +178,9 @@ void csr_ray_depth_launch(TraceDev &td, cudaStream_t s);
 // ---- GBS launchers (gbs.cu) ----
 // Whether a sum carries propagation losses (air absorption or porous surfaces).
 bool has_losses(const gbt_sum_args &a);
-size_t sum_workspace_bytes(const TraceDev &td, const gbt_sum_args &a, int splits);
-int choose_splits(const TraceDev &td, const gbt_sum_args &a);
+size_t sum_workspace_bytes(const TraceDev &td, const gbt_sum_args &a, int splits, bool adjoint = false);
+// `adjoint`: for the adjoint and the sum it differentiates, whose field keeps its grouping.
+int choose_splits(const TraceDev &td, const gbt_sum_args &a, bool adjoint = false);
 void sum_launch(const TraceDev &td, const SceneDev &sd, const gbt_sum_args &a, int splits,
                 void *work, cudaStream_t s, unsigned long long *stats = nullptr,
                 bool differentiable = false,    // with the adjoint's own evaluation (F32)

@@ -381,7 +381,7 @@ __global__ void __launch_bounds__(32 * PairCfg<WarpBuf<NF, LOSSY>, BATCHED, Pair
         int64_t it = 0;
         if (lane == 0) it = atomicAdd(prm.work_counter, 1);
         it = __shfl_sync(0xffffffffu, it, 0);
-        if (it >= prm.n_items) break;
+        if (it >= (BATCHED ? prm.n_items : item_count(prm))) break;
         if (BATCHED) {
             int lo = 0, hi = prm.n_inst - 1;      // last instance with inst_off <= it
             while (lo < hi) {
@@ -464,9 +464,8 @@ __global__ void __launch_bounds__(32 * PairCfg<WarpBuf<NF, LOSSY>, BATCHED, Pair
         }
         const float4 rball = reach_ball(make_float4(cx, cy, cz, rad));
 
-        float4 *const part = p.partial + (int64_t)item.split * p.nf * p.n_recv + item.wbase + lane;
         bool first = true;
-        auto fold_all = [&]() { fold_bands<NF>(p, part, valid, ax, ay, first); };
+        auto fold_all = [&]() { fold_bands<NF>(p, item, lane, valid, ax, ay, first); };
 
         Gather<WINDOW, false> g(item);
         g.issue(p, item, B.in, lane, rball, 0);

@@ -53,7 +53,11 @@ struct alignas(16) FwdParams {
     float kmax_turns;          // largest f / c of the launch's frequencies, turns per metre
     float s_scale;             // staged s is s times this: 1 / b when uniform and forward, else 1
     int splits;
-    int64_t n_items;           // CTA tiles x splits
+    int64_t n_items;           // CTA tiles x splits x warp tiles (weighted: at most)
+    // weighted splits: by dispatch rank (n_tiles + 1), the first tile-split of each CTA tile,
+    // or null; partial is then [tile-split][nf][kCtaRecv]
+    const int32_t *item_off;
+    int n_tiles;
     int *work_counter;         // zero at launch (prepass); warps take items from it
     const int32_t *tile_perm;  // dispatch rank -> CTA tile (heaviest first), or null
     // tile pre-cull: per CTA tile, the segments whose beams can reach its receivers

@@ -401,9 +401,8 @@ __global__ void __maxnreg__(128) gbs_field_kernel(const __grid_constant__ FwdPar
 #pragma unroll
         for (int f = 0; f < NF; ++f) ax[f] = ay[f] = 0ull;
 
-        float4 *const part = p.partial + (int64_t)item.split * p.nf * p.n_recv + item.wbase + lane;
         bool first = true;
-        auto fold_all = [&]() { fold_bands<NF>(p, part, valid, ax, ay, first); };
+        auto fold_all = [&]() { fold_bands<NF>(p, item, lane, valid, ax, ay, first); };
         Gather<WINDOW, true> g(item);
         int group = 0;
         g.issue(p, item, B.in, lane, rball, 0);

@@ -17,23 +17,45 @@ static_assert(kFoldEvery % kScan == 0, "fold groups are whole windows");
 // One item of the queue: a warp tile and a split of the segments it goes through.
 struct Item {
     int64_t wbase;             // first receiver (processing order) of the warp tile
-    int split;
+    int split, splits;         // of the tile's
+    int64_t part;              // first partial of the warp tile's first receiver, band 0
+    int64_t part_band;         // and from band to band
     const int32_t *lst;        // the CTA tile's list, or null: every segment
     const uint32_t *lw;        // this warp tile's words of its chunks
     int64_t n_seg;             // entries of the list, or segments
 };
 // Item `it` of p: CTA tile by dispatch rank, split, warp tile within the CTA tile; false
-// past the last receiver.
+// past the last receiver.  (Items of p: see item_count.)
+__device__ __forceinline__ int64_t item_count(const FwdParams &p)
+{
+    return p.item_off ? (int64_t)p.item_off[p.n_tiles] * kTileWarps : p.n_items;
+}
 __device__ __forceinline__ bool decode_item(const FwdParams &p, int64_t it, Item &m)
 {
-    const int64_t per_tile = (int64_t)kTileWarps * p.splits;
-    const int64_t tile_rank = it / per_tile;
-    const int64_t rem = it - tile_rank * per_tile;
-    m.split = (int)(rem / kTileWarps);
-    const int wl = (int)(rem - (int64_t)m.split * kTileWarps);
+    const int64_t g = it / kTileWarps;         // tile-split
+    const int wl = (int)(it - g * kTileWarps);
+    int64_t tile_rank;
+    if (p.item_off) {
+        int lo = 0, hi = p.n_tiles - 1;        // last rank with item_off <= g
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (p.item_off[mid] <= g) lo = mid;
+            else hi = mid - 1;
+        }
+        tile_rank = lo;
+        m.split = (int)(g - p.item_off[lo]);
+        m.splits = p.item_off[lo + 1] - p.item_off[lo];
+    } else {
+        tile_rank = g / p.splits;
+        m.split = (int)(g - tile_rank * p.splits);
+        m.splits = p.splits;
+    }
     const int64_t tile = p.tile_perm ? (int64_t)p.tile_perm[tile_rank] : tile_rank;
     m.wbase = tile * kCtaRecv + (int64_t)wl * kWarpRecv;
     if (m.wbase >= p.n_recv) return false;
+    m.part_band = p.item_off ? kCtaRecv : p.n_recv;
+    m.part = p.item_off ? g * p.nf * kCtaRecv + (int64_t)wl * kWarpRecv
+                        : (int64_t)m.split * p.nf * p.n_recv + m.wbase;
     m.lst = nullptr;
     m.lw = nullptr;
     m.n_seg = *p.n_seg_ptr;
@@ -87,15 +109,15 @@ struct Gather {
                     if (n > 0 && count % (kFoldEvery / kScan) == 0) break;
                     ++count;
                 }
-                wchunk = wnext + (int64_t)lane * p.splits;
+                wchunk = wnext + (int64_t)lane * m.splits;
                 if (m.lst) {
                     word = wchunk < n_chunks ? m.lw[wchunk * kChunkWords] : 0u;
-                    wnext += (int64_t)32 * p.splits;
+                    wnext += (int64_t)32 * m.splits;
                 } else {
                     float4 q0[kScan], q1[kScan];
 #pragma unroll
                     for (int i = 0; i < kScan; ++i) {
-                        const int64_t sg = (wnext + (int64_t)i * p.splits) * kBatch + lane;
+                        const int64_t sg = (wnext + (int64_t)i * m.splits) * kBatch + lane;
                         q0[i] = q1[i] = make_float4(0.f, 0.f, 0.f, 0.f);
                         if (sg < m.n_seg) {
                             q0[i] = p.crec[2 * sg];
@@ -104,13 +126,13 @@ struct Gather {
                     }
 #pragma unroll
                     for (int i = 0; i < kScan; ++i) {
-                        const int64_t sg = (wnext + (int64_t)i * p.splits) * kBatch + lane;
+                        const int64_t sg = (wnext + (int64_t)i * m.splits) * kBatch + lane;
                         const uint32_t b = __ballot_sync(0xffffffffu,
                             sg < m.n_seg && seg_reaches_ball<WINDOW>(seg_cull(q0[i], q1[i]), rball,
                                                                      p.pre_alpha, p.pre_beta));
                         if (lane == i) word = b;
                     }
-                    wnext += (int64_t)kScan * p.splits;
+                    wnext += (int64_t)kScan * m.splits;
                 }
                 continue;
             }
@@ -182,10 +204,9 @@ __device__ __forceinline__ void fold(float4 *acc, float x, float y, bool first)
     }
 }
 
-// Folds a lane's two receivers' sums per band (valid receivers at part, part + 32) and zeroes
-// them.
+// Folds a lane's two receivers' sums per band into the item's partials and zeroes them.
 template <int NF>
-__device__ __forceinline__ void fold_bands(const FwdParams &p, float4 *part, const bool (&valid)[kR],
+__device__ __forceinline__ void fold_bands(const FwdParams &p, const Item &m, int lane, const bool (&valid)[kR],
                                            f2x (&ax)[NF], f2x (&ay)[NF], bool &first)
 {
 #pragma unroll
@@ -194,8 +215,9 @@ __device__ __forceinline__ void fold_bands(const FwdParams &p, float4 *part, con
             float x0, x1, y0, y1;
             upk(ax[f], x0, x1);
             upk(ay[f], y0, y1);
-            if (valid[0]) fold(part + (int64_t)f * p.n_recv, x0, y0, first);
-            if (valid[1]) fold(part + (int64_t)f * p.n_recv + 32, x1, y1, first);
+            float4 *const part = p.partial + m.part + f * m.part_band + lane;
+            if (valid[0]) fold(part, x0, y0, first);
+            if (valid[1]) fold(part + 32, x1, y1, first);
         }
         ax[f] = ay[f] = 0ull;
     }
