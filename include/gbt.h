@@ -177,6 +177,18 @@ typedef struct gbt_trace_info {
 } gbt_trace_info;
 
 gbt_status gbt_trace_info_get(const gbt_trace_t *trace, gbt_trace_info *info);
+
+/* Copies the arrays of gbt_trace_info, in one launch on `stream`, to device buffers of their
+ * sizes (NULL: not copied).  Reads the segment count as gbt_trace_info_get does if no call has
+ * read it yet; asynchronous otherwise. */
+typedef struct gbt_trace_arrays {
+    int32_t *ray_off;             /* n_rays + 1 */
+    double *seg_o, *seg_t;        /* n_segments * 3 */
+    double *seg_L, *seg_s0;       /* n_segments */
+    int32_t *seg_ray, *seg_depth, *seg_bmat, *seg_hit;    /* n_segments */
+} gbt_trace_arrays;
+gbt_status gbt_trace_copy(const gbt_trace_t *trace, const gbt_trace_arrays *dst, void *stream);
+
 /* Waits for the device (every stream), then frees the trace and its workspace.
  * NULL is a no-op. */
 gbt_status gbt_trace_destroy(gbt_trace_t *trace);

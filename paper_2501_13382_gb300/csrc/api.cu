@@ -638,6 +638,22 @@ gbt_status gbt_trace_info_get(const gbt_trace_t *trace, gbt_trace_info *info)
     });
 }
 
+gbt_status gbt_trace_copy(const gbt_trace_t *trace, const gbt_trace_arrays *dst, void *stream)
+{
+    NvtxRange nvtx_range("gbt_trace_copy");
+    return guarded([&] {
+        GBT_REQUIRE(trace && dst, "trace and dst must be non-NULL");
+        gbt_trace_t *tr = const_cast<gbt_trace_t *>(trace);
+        TraceDev &td = tr->d;
+        if (td.n_seg_host < 0) td.n_seg_host = read_device_i32(td.ray_off + td.n_rays, td.used);
+        cudaStream_t s = static_cast<cudaStream_t>(stream);
+        trace_copy_launch(td, *dst, s);
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        GBT_CUDA(cudaStreamIsCapturing(s, &cs));
+        if (cs == cudaStreamCaptureStatusNone) mark_used(td.used, s);
+    });
+}
+
 gbt_status gbt_trace_destroy(gbt_trace_t *trace)
 {
     return guarded([&] {

@@ -1273,9 +1273,9 @@ __global__ void list_words_kernel(const float4 *crec, const float4 *wball, int64
 // the heavy tiles' items ten times the mean, so that the queue drains well only with three
 // times as many of them, whose per-item work and partial sums then cost more than the tail
 // they save; shares with the cost itself make the last items as long as the first.  Equal
-// (32 items per warp) | root (12) | cost (12), in ms: 1 M rays x 1024^2 x 1 band, city,
+// (32 items per warp) | root (12) | cost (12), in ms: 1 M rays x 512^2 x 1 band, city,
 // 22.4 | 19.4 | 20.4; 192^2 x 8 bands with losses 6.40 | 6.42 | 6.94; batch of 8 sources x
-// 128^2 x 8 bands 4.63 | 3.62 | 3.67; 4,096 scattered receivers .724 | .701 | .697.
+// 128^2 x 8 bands 4.63 | 3.62 | 3.67; 9,973 scattered receivers .724 | .701 | .697.
 __global__ void __launch_bounds__(1024) list_layout_kernel(const unsigned int *total,
                                                            const int32_t *perm, int64_t n_tiles,
                                                            int64_t cap, int64_t *list_off,

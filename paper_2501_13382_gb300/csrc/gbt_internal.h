@@ -172,6 +172,8 @@ struct PaddedRays {
 };
 PaddedRays trace_rays_launch(const SceneDev &sd, TraceDev &td, const gbt_source_desc &src,
                              void *scratch, size_t scratch_bytes, cudaStream_t s);
+// Copies the trace's arrays to dst's buffers (null: not).
+void trace_copy_launch(const TraceDev &td, const gbt_trace_arrays &dst, cudaStream_t s);
 // Fills each segment's ray index and depth from the trace's offsets (imported traces).
 void csr_ray_depth_launch(TraceDev &td, cudaStream_t s);
 

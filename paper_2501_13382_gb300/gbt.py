@@ -69,6 +69,11 @@ class gbt_trace_info(C.Structure):
                 ("seg_depth", C.c_void_p), ("seg_bmat", C.c_void_p), ("seg_hit", C.c_void_p)]
 
 
+class gbt_trace_arrays(C.Structure):
+    _fields_ = [(n, C.c_void_p) for n in ("ray_off", "seg_o", "seg_t", "seg_L", "seg_s0",
+                                          "seg_ray", "seg_depth", "seg_bmat", "seg_hit")]
+
+
 class gbt_sum_args(C.Structure):
     _fields_ = [("recv", C.c_void_p), ("n_recv", C.c_int64), ("recv_order", C.c_void_p),
                 ("n_freq", C.c_int32), ("window", C.c_int32),
@@ -102,6 +107,7 @@ _SIGS = {
     "gbt_trace": (C.c_int, [C.c_void_p, C.POINTER(gbt_source_desc), C.c_void_p,
                             C.POINTER(C.c_void_p)]),
     "gbt_trace_info_get": (C.c_int, [C.c_void_p, C.POINTER(gbt_trace_info)]),
+    "gbt_trace_copy": (C.c_int, [C.c_void_p, C.POINTER(gbt_trace_arrays), C.c_void_p]),
     "gbt_trace_import": (C.c_int, [C.c_void_p, C.POINTER(gbt_source_desc), C.POINTER(gbt_segments),
                                    C.c_void_p, C.POINTER(C.c_void_p)]),
     "gbt_trace_destroy": (C.c_int, [C.c_void_p]),
@@ -210,6 +216,11 @@ def gbt_trace_info_get(trace: int) -> gbt_trace_info:
     info = gbt_trace_info()
     _check(load().gbt_trace_info_get(C.c_void_p(trace), C.byref(info)), "gbt_trace_info_get")
     return info
+
+
+def gbt_trace_copy(trace: int, dst: gbt_trace_arrays, stream: int = 0):
+    _check(load().gbt_trace_copy(C.c_void_p(trace), C.byref(dst), C.c_void_p(stream)),
+           "gbt_trace_copy")
 
 
 def gbt_trace_destroy(trace: int):
@@ -398,12 +409,6 @@ def source_desc(source, ray_begin: int = 0, ray_count: int = 0, dirs=None) -> gb
     return s
 
 
-class _CudaView:
-    def __init__(self, ptr, shape, typestr):
-        self.__cuda_array_interface__ = {"shape": tuple(shape), "typestr": typestr,
-                                         "data": (int(ptr), False), "version": 2, "strides": None}
-
-
 class Trace:
     """Traced fan (CSR of segments) living on the device."""
 
@@ -466,17 +471,16 @@ class Trace:
         n = int(i.n_segments)
         nr = int(i.n_rays)
 
-        def view(ptr, shape, typ):
-            if int(np.prod(shape)) == 0:
-                return torch.zeros(shape, dtype={"<f8": torch.float64, "<i4": torch.int32}[typ],
-                                   device="cuda")
-            return torch.as_tensor(_CudaView(ptr, shape, typ), device="cuda").clone()
-
-        return {"n_segments": n, "ray_off": view(i.ray_off, (nr + 1,), "<i4"),
-                "o": view(i.seg_o, (n, 3), "<f8"), "t": view(i.seg_t, (n, 3), "<f8"),
-                "L": view(i.seg_L, (n,), "<f8"), "s0": view(i.seg_s0, (n,), "<f8"),
-                "ray": view(i.seg_ray, (n,), "<i4"), "depth": view(i.seg_depth, (n,), "<i4"),
-                "bmat": view(i.seg_bmat, (n,), "<i4"), "hit": view(i.seg_hit, (n,), "<i4")}
+        f8 = dict(dtype=torch.float64, device="cuda")
+        i4 = dict(dtype=torch.int32, device="cuda")
+        out = {"n_segments": n, "ray_off": torch.empty(nr + 1, **i4),
+               "o": torch.empty((n, 3), **f8), "t": torch.empty((n, 3), **f8),
+               "L": torch.empty(n, **f8), "s0": torch.empty(n, **f8),
+               "ray": torch.empty(n, **i4), "depth": torch.empty(n, **i4),
+               "bmat": torch.empty(n, **i4), "hit": torch.empty(n, **i4)}
+        gbt_trace_copy(self.handle, gbt_trace_arrays(*(_ptr(v) for k, v in out.items()
+                                                       if k != "n_segments")), _stream_ptr())
+        return out
 
     def close(self):
         if getattr(self, "handle", None):
