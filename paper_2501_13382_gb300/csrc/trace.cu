@@ -85,7 +85,8 @@ struct TraceParams {
     unsigned int *status;
     int chunk;                 // triangles per shared-memory chunk (a multiple of kTriCluster)
     int64_t strip;             // Fibonacci fan: lattice step between a warp's rays (0: none)
-    unsigned long long *counter;   // resident scene: next strip of 32 ray slots (zeroed)
+    unsigned long long *counter;   // next strip of ray slots (zeroed)
+    int lanes;                 // BVH: rays of a strip
     int64_t stride;            // max_refl + 1
     double *po, *pt, *pL, *ps0;
     int32_t *pbmat, *phit, *cnt;
@@ -300,7 +301,10 @@ __device__ __forceinline__ TriGuess tri_guess(float of0, float of1, float of2, f
 // traversal, when the warp's lanes are together again.  262,144 rays, 12,288 triangles: 1.54
 // -> 0.72 ms (exact tests at the leaves to here), 0.63 ms with the packed leaf records; FP64
 // pipe 70 -> 31 % of active cycles, now bound by the latency of the divergent walk.  Four
-// blocks per SM instead of three (64 registers): 1.49 ms.
+// blocks per SM instead of three (64 registers): 1.49 ms.  A stack entry is one 8-byte word
+// (node and distance apart: 2-8 % slower); keeping the nearer child in a register instead of
+// pushing and popping it spares the stack but takes lanes at nodes and at leaves apart
+// (1,048,576 rays through the city: 0.94 -> 1.26 ms).
 constexpr int kCand = 4;
 __device__ __forceinline__ void nearest_in_bvh(const TraceParams &p, const double o[3],
                                                const double d[3], int last_face, double &tbest,
@@ -334,17 +338,17 @@ __device__ __forceinline__ void nearest_in_bvh(const TraceParams &p, const doubl
             if (fine && t - e > 1e-6f) bound = t + e;
         }
     }
-    int32_t sref[kBvhStack];
-    float stn[kBvhStack];
+    int2 stack[kBvhStack];     // node, entry distance
     int sp = 0;
-    sref[sp] = 0;
-    stn[sp] = 0.0f;
-    ++sp;
+    auto push = [&](int32_t r, float t) { stack[sp++] = make_int2(r, __float_as_int(t)); };
+    push(0, 0.0f);
     while (sp > 0) {
         --sp;
-        const int32_t ref = sref[sp];
+        const int2 top = stack[sp];
+        const int32_t ref = top.x;
+        const float tn = __int_as_float(top.y);
         const float wide = bound * 1.000001f + 1e-3f;
-        if (stn[sp] > wide) continue;
+        if (tn > wide) continue;
         if (ref < 0) {
             const int32_t v = -(ref + 1);
             const int32_t first = v >> 3, count = (v & 7) + 1;
@@ -396,12 +400,12 @@ __device__ __forceinline__ void nearest_in_bvh(const TraceParams &p, const doubl
         }
         if (h0 && h1) {
             const bool near0 = tn0 <= tn1;
-            sref[sp] = near0 ? r1 : r0; stn[sp] = near0 ? tn1 : tn0; ++sp;
-            sref[sp] = near0 ? r0 : r1; stn[sp] = near0 ? tn0 : tn1; ++sp;
+            push(near0 ? r1 : r0, near0 ? tn1 : tn0);
+            push(near0 ? r0 : r1, near0 ? tn0 : tn1);
         } else if (h0) {
-            sref[sp] = r0; stn[sp] = tn0; ++sp;
+            push(r0, tn0);
         } else if (h1) {
-            sref[sp] = r1; stn[sp] = tn1; ++sp;
+            push(r1, tn1);
         }
     }
     for (int c = 0; c < nc; ++c)
@@ -548,30 +552,33 @@ __global__ void __launch_bounds__(kTraceBlock) trace_resident_kernel(TraceParams
     }
 }
 
-// Scene in a BVH (global memory, L2-resident): persistent warps take strips of 32 ray
-// slots and trace each ray to its end on its own, like the resident kernel.
+// Scene in a BVH (global memory, L2-resident): persistent warps take strips of p.lanes ray
+// slots, a lane per ray, and trace them bounce by bounce.  The vote brings the lanes together
+// for each walk (1,048,576 rays through the city: 1.17 -> 1.06 ms).  Lanes of rays that have
+// ended stay idle: handing them new rays loses the strip's coherence (refilled at 24, 16, 8
+// or 0 lanes left: 1.23, 1.19, 1.14, 1.06 ms).  What a divergent walk costs grows with the
+// lanes, so few rays are spread over more warps: see the launch.
 __global__ void __launch_bounds__(kTraceBlock) trace_bvh_kernel(TraceParams p)
 {
     const int lane = threadIdx.x & 31;
     for (;;) {
         int64_t q = 0;
         if (lane == 0) q = atomicAdd(p.counter, 1ull);
-        q = __shfl_sync(0xffffffffu, q, 0);
-        if (q * 32 >= p.n_rays) break;
-        const int64_t i = ray_of_slot(p, q * 32 + lane);
-        if (i >= p.n_rays) continue;
-        double o[3] = {p.src[0], p.src[1], p.src[2]};
-        double d[3];
-        ray_direction(p, i, d);
-        double s0 = 0.0;
+        q = __shfl_sync(0xffffffffu, q, 0) * p.lanes;
+        if (q >= p.n_rays) break;
+        bool alive = lane < p.lanes && q + lane < p.n_rays;
+        const int64_t i = alive ? ray_of_slot(p, q + lane) : 0;
+        double o[3] = {p.src[0], p.src[1], p.src[2]}, d[3] = {0.0, 0.0, 1.0}, s0 = 0.0;
+        if (alive) ray_direction(p, i, d);
         int last_face = -1, bmat = -1, nref = 0, nseg = 0;
-        for (bool alive = true; alive;) {
+        while (__any_sync(0xffffffffu, alive)) {
+            if (!alive) continue;
             double tbest = INFINITY;
             int best = -1;
             nearest_in_bvh(p, o, d, last_face, tbest, best);
             alive = record_and_reflect(p, i, o, d, s0, last_face, bmat, nref, nseg, tbest, best);
+            if (!alive) write_count(p, i, nseg);
         }
-        write_count(p, i, nseg);
     }
 }
 
@@ -889,16 +896,22 @@ static void rays_launch(const SceneDev &sd, TraceDev &td, const gbt_source_desc 
     }
     // the BVH (built unless GBT_ACCEL_LINEAR) outran the shared-memory scene already at
     // 768 triangles: 3.2 ms against 5.4 ms for 1,048,576 rays through the synthetic city
-    // (1.5 ms since)
+    // (0.92 ms since)
     const bool use_bvh = sd.n_tri > 0 && sd.bvh && sd.accel != GBT_ACCEL_LINEAR;
     GBT_CUDA(cudaMemsetAsync(p.counter, 0, 256 + (sums ? packs * sizeof(int32_t) : 0), s));
     if (use_bvh) {
         int per_sm = 0;
         GBT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, trace_bvh_kernel, kTraceBlock, 0));
-        const int64_t strips = (n + 31) / 32;
+        // rays of a strip: the fewest (a power of two) that make at most 2.25 strips per
+        // resident warp.  City, us with 1, 2, 4, 8, 16, 32 of them: 1,001 rays 134 187 231
+        // 306 353 422; 16,384: 315 232 230 281 334 397; 65,536: 1106 626 394 330 345 418;
+        // 131,072: 2185 1192 683 447 379 415; 262,144: - - 1268 728 486 441
+        const int64_t resident = (int64_t)std::max(per_sm, 1) * num_sms();
+        p.lanes = 1;
+        while (p.lanes < 32 && 4 * n > 9 * p.lanes * resident * (kTraceBlock / 32)) p.lanes *= 2;
+        const int64_t strips = (n + p.lanes - 1) / p.lanes;
         const int64_t blocks = std::max<int64_t>(
-            1, std::min<int64_t>((int64_t)std::max(per_sm, 1) * num_sms(),
-                                 (strips + kTraceBlock / 32 - 1) / (kTraceBlock / 32)));
+            1, std::min<int64_t>(resident, (strips + kTraceBlock / 32 - 1) / (kTraceBlock / 32)));
         trace_bvh_kernel<<<(unsigned)blocks, kTraceBlock, 0, s>>>(p);
     } else if (sd.n_tri <= p.chunk) {
         // resident scene: a persistent grid whose warps take strips of rays

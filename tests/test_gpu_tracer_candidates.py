@@ -52,3 +52,17 @@ def test_bvh_candidates_match_index_order(stack, gap):
     assert got[0]["n_segments"] == got[1]["n_segments"]
     for k in ("ray_off", "hit", "bmat", "o", "t", "L", "s0"):
         assert torch.equal(got[0][k], got[1][k]), k
+
+
+@pytest.mark.parametrize("rays", [1, 31, 8191, 8209, 16500, 33001, 66003, 132001])
+def test_strips_of_any_length_match_index_order(rays):
+    """One ray of a strip up to 32 by the number of rays; the same segments, to the bit."""
+    import torch
+    from paper_2501_13382_gb300 import gbt as G
+    sc0, _ = I.city_scene(I.SEED_BASE + 3)
+    src = I.Source(np.array([0.3, -0.2, 3.0]), rays, 5, 700.0)
+    a, b = (G.Trace(G.Scene(sc0, accel=m), src).segments() for m in (G.ACCEL_BVH, G.ACCEL_LINEAR))
+    G.gbt_sync()
+    assert a["n_segments"] == b["n_segments"]
+    for k in ("ray_off", "o", "t", "L", "s0", "ray", "depth", "bmat", "hit"):
+        assert torch.equal(a[k], b[k]), k
