@@ -494,7 +494,6 @@ __global__ void __launch_bounds__(kPackRays) pack_kernel(PrepParams p, PaddedRay
 {
     __shared__ int32_t first[kPackRays + 1];     // segments of the block before each ray
     __shared__ int32_t ws[kPackRays / 32];
-    __shared__ int32_t before_s;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (blockIdx.x == 0 && threadIdx.x < kCounters) p.counters[threadIdx.x] = 0;
     auto block_sum = [&](int32_t v) {            // of every thread's v
@@ -1790,117 +1789,78 @@ __global__ void __launch_bounds__(kRadixBlock) radix_scatter_kernel(const unsign
     if (ok) out[base[d] + offs[(int64_t)d * nblocks + blockIdx.x] + wc[wid][d] + rank] = key;
 }
 
-// The whole order in one block, for up to kOrderSmall receivers: bounding box, codes and the
-// four radix passes in shared memory.  Each warp owns a contiguous share of the keys and its
-// own digit counters; ranks within a warp come from the lanes holding the same digit, so
-// every pass is stable.  A few thousand receivers are bound by launches: 15 kernels and 2
-// memsets took 72 us for 4,096 receivers (with the present kernels 65 us), this one 29; at
-// 10,000 the two are even.
-constexpr int kOrderSmall = 8192;
+// The whole order in one launch, for up to kOrderSmall receivers, which are bound by launches
+// and by the latency of passes over few keys: every block forms the bounding box and all codes
+// itself (in shared memory, from L2) and ranks its 128 keys by counting the ones before them,
+// four keys a warp and four codes a load.  That is n^2 comparisons, but spread over the chip:
+// 4,096 receivers 13 us (the radix passes of the large path in their fifteen launches 65 us,
+// in one block 29), 16,384 receivers 45 us (72).
+constexpr int kOrderSmall = 16384;
 constexpr int kOrderThreads = 1024, kOrderWarps = kOrderThreads / 32;
-struct OrderSmem {
-    uint32_t code[2][kOrderSmall];
-    uint16_t idx[2][kOrderSmall];
-};
-struct OrderCounts {
-    uint32_t c[kRadixBuckets][kOrderWarps + 1];   // padded: a digit's counts in different banks
-    uint32_t ws[kOrderWarps];
-    unsigned int bb[6];
-};
+constexpr int kOrderKeys = 4;      // of a warp
 __global__ void __launch_bounds__(kOrderThreads) order_small_kernel(const float *recv, int n, int32_t *order)
 {
-    extern __shared__ __align__(16) unsigned char order_smem[];
-    OrderCounts &K = *reinterpret_cast<OrderCounts *>(order_smem);
-    const int cap = (n + 1) / 2 * 2;
-    uint32_t *code[2];
-    uint16_t *idx[2];
-    code[0] = reinterpret_cast<uint32_t *>(order_smem + sizeof(OrderCounts));
-    code[1] = code[0] + cap;
-    idx[0] = reinterpret_cast<uint16_t *>(code[1] + cap);
-    idx[1] = idx[0] + cap;
+    extern __shared__ uint4 code4[];               // n codes, padded to whole rows of 128
+    uint32_t *const code = reinterpret_cast<uint32_t *>(code4);
+    __shared__ unsigned int bb[6];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (threadIdx.x < 3) { K.bb[threadIdx.x] = 0xffffffffu; K.bb[3 + threadIdx.x] = 0u; }
+    const int rows = (n + 127) / 128;
+    if (threadIdx.x < 3) { bb[threadIdx.x] = 0xffffffffu; bb[3 + threadIdx.x] = 0u; }
     __syncthreads();
     unsigned lo[3] = {~0u, ~0u, ~0u}, hi[3] = {0u, 0u, 0u};
+#pragma unroll 4
     for (int i = threadIdx.x; i < n; i += kOrderThreads)
+#pragma unroll
         for (int a = 0; a < 3; ++a) {
             const unsigned u = ordered_bits(recv[3 * i + a]);
             lo[a] = min(lo[a], u);
             hi[a] = max(hi[a], u);
         }
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
         lo[a] = __reduce_min_sync(0xffffffffu, lo[a]);
         hi[a] = __reduce_max_sync(0xffffffffu, hi[a]);
         if (lane == 0) {
-            atomicMin(&K.bb[a], lo[a]);
-            atomicMax(&K.bb[3 + a], hi[a]);
+            atomicMin(&bb[a], lo[a]);
+            atomicMax(&bb[3 + a], hi[a]);
         }
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < n; i += kOrderThreads) {
-        code[0][i] = morton_code(recv + 3 * i, K.bb);
-        idx[0][i] = (uint16_t)i;
-    }
-    // warp w owns keys [w share, (w + 1) share)
-    const int share = (n + kOrderThreads - 1) / kOrderThreads * 32;
-    const int b = min(n, wid * share), e = min(n, b + share);
-    for (int pass = 0; pass < 4; ++pass) {
-        const int shift = 8 * pass;
-        const uint32_t *ci = code[pass & 1];
-        const uint16_t *ii = idx[pass & 1];
-        for (int q = threadIdx.x; q < kRadixBuckets * kOrderWarps; q += kOrderThreads)
-            K.c[q / kOrderWarps][q % kOrderWarps] = 0u;
-        __syncthreads();
-        for (int i0 = b; i0 < e; i0 += 32) {
-            const bool ok = i0 + lane < e;
-            const unsigned d = ok ? (ci[i0 + lane] >> shift) & 255u : 0u;
-            const unsigned same = same_digit(d, ok);
-            if (ok && (same & ((1u << lane) - 1u)) == 0u) K.c[d][wid] += __popc(same);
-            __syncwarp();
-        }
-        __syncthreads();
-        // exclusive scan over (digit, warp): 8 consecutive counts per thread
-        uint32_t v[8], sum = 0;
-        for (int q = 0; q < 8; ++q) {
-            const int at = threadIdx.x * 8 + q;
-            v[q] = K.c[at / kOrderWarps][at % kOrderWarps];
-            sum += v[q];
-        }
-        uint32_t x = sum;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < 128 * rows; i += kOrderThreads)
+        code[i] = i < n ? morton_code(recv + 3 * i, bb) : 0xffffffffu;     // above any code
+    __syncthreads();
+    const int i0 = (blockIdx.x * kOrderWarps + wid) * kOrderKeys;          // one uint4 of keys
+    if (i0 >= n) return;
+    const uint4 own = code4[i0 / 4];
+    const uint32_t key[kOrderKeys] = {own.x, own.y, own.z, own.w};
+    int before[kOrderKeys] = {0, 0, 0, 0};
+    // earlier keys come first on a tie: code <= key before the own four, code < key after
+    auto row = [&](int r, bool ties) {
+        const uint4 c = code4[32 * r + lane];
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
+        for (int m = 0; m < kOrderKeys; ++m) {
+            const uint32_t k = key[m] + (ties ? 1u : 0u);
+            before[m] += (c.x < k) + (c.y < k) + (c.z < k) + (c.w < k);
         }
-        if (lane == 31) K.ws[wid] = x;
-        __syncthreads();
-        uint32_t run = x - sum;
-        for (int w = 0; w < wid; ++w) run += K.ws[w];
-        for (int q = 0; q < 8; ++q) {
-            const int at = threadIdx.x * 8 + q;
-            K.c[at / kOrderWarps][at % kOrderWarps] = run;
-            run += v[q];
-        }
-        __syncthreads();
-        for (int i0 = b; i0 < e; i0 += 32) {
-            const bool ok = i0 + lane < e;
-            const uint32_t cd = ok ? ci[i0 + lane] : 0u;
-            const unsigned d = (cd >> shift) & 255u;
-            const unsigned same = same_digit(d, ok), below = same & ((1u << lane) - 1u);
-            const uint32_t at = ok ? K.c[d][wid] + __popc(below) : 0u;
-            __syncwarp();
-            if (ok) {
-                if (below == 0u) K.c[d][wid] += __popc(same);
-                if (pass == 3) {
-                    order[at] = ii[i0 + lane];
-                } else {
-                    code[1 - (pass & 1)][at] = cd;
-                    idx[1 - (pass & 1)][at] = ii[i0 + lane];
-                }
-            }
-            __syncwarp();
-        }
-        __syncthreads();
+    };
+    const int r0 = i0 / 128, l0 = (i0 % 128) / 4;
+#pragma unroll 4
+    for (int r = 0; r < r0; ++r) row(r, true);
+    if (lane != l0) {
+        row(r0, lane < l0);
+    } else {
+#pragma unroll
+        for (int m = 0; m < kOrderKeys; ++m)
+#pragma unroll
+            for (int q = 0; q < kOrderKeys; ++q) before[m] += key[q] < key[m] + (q < m ? 1u : 0u);
+    }
+#pragma unroll 4
+    for (int r = r0 + 1; r < rows; ++r) row(r, false);
+#pragma unroll
+    for (int m = 0; m < kOrderKeys; ++m) {
+        const int at = __reduce_add_sync(0xffffffffu, before[m]);
+        if (lane == m && i0 + m < n) order[at] = i0 + m;
     }
 }
 
@@ -2478,17 +2438,18 @@ void recv_order_launch(const float *recv, int64_t n, int32_t *order, void *scrat
 {
     if (n <= 0) return;
     if (n <= kOrderSmall) {
-        const size_t sm = sizeof(OrderCounts) + 2 * ((size_t)n + 1) * (sizeof(uint32_t) + sizeof(uint16_t));
+        const size_t sm = ((size_t)n + 127) / 128 * 128 * sizeof(uint32_t);
         static std::atomic<bool> set[64] = {};
         int dev = 0;
         GBT_CUDA(cudaGetDevice(&dev));
         if (dev < 0 || dev >= 64) fail(GBT_ERR_UNSUPPORTED, "device index >= 64");
         if (!set[dev].load(std::memory_order_acquire)) {
             GBT_CUDA(cudaFuncSetAttribute(order_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)(sizeof(OrderCounts) + sizeof(OrderSmem) + 16)));
+                                          (int)(kOrderSmall * sizeof(uint32_t))));
             set[dev].store(true, std::memory_order_release);
         }
-        order_small_kernel<<<1, kOrderThreads, sm, s>>>(recv, (int)n, order);
+        const unsigned blocks = (unsigned)((n + kOrderWarps * kOrderKeys - 1) / (kOrderWarps * kOrderKeys));
+        order_small_kernel<<<blocks, kOrderThreads, sm, s>>>(recv, (int)n, order);
         note_launches(1);
         GBT_CUDA(cudaGetLastError());
         return;

@@ -95,7 +95,7 @@ def test_f64_kernel_edges(n, rays, nf, window, cutoff):
 
 @pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 1023, 1024, 1025, 5000, 16383, 16384, 16385, 40001])
 def test_receiver_order_is_the_stable_morton_order(n):
-    """One block up to 16,384 receivers, radix passes over the grid beyond; codes and order
+    """Counted ranks up to 16,384 receivers, radix passes beyond; codes and order
     from numpy in the same FP32 steps, ties by index.  Integers: no tolerance."""
     import torch
     from paper_2501_13382_gb300 import gbt as G
