@@ -40,9 +40,10 @@ sys.path.insert(0, ROOT)
 
 METRIC = "GBS segment x receiver evals/s at <=1e-4 rel L2; batched & fwd+bwd vs plain"
 UNIT = "evals/s"
-# Algorithmic work of the method, in FP32/ALU lane issue slots:
-# per tested (receiver, segment) pair about 20 (projection onto the segment, s, n^2, window,
-# the frequency-independent cutoff); per kept (pair, frequency) about 45 FP32 slots for the
+# Algorithmic work of the method, in FP32/ALU lane issue slots: per (receiver, segment) pair
+# inside the union of its bands' cutoffs about 20 (projection onto the segment, s, n^2, window,
+# the frequency-independent cutoff; pairs outside need none of it, since a ball test drops them
+# for a whole group of receivers); per kept (pair, frequency) about 45 FP32 slots for the
 # beam term (1/E, Gaussian amplitude, phase with its range reduction, complex product) plus
 # about 12 for the compensated accumulation, i.e. 57, and 4 MUFU operations (RCP, EX2, SIN,
 # COS) on the separate special-function pipe, whose time at 16-32 lanes per clock per SM
@@ -54,17 +55,8 @@ LANES_PER_SM_CLK = 128          # FP32 lanes per SM per clock (4 SMSPs x 32)
 # Revision of the pair kernel's source.  DRAM bytes (read + write) per launch of the
 # dominant kernel come from an ncu capture of one revision, instantiation and workload;
 # a changed kernel gets a new revision and no entry until it is captured again.
-KERNEL_REV = "rev10"
-KERNEL_TRAFFIC = {
-    ("gbs_fwd_kernel<1,SEGMENT,fwd,plain> tile segment lists [rev10]",
-     "city_1M_rays_512x512_1kHz"): 5284817920,
-    ("gbs_fwd_kernel<1,SEGMENT,fwd,plain> every pair [rev10]",
-     "city_1M_rays_512x512_1kHz"): 241523122432,
-    ("gbs_fwd_kernel<6,LINE,fwd,plain> tile segment lists [rev10]",
-     "open_plane_64k_rays_256x256_6f"): 468206080,
-    ("gbs_fwd_kernel<6,LINE,fwd,plain> every pair [rev10]",
-     "open_plane_64k_rays_256x256_6f"): 195008000,
-}
+KERNEL_REV = "rev11"
+KERNEL_TRAFFIC = {}
 WORKLOADS = ("city", "open_plane_large", "open_plane_small", "diff_city", "big_city")
 
 
@@ -72,8 +64,8 @@ def kernel_tag(nf: int, window: int, cull: bool) -> str:
     """Name of the pair-kernel instantiation a sum with nf frequencies launches."""
     inst = next((v for v in (1, 2, 4, 6, 8) if nf <= v), 8)
     win = "LINE" if window == 1 else "SEGMENT"
-    return (f"gbs_fwd_kernel<{inst},{win},fwd,plain> "
-            f"{'tile segment lists' if cull else 'every pair'} [{KERNEL_REV}]")
+    return (f"gbs_pair_kernel<{inst},{win}> "
+            f"{'tile segment lists' if cull else 'no lists'} [{KERNEL_REV}]")
 
 
 def _env_int(name, default):
@@ -278,7 +270,7 @@ def _peak_tlane(torch, mhz):
 def roofline_of(torch, st, kern_ms, n_launch, tag, workload, mhz):
     """FP32/ALU roofline of the pair kernel: the algorithmic lane operations of one launch
     (from the counting pass) over its CUDA-event duration."""
-    ops = OPS_PER_PAIR * float(st["pairs_tested"]) + OPS_PER_KEPT * float(st["triples_kept"])
+    ops = OPS_PER_PAIR * float(st["pairs_prefiltered"]) + OPS_PER_KEPT * float(st["triples_kept"])
     peak, n_sm = _peak_tlane(torch, mhz)
     achieved = ops / (kern_ms * 1e-3) / 1e12 if kern_ms > 0 else 0.0
     return {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Tlane-op/s",
