@@ -1536,7 +1536,7 @@ struct ReduceParams {
     int accumulate;
     // weighted splits: per tile its first tile-split and their number, or nullptr
     const int32_t *tile_first, *tile_splits;
-    int nf;
+    int nf, part_recv;
 };
 
 // Float-float partials (hi, running FP32 sum of errors) merged into a float-float total with
@@ -1568,8 +1568,8 @@ __global__ void __launch_bounds__(32 * kMergeGroups) reduce_kernel(ReduceParams 
         if (p.tile_first) {
             const int64_t f = i / p.n_recv, r = i - f * p.n_recv, t = r / kCtaRecv;
             n = p.tile_splits[t];
-            stride = (int64_t)p.nf * kCtaRecv;
-            src = p.p32 + p.tile_first[t] * stride + f * kCtaRecv + (r - t * kCtaRecv);
+            stride = (int64_t)p.nf * p.part_recv;
+            src = p.p32 + p.tile_first[t] * stride + f * p.part_recv + (r - t * kCtaRecv);
         }
         const int s0 = (int)(n * g / kMergeGroups), s1 = (int)(n * (g + 1) / kMergeGroups);
 #pragma unroll 8
@@ -2121,9 +2121,12 @@ static bool weighted_splits(const gbt_sum_args &a, const TileWs &t, bool adjoint
 {
     return t.lists && a.seg_split == 0 && !adjoint;
 }
+// Receivers of a tile-split's partials: a CTA tile's, or all of a single tile.
+static int part_receivers(int64_t n_recv) { return (int)std::min<int64_t>(kCtaRecv, n_recv); }
 // Points q at a weighted layout: tile-splits instead of splits per tile.
 static void set_weighted(FwdParams &q, const TileWs &t)
 {
+    q.part_recv = part_receivers(q.n_recv);
     q.item_off = t.item_off;
     q.n_tiles = (int32_t)t.tiles;
     q.n_items = ((int64_t)q.splits + 1) * t.tiles * kTileWarps;     // at most (sizes the grid)
@@ -2132,7 +2135,7 @@ static void set_weighted(FwdParams &q, const TileWs &t)
 // [tile-split][band][receiver of the tile].
 static size_t partial_count(const gbt_sum_args &a, int nf, int splits, bool weighted)
 {
-    return weighted ? ((size_t)splits + 1) * (size_t)cta_tiles(a.n_recv) * kCtaRecv * nf
+    return weighted ? ((size_t)splits + 1) * (size_t)cta_tiles(a.n_recv) * part_receivers(a.n_recv) * nf
                     : (size_t)splits * nf * (size_t)a.n_recv;
 }
 
@@ -2408,6 +2411,7 @@ void sum_launch(const TraceDev &td, const SceneDev &sd, const gbt_sum_args &a, i
         rp.tile_first = weighted ? tw.tile_first : nullptr;
         rp.tile_splits = tw.tile_splits;
         rp.nf = q.nf;
+        rp.part_recv = q.part_recv;
         reduce_launch(rp, s);
     }
 }
@@ -2786,6 +2790,7 @@ static void batch_reduce(BatchImpl &B, int k, cudaStream_t s)
         rp.tile_first = t.tile_first;
         rp.tile_splits = t.tile_splits;
         rp.nf = a.n_freq;
+        rp.part_recv = part_receivers(a.n_recv);
     }
     reduce_launch(rp, s);
 }

@@ -55,9 +55,9 @@ struct alignas(16) FwdParams {
     int splits;
     int64_t n_items;           // CTA tiles x splits x warp tiles (weighted: at most)
     // weighted splits: by dispatch rank (n_tiles + 1), the first tile-split of each CTA tile,
-    // or null; partial is then [tile-split][nf][kCtaRecv]
+    // or null; partial is then [tile-split][nf][part_recv]
     const int32_t *item_off;
-    int n_tiles;
+    int n_tiles, part_recv;
     int *work_counter;         // zero at launch (prepass); warps take items from it
     const int32_t *tile_perm;  // dispatch rank -> CTA tile (heaviest first), or null
     // tile pre-cull: per CTA tile, the segments whose beams can reach its receivers

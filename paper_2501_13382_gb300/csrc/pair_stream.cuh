@@ -53,8 +53,8 @@ __device__ __forceinline__ bool decode_item(const FwdParams &p, int64_t it, Item
     const int64_t tile = p.tile_perm ? (int64_t)p.tile_perm[tile_rank] : tile_rank;
     m.wbase = tile * kCtaRecv + (int64_t)wl * kWarpRecv;
     if (m.wbase >= p.n_recv) return false;
-    m.part_band = p.item_off ? kCtaRecv : p.n_recv;
-    m.part = p.item_off ? g * p.nf * kCtaRecv + (int64_t)wl * kWarpRecv
+    m.part_band = p.item_off ? p.part_recv : p.n_recv;
+    m.part = p.item_off ? g * p.nf * p.part_recv + (int64_t)wl * kWarpRecv
                         : (int64_t)m.split * p.nf * p.n_recv + m.wbase;
     m.lst = nullptr;
     m.lw = nullptr;
