@@ -68,6 +68,9 @@ struct PairShape {
     static constexpr int NS = NF == 1 ? 4 : 1, NP = NF == 1 ? 2 : 1;
     static constexpr int FG = NF >= 6 && !LOSSY ? 2 : 1;
     static constexpr int kWarps = NF == 1 ? 12 : 16;
+    // the fused batch: 8 bands read 14 warps' constants from shared memory (16 sources x 256^2 x
+    // 8 bands, lists: 16 warps 99.6, 14 95.1, 12 97.0 ms)
+    static constexpr int kWarpsBatched = NF >= 6 ? 14 : kWarps;
 };
 
 // Per-warp shared memory: the raw records and the staged batch, every value in both halves of
@@ -94,7 +97,7 @@ struct LaneRecv {
 
 // Adds the beams of the staged slots j .. j + NS - 1 to the lane's two receivers' sums per
 // band.  `cross`: slots with an end of their window inside the warp tile's ball.
-template <int NF, int WINDOW, bool LOSSY, bool PREC, int NS, int FG>
+template <int NF, int WINDOW, bool LOSSY, bool PREC, int NS, int FG, bool BATCHED>
 __device__ __forceinline__ void eval_segments(const FwdParams &p, const WarpBuf<NF, LOSSY> &w,
                                               int j, uint64_t cross, const LaneRecv &x,
                                               f2x (&ax)[NF], f2x (&ay)[NF])
@@ -156,7 +159,14 @@ __device__ __forceinline__ void eval_segments(const FwdParams &p, const WarpBuf<
 #pragma unroll
         for (int i = 0; i < FG; ++i) {
             const int f = f0 + i;
-            const FreqConst &c = p.fc[f];
+            FreqConst cs;
+            if (BATCHED) {      // instance constants in shared memory, by whole words (that batch:
+                                // 103.4 ms by floats, 99.6 by words)
+                const float4 v = reinterpret_cast<const float4 *>(&p.fc[f])[1];
+                cs.rc = v.z;
+                cs.invb = v.w;
+            }
+            const FreqConst &c = BATCHED ? cs : p.fc[f];
             const bool live = NF == 1 || FG == 1 || f < p.nf;
 #pragma unroll
             for (int q = 0; q < NS; ++q) {
@@ -189,7 +199,16 @@ __device__ __forceinline__ void eval_segments(const FwdParams &p, const WarpBuf<
 #pragma unroll
         for (int i = 0; i < FG; ++i) {
             const int f = f0 + i;
-            const FreqConst &c = p.fc[f];
+            FreqConst cs;
+            if (BATCHED) {
+                const float4 u = reinterpret_cast<const float4 *>(&p.fc[f])[0];
+                const float4 v = reinterpret_cast<const float4 *>(&p.fc[f])[1];
+                cs.K_hi = u.z;
+                cs.K_lo = u.w;
+                cs.hK = v.x;
+                cs.ne = v.y;
+            }
+            const FreqConst &c = BATCHED ? cs : p.fc[f];
 #pragma unroll
             for (int q = 0; q < NS; ++q) {
                 const ulonglong2 pp = *reinterpret_cast<const ulonglong2 *>(&w.F[f / 2][j + q]);
@@ -363,9 +382,9 @@ __device__ __forceinline__ StagedBatch stage(const FwdParams &p, WarpBuf<NF, LOS
 }
 
 template <int NF, int WINDOW, bool BATCHED, bool LOSSY>
-__global__ void __launch_bounds__(32 * PairCfg<WarpBuf<NF, LOSSY>, BATCHED, PairShape<NF, LOSSY>::kWarps>::kWarps, 1) gbs_pair_kernel(const __grid_constant__ FwdParams prm)
+__global__ void __launch_bounds__(32 * PairCfg<WarpBuf<NF, LOSSY>, BATCHED, BATCHED ? PairShape<NF, LOSSY>::kWarpsBatched : PairShape<NF, LOSSY>::kWarps>::kWarps, 1) gbs_pair_kernel(const __grid_constant__ FwdParams prm)
 {
-    using Cfg = PairCfg<WarpBuf<NF, LOSSY>, BATCHED, PairShape<NF, LOSSY>::kWarps>;
+    using Cfg = PairCfg<WarpBuf<NF, LOSSY>, BATCHED, BATCHED ? PairShape<NF, LOSSY>::kWarpsBatched : PairShape<NF, LOSSY>::kWarps>;
     static_assert(!(LOSSY && BATCHED), "batches with losses run the single-sum kernel");
     using Shape = PairShape<NF, LOSSY>;
     constexpr int NS = Shape::NS, NP = Shape::NP, FG = Shape::FG;
@@ -480,9 +499,9 @@ __global__ void __launch_bounds__(32 * PairCfg<WarpBuf<NF, LOSSY>, BATCHED, Pair
             __syncwarp();       // the batch is staged
             g.issue(p, item, B.in, lane, rball, buf);   // batch kb + 2 into the buffer just read
             for (int j = 0; j < b.n_plain; j += NS)
-                eval_segments<NF, WINDOW, LOSSY, false, NS, FG>(p, B, j, 0ull, x, ax, ay);
+                eval_segments<NF, WINDOW, LOSSY, false, NS, FG, BATCHED>(p, B, j, 0ull, x, ax, ay);
             for (int j = b.n_plain; j < b.end; j += NP)
-                eval_segments<NF, WINDOW, LOSSY, true, NP, FG>(p, B, j, b.cross, x, ax, ay);
+                eval_segments<NF, WINDOW, LOSSY, true, NP, FG, BATCHED>(p, B, j, b.cross, x, ax, ay);
             if ((kb % kFoldEvery) == kFoldEvery - 1) fold_all();
             __syncwarp();        // before the next batch is staged over this one
         }

@@ -8,7 +8,7 @@ namespace {
 template <int NF, int WINDOW>
 int run(const FwdParams *p, int grid, cudaStream_t s)
 {
-    using Cfg = PairCfg<WarpBuf<NF, false>, true, PairShape<NF, false>::kWarps>;
+    using Cfg = PairCfg<WarpBuf<NF, false>, true, PairShape<NF, false>::kWarpsBatched>;
     static std::atomic<int> known[64] = {};
     auto *fn = gbs_pair_kernel<NF, WINDOW, true, false>;
     const int per_sm = resident_ctas<Cfg>(fn, known);
