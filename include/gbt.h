@@ -232,16 +232,18 @@ gbt_status gbt_trace_import(const gbt_scene_t *scene, const gbt_source_desc *src
  * product of gamma over the reflections before segment j.  The constant
  * k b / (8 pi^2) makes a dense fan sum to the point source exp(ikr)/(4 pi r).
  *
- * F32 precision: FP32 arithmetic with float-float arclength and phase
- * reduction, FP32 MUFU exp/sin/cos, compensated per-receiver accumulation;
- * relative L2 error against an FP64 evaluation measured at 1e-7..4e-7 on the
- * synthetic open-plane and city workloads (tested to 1e-6 with 4 kHz phases
- * over 1 km paths).  Where a receiver group is compact for the call's highest
- * frequency (K max|x'| <= 90 turns), the receivers' projection on a segment is
- * formed in FP32 (a term's phase moves by at most about 1e-4 rad); a pair within
- * that projection's error bound of an end of its window is decided and evaluated
- * in float-float, so the window decisions are those of the exact arithmetic.  F64 precision: every step in FP64 (2.6e-8, the rounding of
- * the complex64 output), at FP64 speed.
+ * F32 precision: FP32 arithmetic per pair relative to the centre of its group of
+ * 64 receivers, whose segment terms are formed in float-float, FP32 MUFU
+ * exp/sin/cos, compensated per-receiver accumulation; relative L2 error against
+ * an FP64 evaluation measured at 1e-7..5e-7 on the synthetic open-plane and city
+ * workloads (tested to 1e-6 with 4 kHz phases over 1 km paths).  Where a group
+ * is compact for the call's highest frequency (K max|x'| <= 16 turns) the
+ * receivers' projection on a segment is one FP32 dot product (a term's phase
+ * moves by at most 1.8e-5 rad); elsewhere, and for a segment that has an end of
+ * its window inside the group's ball, it is split into an exact and a rest part,
+ * so the window decisions are those of the exact arithmetic to 1e-10 m.  F64
+ * precision: every step in FP64 (2.6e-8, the rounding of the complex64 output),
+ * at FP64 speed.
  * With more than 8 frequencies the F32 path runs one pair launch per group of
  * at most 8 (frequencies sorted by value when every b_f is equal, otherwise in
  * the given order); each group costs a full pass over the pairs.
@@ -281,10 +283,13 @@ typedef struct gbt_sum_args {
     double cutoff;                /* C (> 0); 16 drops less than 1.2e-7 of a beam */
     int32_t precision;            /* GBT_PRECISION_F32 / GBT_PRECISION_F64 */
     int32_t accumulate;           /* 0 overwrite, 1 add into out */
-    int32_t seg_split;            /* segment ranges per receiver tile; 0 = automatic */
+    int32_t seg_split;            /* segment ranges per receiver tile; 0 = automatic (with
+                                     tile_cull by the length of the tile's list) */
     int32_t tile_cull;            /* 1: skip, per warp of 64 receivers, segments whose beams
-                                     provably reach none of them (same result, less work);
-                                     0: test every pair */
+                                     provably reach none of them by lists built once for
+                                     every 960 receivers; 0: the same skip tested by each
+                                     warp on its own (no lists: less memory, and less work
+                                     on small sums) */
     int64_t max_device_bytes;     /* gbt_solve only: device budget for one chunk; 0 = auto */
     double absorption[GBT_MAX_FREQ]; /* air's amplitude decay rate per frequency, Np/m
                                      (>= 0; all 0 = lossless air) */
@@ -461,7 +466,8 @@ typedef struct gbt_sum_stats {
     int64_t pairs;
     int64_t pairs_prefiltered;
     int64_t triples_kept;
-    int64_t pairs_tested;         /* pairs that reached the per-pair test (all, unless tile_cull) */
+    int64_t pairs_tested;         /* pairs that reach the counting pass's per-pair test (all,
+                                     unless tile_cull) */
 } gbt_sum_stats;
 
 gbt_status gbt_sum_stats_get(const gbt_trace_t *trace, const gbt_sum_args *args,
