@@ -268,7 +268,10 @@ gbt_status gbt_trace_import(const gbt_scene_t *scene, const gbt_source_desc *src
  * Batches with losses run in the CONCURRENT form; the FUSED form rejects them
  * (GBT_ERR_UNSUPPORTED). */
 typedef struct gbt_sum_args {
-    const float *recv;            /* device, n_recv * 3 (x, y, z), m */
+    const float *recv;            /* device, n_recv * 3 (x, y, z), m.  A receiver with a
+                                     coordinate that is not finite, or of 1e18 m and more,
+                                     gets a zero field and adds nothing to gradients; the
+                                     others are not affected */
     int64_t n_recv;               /* >= 0 */
     const int32_t *recv_order;    /* device permutation of [0, n_recv) or NULL; receivers
                                      are processed in this order (see gbt_recv_order) */
@@ -309,10 +312,11 @@ gbt_status gbt_sum_differentiable(const gbt_trace_t *trace, const gbt_sum_args *
 /* Spatially coherent processing order of receivers (Morton order of their
  * positions quantised to their bounding box), written to order_out (device,
  * n_recv int32).  The order changes results only by rounding: each warp of 64
- * receivers forms its exact geometry relative to its first receiver, so
- * compact warps (neighbouring receivers) are both faster (they see similar
- * beams, which keeps the warp's lanes busy) and the most accurate; a given
- * order always gives the same result. */
+ * receivers forms its geometry relative to their centre (the differentiable sum
+ * and the adjoint: to the first of them), so compact warps (neighbouring
+ * receivers) are both faster (they see similar beams, which keeps the warp's
+ * lanes busy) and the most accurate; a given order always gives the same
+ * result. */
 gbt_status gbt_recv_order(const float *recv, int64_t n_recv, int32_t *order_out, void *stream);
 
 /* Same result as gbt_recv_order (the identical permutation), for callers that

@@ -126,12 +126,9 @@ __global__ void __maxnreg__(128) gbs_count_kernel(const __grid_constant__ FwdPar
         const int64_t n_batches = (n_seg + kBatch - 1) / kBatch;
         const uint32_t nb = split < n_batches ? (uint32_t)((n_batches - 1 - split) / p.splits + 1) : 0u;
         const float alpha = p.pre_alpha, beta = p.pre_beta;
-        // frame of the staged batches: the warp tile's first receiver
-        const int64_t c_idx = p.order ? p.order[wbase] : wbase;
-        const float cx = p.recv[3 * c_idx], cy = p.recv[3 * c_idx + 1], cz = p.recv[3 * c_idx + 2];
-
         // receiver k of the lane at x = c + x', x' = (xp + xl) exactly
         float xa[kR], ya[kR], za[kR], xp[kR], yp[kR], zp[kR], xl[kR], yl[kR], zl[kR], xx[kR];
+        bool part[kR];
         uint32_t valid = 0;
 #pragma unroll
         for (int k = 0; k < kR; ++k) {
@@ -139,9 +136,19 @@ __global__ void __maxnreg__(128) gbs_count_kernel(const __grid_constant__ FwdPar
             // of its Morton patch, so a beam edge splits work evenly over lanes
             const int64_t r = wbase + (int64_t)k * 32 + lane;
             xa[k] = ya[k] = za[k] = xp[k] = yp[k] = zp[k] = xl[k] = yl[k] = zl[k] = xx[k] = 0.0f;
+            part[k] = false;
             if (r < p.n_recv) {
                 const int64_t o = p.order ? p.order[r] : r;
                 xa[k] = p.recv[3 * o]; ya[k] = p.recv[3 * o + 1]; za[k] = p.recv[3 * o + 2];
+                part[k] = takes_part(xa[k], ya[k], za[k]);
+            }
+        }
+        // frame of the staged batches: the warp tile's first receiver
+        const float3 c0 = first_receiver(part, xa, ya, za);
+        const float cx = c0.x, cy = c0.y, cz = c0.z;
+#pragma unroll
+        for (int k = 0; k < kR; ++k) {
+            if (part[k]) {
                 two_sum(xa[k], -cx, xp[k], xl[k]);
                 two_sum(ya[k], -cy, yp[k], yl[k]);
                 two_sum(za[k], -cz, zp[k], zl[k]);
@@ -726,18 +733,19 @@ __global__ void __launch_bounds__(32 * kWarps64) gbs_fwd_f64_kernel(const __grid
     const float xf = valid ? p.recv[3 * ri] : 0.f, yf = valid ? p.recv[3 * ri + 1] : 0.f,
                 zf = valid ? p.recv[3 * ri + 2] : 0.f;
     // ball about the centre c of the receivers' bounding box
+    const bool part = valid && takes_part(xf, yf, zf);
     const float v[3] = {xf, yf, zf};
     float ctr[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         const unsigned u = ordered_bits(v[a]);
-        ctr[a] = 0.5f * from_ordered(__reduce_min_sync(0xffffffffu, valid ? u : ~0u)) +
-                 0.5f * from_ordered(__reduce_max_sync(0xffffffffu, valid ? u : 0u));
+        ctr[a] = 0.5f * from_ordered(__reduce_min_sync(0xffffffffu, part ? u : ~0u)) +
+                 0.5f * from_ordered(__reduce_max_sync(0xffffffffu, part ? u : 0u));
     }
     const float xp = xf - ctr[0], yp = yf - ctr[1], zp = zf - ctr[2];
     const float xx = fmaf(xp, xp, fmaf(yp, yp, zp * zp));
     const float rad = 1.000001f * sqrtf(__uint_as_float(
-        __reduce_max_sync(0xffffffffu, valid ? __float_as_uint(xx) : 0u)));
+        __reduce_max_sync(0xffffffffu, part ? __float_as_uint(xx) : 0u)));
     const float4 rball = reach_ball(make_float4(ctr[0], ctr[1], ctr[2], rad));
     const float alpha = p.g.pre_alpha, beta = p.g.pre_beta, naxx = -alpha * xx;
     const double c2 = 2.0 * p.cutoff;
@@ -775,7 +783,7 @@ __global__ void __launch_bounds__(32 * kWarps64) gbs_fwd_f64_kernel(const __grid
             const float sl = fmaf(xp, a.x, fmaf(yp, a.y, fmaf(zp, a.z, a.w)));
             const float sm = sl + q.x;
             const float nd = fmaf(xp, b.x, fmaf(yp, b.y, fmaf(zp, b.z, naxx + b.w)));
-            bool keep = valid && fmaf(alpha * sl, sl, fmaf(sm, sm, nd)) >= 0.f;
+            bool keep = part && fmaf(alpha * sl, sl, fmaf(sm, sm, nd)) >= 0.f;
             if (WINDOW == GBT_WINDOW_LINE) keep = keep && sm >= 0.f;
             else keep = keep && sl + q.z >= 0.f && sl < q.y;
             const uint32_t b32 = __ballot_sync(0xffffffffu, keep);
@@ -1012,30 +1020,36 @@ constexpr int64_t kOrderTiles = 24;
 __global__ void tile_ball_kernel(const float *recv, const int32_t *order, int64_t n_recv,
                                  float4 *ball, unsigned int *weight, float4 *rball)
 {
-    __shared__ float red[4][8];
+    __shared__ float red[5][8];
     const int64_t base = (int64_t)blockIdx.x * kCtaRecv;
     const int n = (int)(n_recv - base < (int64_t)kCtaRecv ? n_recv - base : (int64_t)kCtaRecv);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    float sx = 0.f, sy = 0.f, sz = 0.f;
+    float sx = 0.f, sy = 0.f, sz = 0.f, nv = 0.f;
     for (int j = threadIdx.x; j < n; j += blockDim.x) {
         const int64_t o = order ? order[base + j] : base + j;
-        sx += recv[3 * o]; sy += recv[3 * o + 1]; sz += recv[3 * o + 2];
+        const float x = recv[3 * o], y = recv[3 * o + 1], z = recv[3 * o + 2];
+        if (takes_part(x, y, z)) { sx += x; sy += y; sz += z; nv += 1.f; }
     }
     for (int o = 16; o > 0; o >>= 1) {
         sx += __shfl_xor_sync(0xffffffffu, sx, o);
         sy += __shfl_xor_sync(0xffffffffu, sy, o);
         sz += __shfl_xor_sync(0xffffffffu, sz, o);
+        nv += __shfl_xor_sync(0xffffffffu, nv, o);
     }
-    if (lane == 0) { red[0][wid] = sx; red[1][wid] = sy; red[2][wid] = sz; }
+    if (lane == 0) { red[0][wid] = sx; red[1][wid] = sy; red[2][wid] = sz; red[4][wid] = nv; }
     __syncthreads();
-    sx = sy = sz = 0.f;
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) { sx += red[0][k]; sy += red[1][k]; sz += red[2][k]; }
-    const float cx = sx / (float)n, cy = sy / (float)n, cz = sz / (float)n;
+    sx = sy = sz = nv = 0.f;
+    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) {
+        sx += red[0][k]; sy += red[1][k]; sz += red[2][k]; nv += red[4][k];
+    }
+    nv = fmaxf(nv, 1.f);
+    const float cx = sx / nv, cy = sy / nv, cz = sz / nv;
     float r2 = 0.f;
     for (int j = threadIdx.x; j < n; j += blockDim.x) {
         const int64_t o = order ? order[base + j] : base + j;
-        const float dx = recv[3 * o] - cx, dy = recv[3 * o + 1] - cy, dz = recv[3 * o + 2] - cz;
-        r2 = fmaxf(r2, fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
+        const float x = recv[3 * o], y = recv[3 * o + 1], z = recv[3 * o + 2];
+        const float dx = x - cx, dy = y - cy, dz = z - cz;
+        if (takes_part(x, y, z)) r2 = fmaxf(r2, fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
     }
     for (int o = 16; o > 0; o >>= 1) r2 = fmaxf(r2, __shfl_xor_sync(0xffffffffu, r2, o));
     __syncthreads();
@@ -1065,8 +1079,9 @@ __global__ void warp_ball_kernel(const float *recv, const int32_t *order, int64_
         if (ok[k]) {
             const int64_t o = order ? order[r] : r;
             x[k] = recv[3 * o]; y[k] = recv[3 * o + 1]; z[k] = recv[3 * o + 2];
-            sx += x[k]; sy += y[k]; sz += z[k]; nv += 1.f;
+            ok[k] = takes_part(x[k], y[k], z[k]);
         }
+        if (ok[k]) { sx += x[k]; sy += y[k]; sz += z[k]; nv += 1.f; }
     }
     for (int o = 16; o > 0; o >>= 1) {
         sx += __shfl_xor_sync(0xffffffffu, sx, o);

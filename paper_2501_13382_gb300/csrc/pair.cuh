@@ -28,7 +28,7 @@
 //    3 x 2^-24 x 16 turns = 1.8e-5 rad where K max|x'| <= kFastTurns.  Beyond that, and for
 //    the segments that have an end of their window inside the warp tile's ball (about one
 //    in five on the city), u = Um + Uc: x' and t are split on grids of 11 and 12 bits of
-//    their largest magnitude, so the three products of Um and their sum are exact in FP32,
+//    their magnitude, so the three products of Um and their sum are exact in FP32,
 //    and Uc holds the rest to about 2^-36 |x'|.  Nine products, where float-float sums took
 //    31 operations; window decisions are then those of the exact arithmetic to 1e-10 m.
 //    Which of the two a segment takes is uniform over the warp.
@@ -381,6 +381,38 @@ __device__ __forceinline__ StagedBatch stage(const FwdParams &p, WarpBuf<NF, LOS
     return b;
 }
 
+// The median of the warp's receivers by coordinate (part: those that count), as the frame of a
+// warp tile with a stray receiver (a point far off the map), whose |x'| then does not coarsen the
+// others'; w > 0 if most of them lie within sqrt(close2) of it.  Out of line: it is seldom
+// called, and its registers are not the kernel's.
+__device__ __noinline__ float4 stray_frame(bool p0, bool p1, float x0, float y0, float z0, float x1,
+                                           float y1, float z1, float close2)
+{
+    const int most = __popc(__ballot_sync(0xffffffffu, p0)) + __popc(__ballot_sync(0xffffffffu, p1));
+    float med[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const unsigned u0 = ordered_bits(a == 0 ? x0 : a == 1 ? y0 : z0);
+        const unsigned u1 = ordered_bits(a == 0 ? x1 : a == 1 ? y1 : z1);
+        unsigned m = 0u;               // the largest value with fewer than half of them below it
+#pragma unroll 1
+        for (unsigned bit = 0x80000000u; bit; bit >>= 1) {
+            const unsigned v = m | bit;
+            const int below = __popc(__ballot_sync(0xffffffffu, p0 && u0 < v)) +
+                              __popc(__ballot_sync(0xffffffffu, p1 && u1 < v));
+            if (below <= (most - 1) / 2) m = v;
+        }
+        med[a] = from_ordered(m);
+    }
+    auto is_close = [&](float x, float y, float z) {
+        const float ex = x - med[0], ey = y - med[1], ez = z - med[2];
+        return fmaf(ex, ex, fmaf(ey, ey, ez * ez)) < close2;
+    };
+    const int close = __popc(__ballot_sync(0xffffffffu, p0 && is_close(x0, y0, z0))) +
+                      __popc(__ballot_sync(0xffffffffu, p1 && is_close(x1, y1, z1)));
+    return make_float4(med[0], med[1], med[2], 2 * close > most ? 1.0f : 0.0f);
+}
+
 template <int NF, int WINDOW, bool BATCHED, bool LOSSY>
 __global__ void __launch_bounds__(32 * PairCfg<WarpBuf<NF, LOSSY>, BATCHED, BATCHED ? PairShape<NF, LOSSY>::kWarpsBatched : PairShape<NF, LOSSY>::kWarps>::kWarps, 1) gbs_pair_kernel(const __grid_constant__ FwdParams prm)
 {
@@ -422,16 +454,20 @@ __global__ void __launch_bounds__(32 * PairCfg<WarpBuf<NF, LOSSY>, BATCHED, BATC
         // the lane's receivers: lane and lane + 32 of the warp tile, the two halves of its
         // Morton patch, so a beam edge splits work evenly over lanes
         float xr[kR], yr[kR], zr[kR];
-        bool valid[kR];
+        bool part[kR];
         unsigned bb[6] = {~0u, ~0u, ~0u, 0u, 0u, 0u};
 #pragma unroll
         for (int k = 0; k < kR; ++k) {
             const int64_t r = item.wbase + (int64_t)k * 32 + lane;
-            valid[k] = r < p.n_recv;
+            part[k] = false;
             xr[k] = yr[k] = zr[k] = 0.0f;
-            if (valid[k]) {
+            if (r < p.n_recv) {
                 const int64_t o = p.order ? p.order[r] : r;
                 xr[k] = p.recv[3 * o]; yr[k] = p.recv[3 * o + 1]; zr[k] = p.recv[3 * o + 2];
+                part[k] = takes_part(xr[k], yr[k], zr[k]);
+                if (!part[k]) no_partials(p, item, 32 * k + lane);
+            }
+            if (part[k]) {
                 const unsigned ux = ordered_bits(xr[k]), uy = ordered_bits(yr[k]), uz = ordered_bits(zr[k]);
                 bb[0] = min(bb[0], ux); bb[1] = min(bb[1], uy); bb[2] = min(bb[2], uz);
                 bb[3] = max(bb[3], ux); bb[4] = max(bb[4], uy); bb[5] = max(bb[5], uz);
@@ -448,30 +484,55 @@ __global__ void __launch_bounds__(32 * PairCfg<WarpBuf<NF, LOSSY>, BATCHED, BATC
             const float hi = from_ordered(__reduce_max_sync(0xffffffffu, bb[3 + a]));
             ctr[a] = 0.5f * lo + 0.5f * hi;
         }
-        const float cx = ctr[0], cy = ctr[1], cz = ctr[2];
-        float xp[kR], yp[kR], zp[kR], xl[kR], yl[kR], zl[kR], xx = 0.0f;
+        float xp[kR], yp[kR], zp[kR], xl[kR], yl[kR], zl[kR], xx[kR];
+        unsigned far2, near2;          // bits of the largest and the smallest |x'|^2
+        auto place = [&]() {
+            far2 = 0u;
+            near2 = ~0u;
 #pragma unroll
-        for (int k = 0; k < kR; ++k) {
-            xp[k] = yp[k] = zp[k] = xl[k] = yl[k] = zl[k] = 0.0f;
-            if (valid[k]) {
-                two_sum(xr[k], -cx, xp[k], xl[k]);
-                two_sum(yr[k], -cy, yp[k], yl[k]);
-                two_sum(zr[k], -cz, zp[k], zl[k]);
-                xx = fmaxf(xx, fmaf(xp[k], xp[k], fmaf(yp[k], yp[k], zp[k] * zp[k])));
+            for (int k = 0; k < kR; ++k) {
+                xp[k] = yp[k] = zp[k] = xl[k] = yl[k] = zl[k] = xx[k] = 0.0f;
+                if (part[k]) {
+                    two_sum(xr[k], -ctr[0], xp[k], xl[k]);
+                    two_sum(yr[k], -ctr[1], yp[k], yl[k]);
+                    two_sum(zr[k], -ctr[2], zp[k], zl[k]);
+                    xx[k] = fmaf(xp[k], xp[k], fmaf(yp[k], yp[k], zp[k] * zp[k]));
+                    far2 = max(far2, __float_as_uint(xx[k]));
+                    near2 = min(near2, __float_as_uint(xx[k]));
+                }
+            }
+            far2 = __reduce_max_sync(0xffffffffu, far2);
+            near2 = __reduce_min_sync(0xffffffffu, near2);
+        };
+        place();
+        const float4 rball = reach_ball(make_float4(ctr[0], ctr[1], ctr[2],
+                                                    1.000001f * sqrtf(__uint_as_float(far2))));
+        // a centre without a receiver within half the radius may lie between the others and a
+        // stray one
+        if (far2 != 0u && __uint_as_float(near2) > 0.25f * __uint_as_float(far2)) {
+            const float4 med = stray_frame(part[0], part[1], xr[0], yr[0], zr[0], xr[1], yr[1], zr[1],
+                                           0.0625f * __uint_as_float(far2));
+            if (med.w > 0.0f) {
+                ctr[0] = med.x; ctr[1] = med.y; ctr[2] = med.z;
+                place();
             }
         }
-        const float rad = 1.000001f * sqrtf(__uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(xx))));
+        const float cx = ctr[0], cy = ctr[1], cz = ctr[2];
+        const float rad = 1.000001f * sqrtf(__uint_as_float(far2));
         const bool fast = rad * p.kmax_turns <= kFastTurns;
-        // grid of x': a power of two q with |x'| <= 2^11 q, by adding 1.5 x 2^23 q
-        const float grid = rad > 1e-25f ? scalbnf(12582912.0f, (int)ceilf(log2f(rad) + 1e-5f) - 11) : 0.0f;
+        // grid of a receiver's x': a power of two q with |x'| <= 2^11 q, by adding 1.5 x 2^23 q
+        float grid[kR];
+#pragma unroll
+        for (int k = 0; k < kR; ++k)
+            grid[k] = xx[k] > 1e-36f ? scalbnf(12582912.0f, (int)ceilf(0.5f * log2f(xx[k]) + 1e-5f) - 11) : 0.0f;
         LaneRecv x;
         {
             float h[3][kR];
 #pragma unroll
             for (int k = 0; k < kR; ++k) {
-                h[0][k] = __fsub_rn(__fadd_rn(xp[k], grid), grid);
-                h[1][k] = __fsub_rn(__fadd_rn(yp[k], grid), grid);
-                h[2][k] = __fsub_rn(__fadd_rn(zp[k], grid), grid);
+                h[0][k] = __fsub_rn(__fadd_rn(xp[k], grid[k]), grid[k]);
+                h[1][k] = __fsub_rn(__fadd_rn(yp[k], grid[k]), grid[k]);
+                h[2][k] = __fsub_rn(__fadd_rn(zp[k], grid[k]), grid[k]);
                 xl[k] = __fadd_rn(__fsub_rn(xp[k], h[0][k]), xl[k]);
                 yl[k] = __fadd_rn(__fsub_rn(yp[k], h[1][k]), yl[k]);
                 zl[k] = __fadd_rn(__fsub_rn(zp[k], h[2][k]), zl[k]);
@@ -481,10 +542,8 @@ __global__ void __launch_bounds__(32 * PairCfg<WarpBuf<NF, LOSSY>, BATCHED, BATC
             x.XH = pk(h[0][0], h[0][1]); x.YH = pk(h[1][0], h[1][1]); x.ZH = pk(h[2][0], h[2][1]);
             x.XL = pk(xl[0], xl[1]); x.YL = pk(yl[0], yl[1]); x.ZL = pk(zl[0], zl[1]);
         }
-        const float4 rball = reach_ball(make_float4(cx, cy, cz, rad));
-
         bool first = true;
-        auto fold_all = [&]() { fold_bands<NF>(p, item, lane, valid, ax, ay, first); };
+        auto fold_all = [&]() { fold_bands<NF>(p, item, lane, part, ax, ay, first); };
 
         Gather<WINDOW, false> g(item);
         g.issue(p, item, B.in, lane, rball, 0);

@@ -168,13 +168,10 @@ __global__ void __maxnreg__(128) gbs_adjoint_kernel(const __grid_constant__ FwdP
         const int64_t n_batches = (n_seg + kBatch - 1) / kBatch;
         const uint32_t nb = split < n_batches ? (uint32_t)((n_batches - 1 - split) / p.splits + 1) : 0u;
         const float alpha = p.pre_alpha, beta = p.pre_beta;
-        // frame of the staged batches: the warp tile's first receiver
-        const int64_t c_idx = p.order ? p.order[wbase] : wbase;
-        const float cx = p.recv[3 * c_idx], cy = p.recv[3 * c_idx + 1], cz = p.recv[3 * c_idx + 2];
-
         // receiver k of the lane at x = c + x', x' = (xp + xl) exactly
         float xa[kR], ya[kR], za[kR], xp[kR], yp[kR], zp[kR], xl[kR], yl[kR], zl[kR], xx[kR];
         int32_t ridx[kR];
+        bool part[kR];
         uint32_t valid = 0;
 #pragma unroll
         for (int k = 0; k < kR; ++k) {
@@ -183,15 +180,25 @@ __global__ void __maxnreg__(128) gbs_adjoint_kernel(const __grid_constant__ FwdP
             const int64_t r = wbase + (int64_t)k * 32 + lane;
             xa[k] = ya[k] = za[k] = xp[k] = yp[k] = zp[k] = xl[k] = yl[k] = zl[k] = xx[k] = 0.0f;
             ridx[k] = -1;
+            part[k] = false;
             if (r < p.n_recv) {
                 const int64_t o = p.order ? p.order[r] : r;
                 xa[k] = p.recv[3 * o]; ya[k] = p.recv[3 * o + 1]; za[k] = p.recv[3 * o + 2];
+                part[k] = takes_part(xa[k], ya[k], za[k]);
+                if (part[k]) ridx[k] = (int32_t)o;
+            }
+        }
+        // frame of the staged batches: the warp tile's first receiver
+        const float3 c0 = first_receiver(part, xa, ya, za);
+        const float cx = c0.x, cy = c0.y, cz = c0.z;
+#pragma unroll
+        for (int k = 0; k < kR; ++k) {
+            if (part[k]) {
                 two_sum(xa[k], -cx, xp[k], xl[k]);
                 two_sum(ya[k], -cy, yp[k], yl[k]);
                 two_sum(za[k], -cz, zp[k], zl[k]);
                 xx[k] = fmaf(xp[k], xp[k], fmaf(yp[k], yp[k], zp[k] * zp[k]));
                 valid |= 1u << k;
-                ridx[k] = (int32_t)o;
             }
 #pragma unroll
             for (int f = 0; f < NF; ++f)

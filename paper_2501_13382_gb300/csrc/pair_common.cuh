@@ -223,6 +223,28 @@ __device__ __forceinline__ float from_ordered(unsigned int u)
     return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
 }
 
+// Whether a receiver takes part: its coordinates are finite and small enough for their squares
+// to be FP32 numbers.  One that does not gets a zero field and leaves its neighbours alone: it
+// stays out of the frames, balls and boxes of its warp and tile.
+__device__ __forceinline__ bool takes_part(float x, float y, float z)
+{
+    return fabsf(x) < 1e18f && fabsf(y) < 1e18f && fabsf(z) < 1e18f;      // false for a NaN
+}
+// The warp's first receiver that takes part (part: per receiver of the lane; 0 when there is
+// none), which is the frame of the float-float kernels.
+__device__ __forceinline__ float3 first_receiver(const bool (&part)[kR], const float (&x)[kR],
+                                                 const float (&y)[kR], const float (&z)[kR])
+{
+    static_assert(kR == 2, "two receivers per lane");
+    const uint32_t m0 = __ballot_sync(0xffffffffu, part[0]), m1 = __ballot_sync(0xffffffffu, part[1]);
+    const int k = m0 ? 0 : 1, src = (m0 | m1) ? __ffs(m0 ? m0 : m1) - 1 : 0;
+    const bool any = (m0 | m1) != 0u;
+    const float cx = __shfl_sync(0xffffffffu, k ? x[1] : x[0], src);
+    const float cy = __shfl_sync(0xffffffffu, k ? y[1] : y[0], src);
+    const float cz = __shfl_sync(0xffffffffu, k ? z[1] : z[0], src);
+    return any ? make_float3(cx, cy, cz) : make_float3(0.f, 0.f, 0.f);
+}
+
 // Two values, each duplicated into both halves of a float pair.
 __device__ __forceinline__ float4 dup2(float a, float b) { return make_float4(a, a, b, b); }
 

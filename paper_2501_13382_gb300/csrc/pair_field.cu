@@ -347,22 +347,29 @@ __global__ void __maxnreg__(128) gbs_field_kernel(const __grid_constant__ FwdPar
         Item item;
         if (!decode_item(p, it, item)) continue;
 
-        // frame of the staged batches: the warp tile's first receiver
-        const int64_t c_idx = p.order ? p.order[item.wbase] : item.wbase;
-        const float cx = p.recv[3 * c_idx], cy = p.recv[3 * c_idx + 1], cz = p.recv[3 * c_idx + 2];
         // receiver k of the lane (lane and lane + 32 of the warp tile) at x = c + x',
         // x' = (xp + xl) exactly
         float xr[kR], yr[kR], zr[kR], xp[kR], yp[kR], zp[kR], xl[kR], yl[kR], zl[kR], xx[kR];
-        bool valid[kR];
+        bool part[kR];
         unsigned bb[6] = {~0u, ~0u, ~0u, 0u, 0u, 0u};
 #pragma unroll
         for (int k = 0; k < kR; ++k) {
             const int64_t r = item.wbase + (int64_t)k * 32 + lane;
-            valid[k] = r < p.n_recv;
+            part[k] = false;
             xr[k] = yr[k] = zr[k] = xp[k] = yp[k] = zp[k] = xl[k] = yl[k] = zl[k] = xx[k] = 0.0f;
-            if (valid[k]) {
+            if (r < p.n_recv) {
                 const int64_t o = p.order ? p.order[r] : r;
                 xr[k] = p.recv[3 * o]; yr[k] = p.recv[3 * o + 1]; zr[k] = p.recv[3 * o + 2];
+                part[k] = takes_part(xr[k], yr[k], zr[k]);
+                if (!part[k]) no_partials(p, item, 32 * k + lane);
+            }
+        }
+        // frame of the staged batches: the warp tile's first receiver
+        const float3 c0 = first_receiver(part, xr, yr, zr);
+        const float cx = c0.x, cy = c0.y, cz = c0.z;
+#pragma unroll
+        for (int k = 0; k < kR; ++k) {
+            if (part[k]) {
                 two_sum(xr[k], -cx, xp[k], xl[k]);
                 two_sum(yr[k], -cy, yp[k], yl[k]);
                 two_sum(zr[k], -cz, zp[k], zl[k]);
@@ -381,7 +388,7 @@ __global__ void __maxnreg__(128) gbs_field_kernel(const __grid_constant__ FwdPar
         float q2 = 0.0f;
 #pragma unroll
         for (int k = 0; k < kR; ++k)
-            if (valid[k]) {
+            if (part[k]) {
                 const float ex = xr[k] - ctr[0], ey = yr[k] - ctr[1], ez = zr[k] - ctr[2];
                 q2 = fmaxf(q2, fmaf(ex, ex, fmaf(ey, ey, ez * ez)));
             }
@@ -404,7 +411,7 @@ __global__ void __maxnreg__(128) gbs_field_kernel(const __grid_constant__ FwdPar
         for (int f = 0; f < NF; ++f) ax[f] = ay[f] = 0ull;
 
         bool first = true;
-        auto fold_all = [&]() { fold_bands<NF>(p, item, lane, valid, ax, ay, first); };
+        auto fold_all = [&]() { fold_bands<NF>(p, item, lane, part, ax, ay, first); };
         Gather<WINDOW, true> g(item);
         int group = 0;
         g.issue(p, item, B.in, lane, rball, 0);
@@ -431,13 +438,13 @@ __global__ void __maxnreg__(128) gbs_field_kernel(const __grid_constant__ FwdPar
             uint32_t mine = 0u;
             for (uint32_t T = smask; T; T &= T - 1u) {
                 const int j = __ffs(T) - 1;
-                if (may_keep<NF, WINDOW>(B, j, x, NAXX, AL2, valid[0], valid[1])) mine |= 1u << j;
+                if (may_keep<NF, WINDOW>(B, j, x, NAXX, AL2, part[0], part[1])) mine |= 1u << j;
             }
             uint32_t T = (all & ~smask) | __reduce_or_sync(0xffffffffu, mine);
             while (T) {
                 const int j = __ffs(T) - 1;
                 T &= T - 1u;
-                eval_field<NF, WINDOW, LOSSY>(p, B, j, x, valid[0], valid[1], fast, eps, ax, ay);
+                eval_field<NF, WINDOW, LOSSY>(p, B, j, x, part[0], part[1], fast, eps, ax, ay);
             }
             __syncwarp();        // before the next batch is staged over this one
         }

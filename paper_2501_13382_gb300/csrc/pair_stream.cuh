@@ -204,9 +204,16 @@ __device__ __forceinline__ void fold(float4 *acc, float x, float y, bool first)
     }
 }
 
+// Zero partials of the item's receiver `at` (of its warp tile), which takes no part.
+__device__ __forceinline__ void no_partials(const FwdParams &p, const Item &m, int at)
+{
+    for (int f = 0; f < p.nf; ++f)
+        __stcg(p.partial + m.part + f * m.part_band + at, make_float4(0.f, 0.f, 0.f, 0.f));
+}
+
 // Folds a lane's two receivers' sums per band into the item's partials and zeroes them.
 template <int NF>
-__device__ __forceinline__ void fold_bands(const FwdParams &p, const Item &m, int lane, const bool (&valid)[kR],
+__device__ __forceinline__ void fold_bands(const FwdParams &p, const Item &m, int lane, const bool (&part_of)[kR],
                                            f2x (&ax)[NF], f2x (&ay)[NF], bool &first)
 {
 #pragma unroll
@@ -216,8 +223,8 @@ __device__ __forceinline__ void fold_bands(const FwdParams &p, const Item &m, in
             upk(ax[f], x0, x1);
             upk(ay[f], y0, y1);
             float4 *const part = p.partial + m.part + f * m.part_band + lane;
-            if (valid[0]) fold(part, x0, y0, first);
-            if (valid[1]) fold(part + 32, x1, y1, first);
+            if (part_of[0]) fold(part, x0, y0, first);
+            if (part_of[1]) fold(part + 32, x1, y1, first);
         }
         ax[f] = ay[f] = 0ull;
     }
