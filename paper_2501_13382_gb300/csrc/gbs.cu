@@ -768,8 +768,13 @@ __global__ void __launch_bounds__(32 * kWarps64) gbs_fwd_f64_kernel(const __grid
             const float oo = fmaf(ox, ox, fmaf(oy, oy, oz * oz));
             const float a2 = 2.f * alpha;
             w.P[0][lane] = make_float4(r1.x, r1.y, r1.z, -ot);
-            w.P[1][lane] = make_float4(a2 * ox, a2 * oy, a2 * oz, fmaf(-alpha, oo, beta));
-            const float mg = kWinMargin + 1e-6f * (fabsf(ox) + fabsf(oy) + fabsf(oz));
+            // What the prefilter's terms may lose: with M = |o'| + |x'| the rounding of o', x' and t
+            // moves n^2 by at most 10 x 2^-24 M^2, that of the sums alpha s_loc^2 and alpha |x' - o'|^2,
+            // which cancel, by about 30 x 2^-24 alpha M^2 more, whatever s is; and s by 6 x 2^-24 M.
+            const float M = sqrtf(oo) + rad;
+            w.P[1][lane] = make_float4(a2 * ox, a2 * oy, a2 * oz,
+                                       fmaf(-alpha, oo, beta) + 3e-6f * alpha * M * M);
+            const float mg = kWinMargin + 1e-6f * (fabsf(ox) + fabsf(oy) + fabsf(oz) + rad);
             w.P[2][lane] = make_float4(r0.w + mg, r1.w + mg, mg, 0.f);
             w.seg[lane] = buf ? g.seg1 : g.seg0;
         }
@@ -783,9 +788,10 @@ __global__ void __launch_bounds__(32 * kWarps64) gbs_fwd_f64_kernel(const __grid
             const float sl = fmaf(xp, a.x, fmaf(yp, a.y, fmaf(zp, a.z, a.w)));
             const float sm = sl + q.x;
             const float nd = fmaf(xp, b.x, fmaf(yp, b.y, fmaf(zp, b.z, naxx + b.w)));
-            bool keep = part && fmaf(alpha * sl, sl, fmaf(sm, sm, nd)) >= 0.f;
-            if (WINDOW == GBT_WINDOW_LINE) keep = keep && sm >= 0.f;
-            else keep = keep && sl + q.z >= 0.f && sl < q.y;
+            // (an overflow leaves the pair a candidate)
+            bool keep = part && !(fmaf(alpha * sl, sl, fmaf(sm, sm, nd)) < 0.f);
+            if (WINDOW == GBT_WINDOW_LINE) keep = keep && !(sm < 0.f);
+            else keep = keep && !(sl + q.z < 0.f) && !(sl >= q.y);
             const uint32_t b32 = __ballot_sync(0xffffffffu, keep);
             if (lane == j) mine = b32;
         }

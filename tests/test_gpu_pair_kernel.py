@@ -139,3 +139,27 @@ def test_splits_by_list_length_against_equal_splits(n, rays, nf, window):
                              tile_cull=True, seg_split=k) for k in (0, 3))
     torch.cuda.synchronize()
     assert float((auto - equal).norm()) <= 1.2e-4 * float(equal.norm())
+
+
+@pytest.mark.parametrize("cutoff,height,b", [(2.0, 1000.0, 1.0), (0.5, 1000.0, 1.0), (2.0, 5000.0, 0.3)])
+def test_f64_candidates_near_an_image_source_seen_from_afar(cutoff, height, b):
+    """Receivers a few metres from the image source, on rays whose reflection lies a kilometre
+    away: the prefilter's terms alpha |x' - o'|^2 are then far above s^2 + b^2, and their FP32
+    rounding must not drop a pair that the FP64 test keeps.  Tolerance: the rounding of the
+    complex64 output, 2^-24, and of FP64 phases, 1e-11 of up to 1e5 rad."""
+    import torch
+    from paper_2501_13382_gb300 import gbt as G
+    sc0 = I.Scene(I.C_AIR, True, 0.0, 0, np.zeros((0, 3, 3)), np.zeros(0, np.int32),
+                  np.zeros(0, np.int32), np.array([0.9], np.float32))
+    src = I.Source(np.array([0.2, -0.3, height]), 4000, 1, 4.0 * height)
+    rng = np.random.default_rng(9)
+    away = rng.uniform(-1.0, 1.0, (96, 3)) * [3.0, 3.0, 2.0] + [0.0, 0.0, 3.0]
+    recv = (np.array([0.2, -0.3, -height]) + away).astype(np.float32)
+    freqs, bs = [4000.0], [b]
+    po = O.gbs_sum(O.trace(sc0, src), recv, freqs, bs, sc0.c, sc0.gamma, window=I.WINDOW_LINE, cutoff=cutoff)
+    tr = G.Trace(G.Scene(sc0), src)
+    p = G.gbs_sum(tr, torch.as_tensor(recv, device="cuda"), freqs, bs, torch.as_tensor(sc0.gamma, device="cuda"),
+                  window=I.WINDOW_LINE, cutoff=cutoff, precision=G.PRECISION_F64)
+    torch.cuda.synchronize()
+    e = p.cpu().numpy().astype(np.complex128) - po
+    assert np.linalg.norm(po) > 0 and np.linalg.norm(e) <= 1e-7 * np.linalg.norm(po)
