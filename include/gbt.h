@@ -236,14 +236,14 @@ gbt_status gbt_trace_import(const gbt_scene_t *scene, const gbt_source_desc *src
  * 64 receivers, whose segment terms are formed in float-float, FP32 MUFU
  * exp/sin/cos, compensated per-receiver accumulation; relative L2 error against
  * an FP64 evaluation measured at 1e-7..5e-7 on the synthetic open-plane and city
- * workloads (tested to 1e-6 with 4 kHz phases over 1 km paths).  Where a group
- * is compact for the call's highest frequency (K max|x'| <= 16 turns) the
- * receivers' projection on a segment is one FP32 dot product (a term's phase
- * moves by at most 1.8e-5 rad); elsewhere, and for a segment that has an end of
- * its window inside the group's ball, it is split into an exact and a rest part,
- * so the window decisions are those of the exact arithmetic to 1e-10 m.  F64
- * precision: every step in FP64 (2.6e-8, the rounding of the complex64 output),
- * at FP64 speed.
+ * workloads (tested to 1e-6 with 4 kHz phases over 1 km paths).  The receivers'
+ * projection on a segment is split into an exact and a rest part, so the window
+ * decisions are those of the exact arithmetic to 1e-10 m; with one frequency, and
+ * where a group is compact for it (K max|x'| <= 16 turns) and no end of the
+ * segment's window lies inside the group's ball, it is one FP32 dot product and
+ * the low words' (a term's phase moves by at most 1.8e-5 rad).  F64 precision:
+ * every step of a kept beam in FP64 (2.6e-8, the rounding of the complex64
+ * output), at FP64 speed.
  * With more than 8 frequencies the F32 path runs one pair launch per group of
  * at most 8 (frequencies sorted by value when every b_f is equal, otherwise in
  * the given order); each group costs a full pass over the pairs.

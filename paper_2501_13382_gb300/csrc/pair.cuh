@@ -1,5 +1,5 @@
 // pair.cuh -- the FP32 pair kernel: beams of Eq. 1 / Eq. 2 summed over (receiver, segment,
-// frequency), forward and adjoint.
+// frequency), forward only (the adjoint is in pair_bwd.cu).
 //
 // Every warp works on its own.  It takes (warp tile of 64 receivers, segment split) items
 // from a global queue (CTA tiles of 960 receivers heaviest first), collects the segments
@@ -18,32 +18,39 @@
 // LOP3: 4.9 cycles); more warps or longer chains change little.  So the number of operands
 // per pair is what counts.
 //  * The frame is the centre of the warp tile's bounding box, x = c + x'.  The staging forms
-//    per segment A = (c - o).t and S = s0 + A in float-float, the compensated
-//    N = (c - o) x t, and per band the phase of S reduced to one turn, so a pair needs
+//    per segment A = (c - o).t and S = s0 + A in float-float, N = (c - o) x t rounded once,
+//    and per band the phase of S reduced to one turn, so a pair needs
 //      u = x'.t,  s = S + u,  n = N + x' x t
 //    and the phase K u + phi_f, reduced by adding and subtracting 1.5 x 2^23: no
-//    float-float arithmetic per pair (32 paired operations with one band, where float-float
+//    float-float arithmetic per pair (38 paired operations with one band, where float-float
 //    geometry and phase took 63).
-//  * u in FP32 is within about 3 x 2^-24 |x'| of x'.t, which moves the phase by at most
-//    3 x 2^-24 x 16 turns = 1.8e-5 rad where K max|x'| <= kFastTurns.  Beyond that, and for
-//    the segments that have an end of their window inside the warp tile's ball (about one
-//    in five on the city), u = Um + Uc: x' and t are split on grids of 11 and 12 bits of
-//    their magnitude, so the three products of Um and their sum are exact in FP32,
-//    and Uc holds the rest to about 2^-36 |x'|.  Nine products, where float-float sums took
-//    31 operations; window decisions are then those of the exact arithmetic to 1e-10 m.
-//    Which of the two a segment takes is uniform over the warp.
-//  * Every sum of the phase is rounded near its smallest size (whole turns go before and
-//    after the second term): against 64 bits the relative L2 error of the open plane with 6
-//    bands is 2.5e-7 (float-float phases 2.9e-7), of scattered receivers 3.7e-7 (4.7e-7), of
-//    8 bands on the city 2.5e-7 to 2.8e-7 (2.5e-7 to 2.9e-7).
+//  * u = Um + Uc: x' and t are split on grids of 11 and 12 bits of their magnitude, so the three
+//    products of Um and their sum are exact in FP32, and Uc holds the rest to about 2^-36 |x'|.
+//    Nine products, where float-float sums took 31 operations; window decisions are those of
+//    the exact arithmetic to 1e-10 m.
+//  * One band, a compact warp (K max|x'| <= kFastTurns) and a segment without an end of its
+//    window inside the warp tile's ball: u is one FP32 dot product plus that of t's low words,
+//    six products.  Its rounding, 3 x 2^-24 |x'| at most, moves the phase by up to 1.8e-5 rad
+//    (small open plane: relative L2 error 2.3e-7, with the split form 1.7e-7), which spares
+//    the 1M-ray city 8 % of its time.  Several bands spend their time on the beams: there the
+//    split form is free.  Which of the two a segment takes is uniform over the warp.
+//  * Precision.  Relative L2 error against 64 bits over 37 inputs (listed, drawn and bench
+//    sizes, 8 seeds each): 0.60 of that of float-float pairs in the geometric mean, 0.24 to
+//    1.005 by input; 1M-ray city 1.3e-7 (1.8e-7), with losses 1.4e-7 (1.8e-7), open plane with 6
+//    bands 1.3e-7 (1.7e-7), 8 bands with losses 1.85e-7 (1.88e-7), scattered receivers 2.8e-7
+//    (4.6e-7).  Dropping t's low word, reducing the phase once and a compensated N with two
+//    roundings gave 0.77 and up to 1.26.  What is left is mostly MUFU's sine and cosine (0.39
+//    with sincospif); their mean loss of amplitude goes into the merge's factor.  n as exact
+//    head products and a rest (15 operations more) would give 0.50, for 8 to 16 % of the time.
 //  * The amplitude's common factor k / (8 pi^2) is left to the merge, the pairs' cutoff test
 //    is one comparison (r <= rc), and receivers past the last are computed and not stored.
-// Summation: FP32 per lane and batch group, folded every kFoldEvery batches into the item's
-// float-float partials, merged in split order by reduce_kernel, so results do not depend on
-// scheduling.
-// Measured (kernel alone, before -> after): city, 1,048,576 rays x 512^2 receivers, lists:
-// 31.0 -> 17.4 ms; open plane, 65,536 rays x 256^2 x 6 bands, no lists: 6.04 -> 1.92 ms;
-// city, 65,536 rays x 200^2 x 2 bands, no lists: 6.79 -> 1.6 ms.
+// Summation: FP32 per lane and batch group, folded into the item's float-float partials every
+// kFoldEvery batches of list entries and, without a list, twice as often (open plane, 6 bands:
+// every 16, 8, 4 batches 1.42e-7, 1.36e-7, 1.32e-7 and 2.08, 2.08, 2.14 ms), merged in split
+// order by reduce_kernel, so results do not depend on scheduling.
+// Measured (kernel alone, with float-float pairs -> now): city, 1,048,576 rays x 512^2
+// receivers, lists: 31.0 -> 15.8 ms; open plane, 65,536 rays x 256^2 x 6 bands, no lists:
+// 6.06 -> 2.01 ms; city, 65,536 rays x 200^2 x 2 bands, no lists: 6.79 -> 1.51 ms.
 #pragma once
 
 #include "pair_stream.cuh"
@@ -51,13 +58,12 @@
 namespace gbt {
 namespace {
 
-// K max|x'| up to which u is plain FP32.  The split form everywhere costs the 1M-ray city
-// step 5 % (26.6 against 25.4 ms) and brings the small open plane's error from 4.3e-7 to
-// 1.9e-7; up to this line the plain form's error stays under that of MUFU sine and cosine.
+// K max|x'| up to which one band's u is a plain dot product (see above).  Everywhere split, the
+// 1M-ray city takes 21.8 ms instead of 20.2, at an error of 1.24e-7 instead of 1.26e-7.
 constexpr float kFastTurns = 16.0f;
 
-// Shape by the number of band slots: segments evaluated together (plain, and of the second
-// class), bands per vote, and warps.  One band needs several segments for independent
+// Shape by the number of band slots: segments evaluated together (plain, which only one band has,
+// and split), bands per vote, and warps.  One band needs several segments for independent
 // chains and shared operands (1M-ray city step: one segment, 16 warps 27.4 ms; two 26.0;
 // four, 12 warps 25.1); two or more bands have the chains themselves.  Bands in pairs spare
 // votes where most bands are kept (open plane, 6 bands: 2.06 -> 1.94 ms), and cost where
@@ -75,14 +81,14 @@ struct PairShape {
 
 // Per-warp shared memory: the raw records and the staged batch, every value in both halves of
 // a float pair (a segment is shared by the warp, so the operands of the paired arithmetic are
-// broadcast loads).  Segments sit in slots: those whose u is plain FP32 first, then the
-// others, padded to whole groups with a slot of zero amplitude.
+// broadcast loads).  Segments sit in slots: those whose u is a plain dot product first, then the
+// split ones, padded to whole groups with a slot of zero amplitude.
 template <int NF, bool LOSSY>
 struct WarpBuf {
     static constexpr int kSlots = kBatch + 1;   // padding
     RawBuf in;
     // D[0] t.x, t.y | D[1] t.z, S (times s_scale) | D[2] N.x, N.y | D[3] N.z, amplitude |
-    // D[4..6] t on its grid (3) and the rest (3)
+    // D[4..6] t on its grid (3) and the rest (3); a plain slot's D[4..5]: t's low words (3)
     float4 D[7][kSlots];
     float4 W[kSlots];               // SEGMENT: A, A - L as (hi, lo); LINE: S as (hi, lo)
     float4 F[(NF + 1) / 2][kSlots]; // bands 2 i, 2 i + 1: phase of S in turns
@@ -141,7 +147,11 @@ __device__ __forceinline__ void eval_segments(const FwdParams &p, const WarpBuf<
                 }
             }
         } else {
+            f2x LX, LY, LZ, none;
+            word(4, q, LX, LY);
+            word(5, q, LZ, none);
             U[q] = u = fma2(x.X, TX, fma2(x.Y, TY, mul2(x.Z, TZ)));
+            UC[q] = fma2(x.X, LX, fma2(x.Y, LY, mul2(x.Z, LZ)));
         }
         s[q] = fma2(u, splat(p.s_scale), S);
         // n = N + x' x t
@@ -223,21 +233,14 @@ __device__ __forceinline__ void eval_segments(const FwdParams &p, const WarpBuf<
                 upk(ex, e0, e1);
                 g = mul2(g, pk(m0[q][i] ? ex2_approx(e0) : 0.0f, m1[q][i] ? ex2_approx(e1) : 0.0f));
                 const f2x KH = splat(c.K_hi);
-                f2x ph = f & 1 ? pp.y : pp.x, tau;
-                if (PREC || NF > 1) ph = fma2(splat(c.K_lo), U[q], ph);
-                if (PREC) ph = fma2(KH, UC[q], ph);
-                if (NF == 1) {
-                    // K u + ph less its whole turns, ph with the second term
-                    ph = fma2(splat(c.hK), rs[q][i], ph);
-                    const f2x nr = sub2(MAGIC, add2(fma2(KH, U[q], ph), MAGIC));
-                    tau = add2(fma2(KH, U[q], nr), ph);
-                } else {
-                    // less whole turns before and after the second term: every sum is rounded
-                    // near its smallest size
-                    const f2x nr = sub2(MAGIC, fma2(KH, U[q], MAGIC));
-                    tau = fma2(splat(c.hK), rs[q][i], add2(fma2(KH, U[q], nr), ph));
-                    tau = add2(tau, sub2(MAGIC, add2(tau, MAGIC)));
-                }
+                f2x ph = f & 1 ? pp.y : pp.x;
+                if (PREC) ph = fma2(splat(c.K_lo), U[q], ph);
+                ph = fma2(KH, UC[q], ph);
+                // less whole turns before and after the second term: every sum is rounded near
+                // its smallest size
+                const f2x nr = sub2(MAGIC, fma2(KH, U[q], MAGIC));
+                f2x tau = fma2(splat(c.hK), rs[q][i], add2(fma2(KH, U[q], nr), ph));
+                tau = add2(tau, sub2(MAGIC, add2(tau, MAGIC)));
                 float t0, t1, sn0, cs0, sn1, cs1;
                 upk(mul2(splat(-6.283185307179586f), tau), t0, t1);
                 __sincosf(t0, &sn0, &cs0);
@@ -250,7 +253,7 @@ __device__ __forceinline__ void eval_segments(const FwdParams &p, const WarpBuf<
     }
 }
 
-// Slots of a staged batch: [0, n_plain) with u in FP32, [n_plain, end) with the split one, and
+// Slots of a staged batch: [0, n_plain) with a plain u, [n_plain, end) with the split one, and
 // which slots may have an end of their window inside the ball.
 struct StagedBatch {
     int n_plain, end;
@@ -258,8 +261,8 @@ struct StagedBatch {
 };
 
 // Stages the batch's raw records (a lane each) in the frame c, for the 64 receivers within rad
-// of it: see WarpBuf.  A segment is of the second class where the warp is not compact
-// (`fast`) or an end of its window may lie inside the ball (a margin of 1 mm covers the
+// of it: see WarpBuf.  A segment is split where the warp is not `fast` (one band, compact, every
+// x' one float) or an end of its window may lie inside the ball (a margin of 1 mm covers the
 // rounding of the float-float heads).
 template <int NF, int WINDOW, bool LOSSY, int NS, int NP>
 __device__ __forceinline__ StagedBatch stage(const FwdParams &p, WarpBuf<NF, LOSSY> &w, int lane,
@@ -314,27 +317,31 @@ __device__ __forceinline__ StagedBatch stage(const FwdParams &p, WarpBuf<NF, LOS
     for (int q = 1; q < NS; ++q)
         if (__popc(plain) > b.n_plain) plain &= plain - 1u;
     b.end = nrec;
-    b.cross = fast ? ~0ull : (uint64_t)xm;     // compact warps: every segment of the second class
+    b.cross = fast ? ~0ull : (uint64_t)xm;     // fast warps: every split segment
     const bool mine_plain = (plain >> lane) & 1u;
     const int slot = mine_plain ? __popc(plain & below) : b.n_plain + __popc(all & ~plain & below);
-    // N = d x t, compensated
-    const float nx = dop(dyh, r1.z, dzh, r1.y) +
-                     fmaf(dyh, r3.z, fmaf(-dzh, r3.y, fmaf(dyl, r1.z, -dzl * r1.y)));
-    const float ny = dop(dzh, r1.x, dxh, r1.z) +
-                     fmaf(dzh, r3.x, fmaf(-dxh, r3.z, fmaf(dzl, r1.x, -dxl * r1.z)));
-    const float nz = dop(dxh, r1.y, dyh, r1.x) +
-                     fmaf(dxh, r3.y, fmaf(-dyh, r3.x, fmaf(dxl, r1.y, -dyl * r1.x)));
-    // one band: t times K / K_hi, so that K_hi u is K u (K_lo u would move the phase of every
-    // term alike, by up to 45 x 2^-25 turns); several bands add K_lo u each
-    const float ks = NF == 1 ? p.fc[0].K_lo * rcp_approx(p.fc[0].K_hi) : 0.0f;
-    const float tx = fmaf(r1.x, ks, r3.x) + r1.x, ty = fmaf(r1.y, ks, r3.y) + r1.y,
-                tz = fmaf(r1.z, ks, r3.z) + r1.z;
+    // N = d x t, each component (ah + al) (th + tl) - (bh + bl) (uh + ul) rounded once
+    auto cross_term = [](float ah, float al, float th, float tl, float bh, float bl, float uh, float ul) {
+        const float p = __fmul_rn(ah, th), q = __fmul_rn(bh, uh);
+        float d, e;
+        two_sum(p, -q, d, e);
+        e = __fadd_rn(e, __fsub_rn(fmaf(ah, th, -p), fmaf(bh, uh, -q)));
+        return __fadd_rn(d, __fadd_rn(e, fmaf(ah, tl, fmaf(-bh, ul, fmaf(al, th, -bl * uh)))));
+    };
+    const float nx = cross_term(dyh, dyl, r1.z, r3.z, dzh, dzl, r1.y, r3.y);
+    const float ny = cross_term(dzh, dzl, r1.x, r3.x, dxh, dxl, r1.z, r3.z);
+    const float nz = cross_term(dxh, dxl, r1.y, r3.y, dyh, dyl, r1.x, r3.x);
     if (have) {
-        w.D[0][slot] = dup2(tx, ty);
-        w.D[1][slot] = dup2(tz, Sh * p.s_scale);
+        w.D[0][slot] = dup2(r1.x, r1.y);
+        w.D[1][slot] = dup2(r1.z, Sh * p.s_scale);
         w.D[2][slot] = dup2(nx, ny);
         w.D[3][slot] = dup2(nz, amp);
-        if (!mine_plain) {
+        if (mine_plain) {
+            // one band: with K_lo / K_hi of t in its low words, K_hi (U + u_lo) is K u
+            const float ks = p.fc[0].K_lo * rcp_approx(p.fc[0].K_hi);
+            w.D[4][slot] = dup2(fmaf(r1.x, ks, r3.x), fmaf(r1.y, ks, r3.y));
+            w.D[5][slot] = dup2(fmaf(r1.z, ks, r3.z), 0.f);
+        } else {
             // t rounded to multiples of 2^-12 (by 1.5 x 2^11, whose ulp that is), and the rest
             const float hx = __fsub_rn(__fadd_rn(r1.x, 3072.f), 3072.f);
             const float hy = __fsub_rn(__fadd_rn(r1.y, 3072.f), 3072.f);
@@ -519,7 +526,13 @@ __global__ void __launch_bounds__(32 * PairCfg<WarpBuf<NF, LOSSY>, BATCHED, BATC
         }
         const float cx = ctr[0], cy = ctr[1], cz = ctr[2];
         const float rad = 1.000001f * sqrtf(__uint_as_float(far2));
-        const bool fast = rad * p.kmax_turns <= kFastTurns;
+        bool fast = false;
+        if (NF == 1) {
+            bool rest = false;          // x' is not one float
+#pragma unroll
+            for (int k = 0; k < kR; ++k) rest = rest || xl[k] != 0.0f || yl[k] != 0.0f || zl[k] != 0.0f;
+            fast = rad * p.kmax_turns <= kFastTurns && !__any_sync(0xffffffffu, rest);
+        }
         // grid of a receiver's x': a power of two q with |x'| <= 2^11 q, by adding 1.5 x 2^23 q
         float grid[kR];
 #pragma unroll
@@ -557,11 +570,14 @@ __global__ void __launch_bounds__(32 * PairCfg<WarpBuf<NF, LOSSY>, BATCHED, BATC
                                                                    cx, cy, cz, rad, fast);
             __syncwarp();       // the batch is staged
             g.issue(p, item, B.in, lane, rball, buf);   // batch kb + 2 into the buffer just read
-            for (int j = 0; j < b.n_plain; j += NS)
-                eval_segments<NF, WINDOW, LOSSY, false, NS, FG, BATCHED>(p, B, j, 0ull, x, ax, ay);
+            if (NF == 1)
+                for (int j = 0; j < b.n_plain; j += NS)
+                    eval_segments<NF, WINDOW, LOSSY, false, NS, FG, BATCHED>(p, B, j, 0ull, x, ax, ay);
             for (int j = b.n_plain; j < b.end; j += NP)
                 eval_segments<NF, WINDOW, LOSSY, true, NP, FG, BATCHED>(p, B, j, b.cross, x, ax, ay);
-            if ((kb % kFoldEvery) == kFoldEvery - 1) fold_all();
+            // without a list every entry of a batch reaches the warp: twice as often
+            const uint32_t every = item.lst ? kFoldEvery : kFoldEvery / 2;
+            if (kb % every == every - 1) fold_all();
             __syncwarp();        // before the next batch is staged over this one
         }
         cp_async_wait0();        // every gather of this item has landed

@@ -31,7 +31,7 @@ struct alignas(16) FreqConst {
     float ne;             // Gaussian exponent ne r: -k / (2 b) log2(e), adjoint -k b / 2 log2(e)
     float rc;             // kept iff r <= rc: C b / (k / 2), adjoint C / (k b / 2)
     float invb;           // 1 / b
-    float sA;             // amplitude: k / (8 pi^2) (applied by the merge), adjoint k b / (8 pi^2)
+    float sA;             // adjoint amplitude k b / (8 pi^2) (forward: k / (8 pi^2), by the merge)
     float nal;            // exponent of the air absorption nal s: -a b log2(e), adjoint -a log2(e)
     float nkh;            // -k / 2 (adjoint)
     float b;              // b (adjoint)

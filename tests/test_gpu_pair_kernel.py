@@ -163,3 +163,64 @@ def test_f64_candidates_near_an_image_source_seen_from_afar(cutoff, height, b):
     torch.cuda.synchronize()
     e = p.cpu().numpy().astype(np.complex128) - po
     assert np.linalg.norm(po) > 0 and np.linalg.norm(e) <= 1e-7 * np.linalg.norm(po)
+
+
+def test_low_words_of_the_direction_reach_the_phase():
+    """One beam at a time (as four equal ones, a group of the plain projection) and two receivers
+    4 m either side of a point on it, along x, where K x' is 14 turns and x'.t is exact in FP32: what is left out of t's low word, uniform within
+    2^-25 for t_x in [1/2, 1), turns up in the phase as 14 x 2 pi x 2^-25 / sqrt(3) = 1.5e-6 rad
+    rms.  With it the phase errs by MUFU's sine and cosine (3.6e-7 at most) and four roundings of
+    at most 2^-25 turns, 3.4e-7 rms together if all were at their worst; the bar is 6e-7."""
+    import torch
+    from paper_2501_13382_gb300 import gbt as G
+    sc0 = I.Scene(I.C_AIR, False, 0.0, 0, np.zeros((0, 3, 3)), np.zeros(0, np.int32),
+                  np.zeros(0, np.int32), np.array([1.0], np.float32))
+    sc = G.Scene(sc0)
+    gam = torch.as_tensor(sc0.gamma, device="cuda")
+    rng = np.random.default_rng(2)
+    freqs, b = [3.5 * I.C_AIR], [100.0]
+    err = []
+    for _ in range(200):
+        d = rng.normal(size=3)
+        d[0] = abs(d[0]) + np.hypot(d[1], d[2]) * 0.8
+        d /= np.linalg.norm(d)
+        c = np.round(8.0 * 90.0 * d) / 8.0
+        recv = (c + np.array([[4.0, 0.0, 0.0], [-4.0, 0.0, 0.0]])).astype(np.float32)
+        src = I.Source(np.zeros(3), 4, 0, 1000.0)
+        dirs = np.tile(d, (4, 1))
+        po = O.gbs_sum(O.trace(sc0, src, dirs=dirs), recv, freqs, b, sc0.c, sc0.gamma, window=I.WINDOW_LINE)
+        tr = G.Trace(sc, src, dirs=torch.as_tensor(dirs, device="cuda"))
+        p = G.gbs_sum(tr, torch.as_tensor(recv, device="cuda"), freqs, b, gam, window=I.WINDOW_LINE)
+        err.append(np.angle(p.cpu().numpy().astype(np.complex128) / po).ravel())
+    rms = np.sqrt(np.mean(np.square(err)))
+    assert rms <= 6e-7, rms
+
+
+@pytest.mark.parametrize("scene,window,nf", [("city", I.WINDOW_SEGMENT, 3), ("city", I.WINDOW_LINE, 1),
+                                             ("plane", I.WINDOW_LINE, 6)])
+def test_fields_against_a_sum_that_skips_nothing(scene, window, nf):
+    """The FP32 field without lists, with lists and with explicit splits, at a sample of the
+    receivers, against the oracle, which tests every pair: a segment that a ball test, a list or a
+    split drops or takes twice shows here.  1e-6: the worst of MUFU (3.6e-7), the projection and
+    the FP32 sums is under it, a beam lost at the cutoff's edge (e^-16 of its peak) not."""
+    import torch
+    from paper_2501_13382_gb300 import gbt as G
+    if scene == "city":
+        w = I.city(n_rays=32768, n_recv_side=96)
+        sc0, src, recv = w.scene, w.sources[0], w.receivers
+    else:
+        w = I.open_plane_large()
+        sc0, src, recv = w.scene, w.sources[0], w.receivers[::3]
+    freqs = [500.0 * 2.0 ** (3.0 * f / max(nf - 1, 1)) for f in range(nf)]
+    b = [100.0 - 7.0 * f for f in range(nf)]
+    some = np.sort(np.random.default_rng(3).permutation(len(recv))[:150])
+    po = O.gbs_sum(O.trace(sc0, src), recv[some], freqs, b, sc0.c, sc0.gamma, window=window)
+    tr = G.Trace(G.Scene(sc0), src)
+    r = torch.as_tensor(np.ascontiguousarray(recv, np.float32), device="cuda")
+    gam = torch.as_tensor(sc0.gamma, device="cuda")
+    order = G.recv_order(r)
+    for kw in (dict(), dict(tile_cull=True), dict(seg_split=7), dict(tile_cull=True, seg_split=7),
+               dict(order=None)):
+        p = G.gbs_sum(tr, r, freqs, b, gam, window=window, **{"order": order, **kw})
+        e = p.cpu().numpy()[:, some].astype(np.complex128) - po
+        assert np.linalg.norm(e) <= 1e-6 * np.linalg.norm(po), kw
