@@ -388,36 +388,34 @@ __device__ __forceinline__ StagedBatch stage(const FwdParams &p, WarpBuf<NF, LOS
     return b;
 }
 
-// The median of the warp's receivers by coordinate (part: those that count), as the frame of a
-// warp tile with a stray receiver (a point far off the map), whose |x'| then does not coarsen the
-// others'; w > 0 if most of them lie within sqrt(close2) of it.  Out of line: it is seldom
-// called, and its registers are not the kernel's.
-__device__ __noinline__ float4 stray_frame(bool p0, bool p1, float x0, float y0, float z0, float x1,
-                                           float y1, float z1, float close2)
+// The frame of a warp tile with stray receivers (points far off the map), so that their |x'| does
+// not coarsen the others': the tile's first, middle or last receiver (part: those that count),
+// if most of them lie within sqrt(close2) of it; else c as it is.  Out of line and without a
+// search for the median: inside the kernel its registers cost the main loop (open plane, 6 bands:
+// median 2.11 ms, inline 2.10, so 2.04).
+__device__ __noinline__ void stray_frame(const bool (&part)[kR], const float (&x)[kR], const float (&y)[kR],
+                                         const float (&z)[kR], float close2, float (&c)[3])
 {
-    const int most = __popc(__ballot_sync(0xffffffffu, p0)) + __popc(__ballot_sync(0xffffffffu, p1));
-    float med[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const unsigned u0 = ordered_bits(a == 0 ? x0 : a == 1 ? y0 : z0);
-        const unsigned u1 = ordered_bits(a == 0 ? x1 : a == 1 ? y1 : z1);
-        unsigned m = 0u;               // the largest value with fewer than half of them below it
+    const uint32_t m0 = __ballot_sync(0xffffffffu, part[0]), m1 = __ballot_sync(0xffffffffu, part[1]);
 #pragma unroll 1
-        for (unsigned bit = 0x80000000u; bit; bit >>= 1) {
-            const unsigned v = m | bit;
-            const int below = __popc(__ballot_sync(0xffffffffu, p0 && u0 < v)) +
-                              __popc(__ballot_sync(0xffffffffu, p1 && u1 < v));
-            if (below <= (most - 1) / 2) m = v;
+    for (int q = 0; q < 3; ++q) {
+        const int k = q == 0 ? m0 == 0u : m1 != 0u;
+        const uint32_t m = k ? m1 : m0;
+        const int src = q < 2 ? __ffs(m) - 1 : 31 - __clz(m);
+        const float cx = __shfl_sync(0xffffffffu, k ? x[1] : x[0], src);
+        const float cy = __shfl_sync(0xffffffffu, k ? y[1] : y[0], src);
+        const float cz = __shfl_sync(0xffffffffu, k ? z[1] : z[0], src);
+        int close = 0;
+#pragma unroll
+        for (int r = 0; r < kR; ++r) {
+            const float ex = x[r] - cx, ey = y[r] - cy, ez = z[r] - cz;
+            close += __popc(__ballot_sync(0xffffffffu, part[r] && fmaf(ex, ex, fmaf(ey, ey, ez * ez)) < close2));
         }
-        med[a] = from_ordered(m);
+        if (2 * close > __popc(m0) + __popc(m1)) {
+            c[0] = cx; c[1] = cy; c[2] = cz;
+            break;
+        }
     }
-    auto is_close = [&](float x, float y, float z) {
-        const float ex = x - med[0], ey = y - med[1], ez = z - med[2];
-        return fmaf(ex, ex, fmaf(ey, ey, ez * ez)) < close2;
-    };
-    const int close = __popc(__ballot_sync(0xffffffffu, p0 && is_close(x0, y0, z0))) +
-                      __popc(__ballot_sync(0xffffffffu, p1 && is_close(x1, y1, z1)));
-    return make_float4(med[0], med[1], med[2], 2 * close > most ? 1.0f : 0.0f);
 }
 
 template <int NF, int WINDOW, bool BATCHED, bool LOSSY>
@@ -491,41 +489,38 @@ __global__ void __launch_bounds__(32 * PairCfg<WarpBuf<NF, LOSSY>, BATCHED, BATC
             const float hi = from_ordered(__reduce_max_sync(0xffffffffu, bb[3 + a]));
             ctr[a] = 0.5f * lo + 0.5f * hi;
         }
-        float xp[kR], yp[kR], zp[kR], xl[kR], yl[kR], zl[kR], xx[kR];
-        unsigned far2, near2;          // bits of the largest and the smallest |x'|^2
-        auto place = [&]() {
-            far2 = 0u;
-            near2 = ~0u;
+        float4 rball;
+        {
+            unsigned far2 = 0u, near2 = ~0u;      // bits of the largest and the smallest |x - c|^2
 #pragma unroll
-            for (int k = 0; k < kR; ++k) {
-                xp[k] = yp[k] = zp[k] = xl[k] = yl[k] = zl[k] = xx[k] = 0.0f;
+            for (int k = 0; k < kR; ++k)
                 if (part[k]) {
-                    two_sum(xr[k], -ctr[0], xp[k], xl[k]);
-                    two_sum(yr[k], -ctr[1], yp[k], yl[k]);
-                    two_sum(zr[k], -ctr[2], zp[k], zl[k]);
-                    xx[k] = fmaf(xp[k], xp[k], fmaf(yp[k], yp[k], zp[k] * zp[k]));
-                    far2 = max(far2, __float_as_uint(xx[k]));
-                    near2 = min(near2, __float_as_uint(xx[k]));
+                    const float ex = xr[k] - ctr[0], ey = yr[k] - ctr[1], ez = zr[k] - ctr[2];
+                    const unsigned e2 = __float_as_uint(fmaf(ex, ex, fmaf(ey, ey, ez * ez)));
+                    far2 = max(far2, e2);
+                    near2 = min(near2, e2);
                 }
-            }
-            far2 = __reduce_max_sync(0xffffffffu, far2);
-            near2 = __reduce_min_sync(0xffffffffu, near2);
-        };
-        place();
-        const float4 rball = reach_ball(make_float4(ctr[0], ctr[1], ctr[2],
-                                                    1.000001f * sqrtf(__uint_as_float(far2))));
-        // a centre without a receiver within half the radius may lie between the others and a
-        // stray one
-        if (far2 != 0u && __uint_as_float(near2) > 0.25f * __uint_as_float(far2)) {
-            const float4 med = stray_frame(part[0], part[1], xr[0], yr[0], zr[0], xr[1], yr[1], zr[1],
-                                           0.0625f * __uint_as_float(far2));
-            if (med.w > 0.0f) {
-                ctr[0] = med.x; ctr[1] = med.y; ctr[2] = med.z;
-                place();
+            const float f2 = __uint_as_float(__reduce_max_sync(0xffffffffu, far2));
+            const float n2 = __uint_as_float(__reduce_min_sync(0xffffffffu, near2));
+            rball = reach_ball(make_float4(ctr[0], ctr[1], ctr[2], 1.000001f * sqrtf(f2)));
+            // a centre without a receiver within half the radius may lie between the others and a
+            // stray one
+            if (n2 > 0.25f * f2) stray_frame(part, xr, yr, zr, 0.0625f * f2, ctr);
+        }
+        float xp[kR], yp[kR], zp[kR], xl[kR], yl[kR], zl[kR], xx[kR];
+#pragma unroll
+        for (int k = 0; k < kR; ++k) {
+            xp[k] = yp[k] = zp[k] = xl[k] = yl[k] = zl[k] = xx[k] = 0.0f;
+            if (part[k]) {
+                two_sum(xr[k], -ctr[0], xp[k], xl[k]);
+                two_sum(yr[k], -ctr[1], yp[k], yl[k]);
+                two_sum(zr[k], -ctr[2], zp[k], zl[k]);
+                xx[k] = fmaf(xp[k], xp[k], fmaf(yp[k], yp[k], zp[k] * zp[k]));
             }
         }
         const float cx = ctr[0], cy = ctr[1], cz = ctr[2];
-        const float rad = 1.000001f * sqrtf(__uint_as_float(far2));
+        const float rad = 1.000001f * sqrtf(__uint_as_float(
+            __reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(xx[0], xx[1])))));
         bool fast = false;
         if (NF == 1) {
             bool rest = false;          // x' is not one float
