@@ -2052,6 +2052,12 @@ int choose_splits(const TraceDev &td, const gbt_sum_args &a, bool adjoint)
         const int64_t tiles = (a.n_recv + 31) / 32;
         int64_t s = (512 * (int64_t)num_sms() + tiles - 1) / (tiles > 0 ? tiles : 1);
         s = std::max<int64_t>(1, std::min<int64_t>(s, (nseg_est + 2 * kBatch - 1) / (2 * kBatch)));
+        // partial sums stay under 1 GiB, and under an eighth of a solve's budget (40 MB a band
+        // without one, and two chunks may hold them)
+        const int64_t room = a.max_device_bytes > 0 ? std::min<int64_t>(1LL << 30, a.max_device_bytes / 8)
+                                                    : 1LL << 30;
+        const int64_t per_split = (int64_t)a.n_freq * std::max<int64_t>(a.n_recv, 1) * (int64_t)sizeof(double2);
+        s = std::min<int64_t>(s, std::max<int64_t>(1, room / per_split));
         return (int)std::min<int64_t>(s, 4096);
     }
     // items are (warp tile, split): about 16 per resident warp, so that the last items to

@@ -139,3 +139,42 @@ def test_synthesis_rejects_bad_arguments_on_host(lib):
     for nf, n_t in ((0, 10), (17, 10), (4, 0), (4, (1 << 20) + 1)):
         assert lib.gbt_synthesize(None, nf, 0, fr, am, 0.0, 1e-4, n_t, None, 0, None) == 1
     assert lib.gbt_synthesize(None, 4, 10, fr, am, 0.0, 1e-4, 10, None, 0, None) == 1   # NULL p
+
+
+@pytest.mark.gpu
+def test_f64_solve_stays_within_its_budget(lib):
+    """A solve's device budget also bounds the FP64 sum's partials (40 MB a band without one):
+    what the library holds at once, of a fan that is one chunk, is under the budget; and the
+    field is the same but for the rounding of FP64 sums in other groups (complex64: 1e-7)."""
+    import torch
+    w = I.open_plane_small()
+    r = torch.as_tensor(w.receivers[:1500].copy(), device="cuda")
+    gam = torch.as_tensor(w.scene.gamma, device="cuda")
+    freqs, b = [100.0 * (f + 1) for f in range(16)], [50.0] * 16
+    sc, src = G.Scene(w.scene), I.Source(np.array([0.0, 0.0, 2.0]), 16384, 2, 200.0)
+    budget, held, most, got = 32 << 20, {}, [0], []
+    for limit in (0, budget):
+        out = torch.zeros((16, len(r)), dtype=torch.complex64, device="cuda")
+        a = G.sum_args(r, freqs, b, gam, out, window=I.WINDOW_LINE, precision=G.PRECISION_F64)
+        a.max_device_bytes = limit
+        most[0] = 0
+
+        def alloc(n, stream):
+            buf = torch.empty(max(n, 1), dtype=torch.uint8, device="cuda")
+            held[buf.data_ptr()] = buf
+            most[0] = max(most[0], sum(v.numel() for v in held.values()))
+            return buf.data_ptr()
+
+        def free(ptr, stream):
+            torch.cuda.synchronize()
+            held.pop(ptr, None)
+
+        G.gbt_set_allocator(alloc, free)
+        try:
+            G.gbt_solve(sc.handle, G.source_desc(src), a, torch.cuda.current_stream().cuda_stream)
+            torch.cuda.synchronize()
+        finally:
+            G.gbt_set_allocator(None)
+        got.append(out)
+    assert 0 < most[0] <= budget
+    assert float((got[0] - got[1]).norm()) <= 1e-7 * float(got[0].norm())
