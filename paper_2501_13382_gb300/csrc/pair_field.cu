@@ -1,9 +1,10 @@
 // pair_field.cu -- the forward sum that the adjoint differentiates (gbt_sum_differentiable).
 //
 // A least-squares gradient depends on the field's rounding, so this kernel evaluates each
-// beam as the adjoint kernel (pair_bwd.cu) does, operation for operation, and sums in the
-// same order and groups whether or not the pre-cull is on: the field does not depend on how
-// the segments that reach nobody are skipped.
+// beam as the adjoint kernel (pair_bwd.cu) does, operation for operation.  Without lists its
+// FP32 sums fold every 16 chunks of all segments, whichever of them reach the warp; with lists
+// every 16 batches of the tile's own entries, and splits stride chunks of the list.  So a call
+// repeats to the bit, and the two forms differ by the rounding of regrouped sums.
 //
 // Same items and gathering as the forward kernel of pair.cuh: a warp goes through the
 // segments whose beams reach its ball.  Each is evaluated for the lane's two receivers in
@@ -330,7 +331,7 @@ __device__ __forceinline__ void eval_field(const FwdParams &p, const FieldBuf<NF
 }
 
 // The FP32 sums fold into the item's float-float partials every kFoldEvery batches of list
-// entries (without a list, of all segments).
+// entries, or without a list every kFoldEvery chunks of all segments.
 template <int NF, int WINDOW, bool LOSSY>
 __global__ void __maxnreg__(128) gbs_field_kernel(const __grid_constant__ FwdParams p)
 {

@@ -224,3 +224,58 @@ def test_fields_against_a_sum_that_skips_nothing(scene, window, nf):
         p = G.gbs_sum(tr, r, freqs, b, gam, window=window, **{"order": order, **kw})
         e = p.cpu().numpy()[:, some].astype(np.complex128) - po
         assert np.linalg.norm(e) <= 1e-6 * np.linalg.norm(po), kw
+
+
+@pytest.mark.parametrize("nf,n", [(1, 700), (3, 1930)])
+def test_differentiable_sum_repeats_and_regroups(nf, n):
+    """The differentiable sum repeats to the bit, with lists and without; the two differ by the
+    rounding of FP32 sums in other groups of at most 512 terms, at random: 1e-6."""
+    import torch
+    from paper_2501_13382_gb300 import gbt as G
+    sc0, _ = I.city_scene(I.SEED_BASE + 3)
+    src = I.Source(np.array([0.3, -0.2, 3.0]), 3000, 4, 600.0)
+    freqs = list(250.0 * 2.0 ** np.arange(nf))
+    tr = G.Trace(G.Scene(sc0), src)
+    r = torch.as_tensor(_receivers("scatter", n, 5), device="cuda")
+    gam = torch.as_tensor(sc0.gamma, device="cuda")
+    kw = dict(order=G.recv_order(r), window=I.WINDOW_SEGMENT)
+    a, b, c, d = (G.gbs_sum_differentiable(tr, r, freqs, [40.0] * nf, gam, tile_cull=cull, **kw)
+                  for cull in (False, False, True, True))
+    assert torch.equal(a, b) and torch.equal(c, d)
+    assert float((a - c).norm()) <= 1e-6 * float(a.norm())
+
+
+@pytest.mark.parametrize("kind,n,rays,nf,uniform,window", [
+    ("compact", 1, 257, 1, True, I.WINDOW_SEGMENT),
+    ("compact", 65, 301, 3, False, I.WINDOW_LINE),
+    ("compact", 959, 500, 1, True, I.WINDOW_SEGMENT),
+    ("compact", 961, 333, 6, False, I.WINDOW_SEGMENT),
+    ("scatter", 64, 1023, 1, True, I.WINDOW_SEGMENT),
+    ("scatter", 961, 512, 5, True, I.WINDOW_LINE),
+    ("scatter", 1921, 400, 8, True, I.WINDOW_SEGMENT),
+    ("scatter", 130, 900, 7, False, I.WINDOW_SEGMENT),
+])
+def test_forward_field_to_a_few_roundings(kind, n, rays, nf, uniform, window):
+    """The forward sum at edges of its tiles and band slots, with lists, splits by list length
+    and equal splits, far under the bar of the differentiable sum.  A term's phase errs by MUFU
+    (3.6e-7) and some six roundings of 2^-25 turns (1.1e-6 rad), its amplitude by 6e-7 (ex2, rcp):
+    2e-6 at worst, which mild cancellation of terms may double; 5e-6.  One band on a compact warp
+    adds 3 x 2^-24 x 8 turns at worst, 9e-6 rad, independently from term to term."""
+    import torch
+    from paper_2501_13382_gb300 import gbt as G
+    sc0, _ = I.city_scene(I.SEED_BASE + 3)
+    src = I.Source(np.array([0.3, -0.2, 3.0]), rays, 4, 600.0)
+    recv = _receivers(kind, n, rays)
+    freqs = list(125.0 * 2.0 ** (np.arange(nf) * (5.0 / max(nf - 1, 1))))[::-1]
+    b = [40.0] * nf if uniform else [20.0 + 9.0 * f for f in range(nf)]
+    po = O.gbs_sum(O.trace(sc0, src), recv, freqs, b, sc0.c, sc0.gamma, window=window)
+    tr = G.Trace(G.Scene(sc0), src)
+    r = torch.as_tensor(recv, device="cuda")
+    gam = torch.as_tensor(sc0.gamma, device="cuda")
+    for kw in (dict(), dict(tile_cull=True), dict(tile_cull=True, seg_split=3)):
+        p = G.gbs_sum(tr, r, freqs, b, gam, order=G.recv_order(r), window=window, **kw)
+        out = torch.ones_like(p)
+        G.gbs_sum(tr, r, freqs, b, gam, order=G.recv_order(r), window=window, out=out, accumulate=True, **kw)
+        for q, ref in ((p, po), (out, po + 1.0)):
+            e = q.cpu().numpy().astype(np.complex128) - ref
+            assert np.linalg.norm(e) <= 5e-6 * np.linalg.norm(ref), kw
