@@ -27,6 +27,7 @@ SOURCES = {
     "trace.cu": ["--fmad=false"],
     "gbs.cu": [],
     "pair_fwd.cu": [],
+    "pair_unordered.cu": [],
     "pair_field.cu": [],
     "pair_bwd.cu": [],
     "pair_batched.cu": [],

@@ -9,7 +9,8 @@
 //    once and gathers the entries whose bit is set;
 //  * no list: the warp tests the 32-byte cull records of four chunks of 32 segments at a
 //    time against its ball.  About 35 instructions per 32 segments, where a test of every
-//    (receiver, segment) pair took 15 per segment.
+//    (receiver, segment) pair took 15 per segment.  That test comes back for receivers that
+//    have no order either (kSmallBeam).
 // Gathered records arrive by per-lane cp.async, double buffered, and each lane stages one.
 //
 // What bounds it: operand reads.  On this chip an FFMA2 with three operand pairs of its own
@@ -62,6 +63,16 @@ namespace {
 // 1M-ray city takes 21.8 ms instead of 20.2, at an error of 1.24e-7 instead of 1.26e-7.
 constexpr float kFastTurns = 16.0f;
 
+// Receivers without an order and without lists: a warp tile's 64 may lie anywhere, nearly every
+// segment reaches its ball and keeps a few of them.  A segment is small if its union cutoff radius
+// at the tile is under kSmallBeam times the ball's radius; where most of a batch are, may_keep marks
+// candidates and every receiver evaluates its own, a slot of its own to each lane and half.
+// 65,536-ray city x 10,000 scattered x 2 bands: every segment for all 64 5.38 ms, so 3.86; 8 bands
+// 10.0, 6.87 (line at 0.5: 8.6, at 1 to 1e6 the same); rows of a 200^2 grid 9.26, 6.15; rows of
+// the 256^2 open plane, 6 bands 4.93, 4.64.  The candidates' loop unrolled 1, 2, 4, 8 times: 8 bands
+// 7.03, 6.92, 6.87, 7.92.  Ordered receivers have kernels of their own without this (registers).
+constexpr float kSmallBeam = 1.0f;
+
 // Shape by the number of band slots: segments evaluated together (plain, which only one band has,
 // and split), bands per vote, and warps.  One band needs several segments for independent
 // chains and shared operands (1M-ray city step: one segment, 16 warps 27.4 ms; two 26.0;
@@ -101,24 +112,40 @@ struct LaneRecv {
     f2x X, Y, Z, NX, NY, NZ, XH, YH, ZH, XL, YL, ZL;
 };
 
+// A staged word's two values as float pairs: of slot j, or (EACH) of slot j for the lane's first
+// receiver and j1 for its second.
+template <bool EACH>
+__device__ __forceinline__ void staged(const float4 *w, int j, int j1, f2x &a, f2x &b)
+{
+    if (EACH) {
+        const float4 u = w[j], v = w[j1];
+        a = pk(u.x, v.x);
+        b = pk(u.z, v.z);
+    } else {
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(w + j);
+        a = v.x;
+        b = v.y;
+    }
+}
+
 // Adds the beams of the staged slots j .. j + NS - 1 to the lane's two receivers' sums per
-// band.  `cross`: slots with an end of their window inside the warp tile's ball.
-template <int NF, int WINDOW, bool LOSSY, bool PREC, int NS, int FG, bool BATCHED>
+// band.  `cross`: slots with an end of their window inside the warp tile's ball.  EACH: of a slot
+// of its own to each receiver (j and j1; h0, h1: whether it has one).
+template <int NF, int WINDOW, bool LOSSY, bool PREC, int NS, int FG, bool BATCHED, bool EACH = false>
 __device__ __forceinline__ void eval_segments(const FwdParams &p, const WarpBuf<NF, LOSSY> &w,
                                               int j, uint64_t cross, const LaneRecv &x,
-                                              f2x (&ax)[NF], f2x (&ay)[NF])
+                                              f2x (&ax)[NF], f2x (&ay)[NF], int j1 = 0,
+                                              bool h0 = true, bool h1 = true)
 {
+    static_assert(!EACH || (PREC && NS == 1), "slots apart are split ones, one at a time");
     const f2x MAGIC = splat(12582912.0f), ONE = splat(1.0f);
     f2x U[NS], UC[NS], s[NS], nn[NS], amp[NS];
     bool k0[NS], k1[NS];
-    auto word = [&](int d, int q, f2x &a, f2x &b) {
-        const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(&w.D[d][j + q]);
-        a = v.x;
-        b = v.y;
-    };
+    auto word = [&](int d, int q, f2x &a, f2x &b) { staged<EACH>(w.D[d], j + q, j1, a, b); };
 #pragma unroll
     for (int q = 0; q < NS; ++q) {
-        k0[q] = k1[q] = true;
+        k0[q] = h0;
+        k1[q] = h1;
         f2x TX, TY, TZ, S, NX, NY, NZ;
         word(0, q, TX, TY);
         word(1, q, TZ, S);
@@ -134,14 +161,14 @@ __device__ __forceinline__ void eval_segments(const FwdParams &p, const WarpBuf<
             UC[q] = fma2(x.XL, TX, fma2(x.YL, TY, fma2(x.ZL, TZ,
                     fma2(x.XH, LX, fma2(x.YH, LY, mul2(x.ZH, LZ))))));
             u = add2(U[q], UC[q]);
-            if ((cross >> (j + q)) & 1u) {
-                const float4 e = w.W[j + q];
+            if (EACH || ((cross >> (j + q)) & 1u)) {
+                const float4 e = w.W[j + q], o = EACH ? w.W[j1] : e;
                 float a0, a1;
-                upk(add2(add2(splat(e.x), U[q]), add2(splat(e.y), UC[q])), a0, a1);
-                k0[q] = a0 >= 0.0f;
-                k1[q] = a1 >= 0.0f;
+                upk(add2(add2(pk(e.x, o.x), U[q]), add2(pk(e.y, o.y), UC[q])), a0, a1);
+                k0[q] = k0[q] && a0 >= 0.0f;
+                k1[q] = k1[q] && a1 >= 0.0f;
                 if (WINDOW == GBT_WINDOW_SEGMENT) {
-                    upk(add2(add2(splat(e.z), U[q]), add2(splat(e.w), UC[q])), a0, a1);
+                    upk(add2(add2(pk(e.z, o.z), U[q]), add2(pk(e.w, o.w), UC[q])), a0, a1);
                     k0[q] = k0[q] && a0 < 0.0f;
                     k1[q] = k1[q] && a1 < 0.0f;
                 }
@@ -221,11 +248,14 @@ __device__ __forceinline__ void eval_segments(const FwdParams &p, const WarpBuf<
             const FreqConst &c = BATCHED ? cs : p.fc[f];
 #pragma unroll
             for (int q = 0; q < NS; ++q) {
-                const ulonglong2 pp = *reinterpret_cast<const ulonglong2 *>(&w.F[f / 2][j + q]);
+                f2x ph, pq;
+                staged<EACH>(w.F[f / 2], j + q, j1, ph, pq);
+                if (f & 1) ph = pq;
                 f2x g = AD[q][i];
                 if (LOSSY) {
-                    const ulonglong2 ra = *reinterpret_cast<const ulonglong2 *>(&w.R[f / 2][j + q]);
-                    g = mul2(f & 1 ? ra.y : ra.x, g);
+                    f2x ra, rb;
+                    staged<EACH>(w.R[f / 2], j + q, j1, ra, rb);
+                    g = mul2(f & 1 ? rb : ra, g);
                 }
                 f2x ex = mul2(splat(c.ne), r[q][i]);
                 if (LOSSY) ex = fma2(splat(c.nal), sc[q][i], ex);
@@ -233,7 +263,6 @@ __device__ __forceinline__ void eval_segments(const FwdParams &p, const WarpBuf<
                 upk(ex, e0, e1);
                 g = mul2(g, pk(m0[q][i] ? ex2_approx(e0) : 0.0f, m1[q][i] ? ex2_approx(e1) : 0.0f));
                 const f2x KH = splat(c.K_hi);
-                f2x ph = f & 1 ? pp.y : pp.x;
                 if (PREC) ph = fma2(splat(c.K_lo), U[q], ph);
                 ph = fma2(KH, UC[q], ph);
                 // less whole turns before and after the second term: every sum is rounded near
@@ -253,18 +282,52 @@ __device__ __forceinline__ void eval_segments(const FwdParams &p, const WarpBuf<
     }
 }
 
+// Whether the staged (split) slot j may keep a beam at the lane's receivers: the union of the
+// bands' cutoffs and the window, in plain FP32 with margins: u, s and n are within 1e-6 of rad and
+// of their own sizes, so n^2 is within 1e-3 of itself and 1e-9 rad^2 (al, be: see the caller).
+// The signs' outcome is shifted into m0, m1.
+template <int NF, int WINDOW, bool LOSSY>
+__device__ __forceinline__ void may_keep(const WarpBuf<NF, LOSSY> &w, int j, const LaneRecv &x, float scale,
+                                         float al, float be, float rad, uint32_t &m0, uint32_t &m1)
+{
+    f2x TX, TY, TZ, S, NX, NY, NZ, amp;
+    staged<false>(w.D[0], j, j, TX, TY);
+    staged<false>(w.D[1], j, j, TZ, S);
+    staged<false>(w.D[2], j, j, NX, NY);
+    staged<false>(w.D[3], j, j, NZ, amp);
+    const f2x u = fma2(x.X, TX, fma2(x.Y, TY, mul2(x.Z, TZ)));
+    const f2x s = fma2(u, splat(scale), S);
+    const f2x nx = fma2(x.Y, TZ, fma2(x.NZ, TY, NX));
+    const f2x ny = fma2(x.Z, TX, fma2(x.NX, TZ, NY));
+    const f2x nz = fma2(x.X, TY, fma2(x.NY, TX, NZ));
+    const f2x nn = fma2(nx, nx, fma2(ny, ny, mul2(nz, nz)));
+    float g0, g1, a0, a1;
+    upk(fma2(s, s, fma2(splat(-al), nn, splat(be))), g0, g1);
+    const float4 e = w.W[j];
+    upk(add2(u, splat(e.x + kWinMargin + 1e-6f * (fabsf(e.x) + rad))), a0, a1);
+    uint32_t b0 = ~(__float_as_uint(g0) | __float_as_uint(a0)), b1 = ~(__float_as_uint(g1) | __float_as_uint(a1));
+    if (WINDOW == GBT_WINDOW_SEGMENT) {
+        upk(add2(u, splat(e.z - kWinMargin - 1e-6f * (fabsf(e.z) + rad))), a0, a1);
+        b0 &= __float_as_uint(a0);
+        b1 &= __float_as_uint(a1);
+    }
+    m0 = __funnelshift_l(b0, m0, 1);
+    m1 = __funnelshift_l(b1, m1, 1);
+}
+
 // Slots of a staged batch: [0, n_plain) with a plain u, [n_plain, end) with the split one, and
 // which slots may have an end of their window inside the ball.
 struct StagedBatch {
     int n_plain, end;
     uint64_t cross;
+    uint32_t small;            // segments whose beam is small against the ball (kSmallBeam)
 };
 
 // Stages the batch's raw records (a lane each) in the frame c, for the 64 receivers within rad
 // of it: see WarpBuf.  A segment is split where the warp is not `fast` (one band, compact, every
 // x' one float) or an end of its window may lie inside the ball (a margin of 1 mm covers the
 // rounding of the float-float heads).
-template <int NF, int WINDOW, bool LOSSY, int NS, int NP>
+template <int NF, int WINDOW, bool LOSSY, int NS, int NP, bool UNORDERED>
 __device__ __forceinline__ StagedBatch stage(const FwdParams &p, WarpBuf<NF, LOSSY> &w, int lane,
                                              int nrec, int buf, int32_t seg, float cx, float cy,
                                              float cz, float rad, bool fast)
@@ -312,6 +375,12 @@ __device__ __forceinline__ StagedBatch stage(const FwdParams &p, WarpBuf<NF, LOS
     const uint32_t below = (1u << lane) - 1u;
     uint32_t plain = fast ? all & ~xm : 0u;
     StagedBatch b;
+    b.small = 0u;
+    if (UNORDERED) {
+        const float smax = fabsf(Sh) + rad;
+        b.small = __ballot_sync(0xffffffffu, have && fmaf(smax, smax, p.pre_beta) <
+                                                         kSmallBeam * kSmallBeam * p.pre_alpha * rad * rad);
+    }
     b.n_plain = __popc(plain) / NS * NS;
 #pragma unroll
     for (int q = 1; q < NS; ++q)
@@ -418,7 +487,7 @@ __device__ __noinline__ void stray_frame(const bool (&part)[kR], const float (&x
     }
 }
 
-template <int NF, int WINDOW, bool BATCHED, bool LOSSY>
+template <int NF, int WINDOW, bool BATCHED, bool LOSSY, bool UNORDERED = false>
 __global__ void __launch_bounds__(32 * PairCfg<WarpBuf<NF, LOSSY>, BATCHED, BATCHED ? PairShape<NF, LOSSY>::kWarpsBatched : PairShape<NF, LOSSY>::kWarps>::kWarps, 1) gbs_pair_kernel(const __grid_constant__ FwdParams prm)
 {
     using Cfg = PairCfg<WarpBuf<NF, LOSSY>, BATCHED, BATCHED ? PairShape<NF, LOSSY>::kWarpsBatched : PairShape<NF, LOSSY>::kWarps>;
@@ -550,6 +619,9 @@ __global__ void __launch_bounds__(32 * PairCfg<WarpBuf<NF, LOSSY>, BATCHED, BATC
             x.XH = pk(h[0][0], h[0][1]); x.YH = pk(h[1][0], h[1][1]); x.ZH = pk(h[2][0], h[2][1]);
             x.XL = pk(xl[0], xl[1]); x.YL = pk(yl[0], yl[1]); x.ZL = pk(zl[0], zl[1]);
         }
+        // the candidates' test in the units of the staged s, with its margins
+        const float al = 0.999f * p.pre_alpha * p.s_scale * p.s_scale;
+        const float be = fmaf(1.001e-9f * al, rad * rad, 1.001f * p.pre_beta * p.s_scale * p.s_scale);
         bool first = true;
         auto fold_all = [&]() { fold_bands<NF>(p, item, lane, part, ax, ay, first); };
 
@@ -561,15 +633,32 @@ __global__ void __launch_bounds__(32 * PairCfg<WarpBuf<NF, LOSSY>, BATCHED, BATC
             const int nrec = buf ? g.n1 : g.n0;
             if (nrec <= 0) break;
             cp_async_wait1();   // this lane's copies of batch kb
-            const StagedBatch b = stage<NF, WINDOW, LOSSY, NS, NP>(p, B, lane, nrec, buf, buf ? g.seg1 : g.seg0,
-                                                                   cx, cy, cz, rad, fast);
+            const StagedBatch b = stage<NF, WINDOW, LOSSY, NS, NP, UNORDERED>(
+                p, B, lane, nrec, buf, buf ? g.seg1 : g.seg0, cx, cy, cz, rad, fast);
             __syncwarp();       // the batch is staged
             g.issue(p, item, B.in, lane, rball, buf);   // batch kb + 2 into the buffer just read
             if (NF == 1)
                 for (int j = 0; j < b.n_plain; j += NS)
                     eval_segments<NF, WINDOW, LOSSY, false, NS, FG, BATCHED>(p, B, j, 0ull, x, ax, ay);
-            for (int j = b.n_plain; j < b.end; j += NP)
-                eval_segments<NF, WINDOW, LOSSY, true, NP, FG, BATCHED>(p, B, j, b.cross, x, ax, ay);
+            if (UNORDERED && !fast && 2 * __popc(b.small) > nrec) {
+                // small beams: each receiver's own candidates, in segment order
+                uint32_t m0 = 0u, m1 = 0u;      // slot j at bit 31 - j
+#pragma unroll 4
+                for (int j = 0; j < nrec; ++j)
+                    may_keep<NF, WINDOW, LOSSY>(B, j, x, p.s_scale, al, be, rad, m0, m1);
+                m0 = part[0] ? m0 << (32 - nrec) : 0u;
+                m1 = part[1] ? m1 << (32 - nrec) : 0u;
+                while (__any_sync(0xffffffffu, (m0 | m1) != 0u)) {
+                    const bool h0 = m0 != 0u, h1 = m1 != 0u;
+                    const int a = __clz(h0 ? m0 : h1 ? m1 : 0x80000000u), c = h1 ? __clz(m1) : a;
+                    eval_segments<NF, WINDOW, LOSSY, true, 1, 1, BATCHED, true>(p, B, a, 0ull, x, ax, ay, c, h0, h1);
+                    m0 &= ~(0x80000000u >> a);
+                    m1 &= ~(0x80000000u >> c);
+                }
+            } else {
+                for (int j = b.n_plain; j < b.end; j += NP)
+                    eval_segments<NF, WINDOW, LOSSY, true, NP, FG, BATCHED>(p, B, j, b.cross, x, ax, ay);
+            }
             // without a list every entry of a batch reaches the warp: twice as often
             const uint32_t every = item.lst ? kFoldEvery : kFoldEvery / 2;
             if (kb % every == every - 1) fold_all();

@@ -279,3 +279,37 @@ def test_forward_field_to_a_few_roundings(kind, n, rays, nf, uniform, window):
         for q, ref in ((p, po), (out, po + 1.0)):
             e = q.cpu().numpy().astype(np.complex128) - ref
             assert np.linalg.norm(e) <= 5e-6 * np.linalg.norm(ref), kw
+
+
+@pytest.mark.parametrize("n,nf,uniform,window,cutoff,lossy", [
+    (1, 1, True, I.WINDOW_SEGMENT, 16.0, False),
+    (63, 2, False, I.WINDOW_SEGMENT, 2.0, False),
+    (65, 3, True, I.WINDOW_LINE, 16.0, False),
+    (130, 6, False, I.WINDOW_SEGMENT, 16.0, False),
+    (961, 8, True, I.WINDOW_SEGMENT, 1e4, False),
+    (700, 8, False, I.WINDOW_LINE, 16.0, True),
+    (2000, 1, True, I.WINDOW_LINE, 0.5, True),
+    (1000, 11, True, I.WINDOW_SEGMENT, 16.0, True),
+])
+def test_receivers_without_an_order(n, nf, uniform, window, cutoff, lossy):
+    """Receivers in no order go through candidates of their own where beams are small against
+    their warp tile; the same receivers in the order given (the identity) do not.  Both against
+    the oracle to 5e-6 (see test_forward_field_to_a_few_roundings; the tiles are 250 m wide, where
+    n errs by 2^-24 of that), wide and narrow cutoffs, every band slot."""
+    import torch
+    from paper_2501_13382_gb300 import gbt as G
+    sc0, _ = I.city_scene(I.SEED_BASE + 3)
+    src = I.Source(np.array([0.3, -0.2, 3.0]), 900, 4, 600.0)
+    recv = _receivers("scatter", n, 11 + n)
+    freqs = list(250.0 * 2.0 ** (np.arange(nf) * (4.0 / max(nf - 1, 1))))
+    b = [40.0] * nf if uniform else [20.0 + 9.0 * f for f in range(nf)]
+    absorption = [1e-3 * (1 + f) for f in range(nf)] if lossy else None
+    ot = O.trace(sc0, src)
+    po = O.gbs_sum(ot, recv, freqs, b, sc0.c, sc0.gamma, window=window, cutoff=cutoff, absorption=absorption)
+    tr = G.Trace(G.Scene(sc0), src)
+    r = torch.as_tensor(recv, device="cuda")
+    gam = torch.as_tensor(sc0.gamma, device="cuda")
+    for order in (None, torch.arange(n, dtype=torch.int32, device="cuda")):
+        p = G.gbs_sum(tr, r, freqs, b, gam, order=order, window=window, cutoff=cutoff, absorption=absorption)
+        e = p.cpu().numpy().astype(np.complex128) - po
+        assert np.linalg.norm(e) <= 5e-6 * np.linalg.norm(po), order is None
