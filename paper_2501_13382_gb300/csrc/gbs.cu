@@ -1986,7 +1986,7 @@ FwdParams make_pair_params(const TraceDev &td, const SceneDev &sd, const gbt_sum
     q.cutoff = (float)a.cutoff;
     q.tile_cull = a.tile_cull ? 1 : 0;
     int perm[GBT_MAX_FREQ];
-    q.uniform_b = freq_order(a, perm) ? 1 : 0;
+    q.uniform_b = freq_order(a, perm) || q.nf == 1 ? 1 : 0;     // one band has one b (the ninth alone)
     double amin = 1e300, bmax = 0.0, kmax = 0.0;
     for (int f = 0; f < GBT_MAX_FREQ; ++f) q.fperm[f] = f;
     for (int f = 0; f < q.nf; ++f) {
@@ -2014,7 +2014,7 @@ FwdParams make_pair_params(const TraceDev &td, const SceneDev &sd, const gbt_sum
         kmax = std::max(kmax, K);
     }
     q.kmax_turns = (float)kmax;
-    q.s_scale = (q.uniform_b && !adjoint) ? (float)(1.0 / a.beam_b[0]) : 1.0f;
+    q.s_scale = (q.uniform_b && !adjoint) ? (float)(1.0 / a.beam_b[perm[g0]]) : 1.0f;
     q.pre_alpha = (float)(amin / (a.cutoff + 1.0));
     q.pre_beta = (float)bmax;
     q.status = status_word();

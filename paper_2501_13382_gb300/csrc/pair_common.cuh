@@ -46,7 +46,7 @@ struct alignas(16) FwdParams {
     const float *rec;          // AoS records, kRecFloats per segment
     const float4 *crec;        // cull records: (o_hi, s0_hi), (t_hi, L_hi) per segment
     int nf;
-    int uniform_b;             // all b equal: frequencies sorted by k, loop stops at first cull
+    int uniform_b;             // all b of the launch equal: frequencies sorted by k, loop stops at first cull
     int tile_cull;             // counting pass: skip segments that reach none of a warp's receivers
     float cutoff;
     float pre_alpha, pre_beta; // union cull: keep iff alpha n^2 <= s^2 + beta

@@ -313,3 +313,31 @@ def test_receivers_without_an_order(n, nf, uniform, window, cutoff, lossy):
         p = G.gbs_sum(tr, r, freqs, b, gam, order=order, window=window, cutoff=cutoff, absorption=absorption)
         e = p.cpu().numpy().astype(np.complex128) - po
         assert np.linalg.norm(e) <= 5e-6 * np.linalg.norm(po), order is None
+
+
+@pytest.mark.parametrize("nf", [7, 8, 9, 10, 15, 16])
+@pytest.mark.parametrize("uniform", [True, False])
+def test_every_band_of_every_group(nf, uniform):
+    """More than eight bands run as groups of at most eight, the last of which may hold one band:
+    each band by itself against the oracle, with equal and unequal beam parameters, with lists,
+    without an order, and differentiable.  5e-6 as for the forward field, per band."""
+    import torch
+    from paper_2501_13382_gb300 import gbt as G
+    sc0, _ = I.city_scene(I.SEED_BASE + 3)
+    src = I.Source(np.array([0.3, -0.2, 3.0]), 3000, 3, 500.0)
+    recv = _receivers("compact", 150, 3)
+    freqs = list(125.0 * 2.0 ** (np.arange(nf) * (4.0 / (nf - 1))))
+    b = [40.0] * nf if uniform else [100.0 / (1.0 + 0.3 * f) for f in range(nf)]
+    po = O.gbs_sum(O.trace(sc0, src), recv, freqs, b, sc0.c, sc0.gamma, window=I.WINDOW_SEGMENT)
+    tr = G.Trace(G.Scene(sc0), src)
+    r = torch.as_tensor(recv, device="cuda")
+    gam = torch.as_tensor(sc0.gamma, device="cuda")
+    o = G.recv_order(r)
+    for name, p in [("plain", G.gbs_sum(tr, r, freqs, b, gam, order=o, window=I.WINDOW_SEGMENT)),
+                    ("lists", G.gbs_sum(tr, r, freqs, b, gam, order=o, window=I.WINDOW_SEGMENT, tile_cull=True)),
+                    ("no order", G.gbs_sum(tr, r, freqs, b, gam, window=I.WINDOW_SEGMENT)),
+                    ("differentiable", G.gbs_sum_differentiable(tr, r, freqs, b, gam, order=o,
+                                                                window=I.WINDOW_SEGMENT))]:
+        e = p.cpu().numpy().astype(np.complex128) - po
+        rel = np.linalg.norm(e, axis=1) / np.linalg.norm(po, axis=1)
+        assert rel.max() <= 5e-6, (name, rel)
