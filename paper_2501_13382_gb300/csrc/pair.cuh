@@ -10,7 +10,7 @@
 //  * no list: the warp tests the 32-byte cull records of four chunks of 32 segments at a
 //    time against its ball.  About 35 instructions per 32 segments, where a test of every
 //    (receiver, segment) pair took 15 per segment.  That test comes back for receivers that
-//    have no order either (kSmallBeam).
+//    have no order either (small_beam).
 // Gathered records arrive by per-lane cp.async, double buffered, and each lane stages one.
 //
 // What bounds it: operand reads.  On this chip an FFMA2 with three operand pairs of its own
@@ -65,13 +65,16 @@ constexpr float kFastTurns = 16.0f;
 
 // Receivers without an order and without lists: a warp tile's 64 may lie anywhere, nearly every
 // segment reaches its ball and keeps a few of them.  A segment is small if its union cutoff radius
-// at the tile is under kSmallBeam times the ball's radius; where most of a batch are, may_keep marks
-// candidates and every receiver evaluates its own, a slot of its own to each lane and half.
-// 65,536-ray city x 10,000 scattered x 2 bands: every segment for all 64 5.38 ms, so 3.86; 8 bands
-// 10.0, 6.87 (line at 0.5: 8.6, at 1 to 1e6 the same); rows of a 200^2 grid 9.26, 6.15; rows of
-// the 256^2 open plane, 6 bands 4.93, 4.64.  The candidates' loop unrolled 1, 2, 4, 8 times: 8 bands
-// 7.03, 6.92, 6.87, 7.92.  Ordered receivers have kernels of their own without this (registers).
-constexpr float kSmallBeam = 1.0f;
+// at the tile is under small_beam() times the ball's radius; where most of a batch are, may_keep
+// marks candidates and every receiver evaluates its own, a slot of its own to each lane and half.
+// 65,536-ray city x 10,000 scattered x 2 bands: every segment for all 64 5.36 ms, so 3.85; 8 bands
+// 10.0, 6.87; rows of a 200^2 grid 9.26, 6.13; rows of the 256^2 open plane, 6 bands 4.91, 4.58.  Line
+// at 0.5, 1, 2, 4: 8 bands 8.62, 6.86, 6.87, 6.87, with a cutoff of 100 (23,296 rays x 17,737 x 5) -,
+// 10.43, 7.81, 7.84.  A few hundred ordered receivers (a CTA tile or less) take it too, as they may
+// be as far apart, with the line at 1: 56 over 1 km, one split 7.66, 3.01; 900 on 40 m, 6 bands .19,
+// .20 (.22 at 2).  The candidates' loop unrolled 1, 2, 4, 8 times: 8 bands 7.03, 6.92, 6.87, 7.92.
+// Other ordered receivers have kernels of their own without this (registers).
+__device__ __forceinline__ float small_beam(const FwdParams &p) { return p.order ? 1.0f : 2.0f; }
 
 // Shape by the number of band slots: segments evaluated together (plain, which only one band has,
 // and split), bands per vote, and warps.  One band needs several segments for independent
@@ -111,22 +114,6 @@ struct WarpBuf {
 struct LaneRecv {
     f2x X, Y, Z, NX, NY, NZ, XH, YH, ZH, XL, YL, ZL;
 };
-
-// A staged word's two values as float pairs: of slot j, or (EACH) of slot j for the lane's first
-// receiver and j1 for its second.
-template <bool EACH>
-__device__ __forceinline__ void staged(const float4 *w, int j, int j1, f2x &a, f2x &b)
-{
-    if (EACH) {
-        const float4 u = w[j], v = w[j1];
-        a = pk(u.x, v.x);
-        b = pk(u.z, v.z);
-    } else {
-        const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(w + j);
-        a = v.x;
-        b = v.y;
-    }
-}
 
 // Adds the beams of the staged slots j .. j + NS - 1 to the lane's two receivers' sums per
 // band.  `cross`: slots with an end of their window inside the warp tile's ball.  EACH: of a slot
@@ -320,7 +307,7 @@ __device__ __forceinline__ void may_keep(const WarpBuf<NF, LOSSY> &w, int j, con
 struct StagedBatch {
     int n_plain, end;
     uint64_t cross;
-    uint32_t small;            // segments whose beam is small against the ball (kSmallBeam)
+    uint32_t small;            // segments whose beam is small against the ball (small_beam)
 };
 
 // Stages the batch's raw records (a lane each) in the frame c, for the 64 receivers within rad
@@ -378,8 +365,8 @@ __device__ __forceinline__ StagedBatch stage(const FwdParams &p, WarpBuf<NF, LOS
     b.small = 0u;
     if (UNORDERED) {
         const float smax = fabsf(Sh) + rad;
-        b.small = __ballot_sync(0xffffffffu, have && fmaf(smax, smax, p.pre_beta) <
-                                                         kSmallBeam * kSmallBeam * p.pre_alpha * rad * rad);
+        const float line = small_beam(p) * rad;
+        b.small = __ballot_sync(0xffffffffu, have && fmaf(smax, smax, p.pre_beta) < p.pre_alpha * line * line);
     }
     b.n_plain = __popc(plain) / NS * NS;
 #pragma unroll

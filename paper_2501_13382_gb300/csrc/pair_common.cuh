@@ -91,7 +91,7 @@ static_assert(sizeof(FwdParams) % 16 == 0, "instance parameters are copied as 16
 
 // Launchers of the pair kernel (pair_fwd.cu, pair_bwd.cu, pair_batched.cu).
 void pair_fwd_launch(const FwdParams &p, int window, cudaStream_t s, bool timed);
-void pair_unordered_launch(const FwdParams &p, int window, cudaStream_t s, bool timed);   // no order, no lists
+void pair_unordered_launch(const FwdParams &p, int window, cudaStream_t s, bool timed);   // no lists, no order or few
 void pair_bwd_launch(const FwdParams &p, int window, cudaStream_t s, bool timed);
 void pair_field_launch(const FwdParams &p, int window, cudaStream_t s, bool timed);   // its forward
 int pair_batched_prepare(int nf_max, int window);                  // resident CTAs per SM

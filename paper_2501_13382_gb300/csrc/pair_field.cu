@@ -25,6 +25,10 @@ constexpr float kFastTurnsField = 90.0f;   // K max|x'| up to which u is plain F
 // rays x 4,000 scattered receivers x 4 bands with the line at 0.7, 1, 2, 100: 9.18, 8.54, 8.43,
 // 8.42 ms; x 64^2 receivers on a grid 3.92, 3.89, 3.89, 3.89.
 constexpr float kSmallBeam = 2.0f;
+// Receivers without an order and without lists: where most of a batch's segments are small, every
+// receiver evaluates its own candidates, a segment of its own to each lane and half (30,000-ray
+// city x 4,000 scattered x 4 bands 1.50 ms with one segment for the warp, 1.10 so; the same bits).
+// A kernel of its own, since its registers cost the others.
 
 template <int NF>
 struct FieldBuf {
@@ -137,49 +141,44 @@ __device__ __forceinline__ bool stage_field(const FwdParams &p, FieldBuf<NF> &w,
 //   s_loc = x'.t - o'.t,  sm = s_loc + s0 + margin,
 //   g = sm^2 + beta - alpha |x' - o'|^2 + alpha s_loc^2  (= q - alpha n^2) >= 0, window.
 template <int NF, int WINDOW>
-__device__ __forceinline__ bool may_keep(const FieldBuf<NF> &w, int j, const FieldRecv &x, f2x NAXX,
-                                         f2x AL2, bool v0, bool v1)
+__device__ __forceinline__ void may_keep(const FieldBuf<NF> &w, int j, const FieldRecv &x, f2x NAXX,
+                                         f2x AL2, bool &k0, bool &k1)
 {
-    auto word = [](const float4 &v, f2x &a, f2x &b) {
-        const ulonglong2 q = *reinterpret_cast<const ulonglong2 *>(&v);
-        a = q.x;
-        b = q.y;
-    };
     f2x TX, TY, TZ, OT, OX, OY, OZ, C7, S0, LM;
-    word(w.D[0][j], TX, TY);
-    word(w.P[0][j], TZ, OT);
-    word(w.P[1][j], OX, OY);
-    word(w.P[2][j], OZ, C7);
-    word(w.P[3][j], S0, LM);
+    staged<false>(w.D[0], j, j, TX, TY);
+    staged<false>(w.P[0], j, j, TZ, OT);
+    staged<false>(w.P[1], j, j, OX, OY);
+    staged<false>(w.P[2], j, j, OZ, C7);
+    staged<false>(w.P[3], j, j, S0, LM);
     const f2x sl = fma2(x.X, TX, fma2(x.Y, TY, fma2(x.Z, TZ, OT)));
     const f2x sm = add2(sl, S0);
     const f2x nd = fma2(x.X, OX, fma2(x.Y, OY, fma2(x.Z, OZ, add2(NAXX, C7))));
     const f2x g = fma2(mul2(sl, AL2), sl, fma2(sm, sm, nd));
     float g0, g1, a0, a1;
     upk(g, g0, g1);
-    bool k0 = v0 && g0 >= 0.f, k1 = v1 && g1 >= 0.f;
+    k0 = g0 >= 0.f;
+    k1 = g1 >= 0.f;
     if (WINDOW == GBT_WINDOW_LINE) {
         upk(sm, a0, a1);
-        return (k0 && a0 >= 0.f) || (k1 && a1 >= 0.f);
+        k0 = k0 && a0 >= 0.f;
+        k1 = k1 && a1 >= 0.f;
+        return;
     }
     float b0, b1;
     upk(add2(sl, splat(kWinMargin)), a0, a1);
     upk(sub2(sl, LM), b0, b1);
-    return (k0 && a0 >= 0.f && b0 < 0.f) || (k1 && a1 >= 0.f && b1 < 0.f);
+    k0 = k0 && a0 >= 0.f && b0 < 0.f;
+    k1 = k1 && a1 >= 0.f && b1 < 0.f;
 }
 
-// Exact geometry of the staged segment j and the lane's two receivers: s = (s + sl), n^2, and
-// which receivers (of v0, v1) lie in the window.
-template <int NF, int WINDOW>
-__device__ __forceinline__ void field_geometry(const FieldBuf<NF> &w, int j, const FieldRecv &x, bool v0,
-                                             bool v1, bool fast, float eps, f2x &s, f2x &sl, f2x &n2,
+// Exact geometry of the staged segment j (EACH: and j1 for the second) and the lane's two
+// receivers: s = (s + sl), n^2, and which receivers (of v0, v1) lie in the window.
+template <int NF, int WINDOW, bool EACH>
+__device__ __forceinline__ void field_geometry(const FieldBuf<NF> &w, int j, int j1, const FieldRecv &x,
+                                             bool v0, bool v1, bool fast, float eps, f2x &s, f2x &sl, f2x &n2,
                                              f2x &amp, bool &k0, bool &k1)
 {
-    auto word = [&](int d, f2x &a, f2x &b) {
-        const ulonglong2 q = *reinterpret_cast<const ulonglong2 *>(&w.D[d][j]);
-        a = q.x;
-        b = q.y;
-    };
+    auto word = [&](int d, f2x &a, f2x &b) { staged<EACH>(w.D[d], j, j1, a, b); };
     f2x TX, TY, TZ, S, TLX, TLY, TLZ, SL, NX, NY, NZ, AH, AL, BH, BL;
     word(0, TX, TY);
     word(1, TZ, S);
@@ -285,15 +284,16 @@ __device__ __forceinline__ void sincos_turns(f2x tau, f2x &sn, f2x &cs)
     cs = pk(cs0, cs1);
 }
 
-// Adds the beams of the staged segment j to the lane's receivers' sums per band.
-template <int NF, int WINDOW, bool LOSSY>
-__device__ __forceinline__ void eval_field(const FwdParams &p, const FieldBuf<NF> &w, int j,
+// Adds the beams of the staged segment j (EACH: and j1 for the second) to the lane's receivers'
+// sums per band.
+template <int NF, int WINDOW, bool LOSSY, bool EACH>
+__device__ __forceinline__ void eval_field(const FwdParams &p, const FieldBuf<NF> &w, int j, int j1,
                                            const FieldRecv &x, bool v0, bool v1, bool fast, float eps,
                                            f2x (&ax)[NF], f2x (&ay)[NF])
 {
     f2x s, sl, n2, amp;
     bool k0, k1;
-    field_geometry<NF, WINDOW>(w, j, x, v0, v1, fast, eps, s, sl, n2, amp, k0, k1);
+    field_geometry<NF, WINDOW, EACH>(w, j, j1, x, v0, v1, fast, eps, s, sl, n2, amp, k0, k1);
     f2x invD, n2invD;
     float d0 = 1.f, d1 = 1.f, n20, n21, r0 = 0.f, r1 = 0.f;
     upk(n2, n20, n21);
@@ -315,9 +315,9 @@ __device__ __forceinline__ void eval_field(const FwdParams &p, const FieldBuf<NF
         }
         f2x ex = mul2(splat(c.ne), n2invD), RPH = 0ull;
         if (LOSSY) {
-            const float2 r = w.rf[f][j];
-            ex = fma2(splat(c.nal), s, add2(ex, splat(r.x)));
-            RPH = splat(r.y);
+            const float2 ra = w.rf[f][j], rb = EACH ? w.rf[f][j1] : ra;
+            ex = fma2(splat(c.nal), s, add2(ex, pk(ra.x, rb.x)));
+            RPH = pk(ra.y, rb.y);
         }
         float e0, e1;
         upk(ex, e0, e1);
@@ -332,7 +332,7 @@ __device__ __forceinline__ void eval_field(const FwdParams &p, const FieldBuf<NF
 
 // The FP32 sums fold into the item's float-float partials every kFoldEvery batches of list
 // entries, or without a list every kFoldEvery chunks of all segments.
-template <int NF, int WINDOW, bool LOSSY>
+template <int NF, int WINDOW, bool LOSSY, bool UNORDERED>
 __global__ void __maxnreg__(128) gbs_field_kernel(const __grid_constant__ FwdParams p)
 {
     using Cfg = PairCfg<FieldBuf<NF>, false>;
@@ -436,16 +436,37 @@ __global__ void __maxnreg__(128) gbs_field_kernel(const __grid_constant__ FwdPar
             g.issue(p, item, B.in, lane, rball, buf);   // batch kb + 2 into the buffer just read
 
             const uint32_t all = nrec < 32 ? (1u << nrec) - 1u : 0xffffffffu;
-            uint32_t mine = 0u;
-            for (uint32_t T = smask; T; T &= T - 1u) {
-                const int j = __ffs(T) - 1;
-                if (may_keep<NF, WINDOW>(B, j, x, NAXX, AL2, part[0], part[1])) mine |= 1u << j;
-            }
-            uint32_t T = (all & ~smask) | __reduce_or_sync(0xffffffffu, mine);
-            while (T) {
-                const int j = __ffs(T) - 1;
-                T &= T - 1u;
-                eval_field<NF, WINDOW, LOSSY>(p, B, j, x, part[0], part[1], fast, eps, ax, ay);
+            if (UNORDERED && 2 * __popc(smask) > nrec) {
+                // each receiver's own, in segment order
+                uint32_t m0 = part[0] ? all & ~smask : 0u, m1 = part[1] ? all & ~smask : 0u;
+                for (uint32_t T = smask; T; T &= T - 1u) {
+                    const int j = __ffs(T) - 1;
+                    bool k0, k1;
+                    may_keep<NF, WINDOW>(B, j, x, NAXX, AL2, k0, k1);
+                    m0 |= (uint32_t)(part[0] && k0) << j;
+                    m1 |= (uint32_t)(part[1] && k1) << j;
+                }
+                while (__any_sync(0xffffffffu, (m0 | m1) != 0u)) {
+                    const bool h0 = m0 != 0u, h1 = m1 != 0u;
+                    const int a = h0 ? __ffs(m0) - 1 : h1 ? __ffs(m1) - 1 : 0, c = h1 ? __ffs(m1) - 1 : a;
+                    eval_field<NF, WINDOW, LOSSY, true>(p, B, a, c, x, h0, h1, fast, eps, ax, ay);
+                    m0 &= m0 - 1u;
+                    m1 &= m1 - 1u;
+                }
+            } else {
+                uint32_t mine = 0u;
+                for (uint32_t T = smask; T; T &= T - 1u) {
+                    const int j = __ffs(T) - 1;
+                    bool k0, k1;
+                    may_keep<NF, WINDOW>(B, j, x, NAXX, AL2, k0, k1);
+                    if ((part[0] && k0) || (part[1] && k1)) mine |= 1u << j;
+                }
+                uint32_t T = (all & ~smask) | __reduce_or_sync(0xffffffffu, mine);
+                while (T) {
+                    const int j = __ffs(T) - 1;
+                    T &= T - 1u;
+                    eval_field<NF, WINDOW, LOSSY, false>(p, B, j, j, x, part[0], part[1], fast, eps, ax, ay);
+                }
             }
             __syncwarp();        // before the next batch is staged over this one
         }
@@ -457,8 +478,11 @@ __global__ void __maxnreg__(128) gbs_field_kernel(const __grid_constant__ FwdPar
 template <int NF, int WINDOW, bool LOSSY>
 void launch(const FwdParams &p, cudaStream_t s, bool timed)
 {
-    static std::atomic<int> known[64] = {};
-    launch_items<PairCfg<FieldBuf<NF>, false>>(gbs_field_kernel<NF, WINDOW, LOSSY>, known, p, s, timed);
+    static std::atomic<int> known[2][64] = {};
+    if (!p.order && !p.list)
+        launch_items<PairCfg<FieldBuf<NF>, false>>(gbs_field_kernel<NF, WINDOW, LOSSY, true>, known[1], p, s, timed);
+    else
+        launch_items<PairCfg<FieldBuf<NF>, false>>(gbs_field_kernel<NF, WINDOW, LOSSY, false>, known[0], p, s, timed);
 }
 
 // Frequency slots: 1, 2, 4, 6 (lossless) and 8.

@@ -32,7 +32,7 @@ void launch_nf(const FwdParams &p, cudaStream_t s, bool timed)
 
 void pair_fwd_launch(const FwdParams &p, int window, cudaStream_t s, bool timed)
 {
-    if (!p.order && !p.list) pair_unordered_launch(p, window, s, timed);
+    if ((!p.order || p.n_recv <= kCtaRecv) && !p.list) pair_unordered_launch(p, window, s, timed);
     else if (window == GBT_WINDOW_LINE) launch_nf<GBT_WINDOW_LINE>(p, s, timed);
     else launch_nf<GBT_WINDOW_SEGMENT>(p, s, timed);
 }

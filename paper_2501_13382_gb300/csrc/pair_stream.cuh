@@ -185,6 +185,22 @@ struct Gather {
     }
 };
 
+// A staged word's two values as float pairs: of slot j, or (EACH) of slot j for the lane's first
+// receiver and j1 for its second.
+template <bool EACH>
+__device__ __forceinline__ void staged(const float4 *w, int j, int j1, f2x &a, f2x &b)
+{
+    if (EACH) {
+        const float4 u = w[j], v = w[j1];
+        a = pk(u.x, v.x);
+        b = pk(u.z, v.z);
+    } else {
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(w + j);
+        a = v.x;
+        b = v.y;
+    }
+}
+
 // Adds an FP32 partial sum (x, y) into a float-float accumulator (hi, hi, lo, lo); the
 // item's first fold only writes it.
 __device__ __forceinline__ void fold(float4 *acc, float x, float y, bool first)

@@ -1,5 +1,5 @@
-// pair_unordered.cu -- instantiations of the pair kernel for receivers without an order and
-// without lists (see kSmallBeam).
+// pair_unordered.cu -- instantiations of the pair kernel for receivers without an order, or few
+// of them, and without lists (see small_beam).
 #include "pair.cuh"
 
 namespace gbt {

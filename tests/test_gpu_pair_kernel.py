@@ -341,3 +341,19 @@ def test_every_band_of_every_group(nf, uniform):
         e = p.cpu().numpy().astype(np.complex128) - po
         rel = np.linalg.norm(e, axis=1) / np.linalg.norm(po, axis=1)
         assert rel.max() <= 5e-6, (name, rel)
+
+
+@pytest.mark.parametrize("n,nf,window", [(65, 1, I.WINDOW_SEGMENT), (700, 3, I.WINDOW_LINE), (1500, 8, I.WINDOW_SEGMENT)])
+def test_differentiable_sum_is_the_same_without_an_order(n, nf, window):
+    """Without an order the differentiable sum gives each receiver its own candidates; given the
+    identity as an order it does not.  The same terms in the same order: the same bits."""
+    import torch
+    from paper_2501_13382_gb300 import gbt as G
+    sc0, _ = I.city_scene(I.SEED_BASE + 3)
+    tr = G.Trace(G.Scene(sc0), I.Source(np.array([0.3, -0.2, 3.0]), 1500, 4, 600.0))
+    r = torch.as_tensor(_receivers("scatter", n, 2), device="cuda")
+    gam = torch.as_tensor(sc0.gamma, device="cuda")
+    freqs = list(500.0 * 2.0 ** (np.arange(nf) / 2.0))
+    a, b = (G.gbs_sum_differentiable(tr, r, freqs, [30.0] * nf, gam, order=o, window=window)
+            for o in (None, torch.arange(n, dtype=torch.int32, device="cuda")))
+    assert torch.equal(torch.view_as_real(a), torch.view_as_real(b))
