@@ -15,7 +15,7 @@ method (the pre-cull skips only pairs that provably contribute nothing).  L2 is 
 
 Prints one JSON line (rank 0).  Under torchrun each rank runs its own replica of the
 workload (weak scaling, no collective on the data path).  On the default workload the
-line also carries `forms` (rank 0, outside the timed steps): the city testing every pair;
+line also carries `forms` (rank 0, outside the timed steps): the city without lists;
 the large open plane (65,536 rays, 256^2 receivers, 6 bands) with and without the
 pre-cull and on the all-FP64 GPU path; the small open plane; the 32-source batched city
 at 512^2 receivers against one launch per source and per (source, frequency); the
@@ -55,8 +55,17 @@ LANES_PER_SM_CLK = 128          # FP32 lanes per SM per clock (4 SMSPs x 32)
 # Revision of the pair kernel's source.  DRAM bytes (read + write) per launch of the
 # dominant kernel come from an ncu capture of one revision, instantiation and workload;
 # a changed kernel gets a new revision and no entry until it is captured again.
-KERNEL_REV = "rev11"
-KERNEL_TRAFFIC = {}
+KERNEL_REV = "rev12"
+KERNEL_TRAFFIC = {
+    ("gbs_pair_kernel<1,SEGMENT> tile segment lists [rev12]",
+     "city_1M_rays_512x512_1kHz"): 4990984704,
+    ("gbs_pair_kernel<1,SEGMENT> no lists [rev12]",
+     "city_1M_rays_512x512_1kHz"): 23497542144,
+    ("gbs_pair_kernel<6,LINE> tile segment lists [rev12]",
+     "open_plane_64k_rays_256x256_6f"): 149987840,
+    ("gbs_pair_kernel<6,LINE> no lists [rev12]",
+     "open_plane_64k_rays_256x256_6f"): 194871808,
+}
 WORKLOADS = ("city", "open_plane_large", "open_plane_small", "diff_city", "big_city")
 
 
@@ -610,7 +619,7 @@ def main():
     ap.add_argument("--no-e2e", action="store_true", help="skip the host-buffer end-to-end loop")
     ap.add_argument("--workload", default="city", choices=WORKLOADS)
     ap.add_argument("--cull", default="tile", choices=["tile", "none"],
-                    help="tile: the exact tile pre-cull (default); none: test every pair")
+                    help="tile: the exact tile pre-cull (default); none: no lists")
     ap.add_argument("--rays", type=int, default=0,
                     help="city only: rays of the fan (default 1,048,576; smaller for profiling)")
     ap.add_argument("--recv-side", type=int, default=0,

@@ -293,7 +293,8 @@ typedef struct gbt_sum_args {
                                      every 960 receivers; 0: the same skip tested by each
                                      warp on its own (no lists: less memory, and less work
                                      on small sums) */
-    int64_t max_device_bytes;     /* gbt_solve only: device budget for one chunk; 0 = auto */
+    int64_t max_device_bytes;     /* gbt_solve only: device budget for one chunk (the FP64
+                                     sum's partials keep to an eighth of it); 0 = auto */
     double absorption[GBT_MAX_FREQ]; /* air's amplitude decay rate per frequency, Np/m
                                      (>= 0; all 0 = lossless air) */
     const float *flow_resistivity; /* device, n_materials effective flow resistivities,

@@ -50,8 +50,8 @@
 // every 16, 8, 4 batches 1.42e-7, 1.36e-7, 1.32e-7 and 2.08, 2.08, 2.14 ms), merged in split
 // order by reduce_kernel, so results do not depend on scheduling.
 // Measured (kernel alone, with float-float pairs -> now): city, 1,048,576 rays x 512^2
-// receivers, lists: 31.0 -> 15.8 ms; open plane, 65,536 rays x 256^2 x 6 bands, no lists:
-// 6.06 -> 2.01 ms; city, 65,536 rays x 200^2 x 2 bands, no lists: 6.79 -> 1.51 ms.
+// receivers, lists: 31.0 -> 15.6 ms; open plane, 65,536 rays x 256^2 x 6 bands, no lists:
+// 6.06 -> 1.93 ms; city, 65,536 rays x 200^2 x 2 bands, no lists: 6.79 -> 1.49 ms.
 #pragma once
 
 #include "pair_stream.cuh"
